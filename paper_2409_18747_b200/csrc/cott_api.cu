@@ -176,9 +176,13 @@ static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv
             if (g8 <= 4096 && (N + g8 - 1) / g8 == 8) group = g8;
         }
     } else {
-        p->chunk = 16;
+        p->chunk = 32;
         group = 1024;
         while (group > 128 && BH * ((N + group - 1) / group) < 4 * 148) group >>= 1;
+        // Short sequences of few heads: groups down to one chunk, as long as they do not yet give two
+        // CTAs per SM and the group states stay small (2 MiB).
+        while (group > 32 && BH * ((N + group - 1) / group) < 2 * 148 &&
+               BH * ((N + group / 2 - 1) / (group / 2)) * d * d * 4 <= (2L << 20)) group >>= 1;
     }
     if (forced > 0) group = (forced + p->chunk - 1) / p->chunk * p->chunk;
     if (group >= N) group = (N + p->chunk - 1) / p->chunk * p->chunk;
@@ -323,29 +327,70 @@ static WalkArgs base_walk(const cott_scale_params* sp, int H, int N, const Plan&
     return w;
 }
 
-// One gradient / output stream through the generic walk: (optional) per-group partial
-// states, their scan, then the walk that produces rows.
-static cott_status run_stream(WalkArgs w, const Plan& p, int BH, int d, cott_dtype dt, int causal,
-                              float* states, float* total_out, cudaStream_t st,
-                              const float* state_in = nullptr) {
-    const bool single = causal && p.n_groups == 1 && !state_in;
-    if (single) {
-        w.init = nullptr; w.update = 1; w.write_out = 1;
-        w.final_state = total_out; w.final_grouped = 0;
-        COTT_CUDA(launch_walk_simt(w, BH, d, dt, st));
+// The running-sum streams of one call (one for a forward, the three gradients for a backward)
+// through the fp32-accumulating walk, side by side in each launch: (optional) per-group partial
+// states, their sum, then the walks that produce rows.
+struct SimtStream {
+    WalkArgs w;
+    float* states;             // [BH, n_groups, d, d]
+    const float* state_in;     // caller's initial state or NULL
+    float* total_out;          // receives the sum over everything, or NULL
+    int sibling;               // >= 0: this stream's partial states are the transposes of that stream's
+};
+
+static cott_status run_streams(const SimtStream* s, int n, const Plan& p, int BH, int d, cott_dtype dt, int causal,
+                               int* status, cudaStream_t st) {
+    WalkBatch wb;
+    memset(&wb, 0, sizeof(wb));
+    wb.status = status;
+    bool wants_dm = false;
+    for (int i = 0; i < n; ++i) wants_dm |= s[i].w.dm_partial != nullptr;
+    if (causal && p.n_groups == 1) {
+        for (int i = 0; i < n; ++i) {
+            wb.w[i] = s[i].w;
+            wb.w[i].init_extra = s[i].state_in; wb.w[i].update = 1; wb.w[i].write_out = 1;
+            wb.w[i].final_state = s[i].total_out;
+        }
+        if (wants_dm) COTT_CUDA(cudaMemsetAsync(status, 0, kWsHeaderBytes, st));   // (the CTA counter of dm)
+        wb.clear_status = wants_dm ? 0 : 1;
+        COTT_CUDA(launch_walk_simt(wb, n, BH, d, dt, st, false));
         return COTT_OK;
     }
-    WalkArgs a = w;  // phase A: partial state of every group, no rows
-    a.init = nullptr; a.update = 1; a.write_out = 0; a.out = nullptr; a.proj = nullptr;
-    a.epilogue = EPI_PLAIN; a.dm_partial = nullptr;
-    a.final_state = states; a.final_grouped = 1;
-    COTT_CUDA(launch_walk_simt(a, BH, d, dt, st));
-    const int mode = !causal ? SCAN_TOTAL : (w.reverse ? SCAN_SUFFIX : SCAN_PREFIX);
-    // (these states contain c, like a caller's initial state, which the scan starts from)
-    COTT_CUDA(launch_scan(states, total_out, BH, p.n_groups, d, mode, st, nullptr, nullptr, 0.f, 1, 1,
-                          state_in));
-    w.init = states; w.update = causal ? 1 : 0; w.write_out = 1; w.final_state = nullptr;
-    COTT_CUDA(launch_walk_simt(w, BH, d, dt, st));
+    // Every walk CTA sums the partial states before its group itself while they are few: at most
+    // 16 states of d x d floats out of L2 (measured at d = 64, 16 groups: the sums add 2 us to the walk,
+    // a scan launch takes 4 us and the gap in front of it).
+    const bool in_walk = p.n_groups <= 16;
+    int n_a = 0;
+    for (int i = 0; i < n; ++i) {      // phase A: partial state of every group, no rows
+        if (s[i].sibling >= 0) continue;
+        WalkArgs a = s[i].w;
+        a.update = 1; a.write_out = 0; a.out = nullptr; a.proj = nullptr;
+        a.epilogue = EPI_PLAIN; a.dm_partial = nullptr; a.dm_out = nullptr;
+        a.final_state = s[i].states; a.final_grouped = 1;
+        wb.w[n_a++] = a;
+    }
+    wb.clear_status = 1;
+    COTT_CUDA(launch_walk_simt(wb, n_a, BH, d, dt, st, false));
+    wb.clear_status = 0;
+    if (!in_walk)
+        for (int i = 0; i < n; ++i) {
+            if (s[i].sibling >= 0) continue;
+            const int mode = !causal ? SCAN_TOTAL : (s[i].w.reverse ? SCAN_SUFFIX : SCAN_PREFIX);
+            // (these states contain c, like a caller's initial state, which the scan starts from)
+            COTT_CUDA(launch_scan(s[i].states, s[i].total_out, BH, p.n_groups, d, mode, st, nullptr, nullptr, 0.f, 1, 1,
+                                  s[i].state_in));
+        }
+    for (int i = 0; i < n; ++i) {
+        WalkArgs w = s[i].w;
+        w.update = causal ? 1 : 0; w.write_out = 1;
+        w.init = s[i].sibling >= 0 ? s[s[i].sibling].states : s[i].states;
+        w.init_transposed = s[i].sibling >= 0 ? 1 : 0;
+        w.init_sum = in_walk ? 1 : 0;
+        w.init_extra = in_walk ? s[i].state_in : nullptr;
+        w.final_state = in_walk ? s[i].total_out : nullptr;
+        wb.w[i] = w;
+    }
+    COTT_CUDA(launch_walk_simt(wb, n, BH, d, dt, st, in_walk));
     return COTT_OK;
 }
 
@@ -440,8 +485,6 @@ static cott_status fwd_impl(const void* q, const void* k, const void* v, void* o
     CallLayouts lay{to_layout(s_qkv), to_layout(s_o), RowLayout{0, 0, 0}, q, k, v, o};
     lay.dk = p.dk; lay.dv = p.dv;
     if (p.dk != p.dv || s_v) { lay.own_v = true; lay.vl = to_layout(s_v); }
-    // The tensor-core path clears the status words in its first kernel.
-    if (p.path != 1) COTT_CUDA(cudaMemsetAsync(ws, 0, kWsHeaderBytes, st));
     float* states = reinterpret_cast<float*>(static_cast<char*>(ws) + kWsHeaderBytes);
     // Zero-padded head sizes: the kernels read and write states of their own size.
     float* user_state_out = state_out;
@@ -503,7 +546,8 @@ static cott_status fwd_impl(const void* q, const void* k, const void* v, void* o
     lay.assign(w);
     w.mode_x = ROW_NORM; w.mode_a = ROW_NORM; w.mode_b = ROW_SCALE;
     w.epilogue = EPI_PLAIN; w.reverse = 0;
-    return run_stream(w, p, B * H, d, dt, causal, states, state_out, st, state_in);
+    const SimtStream s{w, states, state_in, state_out, -1};
+    return run_streams(&s, 1, p, B * H, d, dt, causal, static_cast<int*>(ws), st);
 }
 
 // Side streams and events for launches of one call that run next to each other on the GPU:
@@ -559,8 +603,6 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
     CallLayouts lay{to_layout(s_qkv), to_layout(s_do), to_layout(s_dqkv), q, k, v, d_o};
     lay.dk = p.dk; lay.dv = p.dv; lay.dv_ptr = dv;
     if (p.dk != p.dv || s_v || s_dv) { lay.own_v = true; lay.vl = to_layout(s_v); lay.dvl = to_layout(s_dv); }
-    // The tensor-core path clears the status words in its first kernel.
-    if (p.path != 1) COTT_CUDA(cudaMemsetAsync(ws, 0, kWsHeaderBytes, st));
     char* base = static_cast<char*>(ws) + kWsHeaderBytes;
     const size_t sb = states_bytes(p, B, H, d);
     float* st0 = reinterpret_cast<float*>(base);
@@ -798,6 +840,7 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
         }
         seg_total = seg.d_state_in;
     }
+    SimtStream s[3];
     {   // dQ^_t = S_t dO_t : the forward walk with (dO, V', K^) in the roles of (Q, K, V)
         WalkArgs w = base_walk(sp, H, N, p);
         w.x = d_o; w.a = v; w.bv = k; w.proj = q; w.out = dq;
@@ -805,7 +848,7 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
         lay.assign(w);
         w.mode_x = ROW_RAW; w.mode_a = ROW_SCALE; w.mode_b = ROW_NORM;
         w.epilogue = EPI_PROJ; w.reverse = 0;
-        if ((rc = run_stream(w, p, BH, d, dt, causal, st0, nullptr, st, seg_q)) != COTT_OK) return rc;
+        s[0] = SimtStream{w, st0, seg_q, nullptr, -1};
     }
     {   // dK^_j = R_j v'_j : running sum of dO_t q^_t^T accumulated backward in time
         WalkArgs w = base_walk(sp, H, N, p);
@@ -814,20 +857,20 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
         lay.assign(w);
         w.mode_x = ROW_SCALE; w.mode_a = ROW_RAW; w.mode_b = ROW_NORM;
         w.epilogue = EPI_PROJ; w.reverse = 1;
-        if ((rc = run_stream(w, p, BH, d, dt, causal, st1, nullptr, st, seg_k)) != COTT_OK) return rc;
+        s[1] = SimtStream{w, st1, seg_k, nullptr, -1};
     }
-    {   // dV'_j = R_j^T k^_j, dV = c dV', and <dV', V> for dm
+    {   // dV'_j = R_j^T k^_j, dV = c dV', and <dV', V> for dm.  Its running sum is the transpose of
+        // the dK^ stream's, in the same direction of time: without a segment's states around it,
+        // that stream's partial states serve both.
         WalkArgs w = base_walk(sp, H, N, p);
         w.x = k; w.a = q; w.bv = d_o; w.proj = v; w.out = dv;
         w.cu_seqlens = packed.cu_seqlens;
         lay.assign(w);
         w.mode_x = ROW_NORM; w.mode_a = ROW_NORM; w.mode_b = ROW_RAW;
-        w.epilogue = EPI_DV; w.reverse = 1; w.dm_partial = dm_partial;
-        if ((rc = run_stream(w, p, BH, d, dt, causal, st2, seg_total, st, seg_v)) != COTT_OK) return rc;
+        w.epilogue = EPI_DV; w.reverse = 1; w.dm_partial = dm_partial; w.dm_out = dm;
+        s[2] = SimtStream{w, st2, seg_v, seg_total, seg.on ? -1 : 1};
     }
-    COTT_CUDA(launch_dm_finalize(dm_partial, dm, sp->m, sp->seq_len, sp->seq_len_scalar, B, H,
-                                 p.n_groups, N, st, packed.cu_seqlens));
-    return COTT_OK;
+    return run_streams(s, 3, p, BH, d, dt, causal, static_cast<int*>(ws), st);
 }
 
 }  // namespace cott

@@ -46,10 +46,15 @@ struct WalkArgs {
     const void* x; const void* a; const void* bv; const void* proj;
     void* out;
     RowLayout lx, la, lbv, lproj, lout;   // layouts of the five tensors (all zero: dense)
-    const float* init;   // [BH, n_groups, d*d] or NULL (zero initial state)
-    float* final_state;  // NULL, or [BH, n_groups, d*d] (final_grouped) / [BH, d*d] (one group)
+    // Initial state: init_extra ([BH, d*d] or NULL, a caller's) plus what `init` ([BH, n_groups, d*d]
+    // or NULL) holds for the group -- its own entry when a scan launch has been over it, the sum of
+    // the partial states before it when init_sum is set (all of them without update).
+    const float* init; const float* init_extra;
+    int init_sum; int init_transposed;   // init_transposed: the entries of `init` are transposes
+    float* final_state;  // NULL, or [BH, n_groups, d*d] (final_grouped) / [BH, d*d] (the total)
     int final_grouped;
     float* dm_partial;   // [BH, n_groups] or NULL
+    float* dm_out;       // dm[H], written by the last CTA of the stream that has dm_partial
     const float* m; const float* seq_len; float seq_len_scalar;
     int H; int N; int group; int n_groups;
     int mode_x, mode_a, mode_b;
@@ -59,7 +64,16 @@ struct WalkArgs {
     const int* cu_seqlens;
 };
 
-cudaError_t launch_walk_simt(const WalkArgs& w, int BH, int d, cott_dtype dt, cudaStream_t st);
+// Streams that run in one launch: the walks of one call, all over the same groups.
+struct WalkBatch {
+    WalkArgs w[3];
+    int* status;         // the workspace's status words (word 4 counts CTAs for dm)
+    int clear_status;    // 1: the first kernel of a call
+};
+
+// `dependent`: may start while the previous kernel of the stream drains (it reads nothing before
+// that one has finished).
+cudaError_t launch_walk_simt(const WalkBatch& wb, int n, int BH, int d, cott_dtype dt, cudaStream_t st, bool dependent);
 // `total_scale_m` non-NULL: the total written to total_out is multiplied by the stabilisation
 // factor c[b,h] (the tensor-core path keeps its states unscaled).
 cudaError_t launch_scan(float* states, float* total_out, int BH, int n_groups, int d, int mode,

@@ -2,6 +2,7 @@
 // states, the dm reduction and the recurrent decode step.  These serve fp32 I/O (tensor
 // cores in TF32 cannot meet the fp32 tolerance) and every shape the tensor-core kernels do
 // not cover.
+#include <initializer_list>
 #include "cott_internal.h"
 
 namespace cott {
@@ -9,20 +10,17 @@ namespace cott {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kTile = 16;  // tokens staged per shared-memory tile
+constexpr int kChunk = 32;  // tokens per chunk of the walk
 
-template <typename T> __device__ __forceinline__ void load4(const T* p, float (&f)[4]);
-template <> __device__ __forceinline__ void load4<float>(const float* p, float (&f)[4]) {
-    float4 v = *reinterpret_cast<const float4*>(p);
-    f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
+template <typename T> __device__ __forceinline__ float4 load4(const T* p);
+template <> __device__ __forceinline__ float4 load4<float>(const float* p) {
+    return *reinterpret_cast<const float4*>(p);
 }
-template <> __device__ __forceinline__ void load4<__nv_bfloat16>(const __nv_bfloat16* p,
-                                                                 float (&f)[4]) {
+template <> __device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16* p) {
     uint2 v = *reinterpret_cast<const uint2*>(p);
-    __nv_bfloat162 lo = *reinterpret_cast<__nv_bfloat162*>(&v.x);
-    __nv_bfloat162 hi = *reinterpret_cast<__nv_bfloat162*>(&v.y);
-    f[0] = __low2float(lo); f[1] = __high2float(lo);
-    f[2] = __low2float(hi); f[3] = __high2float(hi);
+    const float2 lo = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&v.x));
+    const float2 hi = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&v.y));
+    return make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 template <typename T> __device__ __forceinline__ float to_f32(T v);
 template <> __device__ __forceinline__ float to_f32<float>(float v) { return v; }
@@ -34,14 +32,13 @@ template <> __device__ __forceinline__ float from_f32<float>(float v) { return v
 template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float v) {
     return __float2bfloat16_rn(v);
 }
-template <typename T> __device__ __forceinline__ void store4(T* p, const float (&f)[4]);
-template <> __device__ __forceinline__ void store4<float>(float* p, const float (&f)[4]) {
-    *reinterpret_cast<float4*>(p) = make_float4(f[0], f[1], f[2], f[3]);
+template <typename T> __device__ __forceinline__ void store4(T* p, float4 f);
+template <> __device__ __forceinline__ void store4<float>(float* p, float4 f) {
+    *reinterpret_cast<float4*>(p) = f;
 }
-template <> __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* p,
-                                                                  const float (&f)[4]) {
-    __nv_bfloat162 lo = __floats2bfloat162_rn(f[0], f[1]);
-    __nv_bfloat162 hi = __floats2bfloat162_rn(f[2], f[3]);
+template <> __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* p, float4 f) {
+    __nv_bfloat162 lo = __floats2bfloat162_rn(f.x, f.y);
+    __nv_bfloat162 hi = __floats2bfloat162_rn(f.z, f.w);
     uint2 v;
     v.x = *reinterpret_cast<uint32_t*>(&lo);
     v.y = *reinterpret_cast<uint32_t*>(&hi);
@@ -54,166 +51,277 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Stage rows [t0, t0+kTile) of one (b,h) slice (rows `sn` elements apart) as fp32; rows outside
-// [lo,hi) become zero.
-template <int D, typename T>
-__device__ __forceinline__ void stage_tile(float (*dst)[D], const T* src, long long sn, int t0, int lo,
-                                           int hi, int tid) {
-    constexpr int V4 = D / 4;
-    for (int i = tid; i < kTile * V4; i += kThreads) {
-        int r = i / V4, c4 = i % V4;
-        int t = t0 + r;
-        float f[4] = {0.f, 0.f, 0.f, 0.f};
-        if (t >= lo && t < hi) load4<T>(src + (size_t)t * sn + c4 * 4, f);
-        *reinterpret_cast<float4*>(&dst[r][c4 * 4]) = make_float4(f[0], f[1], f[2], f[3]);
-    }
+__device__ __forceinline__ float dot4(float4 a, float4 b) {
+    return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w)));
+}
+__device__ __forceinline__ void axpy4(float4& y, float a, float4 x) {
+    y.x = fmaf(a, x.x, y.x); y.y = fmaf(a, x.y, y.y); y.z = fmaf(a, x.z, y.z); y.w = fmaf(a, x.w, y.w);
 }
 
-// Apply the row treatment to a staged tile: one warp per row.
-template <int D>
-__device__ __forceinline__ void treat_rows(float (*tile)[D], int mode, float c, int warp,
-                                           int lane) {
-    if (mode == ROW_RAW) return;
-    for (int r = warp; r < kTile; r += kThreads / 32) {
-        float scale = c;
-        if (mode == ROW_NORM) {
-            float ss = 0.f;
-            for (int e = lane; e < D; e += 32) ss += tile[r][e] * tile[r][e];
-            ss = warp_sum(ss);
-            scale = 1.0f / fmaxf(sqrtf(ss), kEps);
-        }
-        for (int e = lane; e < D; e += 32) tile[r][e] *= scale;
-    }
-}
+// Shared memory of the walk: three chunk tiles (rows padded by four words: threads that read 16
+// consecutive rows at the same column then hit different banks), the chunk's masked scores and
+// the state.
+template <int D> struct WalkSmem {
+    static constexpr int kRow = D + 4, kScoreRow = kChunk + 4;
+    static constexpr int kX = 0, kA = kX + kChunk * kRow, kB = kA + kChunk * kRow;
+    static constexpr int kP = kB + kChunk * kRow, kS = kP + kChunk * kScoreRow;
+    static constexpr int kBytes = (kS + D * D) * 4;
+};
 
+// One pass of the running-sum walk (WalkArgs) over one sequence group, 32 tokens at a time:
+//     P = X A^T, masked to the pairs the running sum holds (Eq. 6) ;  Out = P Bv + X S ;  S += A^T Bv
+// in fp32 multiply-adds throughout.  What bounds it is the multiply-add rate (per token 2 * 32 * d
+// for the scores side, 2 d^2 for the state side), and for the small problems this path serves the
+// chain of launches and the fill of the SMs; the token-by-token recurrence it replaces was one
+// serial chain (0.35 us a token) on the same SMs.  32 tokens a chunk: a 64-token chunk does 1.3
+// times the multiply-adds at d = 64 and halves the number of CTAs a short sequence gives.
+// Measured, forward and backward at B=2, H=8, N=509, d=64: 303 us and 13 launches with the
+// recurrence, 88 us and 4 launches (state pass and walk each way) here.
+// Thread (ty, tx) owns columns 4 tx .. + 3 everywhere: rows ty, ty + TY, .. of the chunk (it loads,
+// normalises and produces them; the TX threads of a row sit in one warp, so row sums are
+// shuffles) and rows SR ty .. + SR - 1 of the state, which stays in its registers and is copied
+// to shared memory once per chunk.  The next chunk's rows are loaded while this one is computed.
+// blockIdx.y picks one of up to three streams (the three gradients of a backward call).
 template <int D, typename T>
-__global__ void __launch_bounds__(kThreads) walk_kernel(WalkArgs w) {
-    constexpr int NSPLIT = kThreads / D;  // threads sharing one state column
-    constexpr int AR = D / NSPLIT;        // state rows owned by one thread
-    __shared__ __align__(16) float xs[kTile][D];
-    __shared__ __align__(16) float as[kTile][D];
-    __shared__ __align__(16) float bs[kTile][D];
-    __shared__ __align__(16) float part[kTile][NSPLIT][D];
+__global__ void __launch_bounds__(kThreads) walk_kernel(const __grid_constant__ WalkBatch batch) {
+    using M = WalkSmem<D>;
+    constexpr int TX = D / 4, TY = kThreads / TX;
+    constexpr int RPT = kChunk / TY;      // chunk rows per thread
+    constexpr int SR = D / TY;            // state rows per thread
+    extern __shared__ __align__(16) float sm[];
     __shared__ float dm_red[kThreads / 32];
+    __shared__ int last_flag;
+    const WalkArgs& w = batch.w[blockIdx.y];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tx = tid % TX, ty = tid / TX;
     const int g = blockIdx.x % w.n_groups;
     const int bh = blockIdx.x / w.n_groups;
     const int b = bh / w.H, h = bh % w.H;
+    // (the walk of a call may start while its state pass drains)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!w.write_out) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (batch.clear_status && blockIdx.x == 0 && blockIdx.y == 0 && tid < 8) batch.status[tid] = 0;
     // (a packed batch: the rows of sequence b, one group)
     const int lo = w.cu_seqlens ? w.cu_seqlens[b] : g * w.group;
     const int hi = w.cu_seqlens ? w.cu_seqlens[b + 1] : min(w.N, lo + w.group);
     // (the launcher has resolved the layouts: strides are never all zero here)
     auto slice = [&](const RowLayout& l) { return (w.cu_seqlens ? (size_t)0 : (size_t)b * l.sb) + (size_t)h * l.sh; };
-    const T* X = static_cast<const T*>(w.x) + slice(w.lx);
+    const bool write_out = w.write_out, update = w.update;
+    const T* X = write_out ? static_cast<const T*>(w.x) + slice(w.lx) : nullptr;
     const T* A = static_cast<const T*>(w.a) + slice(w.la);
     const T* Bv = static_cast<const T*>(w.bv) + slice(w.lbv);
     const T* P = w.proj ? static_cast<const T*>(w.proj) + slice(w.lproj) : nullptr;
-    T* O = w.out ? static_cast<T*>(w.out) + slice(w.lout) : nullptr;
+    T* O = write_out ? static_cast<T*>(w.out) + slice(w.lout) : nullptr;
 
     const float s_b = w.seq_len ? w.seq_len[b]
                                 : (w.seq_len_scalar > 0.f ? w.seq_len_scalar
                                                           : (float)(w.cu_seqlens ? max(hi - lo, 1) : w.N));
     const float c = stab_factor(w.m[h], s_b);
 
-    const int col = tid % D, split = tid / D, a0 = split * AR;
-    float S[AR];
+    const int n_chunks = (hi - lo + kChunk - 1) / kChunk;
+    auto chunk_row = [&](int it) { return lo + (w.reverse ? n_chunks - 1 - it : it) * kChunk; };
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto load_rows = [&](float4 (&r)[RPT], const T* src, long long sn, int t0) {
+#pragma unroll
+        for (int u = 0; u < RPT; ++u) {
+            const int t = t0 + ty + TY * u;
+            r[u] = t < hi ? load4<T>(src + (long long)t * sn + tx * 4) : zero4;
+        }
+    };
+    float4 rx[RPT], ra[RPT], rb[RPT];
+    auto load_chunk = [&](int t0) {
+        if (write_out) load_rows(rx, X, w.lx.sn, t0);
+        if (update) { load_rows(ra, A, w.la.sn, t0); load_rows(rb, Bv, w.lbv.sn, t0); }
+    };
+    if (n_chunks > 0) load_chunk(chunk_row(0));
+
+    // The state before this group's first chunk: the sum of the partial states before it in the
+    // walk's direction of time (all of them when the mask is all ones), or what a scan launch has
+    // left in the group's own place.
+    float4 S[SR];
+#pragma unroll
+    for (int r = 0; r < SR; ++r) S[r] = zero4;
+    bool have_state = false;
+    auto add_state = [&](const float* src, bool transposed) {
+        have_state = true;
+        if (!transposed) {
+#pragma unroll
+            for (int r = 0; r < SR; ++r) {
+                const float4 v = *reinterpret_cast<const float4*>(src + (size_t)(ty * SR + r) * D + tx * 4);
+                S[r].x += v.x; S[r].y += v.y; S[r].z += v.z; S[r].w += v.w;
+            }
+        } else {
+            const float* s0 = src + (size_t)(tx * 4) * D + ty * SR;
+#pragma unroll
+            for (int r = 0; r < SR; ++r) {
+                S[r].x += s0[r]; S[r].y += s0[D + r]; S[r].z += s0[2 * D + r]; S[r].w += s0[3 * D + r];
+            }
+        }
+    };
+    if (w.init_extra) add_state(w.init_extra + (size_t)bh * D * D, false);
     if (w.init) {
-        const float* src = w.init + ((size_t)bh * w.n_groups + g) * D * D;
-#pragma unroll
-        for (int i = 0; i < AR; ++i) S[i] = src[(size_t)(a0 + i) * D + col];
-    } else {
-#pragma unroll
-        for (int i = 0; i < AR; ++i) S[i] = 0.f;
+        const float* part = w.init + (size_t)bh * w.n_groups * D * D;
+        if (w.init_sum) {
+            const int g0 = (w.reverse && update) ? g + 1 : 0, g1 = (w.reverse || !update) ? w.n_groups : g;
+            for (int gg = g0; gg < g1; ++gg) add_state(part + (size_t)gg * D * D, w.init_transposed);
+        } else {
+            add_state(part + (size_t)g * D * D, w.init_transposed);
+        }
     }
+    auto put_state = [&]() {
+#pragma unroll
+        for (int r = 0; r < SR; ++r) *reinterpret_cast<float4*>(sm + M::kS + (ty * SR + r) * D + tx * 4) = S[r];
+    };
+    if (write_out && have_state) put_state();
+
+    // Row treatment of a loaded row piece: scale by c, or by 1 / max(||row||, eps).
+    auto treat = [&](float4& v, int mode) {
+        float s = 1.f;
+        if (mode == ROW_SCALE) s = c;
+        if (mode == ROW_NORM) {
+            float ss = dot4(v, v);
+#pragma unroll
+            for (int o = TX / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+            s = 1.0f / fmaxf(sqrtf(ss), kEps);
+        }
+        if (mode != ROW_RAW) { v.x *= s; v.y *= s; v.z *= s; v.w *= s; }
+    };
+    auto put_rows = [&](float4 (&r)[RPT], int off, int mode) {
+#pragma unroll
+        for (int u = 0; u < RPT; ++u) {
+            treat(r[u], mode);
+            *reinterpret_cast<float4*>(sm + off + (ty + TY * u) * M::kRow + tx * 4) = r[u];
+        }
+    };
 
     float dm_acc = 0.f;
-    const int n_tiles = (hi - lo + kTile - 1) / kTile;
-    for (int it = 0; it < n_tiles; ++it) {
-        const int tile_idx = w.reverse ? (n_tiles - 1 - it) : it;
-        const int t0 = lo + tile_idx * kTile;
-        __syncthreads();  // previous tile fully consumed
-        stage_tile<D, T>(xs, X, w.lx.sn, t0, lo, hi, tid);
-        stage_tile<D, T>(as, A, w.la.sn, t0, lo, hi, tid);
-        stage_tile<D, T>(bs, Bv, w.lbv.sn, t0, lo, hi, tid);
+    for (int it = 0; it < n_chunks; ++it) {
+        const int t0 = chunk_row(it);
+        if (write_out) put_rows(rx, M::kX, w.mode_x);
+        if (update) { put_rows(ra, M::kA, w.mode_a); put_rows(rb, M::kB, w.mode_b); }
         __syncthreads();
-        treat_rows<D>(xs, w.mode_x, c, warp, lane);
-        treat_rows<D>(as, w.mode_a, c, warp, lane);
-        treat_rows<D>(bs, w.mode_b, c, warp, lane);
-        __syncthreads();
+        float4 rp[RPT];
+        if (w.epilogue != EPI_PLAIN) load_rows(rp, P, w.lproj.sn, t0);
+        if (it + 1 < n_chunks) load_chunk(chunk_row(it + 1));
 
-        for (int s = 0; s < kTile; ++s) {
-            const int tt = w.reverse ? (kTile - 1 - s) : s;
-            const float bval = bs[tt][col];
-            float acc = 0.f;
-            if (w.update) {
+        float4 out[RPT];
+        if (write_out) {
+            if (update) {
+                // scores: rows pi, pi + 16 against keys pj, pj + 16
+                const int pi = tid >> 4, pj = tid & 15;
+                float4 acc[2][2];
 #pragma unroll
-                for (int i = 0; i < AR; i += 4) {
-                    float4 av = *reinterpret_cast<const float4*>(&as[tt][a0 + i]);
-                    S[i] += av.x * bval; S[i + 1] += av.y * bval;
-                    S[i + 2] += av.z * bval; S[i + 3] += av.w * bval;
+                for (int u = 0; u < 2; ++u) { acc[u][0] = zero4; acc[u][1] = zero4; }
+#pragma unroll 4
+                for (int k = 0; k < D; k += 4) {
+                    const float4 x0 = *reinterpret_cast<const float4*>(sm + M::kX + pi * M::kRow + k);
+                    const float4 x1 = *reinterpret_cast<const float4*>(sm + M::kX + (pi + 16) * M::kRow + k);
+                    const float4 a0 = *reinterpret_cast<const float4*>(sm + M::kA + pj * M::kRow + k);
+                    const float4 a1 = *reinterpret_cast<const float4*>(sm + M::kA + (pj + 16) * M::kRow + k);
+                    auto fma4 = [](float4& d, float4 p, float4 q) {
+                        d.x = fmaf(p.x, q.x, d.x); d.y = fmaf(p.y, q.y, d.y);
+                        d.z = fmaf(p.z, q.z, d.z); d.w = fmaf(p.w, q.w, d.w);
+                    };
+                    fma4(acc[0][0], x0, a0); fma4(acc[0][1], x0, a1); fma4(acc[1][0], x1, a0); fma4(acc[1][1], x1, a1);
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) {
+                        const int i = pi + 16 * u, j = pj + 16 * v;
+                        const bool keep = w.reverse ? j >= i : j <= i;
+                        const float4 s = acc[u][v];
+                        sm[M::kP + i * M::kScoreRow + j] = keep ? (s.x + s.y) + (s.z + s.w) : 0.f;
+                    }
+            }
+#pragma unroll
+            for (int u = 0; u < RPT; ++u) out[u] = zero4;
+            if (have_state) {
+#pragma unroll 4
+                for (int k = 0; k < D; k += 4) {
+                    float4 x[RPT];
+#pragma unroll
+                    for (int u = 0; u < RPT; ++u) x[u] = *reinterpret_cast<const float4*>(sm + M::kX + (ty + TY * u) * M::kRow + k);
+                    const float* s0 = sm + M::kS + k * D + tx * 4;
+                    const float4 v0 = *reinterpret_cast<const float4*>(s0), v1 = *reinterpret_cast<const float4*>(s0 + D);
+                    const float4 v2 = *reinterpret_cast<const float4*>(s0 + 2 * D), v3 = *reinterpret_cast<const float4*>(s0 + 3 * D);
+#pragma unroll
+                    for (int u = 0; u < RPT; ++u) {
+                        axpy4(out[u], x[u].x, v0); axpy4(out[u], x[u].y, v1); axpy4(out[u], x[u].z, v2); axpy4(out[u], x[u].w, v3);
+                    }
                 }
             }
-            if (w.write_out) {
+            if (update) {
+                __syncthreads();
+#pragma unroll 2
+                for (int k = 0; k < kChunk; k += 4) {
+                    float4 x[RPT];
 #pragma unroll
-                for (int i = 0; i < AR; i += 4) {
-                    float4 xv = *reinterpret_cast<const float4*>(&xs[tt][a0 + i]);
-                    acc += xv.x * S[i]; acc += xv.y * S[i + 1];
-                    acc += xv.z * S[i + 2]; acc += xv.w * S[i + 3];
+                    for (int u = 0; u < RPT; ++u)
+                        x[u] = *reinterpret_cast<const float4*>(sm + M::kP + (ty + TY * u) * M::kScoreRow + k);
+                    const float* b0 = sm + M::kB + k * M::kRow + tx * 4;
+                    const float4 v0 = *reinterpret_cast<const float4*>(b0), v1 = *reinterpret_cast<const float4*>(b0 + M::kRow);
+                    const float4 v2 = *reinterpret_cast<const float4*>(b0 + 2 * M::kRow), v3 = *reinterpret_cast<const float4*>(b0 + 3 * M::kRow);
+#pragma unroll
+                    for (int u = 0; u < RPT; ++u) {
+                        axpy4(out[u], x[u].x, v0); axpy4(out[u], x[u].y, v1); axpy4(out[u], x[u].z, v2); axpy4(out[u], x[u].w, v3);
+                    }
                 }
-                part[tt][split][col] = acc;
+            }
+#pragma unroll
+            for (int u = 0; u < RPT; ++u) {
+                const int t = t0 + ty + TY * u;
+                if (w.epilogue == EPI_PROJ) {
+                    // dx = (dx^ - x^ <x^, dx^>) / ||x||, or dx^ / eps on the clamped branch
+                    float ss = dot4(rp[u], rp[u]), dp = dot4(rp[u], out[u]);
+#pragma unroll
+                    for (int o = TX / 2; o > 0; o >>= 1) {
+                        ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                        dp += __shfl_xor_sync(0xffffffffu, dp, o);
+                    }
+                    const float nrm = sqrtf(ss);
+                    const float rinv = 1.0f / fmaxf(nrm, kEps);
+                    const float coef = nrm > kEps ? dp * rinv * rinv : 0.f;  // <x^,dx^> * rinv
+                    out[u].x = (out[u].x - rp[u].x * coef) * rinv; out[u].y = (out[u].y - rp[u].y * coef) * rinv;
+                    out[u].z = (out[u].z - rp[u].z * coef) * rinv; out[u].w = (out[u].w - rp[u].w * coef) * rinv;
+                } else if (w.epilogue == EPI_DV) {
+                    dm_acc += dot4(rp[u], out[u]);  // (rows past the end are zero)
+                    out[u].x *= c; out[u].y *= c; out[u].z *= c; out[u].w *= c;
+                }
+                if (t < hi) store4<T>(O + (long long)t * w.lout.sn + tx * 4, out[u]);
             }
         }
-        if (!w.write_out) continue;
+        if (update) {
+            have_state = true;
+#pragma unroll 4
+            for (int k = 0; k < kChunk; ++k) {
+                const float4 v = *reinterpret_cast<const float4*>(sm + M::kB + k * M::kRow + tx * 4);
+                const float* ap = sm + M::kA + k * M::kRow + ty * SR;
+                if constexpr (SR >= 4) {
+#pragma unroll
+                    for (int r = 0; r < SR; r += 4) {
+                        const float4 a = *reinterpret_cast<const float4*>(ap + r);
+                        axpy4(S[r], a.x, v); axpy4(S[r + 1], a.y, v); axpy4(S[r + 2], a.z, v); axpy4(S[r + 3], a.w, v);
+                    }
+                } else {
+#pragma unroll
+                    for (int r = 0; r < SR; ++r) axpy4(S[r], ap[r], v);
+                }
+            }
+            // (every read of the previous copy came before this chunk's second barrier)
+            if (write_out && it + 1 < n_chunks) put_state();
+        }
         __syncthreads();
-        // Sum the partial read-outs of the NSPLIT thread groups into part[.][0][.].
-        for (int i = tid; i < kTile * D; i += kThreads) {
-            int r = i / D, e = i % D;
-            float v = part[r][0][e];
-#pragma unroll
-            for (int sp = 1; sp < NSPLIT; ++sp) v += part[r][sp][e];
-            part[r][0][e] = v;
-        }
-        if (w.epilogue != EPI_PLAIN) stage_tile<D, T>(xs, P, w.lproj.sn, t0, lo, hi, tid);  // xs is dead now
-        __syncthreads();
-        // Epilogue: one warp per row.
-        for (int r = warp; r < kTile; r += kThreads / 32) {
-            const int t = t0 + r;
-            if (t >= hi) continue;
-            float* row = part[r][0];
-            if (w.epilogue == EPI_PROJ) {
-                // dx = (dx^ - x^ <x^, dx^>) / ||x||, or dx^ / eps on the clamped branch
-                float ss = 0.f, dp = 0.f;
-                for (int e = lane; e < D; e += 32) {
-                    ss += xs[r][e] * xs[r][e];
-                    dp += xs[r][e] * row[e];
-                }
-                ss = warp_sum(ss); dp = warp_sum(dp);
-                const float nrm = sqrtf(ss);
-                const float rinv = 1.0f / fmaxf(nrm, kEps);
-                const float coef = nrm > kEps ? dp * rinv * rinv : 0.f;  // <x^,dx^> * rinv
-                for (int e = lane; e < D; e += 32) row[e] = (row[e] - xs[r][e] * coef) * rinv;
-            } else if (w.epilogue == EPI_DV) {
-                float dp = 0.f;
-                for (int e = lane; e < D; e += 32) {
-                    dp += xs[r][e] * row[e];
-                    row[e] *= c;
-                }
-                dm_acc += dp;  // per-lane partial; summed over the warp at the end
-            }
-            __syncwarp();
-            for (int e4 = lane; e4 < D / 4; e4 += 32) {
-                float f[4] = {row[e4 * 4], row[e4 * 4 + 1], row[e4 * 4 + 2], row[e4 * 4 + 3]};
-                store4<T>(O + (size_t)t * w.lout.sn + e4 * 4, f);
-            }
-        }
     }
 
-    if (w.final_state) {
-        float* dst = w.final_state +
-                     (w.final_grouped ? ((size_t)bh * w.n_groups + g) : (size_t)bh) * D * D;
+    // The group's partial state, or the total where this group is the last one the walk visits.
+    if (w.final_state && (w.final_grouped || w.n_groups == 1 || !update || g == (w.reverse ? 0 : w.n_groups - 1))) {
+        float* dst = w.final_state + (w.final_grouped ? ((size_t)bh * w.n_groups + g) : (size_t)bh) * D * D;
+        if (w.final_grouped || update || g == 0) {
 #pragma unroll
-        for (int i = 0; i < AR; ++i) dst[(size_t)(a0 + i) * D + col] = S[i];
+            for (int r = 0; r < SR; ++r) *reinterpret_cast<float4*>(dst + (size_t)(ty * SR + r) * D + tx * 4) = S[r];
+        }
     }
     if (w.dm_partial) {
         dm_acc = warp_sum(dm_acc);
@@ -223,6 +331,30 @@ __global__ void __launch_bounds__(kThreads) walk_kernel(WalkArgs w) {
             float t = 0.f;
             for (int i = 0; i < kThreads / 32; ++i) t += dm_red[i];
             w.dm_partial[(size_t)bh * w.n_groups + g] = t;
+            __threadfence();
+            last_flag = atomicAdd(&batch.status[4], 1) == (int)gridDim.x - 1;
+        }
+        __syncthreads();
+        if (last_flag) {
+            // dm_h = sum_b dc/dm * <dV', V>_{b,h},  dc/dm = -ln(s_b) sigma(m_h)(1-sigma(m_h)) c_{b,h}.
+            // Fixed summation order (deterministic); one warp per head.
+            __threadfence();
+            const int n_b = (int)gridDim.x / (w.n_groups * w.H), per = n_b * w.n_groups;
+            for (int hh = warp; hh < w.H; hh += kThreads / 32) {
+                const float sg = 1.0f / (1.0f + expf(-w.m[hh]));
+                float sum = 0.f;
+                for (int i = lane; i < per; i += 32) {
+                    const int bb = i / w.n_groups, gg = i - bb * w.n_groups;
+                    const float sb2 = w.seq_len ? w.seq_len[bb]
+                                                : (w.seq_len_scalar > 0.f ? w.seq_len_scalar
+                                                   : (float)(w.cu_seqlens ? max(w.cu_seqlens[bb + 1] - w.cu_seqlens[bb], 1) : w.N));
+                    const float ls = logf(sb2);
+                    sum += __ldcg(&w.dm_partial[((size_t)bb * w.H + hh) * w.n_groups + gg]) * (-ls * sg * (1.0f - sg) * expf(-sg * ls));
+                }
+                sum = warp_sum(sum);
+                if (lane == 0) w.dm_out[hh] = sum;
+            }
+            if (tid == 0) batch.status[4] = 0;
         }
     }
 }
@@ -377,17 +509,33 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const T* q, const T* k
     }
 }
 
+template <int D, typename T>
+cudaError_t launch_walk_dt(const WalkBatch& wb, int n, int BH, cudaStream_t st, bool dependent) {
+    if (cudaError_t e = configure_smem_once(reinterpret_cast<const void*>(walk_kernel<D, T>), WalkSmem<D>::kBytes); e != cudaSuccess)
+        return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(BH * wb.w[0].n_groups), (unsigned)n);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = WalkSmem<D>::kBytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, walk_kernel<D, T>, wb);
+    note_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <typename T>
-cudaError_t launch_walk_t(const WalkArgs& w, int BH, int d, cudaStream_t st) {
-    dim3 grid((unsigned)(BH * w.n_groups));
+cudaError_t launch_walk_t(const WalkBatch& wb, int n, int BH, int d, cudaStream_t st, bool dependent) {
     switch (d) {
-        case 32: walk_kernel<32, T><<<grid, kThreads, 0, st>>>(w); break;
-        case 64: walk_kernel<64, T><<<grid, kThreads, 0, st>>>(w); break;
-        case 128: walk_kernel<128, T><<<grid, kThreads, 0, st>>>(w); break;
+        case 32: return launch_walk_dt<32, T>(wb, n, BH, st, dependent);
+        case 64: return launch_walk_dt<64, T>(wb, n, BH, st, dependent);
+        case 128: return launch_walk_dt<128, T>(wb, n, BH, st, dependent);
         default: return cudaErrorInvalidValue;
     }
-    note_launch();
-    return cudaGetLastError();
 }
 
 template <typename T>
@@ -409,13 +557,14 @@ cudaError_t launch_decode_t(const void* q, const void* k, const void* v, float* 
 
 }  // namespace
 
-cudaError_t launch_walk_simt(const WalkArgs& w0, int BH, int d, cott_dtype dt, cudaStream_t st) {
-    WalkArgs w = w0;   // resolve "all zero = dense [B,H,N,d]" once, on the host
-    w.lx = resolve_layout(w0.lx, w0.H, w0.N, d); w.la = resolve_layout(w0.la, w0.H, w0.N, d);
-    w.lbv = resolve_layout(w0.lbv, w0.H, w0.N, d); w.lproj = resolve_layout(w0.lproj, w0.H, w0.N, d);
-    w.lout = resolve_layout(w0.lout, w0.H, w0.N, d);
-    return dt == COTT_F32 ? launch_walk_t<float>(w, BH, d, st)
-                          : launch_walk_t<__nv_bfloat16>(w, BH, d, st);
+cudaError_t launch_walk_simt(const WalkBatch& wb0, int n, int BH, int d, cott_dtype dt, cudaStream_t st, bool dependent) {
+    WalkBatch wb = wb0;   // resolve "all zero = dense [B,H,N,d]" once, on the host
+    for (int i = 0; i < n; ++i) {
+        WalkArgs& w = wb.w[i];
+        for (RowLayout* l : {&w.lx, &w.la, &w.lbv, &w.lproj, &w.lout}) *l = resolve_layout(*l, w.H, w.N, d);
+    }
+    return dt == COTT_F32 ? launch_walk_t<float>(wb, n, BH, d, st, dependent)
+                          : launch_walk_t<__nv_bfloat16>(wb, n, BH, d, st, dependent);
 }
 
 cudaError_t launch_scan(float* states, float* total_out, int BH, int n_groups, int d, int mode,

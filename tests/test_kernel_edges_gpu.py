@@ -1,0 +1,44 @@
+"""GPU parity at the sizes where a kernel or a branch of its dispatch can go wrong: edges of its
+tiles, remainders, the smallest and the largest of its range.  Oracle, metrics and gates are those
+of test_parity_gpu.py."""
+import pytest
+import torch
+
+import oracle
+import paper_2409_18747_b200 as cott
+from paper_2409_18747_b200 import synth
+from test_parity_gpu import (DM_COND_F32, TOL_STATE_F32, dev, dm_condition, force_group, gate, gate_dm, option)  # noqa: F401
+from _metrics import norm_max_err
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d", [32, 64, 128])
+@pytest.mark.parametrize("N,group", [(1, 0), (31, 0), (33, 32), (64, 32), (97, 0), (500, 32), (545, 32), (300, 4096)])
+@pytest.mark.parametrize("causal", [True, False])
+def test_fp32_walk_chunk_and_group_edges(d, N, group, causal, force_group):
+    """The fp32 walk (32 tokens a chunk): single rows, one row short of and one past a chunk, 16 groups
+    (each walk sums the partial states before its own), 18 groups (a scan launch does), one group."""
+    force_group(group)
+    B, H = 2, 3
+    c = synth.make_qkv(B, H, N, d, torch.float32, 7100 + N + d, row_lognormal=True, with_do=True)
+    args = [dev(c[x]) for x in ("q", "k", "v")]
+    o, st = cott.fwd(*args, dev(c["m"]), causal=causal, return_state=True)
+    ref_o = oracle.fwd_quadratic(c["q"], c["k"], c["v"], c["m"], None, causal)
+    _, ref_state = oracle.fwd_bidir_assoc(c["q"], c["k"], c["v"], c["m"], None)
+    assert norm_max_err(st, ref_state) <= TOL_STATE_F32
+    dq, dk, dv, dm = cott.bwd(*args, dev(c["d_o"]), dev(c["m"]), causal=causal)
+    rq, rk, rv, rm = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, causal)
+    if N > 1:
+        for x, r in ((o, ref_o), (dq, rq), (dk, rk), (dv, rv)):
+            gate(x, r, torch.float32)
+        gate_dm(dm, rm, 1e-4, dm_condition(rv, c["v"], c["m"], None), DM_COND_F32)
+        return
+    # One token (c = 1, dm = 0): every row is one dot product of unit or raw rows times a row, and
+    # where that dot product cancels the relative error has no bound.  Absolute: a dot product of d
+    # terms is off by at most (d + 8) u |x| |y| (u = 2^-24, the norms and scalings included), and dq,
+    # dk go through two of them and a division by the row's norm.
+    u = (d + 8) * 2.0 ** -24
+    nq, nk, nv, nd = (c[x].double().norm(dim=-1, keepdim=True).numpy() for x in ("q", "k", "v", "d_o"))
+    for x, r, bound in ((o, ref_o, nv), (dv, rv, nd), (dq, rq, 2 * nd * nv / nq), (dk, rk, 2 * nd * nv / nk)):
+        assert (abs(x.double().cpu().numpy() - r) <= u * bound).all()
