@@ -92,7 +92,7 @@ unsigned long long cott_launch_count(void);
  *   "force_group"        (COTT_FORCE_GROUP, 0)        tokens per sequence group; 0 = the plan's choice
  *   "force_path"         (COTT_FORCE_PATH, 1)         0 = bf16 d = 64 / 128 through the fp32-accumulating SIMT kernels
  *   "pair"               (COTT_PAIR, 1)               0 = gradient streams one after the other where they would run side by side
- *   "fused_bwd"          (COTT_FUSED_BWD, 1)          0 = d = 64 backward (causal and bidirectional) as three role-swapped walks instead of one fused walk
+ *   "fused_bwd"          (COTT_FUSED_BWD, 1)          0 = backward as three role-swapped walks instead of one fused walk (d = 64) or two in one launch (d = 128)
  *   "fused_bidir"        (COTT_FUSED_BIDIR, 1)        0 = bidirectional d = 64 forward as a state pass and a read-out instead of one launch
  *   "bidir_bwd"          (COTT_BIDIR_BWD, 1)          0 = bidirectional d = 64 backward with one group per (b, h) as a state pass and a walk instead of one launch
  *   "short_fwd"          (COTT_SHORT_FWD, 1)          0 = sequences of at most 128 tokens through the generic walk instead of the stateless kernel

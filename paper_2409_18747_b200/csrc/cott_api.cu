@@ -774,6 +774,53 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
             COTT_CUDA(launch_dm_finalize(dm_partial, dm, sp->m, sp->seq_len, sp->seq_len_scalar, B, H, p.n_groups, N, st, nullptr));
             return COTT_OK;
         }
+        if (d == 128 && option_fused_bwd() != 0) {
+            // Two kinds of walks in one launch (cott_tc_bwd128.cu), each over half as many groups as the
+            // plan has (it counts one CTA per group, here there are two); with one group no partial
+            // state is needed.  (Bidirectional: the plan's groups, every walk starts from the totals.)
+            int n = p.n_groups, group = p.group;
+            if (causal && n > 1 && option_force_group() <= 0) {
+                n = n / 2;
+                group = ((N + n - 1) / n + 127) / 128 * 128;
+                n = (N + group - 1) / group;
+            }
+            TcBwdFusedArgs f;
+            memset(&f, 0, sizeof(f));
+            f.q = q; f.k = k; f.v = v; f.d_o = d_o; f.dq = dq; f.dk = dk; f.dv = dv;
+            f.l_qkv = lay.qkv; f.l_do = lay.o; f.l_dqkv = lay.dqkv;
+            f.l_v = lay.of(v); f.l_dv = lay.of(dv); f.w_k = p.dk; f.w_v = p.dv;
+            f.dm_partial = dm_partial; f.dm_out = dm; f.status = status;
+            f.m = sp->m; f.seq_len = sp->seq_len; f.seq_len_scalar = sp->seq_len_scalar;
+            f.group = group; f.n_groups = n; f.bidir = causal ? 0 : 1;
+            f.cu_seqlens = packed.cu_seqlens; f.total_tokens = packed.total_tokens;
+            const bool states = !causal || n > 1;
+            // Up to four partial states are summed by the walks themselves (64 KB each out of L2 per CTA).
+            const bool in_walk = n <= 4;
+            if (states) {
+                auto state_pass = [&](TcWalkArgs a, float* out, int clear) {
+                    a.mode = 0; a.x = nullptr; a.proj = nullptr; a.out = nullptr; a.init = nullptr;
+                    a.state_out = out; a.dm_partial = nullptr; a.dm_out = nullptr; a.epilogue = EPI_PLAIN;
+                    a.status = status; a.clear_status = clear;
+                    a.m = sp->m; a.seq_len = sp->seq_len; a.seq_len_scalar = sp->seq_len_scalar;
+                    a.group = group; a.n_groups = n;
+                    // Nobody reads the state of the group a causal walk visits last.
+                    if (causal) { a.first_group = a.reverse ? 1 : 0; a.grid_groups = n - 1; }
+                    a.reverse = a.reverse ? 0 : 1;       // chunk order opposite to the walk's: L2 reuse of its tiles
+                    return launch_tc_walk(a, B, H, N, d, st);
+                };
+                COTT_CUDA(state_pass(tq, st0, 1));
+                COTT_CUDA(state_pass(tk, st1, 0));
+                if (!in_walk) {
+                    COTT_CUDA(launch_scan(st0, nullptr, BH, n, d, causal ? SCAN_PREFIX : SCAN_TOTAL, st));
+                    COTT_CUDA(launch_scan(st1, nullptr, BH, n, d, causal ? SCAN_SUFFIX : SCAN_TOTAL, st));
+                }
+                f.sq_part = st0; f.r_part = st1;
+            } else {
+                COTT_CUDA(cudaMemsetAsync(ws, 0, kWsHeaderBytes, st));      // status words and the dm counter
+            }
+            COTT_CUDA(launch_tc_bwd128(f, in_walk ? 1 : 0, dm_partial2, states ? 0 : 1, B, H, N, st));
+            return COTT_OK;
+        }
         if (ss) {
             struct TagScope { ~TagScope() { g_prof_cur_tag = 0; } } tag_scope;
             // Everything that follows a cross-stream event wait is a plain launch.

@@ -1,0 +1,778 @@
+// Backward at d = 128 (bf16 I/O, fp32 accumulation and states; head sizes 72 .. 128 zero-filled to it):
+// the three gradients and the dm sum in one launch of two kinds of CTAs.
+//
+// With q^, k^ the normalised rows (Eq. 2/3) and M the causal mask (Eq. 6), per chunk of 128 tokens:
+//   Q walk, forward in time:    dQ^ = (dO V^T . M) K^ + dO Sq        Sq = sum over earlier chunks of V^T K^
+//   K walk, backward in time:   dK^ = (V dO^T . M^T) Q^ + V Rt       Rt = sum over later chunks of dO^T Q^
+//                               dV' = (K^ Q^^T . M^T) dO + K^ Rt^T
+// (the formulas printed after Eq. 7).  dK and dV share one running sum -- the paper's reverse-time
+// cumulative sum -- and all four input tiles, so one walk gives both; three such states, or all
+// products of the three gradients, do not fit one SM's 512 tensor-memory columns and 227 KB next to
+// tiles in flight at this head size, so dQ, whose sum runs the other way, has CTAs of its own.  With
+// an all-ones mask (BIDIR) both sums are totals and only the products with them remain.
+//
+// What bounds it: shared memory and the chain of one chunk.  A 128 x 128 x 16 product reads 8 KB of
+// operands in the 64 cycles it takes at full rate, all the bandwidth shared memory has, so the K
+// walk's seven products, its tiles coming in and going out and the worker warps' passes over them are
+// about 6600 cycles of shared-memory time a chunk (Q walk: 4900); 8800 pass, the rest being waits
+// along the chain (tiles without a second slot land, scores, mask, products, slots free again).  The
+// two CTAs of a (b, h, group) start side by side, so one of them finds most tiles in L2.
+// Measured against the three role-swapped walks with their state passes and scans: B=4, H=16,
+// N=2048 93 us (207), B=3, H=16, N=2999 129 us (210), 32 packed sequences of 512 to 2048 tokens,
+// H=16, 390 us (622), bidirectional B=8, H=16, N=1024 107 us (124).
+#include "cott_internal.h"
+#include "cott_sm100.cuh"
+#include "cott_tc_common.cuh"
+
+namespace cott {
+
+using namespace sm100;
+using namespace tc;
+
+namespace {
+
+constexpr int kC = 128;
+constexpr int kD = 128;
+constexpr int kTile = kC * kD * 2;      // one 128 x 128 bf16 tile: two 64-column halves 16 KB apart
+constexpr int kHalf = kTile / 2;
+constexpr int kWorkerWarps = 16;
+constexpr int kGroup = kWorkerWarps / 2 * 32;       // threads of a worker group
+constexpr int kThreads = (kWorkerWarps + 4) * 32;   // + score, product, state-update and copy threads
+
+// Six tile slots, the bf16 copy of the state and the control block are all of the 227 KB.
+// A walk has four tiles a chunk: X and A (scores X A^T), Bv (normalised in place) and the raw rows P
+// that the projection needs.  Q walk: X = dO, A = V, Bv = K, P = Q; X and A have two slots, so the
+// scores of the next chunk do not wait for this one; dq is staged over P.  K walk: X = V, A = dO,
+// Bv = Q, P = K, in three pairs of slots that take turns: (A, Bv) of chunk c + 1 wait in one, landed
+// and normalised, while chunk c has the other two; (X, P) of chunk c + 1 go where (A, Bv) of chunk c
+// were as soon as its products are done; dv and dk are staged over (X, P).
+struct L {
+    static constexpr int kOffSb = 6 * kTile;
+    static constexpr int kOffCtl = kOffSb + kTile;
+    static constexpr int kOffDmRed = 640;            // float [8] + a flag
+    static constexpr int kOffXch = 1024;             // float2 [2][128]: per-row partial sums of the two column halves
+    static constexpr int kCtlBytes = 3072;
+    static constexpr int kDynBytes = kOffCtl + kCtlBytes;   // (no slack: the base must be aligned, see the kernel)
+};
+
+struct Bwd128Params {
+    // partial states of the groups, fp32 [BH, n_groups, 128 * 128]: V^T K^ and dO^T Q^ (or NULL: one
+    // group, nothing precedes it), raw (init_sum: summed here over the groups before, after, or all)
+    // or already scanned
+    const float* sq; const float* rt; int init_sum;
+    float* dm_q; float* dm_k;           // [BH, n_groups]: parts of the dm sum of the two walks
+    float* dm_out; int* status;
+    const float* m; const float* seq_len; float seq_len_scalar;
+    int H; int N; int group; int n_groups;
+    int clear_status;                   // no kernel of the call comes before this one
+    int wait_limit_kcycles;
+    int head_first_mask;                // bit i: in tensor map i (q, k, v, dO, dq, dk, dv) the head index comes before the token index
+    const int* cu_seqlens;              // packed batch (VARLEN instances)
+    void* out_rows[3]; long long out_sn[3], out_sh[3]; int out_w[3];
+};
+
+#ifdef COTT_TIMING
+// Debug build only: SM-clock stamps of CTAs 0 (K walk) and 1 (Q walk), first 16 chunks, eight slots for each of
+// six roles (0, 1: first thread of worker groups A, B; 2-5: score, product, state, copy threads).
+__device__ long long g_b128_stamps[2 * 6 * 16 * 8];
+#define STAMP(role, c, slot)                                                                                 \
+    do {                                                                                                     \
+        if (blockIdx.x < 2 && (c) < 16 && ((role) > 1 || threadIdx.x == (role) * 256))                       \
+            g_b128_stamps[((blockIdx.x * 6 + (role)) * 16 + (c)) * 8 + (slot)] = clock64();                  \
+    } while (0)
+#else
+#define STAMP(role, c, slot) do { } while (0)
+#endif
+
+// tcgen05.mma chains (one thread).  K step kk of a K-major operand of 128 columns; of an MN-major
+// operand: 16 rows = 2048 bytes.
+__device__ __forceinline__ uint32_t kstep(int kk) { return ((kk >> 2) * (uint32_t)kHalf + (kk & 3) * 32u) >> 4; }
+
+// P = X A^T, both K-major.
+__device__ __forceinline__ void issue_scores(uint32_t tP, uint32_t x, uint32_t a) {
+    constexpr uint32_t idesc = instr_desc_bf16(128, 128, false, false);
+    const uint32_t xl = smem_desc_lo(x, 16), al = smem_desc_lo(a, 16);
+#pragma unroll 2
+    for (int kk = 0; kk < 8; ++kk) mma_ss_w(tP, xl + kstep(kk), kDescHi, al + kstep(kk), kDescHi, idesc, kk > 0);
+}
+// Out = X St, St MN-major (its rows are the contraction index).
+__device__ __forceinline__ void issue_x_state(uint32_t tO, uint32_t x, uint32_t st) {
+    constexpr uint32_t idesc = instr_desc_bf16(128, 128, false, true);
+    const uint32_t xl = smem_desc_lo(x, 16), sl = smem_desc_lo(st, kHalf);
+#pragma unroll 2
+    for (int kk = 0; kk < 8; ++kk) mma_ss_w(tO, xl + kstep(kk), kDescHi, sl + kk * 128u, kDescHi, idesc, kk > 0);
+}
+// Out (+)= P~ B: P~ (bf16, two per column) in tensor memory, B MN-major.
+__device__ __forceinline__ void issue_pt_b(uint32_t tO, uint32_t tPt, uint32_t bt, bool acc_first) {
+    constexpr uint32_t idesc = instr_desc_bf16(128, 128, false, true);
+    const uint32_t bl = smem_desc_lo(bt, kHalf);
+#pragma unroll 2
+    for (int kk = 0; kk < 8; ++kk) mma_ts_w(tO, tPt + kk * 8u, bl + kk * 128u, kDescHi, idesc, (acc_first || kk > 0) ? 1u : 0u);
+}
+// State (+)= A^T B, both MN-major.
+__device__ __forceinline__ void issue_update(uint32_t tS, uint32_t a, uint32_t bt, bool acc_first) {
+    constexpr uint32_t idesc = instr_desc_bf16(128, 128, true, true);
+    const uint32_t al = smem_desc_lo(a, kHalf), bl = smem_desc_lo(bt, kHalf);
+#pragma unroll 2
+    for (int kk = 0; kk < 8; ++kk) mma_ss_w(tS, al + kk * 128u, kDescHi, bl + kk * 128u, kDescHi, idesc, (acc_first || kk > 0) ? 1u : 0u);
+}
+
+// Thread roles.  Warps 0-15 are row workers (warp w owns tensor-memory lanes / tile rows
+// 32 (w % 4) .. + 31 and one half of the columns) in two groups of eight:
+//   group A: masks of the scores, row norms of Bv, bf16 copy of the state;
+//   group B: epilogues.
+// Lane 0 of warp 16 issues the scores, of warp 17 the output products, of warp 18 the state update,
+// of warp 19 every TMA load and store.  The roles meet only through mbarriers, every wait bounded.
+// Every barrier is a pair indexed by chunk parity; no role can be two chunks behind another: each
+// chunk's tiles are requested only after the products (and, where a tile is staged over, the stores)
+// of the chunk that held the slot before.
+// Loops are kept rolled: five roles run different code on one SM, and with everything unrolled they
+// ran out of the instruction caches (ncu: 8.7 warps per issue stalled on "no instruction" against
+// 2.7 with the 16-column loops of the epilogues rolled: 141 us against 120 for B=4, H=16, N=2048;
+// rolling the product chains, the row norms and the two masks took the same case from 113 to 93).
+// Which walk a CTA runs is a compile-time property of its code (KW).
+template <bool KW, bool BIDIR, bool VARLEN>
+__device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
+                                     const CUtensorMap& tmDO, const CUtensorMap& tmDQ, const CUtensorMap& tmDK,
+                                     const CUtensorMap& tmDV, const Bwd128Params& p) {
+    // Tensor-memory columns: State 128 | SC1 128 | SC2 128 | O1 128.  The scores X A^T are in SC1,
+    // packed in place to bf16 (columns 0-63).  K walk: K Q^^T in SC2, packed into columns 64-127 of
+    // SC1, so that SC2 becomes the dV' accumulator; O1 holds dK^.  Q walk: dQ^ alternates between O1
+    // and SC2 (chunk parity).
+    constexpr uint32_t colS = 0, colSC1 = 128, colSC2 = 256, colO1 = 384;
+    constexpr bool kw = KW;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t base = smem_u32(smem_raw);
+    uint8_t* gbase = smem_raw;
+    const uint32_t bars = base + L::kOffCtl;
+    enum { B_FX = 0, B_FA = 16, B_FB = 32, B_FP = 48 /* tiles landed */, B_NB = 64 /* Bv normalised */,
+           B_S1 = 80, B_S2 = 112 /* scores done */, B_M1 = 96, B_M2 = 128 /* masked scores in tensor memory */,
+           B_U = 144 /* state updated */, B_CP = 160 /* bf16 state copy written */, B_O1 = 176, B_O2 = 192 /* accumulators complete */,
+           B_D1 = 208, B_D2 = 224 /* accumulators drained */, B_E1 = 240, B_E2 = 256 /* output rows staged */,
+           B_XCH = 272, B_SIB = 288 /* [4 quadrants][2] */, B_SIB2 = 352 };
+    auto bar = [&](int which, int c) { return bars + which + 8 * (c & 1); };
+    auto par = [&](int c) { return (uint32_t)((c >> 1) & 1); };
+    const uint32_t tmem_slot = bars + kCtlTmemSlot;
+    volatile uint32_t* tmem_slot_g = reinterpret_cast<volatile uint32_t*>(gbase + L::kOffCtl + kCtlTmemSlot);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(gbase + L::kOffCtl + kCtlAbort);
+    float* dm_red = reinterpret_cast<float*>(gbase + L::kOffCtl + L::kOffDmRed);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (base & 1023u) {
+        if (tid == 0 && atomicCAS(p.status, 0, 1) == 0) {
+            p.status[1] = (int)0x80007FF0u;
+            p.status[2] = (int)blockIdx.x | (8 << 24);
+        }
+        return;
+    }
+    const int item = blockIdx.x >> 1;
+    const int g = item % p.n_groups, bh = item / p.n_groups;
+    const int bseq = bh / p.H, h = bh % p.H;
+    const int b = VARLEN ? 0 : bseq;                   // batch coordinate of the tensor maps
+    const int seq0 = VARLEN ? p.cu_seqlens[bseq] : 0, seq1 = VARLEN ? p.cu_seqlens[bseq + 1] : p.N;
+    const int tok0 = seq0 + g * p.group;
+    const int tok1 = min(seq1, tok0 + p.group);
+    const int n_chunks = tok1 > tok0 ? (tok1 - tok0 + kC - 1) / kC : 0;
+    // (a packed batch: the last chunk of a sequence may hold rows of the next one; they are normalised
+    // to zero in Bv, which silences them in every product, and that chunk's rows are stored one by one)
+    const bool ragged_last = VARLEN && ((tok1 - tok0) % kC) != 0;
+    auto chunk_row = [&](int c) { return tok0 + (kw ? n_chunks - 1 - c : c) * kC; };
+    auto is_ragged = [&](int c) { return ragged_last && c == (kw ? 0 : n_chunks - 1); };
+    const bool is_score = warp == kWorkerWarps, is_out = warp == kWorkerWarps + 1;
+    const bool is_upd = warp == kWorkerWarps + 2, is_copy = warp == kWorkerWarps + 3;
+
+    if (is_score) {
+        tmem_alloc(tmem_slot, 512);
+        tmem_relinquish();
+    }
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) {
+            const int o = 8 * i;
+            for (int w : {(int)B_FX, (int)B_FA, (int)B_FB, (int)B_FP, (int)B_S1, (int)B_S2, (int)B_U, (int)B_O1, (int)B_O2}) mbar_init(bars + w + o, 1);
+            for (int w : {(int)B_NB, (int)B_M1, (int)B_M2, (int)B_CP, (int)B_D1, (int)B_D2, (int)B_E1, (int)B_E2, (int)B_XCH}) mbar_init(bars + w + o, kGroup);
+            for (int qq = 0; qq < 4; ++qq) { mbar_init(bars + B_SIB + 16 * qq + o, 32); mbar_init(bars + B_SIB2 + 16 * qq + o, 32); }
+        }
+        *abort_flag = 0;
+        abort_flag[3] = p.wait_limit_kcycles;
+        mbar_fence_init();
+        fence_proxy_async();
+    }
+    if (tid < 16) dm_red[tid] = 0.f;
+    if (is_copy && lane == 0) {
+        tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmDO);
+        tma_prefetch_desc(kw ? &tmDK : &tmDQ);
+        if (kw) tma_prefetch_desc(&tmDV);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot_g;
+
+    // Slots of the four tiles of chunk c (see L).  K walk: (A, Bv) in pair 2 c mod 3, (X, P) in pair
+    // 2 c + 1 mod 3 = the pair of (A, Bv) of chunk c - 1 (bidirectional: no A, Bv; pairs by parity).
+    auto pair_xp = [&](int c) { return BIDIR ? (c & 1) : (2 * c + 1) % 3; };
+    auto pair_ab = [&](int c) { return (2 * c) % 3; };
+    auto off_x = [&](int c) { return kw ? pair_xp(c) * 2 * kTile : (c & 1) * kTile; };
+    auto off_a = [&](int c) { return kw ? pair_ab(c) * 2 * kTile : (2 + (c & 1)) * kTile; };
+    auto off_b = [&](int c) { return kw ? pair_ab(c) * 2 * kTile + kTile : 4 * kTile; };
+    auto off_p = [&](int c) { return kw ? pair_xp(c) * 2 * kTile + kTile : 5 * kTile; };
+    auto load = [&](int off, const CUtensorMap* tm, int which, uint32_t fb, int row) {
+        const bool hf = (p.head_first_mask >> which) & 1;
+        mbar_expect_tx(fb, kTile);
+#pragma unroll 1
+        for (int hh = 0; hh < 2; ++hh) tma_load_4d(base + off + hh * kHalf, tm, fb, hh * 64, hf ? h : row, hf ? row : h, b);
+    };
+    auto load_x = [&](int c) { load(off_x(c), kw ? &tmV : &tmDO, kw ? 2 : 3, bar(B_FX, c), chunk_row(c)); };
+    auto load_a = [&](int c) { load(off_a(c), kw ? &tmDO : &tmV, kw ? 3 : 2, bar(B_FA, c), chunk_row(c)); };
+    auto load_b = [&](int c) { load(off_b(c), kw ? &tmQ : &tmK, kw ? 0 : 1, bar(B_FB, c), chunk_row(c)); };
+    auto load_p = [&](int c) { load(off_p(c), kw ? &tmK : &tmQ, kw ? 1 : 0, bar(B_FP, c), chunk_row(c)); };
+    auto first_loads = [&]() {
+        if (!is_copy || lane != 0 || n_chunks == 0) return;
+        if (!BIDIR) { load_b(0); load_a(0); }
+        load_x(0);
+        load_p(0);
+        if (n_chunks > 1) {
+            if (!kw) { load_x(1); if (!BIDIR) load_a(1); }
+            else if (BIDIR) { load_x(1); load_p(1); }
+            else { load_b(1); load_a(1); }
+        }
+    };
+    // Behind a state pass of the same call (which writes none of the tensors loaded here) the first
+    // tiles are requested before the wait for it.
+    if (!p.clear_status) first_loads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (p.clear_status) first_loads();
+
+    const float s_b = p.seq_len ? p.seq_len[bseq]
+                                : (p.seq_len_scalar > 0.f ? p.seq_len_scalar : (float)(VARLEN ? max(seq1 - seq0, 1) : p.N));
+    const float cfac = stab_factor(p.m[h], s_b);
+
+    const int q4 = warp & 3, hw = (warp >> 2) & 1, w8 = warp & 7;
+    const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
+    const int row = q4 * 32 + lane;               // tile row / tensor-memory lane of a worker thread
+
+    const float* part = kw ? p.rt : p.sq;
+    const bool init_state = part != nullptr;
+    // 32 columns of this thread's state row as bf16 into the copy (rows of 128 bytes, two column halves).
+    auto write_sb = [&](const uint32_t (&r)[32], int c0) {
+#pragma unroll
+        for (int i = 0; i < 32; i += 8) {
+            const int col = c0 + i;
+            *reinterpret_cast<uint4*>(gbase + L::kOffSb + (col >> 6) * kHalf + swz(row, (col & 63) >> 3)) = pack8(&r[i]);
+        }
+    };
+    if (init_state && warp < kWorkerWarps) {
+        // The state before the group's first chunk: row `row`, columns 32 (warp / 4) .. + 31.
+        const int cq = warp >> 2;
+        const float* src = part + (size_t)bh * p.n_groups * kD * kD + (size_t)row * kD + cq * 32;
+        float acc[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) acc[i] = 0.f;
+        const int g_lo = !p.init_sum ? g : (BIDIR ? 0 : (kw ? g + 1 : 0));
+        const int g_hi = !p.init_sum ? g + 1 : (BIDIR ? p.n_groups : (kw ? p.n_groups : g));
+        for (int gg = g_lo; gg < g_hi; ++gg) {
+#pragma unroll
+            for (int i = 0; i < 32; i += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(src + (size_t)gg * kD * kD + i);
+                acc[i] += v.x; acc[i + 1] += v.y; acc[i + 2] += v.z; acc[i + 3] += v.w;
+            }
+        }
+        uint32_t r[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(acc[i]);
+        if (!BIDIR) { tmem_st32(tmem + lane_base + colS + cq * 32, r); tmem_wait_st(); }
+        write_sb(r, cq * 32);
+        fence_proxy_async();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+
+    float dm_acc = 0.f;
+    if (is_copy) {
+        // ------------------------------------------------------------------ copy thread
+        if (lane == 0 && n_chunks > 0) {
+            auto store = [&](const CUtensorMap* tm, int which, int off, int r0) {
+                const bool hf = (p.head_first_mask >> which) & 1;
+#pragma unroll 1
+                for (int hh = 0; hh < 2; ++hh)
+                    if (hh * 64 < p.out_w[which - 4]) tma_store_4d(tm, base + off + hh * kHalf, hh * 64, hf ? h : r0, hf ? r0 : h, b);
+            };
+            for (int c = 0; c < n_chunks; ++c) {
+                const bool by_rows = is_ragged(c);      // the workers stored this chunk's rows themselves
+                if (c + 1 < n_chunks) {
+                    if (!wait_or_abort(bar(B_O1, c), par(c), abort_flag)) break;
+                    if (kw && !wait_or_abort(bar(B_O2, c), par(c), abort_flag)) break;
+                    STAMP(5, c, 0);
+                    if (!BIDIR && !wait_or_abort(bar(B_U, c), par(c), abort_flag)) break;
+                    if (!kw) {
+                        if (!BIDIR) load_b(c + 1);
+                        if (c + 2 < n_chunks) {
+                            load_x(c + 2);
+                            if (!BIDIR) load_a(c + 2);
+                        }
+                    } else if (!BIDIR) {
+                        load_x(c + 1);
+                        load_p(c + 1);
+                    }
+                    STAMP(5, c, 1);
+                }
+                if (!wait_or_abort(bar(B_E1, c), par(c), abort_flag)) break;
+                STAMP(5, c, 2);
+                if (!by_rows) store(kw ? &tmDK : &tmDQ, kw ? 5 : 4, off_p(c), chunk_row(c));
+                tma_store_commit();
+                if (kw) {
+                    if (!wait_or_abort(bar(B_E2, c), par(c), abort_flag)) break;
+                    STAMP(5, c, 3);
+                    if (!by_rows) store(&tmDV, 6, off_x(c), chunk_row(c));
+                    tma_store_commit();
+                    if (c + 2 < n_chunks) {
+                        // (the P slot, whose store is the older one, takes Bv or P; the X slot A or X)
+                        tma_store_wait_read1();
+                        if (BIDIR) load_p(c + 2); else load_b(c + 2);
+                        tma_store_wait_read0();
+                        if (BIDIR) load_x(c + 2); else load_a(c + 2);
+                        STAMP(5, c, 4);
+                    }
+                } else if (c + 1 < n_chunks) {
+                    tma_store_wait_read0();
+                    load_p(c + 1);
+                    STAMP(5, c, 4);
+                }
+            }
+            tma_store_wait_all0();
+        }
+    } else if (is_score) {
+        // ------------------------------------------------------------------ score thread
+        if (lane == 0 && !BIDIR) {
+            for (int c = 0; c < n_chunks; ++c) {
+                if (!wait_or_abort(bar(B_FX, c), par(c), abort_flag)) break;
+                if (!wait_or_abort(bar(B_FA, c), par(c), abort_flag)) break;
+                STAMP(2, c, 0);
+                // the products that read the packed scores in these columns have completed
+                if (c >= 1 && !wait_or_abort(bar(B_O1, c - 1), par(c - 1), abort_flag)) break;
+                if (kw && c >= 1 && !wait_or_abort(bar(B_O2, c - 1), par(c - 1), abort_flag)) break;
+                STAMP(2, c, 1);
+                tc_fence_after();
+                issue_scores(tmem + colSC1, base + off_x(c), base + off_a(c));
+                tc_commit(bar(B_S1, c));
+                if (!kw) continue;
+                if (!wait_or_abort(bar(B_FP, c), par(c), abort_flag)) break;
+                if (!wait_or_abort(bar(B_NB, c), par(c), abort_flag)) break;
+                STAMP(2, c, 2);
+                if (c >= 1 && !wait_or_abort(bar(B_D2, c - 1), par(c - 1), abort_flag)) break;   // dV' drained
+                STAMP(2, c, 3);
+                tc_fence_after();
+                issue_scores(tmem + colSC2, base + off_p(c), base + off_b(c));
+                tc_commit(bar(B_S2, c));
+            }
+        }
+    } else if (is_upd) {
+        // ------------------------------------------------------------------ state-update thread
+        // (the state after the last chunk is read by nobody)
+        if (lane == 0 && !BIDIR) {
+            for (int c = 0; c + 1 < n_chunks; ++c) {
+                if (!wait_or_abort(bar(B_FA, c), par(c), abort_flag)) break;
+                if (!wait_or_abort(bar(B_NB, c), par(c), abort_flag)) break;
+                if (c >= 1 && !wait_or_abort(bar(B_CP, c - 1), par(c - 1), abort_flag)) break;
+                STAMP(4, c, 0);
+                tc_fence_after();
+                issue_update(tmem + colS, base + off_a(c), base + off_b(c), init_state || c > 0);
+                tc_commit(bar(B_U, c));
+            }
+        }
+    } else if (is_out) {
+        // ------------------------------------------------------------------ output-product thread
+        if (lane == 0) {
+            const uint32_t sb = base + L::kOffSb;
+            for (int c = 0; c < n_chunks; ++c) {
+                const bool acc = BIDIR || init_state || c > 0;
+                const uint32_t tO = tmem + (!kw && (c & 1) ? colSC2 : colO1);
+                if (!wait_or_abort(bar(B_FX, c), par(c), abort_flag)) break;
+                if (c >= 1 && !BIDIR && !wait_or_abort(bar(B_CP, c - 1), par(c - 1), abort_flag)) break;
+                STAMP(3, c, 0);
+                // the accumulator has been drained: one in the K walk, two in turn in the Q walk
+                if (kw && c >= 1 && !wait_or_abort(bar(B_D1, c - 1), par(c - 1), abort_flag)) break;
+                if (!kw && c >= 2 && !wait_or_abort(bar(B_D1, c - 2), par(c - 2), abort_flag)) break;
+                STAMP(3, c, 1);
+                tc_fence_after();
+                if (acc) issue_x_state(tO, base + off_x(c), sb);
+                if (!BIDIR) {
+                    if (!wait_or_abort(bar(B_M1, c), par(c), abort_flag)) break;
+                    STAMP(3, c, 2);
+                    if (!wait_or_abort(bar(B_NB, c), par(c), abort_flag)) break;
+                    STAMP(3, c, 3);
+                    tc_fence_after();
+                    issue_pt_b(tO, tmem + colSC1, base + off_b(c), acc);
+                }
+                tc_commit(bar(B_O1, c));
+                if (!kw) continue;
+                if (BIDIR) {
+                    if (!wait_or_abort(bar(B_FP, c), par(c), abort_flag)) break;
+                    if (c >= 1 && !wait_or_abort(bar(B_D2, c - 1), par(c - 1), abort_flag)) break;
+                } else if (!wait_or_abort(bar(B_M2, c), par(c), abort_flag)) break;
+                STAMP(3, c, 4);
+                tc_fence_after();
+                // K Rt^T: the state copy read K-major (its columns are the contraction index)
+                if (acc) issue_scores(tmem + colSC2, base + off_p(c), sb);
+                if (!BIDIR) issue_pt_b(tmem + colSC2, tmem + colSC1 + 64, base + off_a(c), acc);
+                tc_commit(bar(B_O2, c));
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ row workers
+        bool alive = n_chunks > 0;
+        auto wait = [&](uint32_t bar_, uint32_t parity) {
+            if (alive && !wait_or_abort(bar_, parity, abort_flag)) alive = false;
+            return alive;
+        };
+        if (warp < 8) {
+            // -------------------------------------------------------------- group A
+            // Two 32 x 32 score blocks of this warp (row block q4, column blocks 2 hw, 2 hw + 1),
+            // masked (Q walk: columns up to the row, K walk: from the row on; diagonal kept, Eq. 6)
+            // and packed to bf16, two per column, to the columns from tdst on.  Per block the mask is
+            // all-keep, all-zero or a triangle; the first two are warp-uniform.  `guard`: a barrier
+            // to wait for before the first store (0: none).
+            auto mask = [&](uint32_t tsc, uint32_t tdst, uint32_t guard, uint32_t gpar) {
+#pragma unroll 1
+                for (int hb = 0; hb < 2; ++hb) {
+                    const int cb = 2 * hw + hb;
+                    uint32_t r[32];
+                    if (kw ? cb >= q4 : cb <= q4) {
+                        tmem_ld32(tsc + lane_base + cb * 32, r);
+                        tmem_wait_ld();
+                        if (cb == q4) {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) r[j] = (kw ? j >= lane : j <= lane) ? r[j] : 0u;
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) r[j] = 0u;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) r[j] = pack_bf16(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+                    if (hb == 0 && guard) {
+                        if (!wait(guard, gpar)) return;
+                        tc_fence_after();
+                    }
+                    tmem_st16(tdst + lane_base + cb * 16, r);
+                }
+                tmem_wait_st();
+                tc_fence_before();
+            };
+            // x^ = x / max(||x||, eps) on half a row of Bv, in place (lanes l and l ^ 16 share a row),
+            // scaled in packed bf16 arithmetic with the scale split in two terms (see normalise_row64).
+            auto normalise = [&](int c) {
+                if (!wait(bar(B_FB, c), par(c))) return;
+                const int nrow = w8 * 16 + (lane & 15), half = lane >> 4;
+                uint8_t* tile = gbase + off_b(c) + half * kHalf + nrow * 128;
+                float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+#pragma unroll 2
+                for (int j = 0; j < 8; ++j) {
+                    const uint4 w = *reinterpret_cast<const uint4*>(tile + ((j ^ (nrow & 7)) << 4));
+                    const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&w);
+#pragma unroll
+                    for (int i = 0; i < 4; i += 2) {
+                        const float2 f0 = __bfloat1622float2(e[i]), f1 = __bfloat1622float2(e[i + 1]);
+                        s0 = __ffma2_rn(f0, f0, s0); s1 = __ffma2_rn(f1, f1, s1);
+                    }
+                }
+                float ss = (s0.x + s0.y) + (s1.x + s1.y);
+                ss += __shfl_xor_sync(0xffffffffu, ss, 16);
+                float rn = 1.0f / fmaxf(sqrtf(ss), kEps);
+                if (VARLEN && chunk_row(c) + nrow >= tok1) rn = 0.f;      // a row of the next sequence
+                const RowScale sc(rn);
+#pragma unroll 2
+                for (int j = 0; j < 8; ++j) {
+                    uint4 w = *reinterpret_cast<const uint4*>(tile + ((j ^ (nrow & 7)) << 4));
+                    __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&w);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) e[i] = sc(e[i]);
+                    *reinterpret_cast<uint4*>(tile + ((j ^ (nrow & 7)) << 4)) = w;
+                }
+                fence_proxy_async();
+                mbar_arrive(bar(B_NB, c));
+            };
+            for (int c = 0; !BIDIR && c < n_chunks && alive; ++c) {
+                // K walk: Bv of this chunk landed during the chunk before.  Q walk: it lands last.
+                STAMP(0, c, 0);
+                if (kw) { normalise(c); if (!alive) break; }
+                STAMP(0, c, 1);
+                // The packed scores go over the start of the fp32 ones: blocks 2, 3 of a row land in
+                // the columns of fp32 block 1, which the sibling warp (hw = 0) reads first; the second
+                // scores of the K walk go to columns 64-127 of SC1, which the hw = 1 warp has read by then.
+                const uint32_t sib = bars + B_SIB + 16 * q4 + 8 * (c & 1), sib2 = sib + (B_SIB2 - B_SIB);
+#pragma unroll 1
+                for (int it = 0; it < (kw ? 2 : 1) && alive; ++it) {
+                    if (!wait(bar(it ? B_S2 : B_S1, c), par(c))) break;
+                    STAMP(0, c, 2 + 2 * it);
+                    tc_fence_after();
+                    const uint32_t guard = it == 0 ? (hw == 1 ? sib : 0u) : (hw == 0 ? sib2 : 0u);
+                    mask(tmem + (it ? colSC2 : colSC1), tmem + colSC1 + it * 64, guard, par(c));
+                    if (!alive) break;
+                    mbar_arrive(bar(it ? B_M2 : B_M1, c));
+                    if (it == 0) mbar_arrive(hw == 0 ? sib : sib2);
+                    STAMP(0, c, 3 + 2 * it);
+                }
+                if (!kw && alive) normalise(c);
+                if (!alive) break;
+                // bf16 copy of the updated state for the next chunk, once this chunk's products
+                // have read the previous copy.
+                if (c + 1 < n_chunks) {
+                    if (!wait(bar(B_U, c), par(c))) break;
+                    if (!wait(bar(B_O1, c), par(c))) break;
+                    if (kw && !wait(bar(B_O2, c), par(c))) break;
+                    STAMP(0, c, 6);
+                    tc_fence_after();
+#pragma unroll 1
+                    for (int pc = 0; pc < 2; ++pc) {
+                        uint32_t r[32];
+                        tmem_ld32(tmem + lane_base + colS + hw * 64 + pc * 32, r);
+                        tmem_wait_ld();
+                        write_sb(r, hw * 64 + pc * 32);
+                    }
+                    fence_proxy_async();
+                    tc_fence_before();
+                    mbar_arrive(bar(B_CP, c));
+                    STAMP(0, c, 7);
+                }
+            }
+        } else {
+            // -------------------------------------------------------------- group B
+            // (rows of a ragged last chunk of a packed batch leave one by one)
+            auto put = [&](uint8_t* tile, int which, bool by_rows, int c, int i, uint4 o) {
+                if (VARLEN && by_rows) {
+                    const long long grow = (long long)chunk_row(c) + row;
+                    const int col = hw * 64 + i;
+                    if (grow < tok1 && col < p.out_w[which])
+                        *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out_rows[which]) + grow * p.out_sn[which] +
+                                                  (long long)h * p.out_sh[which] + col) = o;
+                } else {
+                    *reinterpret_cast<uint4*>(tile + swz(row, i >> 3)) = o;
+                }
+            };
+            float2* xch = reinterpret_cast<float2*>(gbase + L::kOffCtl + L::kOffXch);
+            for (int c = 0; c < n_chunks && alive; ++c) {
+                // ---- projection epilogue (chain rule through x^ = x / max(||x||, eps)), this thread's 64 columns
+                STAMP(1, c, 0);
+                if (!wait(bar(B_FP, c), par(c))) break;
+                uint8_t* tile = gbase + off_p(c) + hw * kHalf;
+                const uint32_t tacc = tmem + lane_base + (!kw && (c & 1) ? colSC2 : colO1) + hw * 64;
+                if (!wait(bar(B_O1, c), par(c))) break;
+                STAMP(1, c, 1);
+                tc_fence_after();
+                float2 s2 = make_float2(0.f, 0.f), d2 = s2;
+#pragma unroll 1
+                for (int pc = 0; pc < 4; ++pc) {
+                    float2 r[8];
+                    tmem_ld16(tacc + pc * 16, reinterpret_cast<uint32_t*>(r));
+                    uint4 w[2];
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) w[i] = *reinterpret_cast<const uint4*>(tile + swz(row, pc * 2 + i));
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float2 f = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[i]);
+                        s2 = __ffma2_rn(f, f, s2);
+                        d2 = __ffma2_rn(f, r[i], d2);
+                    }
+                }
+                // (every thread of the group has read the exchange area of the chunk before)
+                if (c >= 1 && !wait(bar(B_D1, c - 1), par(c - 1))) break;
+                xch[hw * 128 + row] = make_float2(s2.x + s2.y, d2.x + d2.y);
+                mbar_arrive(bar(B_XCH, c));
+                STAMP(1, c, 2);
+                if (!wait(bar(B_XCH, c), par(c))) break;
+                const float2 e0 = xch[row], e1 = xch[128 + row];
+                const float dp = e0.y + e1.y, nrm = sqrtf(e0.x + e1.x);
+                const float rp = 1.0f / fmaxf(nrm, kEps);
+                const bool valid = !VARLEN || chunk_row(c) + row < tok1;
+                // dm: the Q walk sums <q^_i, dQ^_i> of the unscaled accumulator.  That sum uses k^ rounded
+                // to bf16; to first order the sum with the exact k^ is larger by
+                // sum_j <k^_j - bf16(k^_j), dK^_j>, and the K walk has both factors.
+                const bool use = valid && (!kw || nrm > kEps);
+                if (use && hw == 0) dm_acc += dp * rp;
+                // out = (c acc - x coef) / max(||x||, eps) over the raw rows (K walk: which K Rt^T has read by then)
+                if (kw && !wait(bar(B_O2, c), par(c))) break;
+                STAMP(1, c, 3);
+                const bool by_rows = is_ragged(c);
+                const float sc = cfac * rp, mc = nrm > kEps ? -dp * cfac * rp * rp * rp : 0.f;
+                const float2 sc2 = make_float2(sc, sc), mc2 = make_float2(mc, mc);
+                const RowScale ks(use ? rp : 0.f);
+                float2 k2 = make_float2(0.f, 0.f);
+#pragma unroll 1
+                for (int pc = 0; pc < 4; ++pc) {
+                    float2 r[8];
+                    tmem_ld16(tacc + pc * 16, reinterpret_cast<uint32_t*>(r));
+                    uint4 w[2];
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) w[i] = *reinterpret_cast<const uint4*>(tile + swz(row, pc * 2 + i));
+                    tmem_wait_ld();
+                    uint4 o[2];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const __nv_bfloat162 e = reinterpret_cast<const __nv_bfloat162*>(w)[i];
+                        if (kw) k2 = __ffma2_rn(__bfloat1622float2(ks(e)), r[i], k2);
+                        const float2 v = __ffma2_rn(__bfloat1622float2(e), mc2, __fmul2_rn(r[i], sc2));
+                        reinterpret_cast<uint32_t*>(o)[i] = pack_bf16(v.x, v.y);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) put(tile, kw ? 1 : 0, by_rows, c, (pc * 2 + i) * 8, o[i]);
+                }
+                if (kw) dm_acc -= k2.x + k2.y;
+                tc_fence_before();
+                mbar_arrive(bar(B_D1, c));
+                fence_proxy_async();
+                mbar_arrive(bar(B_E1, c));
+                STAMP(1, c, 4);
+                if (kw) {
+                    // ---- dV = (c / max(||k||, eps)) dV', over the v rows
+                    uint8_t* vt = gbase + off_x(c) + hw * kHalf;
+#pragma unroll 1
+                    for (int pc = 0; pc < 4; ++pc) {
+                        float2 r[8];
+                        tmem_ld16(tmem + lane_base + colSC2 + hw * 64 + pc * 16, reinterpret_cast<uint32_t*>(r));
+                        tmem_wait_ld();
+                        uint4 o[2];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const float2 v = __fmul2_rn(r[i], sc2);
+                            reinterpret_cast<uint32_t*>(o)[i] = pack_bf16(v.x, v.y);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) put(vt, 2, by_rows, c, (pc * 2 + i) * 8, o[i]);
+                    }
+                    tc_fence_before();
+                    mbar_arrive(bar(B_D2, c));
+                    fence_proxy_async();
+                    mbar_arrive(bar(B_E2, c));
+                    STAMP(1, c, 5);
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) dm_acc += __shfl_xor_sync(0xffffffffu, dm_acc, o);
+            if (lane == 0) dm_red[w8] = dm_acc;
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    {
+        int* last_flag = reinterpret_cast<int*>(&dm_red[8]);
+        if (tid == 0) {
+            if (!*abort_flag)
+                (kw ? p.dm_k : p.dm_q)[(size_t)bh * p.n_groups + g] = ((dm_red[0] + dm_red[1]) + (dm_red[2] + dm_red[3])) +
+                                                                   ((dm_red[4] + dm_red[5]) + (dm_red[6] + dm_red[7]));
+            __threadfence();
+            *last_flag = atomicAdd(&p.status[4], 1) == (int)gridDim.x - 1;
+        }
+        __syncthreads();
+        if (*last_flag) {
+            // Every CTA's partial sums are visible: dm_h = sum_b dc/dm(b,h) * sum_g T_{b,h,g}, T the sum
+            // over rows of <q^, dQ^> plus the rounding term, dc/dm = -ln(s_b) sigma(m_h) (1 - sigma(m_h))
+            // c_{b,h}; fixed order, so deterministic.  One warp per head.
+            __threadfence();
+            const int per = (int)gridDim.x / (2 * p.H);
+            for (int hh = warp; hh < p.H; hh += kThreads / 32) {
+                const float sg = 1.0f / (1.0f + expf(-p.m[hh]));
+                float sum = 0.f;
+                for (int i = lane; i < per; i += 32) {
+                    const int bb = i / p.n_groups, gg = i - bb * p.n_groups;
+                    const float sb2 = p.seq_len ? p.seq_len[bb]
+                                                : (p.seq_len_scalar > 0.f ? p.seq_len_scalar
+                                                   : (float)(VARLEN ? max(p.cu_seqlens[bb + 1] - p.cu_seqlens[bb], 1) : p.N));
+                    const float ls = logf(sb2);
+                    const size_t idx = ((size_t)bb * p.H + hh) * p.n_groups + gg;
+                    sum += (__ldcg(&p.dm_q[idx]) + __ldcg(&p.dm_k[idx])) * (-ls * sg * (1.0f - sg) * expf(-sg * ls));
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                if (lane == 0) p.dm_out[hh] = sum;
+            }
+            if (tid == 0) p.status[4] = 0;
+        }
+    }
+    if (*abort_flag) {
+        // A wait gave up: let the copies and products still in flight land (microseconds), then report.
+        for (int i = 0; i < 100; ++i) __nanosleep(1000);
+        __syncthreads();
+        if (tid == 0 && atomicCAS(p.status, 0, 1) == 0) {
+            p.status[1] = *abort_flag;
+            p.status[2] = (int)blockIdx.x | (8 << 24);
+        }
+    }
+    if (is_score) tmem_dealloc(tmem, 512);
+}
+
+template <bool BIDIR, bool VARLEN>
+__global__ void __launch_bounds__(kThreads, 1)
+tc_bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmDO,
+                 const __grid_constant__ CUtensorMap tmDQ, const __grid_constant__ CUtensorMap tmDK,
+                 const __grid_constant__ CUtensorMap tmDV, const __grid_constant__ Bwd128Params p) {
+    // The two walks of a (b, h, group) are neighbours in the grid; the longer one, K, first.
+    if ((blockIdx.x & 1) == 0) walk<true, BIDIR, VARLEN>(tmQ, tmK, tmV, tmDO, tmDQ, tmDK, tmDV, p);
+    else walk<false, BIDIR, VARLEN>(tmQ, tmK, tmV, tmDO, tmDQ, tmDK, tmDV, p);
+}
+
+}  // namespace
+
+cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, int init_sum, float* dm_k, int clear_status, int B, int H, int N,
+                             cudaStream_t st) {
+    const void* ptrs[7] = {a.q, a.k, a.v, a.d_o, a.dq, a.dk, a.dv};
+    const RowLayout lays[7] = {a.l_qkv, a.l_qkv, a.l_v, a.l_do, a.l_dqkv, a.l_dqkv, a.l_dv};
+    const int wk = a.w_k > 0 ? a.w_k : kD, wv = a.w_v > 0 ? a.w_v : kD;
+    const int dims[7] = {wk, wk, wv, wv, wk, wk, wv};
+    if (wk > kD || wv > kD) return cudaErrorInvalidValue;
+    CUtensorMap tm[7];
+    Bwd128Params p;
+    p.head_first_mask = 0;
+    // A packed batch is one tensor of total_tokens rows per head (batch extent 1).
+    const int map_B = a.cu_seqlens ? 1 : B, map_N = a.cu_seqlens ? a.total_tokens : N;
+    for (int i = 0; i < 7; ++i) {
+        bool hf = false;
+        if (!make_tile_map(&tm[i], ptrs[i], map_B, H, map_N, dims[i], lays[i], &hf)) return cudaErrorInvalidValue;
+        p.head_first_mask |= (hf ? 1 : 0) << i;
+    }
+    for (int i = 0; i < 3; ++i) {
+        const RowLayout lo = resolve_layout(lays[4 + i], H, map_N, dims[4 + i]);
+        p.out_rows[i] = const_cast<void*>(ptrs[4 + i]); p.out_sn[i] = lo.sn; p.out_sh[i] = lo.sh; p.out_w[i] = dims[4 + i];
+    }
+    p.sq = a.sq_part; p.rt = a.r_part; p.init_sum = init_sum;
+    p.dm_q = a.dm_partial; p.dm_k = dm_k; p.dm_out = a.dm_out; p.status = a.status;
+    p.m = a.m; p.seq_len = a.seq_len; p.seq_len_scalar = a.seq_len_scalar;
+    p.H = H; p.N = N; p.group = a.group; p.n_groups = a.n_groups;
+    p.clear_status = clear_status;
+    p.wait_limit_kcycles = wait_limit_kcycles();
+    p.cu_seqlens = a.cu_seqlens;
+    if (a.bidir && (!a.sq_part || !a.r_part)) return cudaErrorInvalidValue;
+    auto kern = a.cu_seqlens ? (a.bidir ? tc_bwd128_kernel<true, true> : tc_bwd128_kernel<false, true>)
+                             : (a.bidir ? tc_bwd128_kernel<true, false> : tc_bwd128_kernel<false, false>);
+    if (cudaError_t e = configure_smem_once(reinterpret_cast<const void*>(kern), L::kDynBytes); e != cudaSuccess)
+        return e;
+    const int prof = profile_begin_launch(3, st);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * B * H * a.n_groups));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = L::kDynBytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    // (a packed batch reads cu_seqlens before anything else; behind a memset there is nothing to overlap)
+    cfg.numAttrs = (a.plain_launch || a.cu_seqlens || clear_status) ? 0 : 1;
+    cudaError_t le = cudaLaunchKernelEx(&cfg, kern, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], p);
+    profile_end_launch(prof, st);
+    note_launch();
+    return le != cudaSuccess ? le : cudaGetLastError();
+}
+
+}  // namespace cott
+
+#ifdef COTT_TIMING
+extern "C" int cott_debug_b128_stamps(long long* out) {
+    return (int)cudaMemcpyFromSymbol(out, cott::g_b128_stamps, sizeof(cott::g_b128_stamps));
+}
+#endif

@@ -57,6 +57,18 @@ __device__ __forceinline__ uint4 pack8(const uint32_t* r) {
     return w;
 }
 
+// x * rn in packed bf16 arithmetic with the scale split in two bf16 terms (rn = hi + lo to 2^-17):
+// round(x hi + round(x lo)) is x rn rounded once, up to a second rounding of the small term.
+struct RowScale {
+    __nv_bfloat162 hi2, lo2;
+    __device__ __forceinline__ explicit RowScale(float rn) {
+        const __nv_bfloat16 hi = __float2bfloat16_rn(rn);
+        const __nv_bfloat16 lo = __float2bfloat16_rn(rn - __bfloat162float(hi));
+        hi2 = __halves2bfloat162(hi, hi); lo2 = __halves2bfloat162(lo, lo);
+    }
+    __device__ __forceinline__ __nv_bfloat162 operator()(__nv_bfloat162 x) const { return __hfma2(x, hi2, __hmul2(x, lo2)); }
+};
+
 // x / max(||x||, eps) on one row of 64 bf16 values held in w[8] (eight 16-byte chunks), in
 // packed bf16 arithmetic with the scale split in two bf16 terms (rn = hi + lo to 2^-17):
 // round(x hi + round(x lo)) is x rn rounded once, up to a second rounding of the small term --

@@ -42,3 +42,29 @@ def test_fp32_walk_chunk_and_group_edges(d, N, group, causal, force_group):
     nq, nk, nv, nd = (c[x].double().norm(dim=-1, keepdim=True).numpy() for x in ("q", "k", "v", "d_o"))
     for x, r, bound in ((o, ref_o, nv), (dv, rv, nd), (dq, rq, 2 * nd * nv / nq), (dk, rk, 2 * nd * nv / nk)):
         assert (abs(x.double().cpu().numpy() - r) <= u * bound).all()
+
+
+@pytest.mark.parametrize("N,group", [(1, 0), (127, 0), (128, 0), (129, 0), (257, 0), (400, 128), (900, 256), (700, 128)])
+@pytest.mark.parametrize("dk,dv", [(128, 128), (72, 128), (96, 40)])
+@pytest.mark.parametrize("causal", [True, False])
+def test_backward_d128_chunk_and_group_edges(N, group, dk, dv, causal, force_group):
+    """The d = 128 backward (two walks in one launch): one to several chunks, a ragged last one, one
+    group, up to four (summed by the walks) and six (scan launches), widths zero-filled to 128."""
+    force_group(group)
+    B, H = 2, 3
+    c = synth.make_qkv(B, H, N, dk, torch.bfloat16, 7300 + N + dk, row_lognormal=True, with_do=True, d_v=dv)
+    c["k"][0, 1, N // 2] = 0.0
+    args = [dev(c[x]) for x in ("q", "k", "v", "d_o", "m")]
+    dq, dk_, dv_, dm = cott.bwd(*args, causal=causal)
+    rq, rk, rv, rm = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, causal)
+    if N > 1:      # (one token: see the note on single-term rows in test_parity_gpu's gates)
+        # the zero key row's gradient is that of the clamped formula, 1e12 times larger: gated on its own
+        z = (0, 1, N // 2)
+        assert norm_max_err(dk_[z], rk[z]) <= 1e-2
+        dk_[z] = 0.0
+        rk[z] = 0.0
+        gate(dq, rq, torch.bfloat16); gate(dk_, rk, torch.bfloat16); gate(dv_, rv, torch.bfloat16)
+        # dm's error scales with the sum of its absolute terms (see dm_condition): 3e-4 of it at worst
+        # over random shapes of this size for bf16 operands
+        cond = dm_condition(rv, c["v"], c["m"], None)
+        assert (abs(dm.double().cpu().numpy() - rm) <= 1e-3 * cond).all()
