@@ -135,35 +135,35 @@ __device__ __forceinline__ uint32_t kstep128(int kk) { return ((kk >> 2) * 16384
 __device__ __forceinline__ void issue_scores(uint32_t tP, uint32_t x, uint32_t a) {
     constexpr uint32_t idesc = instr_desc_bf16(128, 128, false, false);
     const uint32_t xl = smem_desc_lo(x, 16), al = smem_desc_lo(a, 16);
-#pragma unroll
+#pragma unroll 2
     for (int kk = 0; kk < kD / 16; ++kk) mma_ss_w(tP, xl + kk * 2u, kDescHi, al + kk * 2u, kDescHi, idesc, kk > 0);
 }
 // Out[128 x 64] = G[128 x 128] B[128 x 64]: G K-major from shared memory, B MN-major.
 __device__ __forceinline__ void issue_g_b(uint32_t tO, uint32_t g, uint32_t bt) {
     constexpr uint32_t idesc = instr_desc_bf16(128, kD, false, true);
     const uint32_t gl = smem_desc_lo(g, 16), bl = smem_desc_lo(bt, 16384);
-#pragma unroll
+#pragma unroll 2
     for (int kk = 0; kk < kC / 16; ++kk) mma_ss_w(tO, gl + kstep128(kk), kDescHi, bl + kk * 128u, kDescHi, idesc, kk > 0);
 }
 // Out[128 x 64] = G^T[128 x 128] B[128 x 64]: G read MN-major (its columns are the M index), B MN-major.
 __device__ __forceinline__ void issue_gt_b(uint32_t tO, uint32_t g, uint32_t bt) {
     constexpr uint32_t idesc = instr_desc_bf16(128, kD, true, true);
     const uint32_t gl = smem_desc_lo(g, 16384), bl = smem_desc_lo(bt, 16384);
-#pragma unroll
+#pragma unroll 2
     for (int kk = 0; kk < kC / 16; ++kk) mma_ss_w(tO, gl + kk * 128u, kDescHi, bl + kk * 128u, kDescHi, idesc, kk > 0);
 }
 // Out[128 x 64] = P~[128 x 128] B[128 x 64]: P~ (bf16, two per column) in tensor memory, B MN-major.
 __device__ __forceinline__ void issue_pt_b(uint32_t tO, uint32_t tPt, uint32_t bt) {
     constexpr uint32_t idesc = instr_desc_bf16(128, kD, false, true);
     const uint32_t bl = smem_desc_lo(bt, 16384);
-#pragma unroll
+#pragma unroll 2
     for (int kk = 0; kk < kC / 16; ++kk) mma_ts_w(tO, tPt + kk * 8u, bl + kk * 128u, kDescHi, idesc, kk > 0);
 }
 // Out[128 x 64] += X[128 x 64] St[64 x 64], St read MN-major (its rows are the contraction index).
 __device__ __forceinline__ void issue_x_state(uint32_t tO, uint32_t x, uint32_t st, bool acc_first = true) {
     constexpr uint32_t idesc = instr_desc_bf16(128, kD, false, true);
     const uint32_t xl = smem_desc_lo(x, 16), sl = smem_desc_lo(st, kD * 128u);
-#pragma unroll
+#pragma unroll 2
     for (int kk = 0; kk < kD / 16; ++kk)
         mma_ss_w(tO, xl + kk * 2u, kDescHi, sl + kk * 128u, kDescHi, idesc, (acc_first || kk > 0) ? 1u : 0u);
 }
@@ -171,7 +171,7 @@ __device__ __forceinline__ void issue_x_state(uint32_t tO, uint32_t x, uint32_t 
 __device__ __forceinline__ void issue_x_state_t(uint32_t tO, uint32_t x, uint32_t st, bool acc_first = true) {
     constexpr uint32_t idesc = instr_desc_bf16(128, kD, false, false);
     const uint32_t xl = smem_desc_lo(x, 16), sl = smem_desc_lo(st, 16);
-#pragma unroll
+#pragma unroll 2
     for (int kk = 0; kk < kD / 16; ++kk)
         mma_ss_w(tO, xl + kk * 2u, kDescHi, sl + kk * 2u, kDescHi, idesc, (acc_first || kk > 0) ? 1u : 0u);
 }
@@ -179,7 +179,7 @@ __device__ __forceinline__ void issue_x_state_t(uint32_t tO, uint32_t x, uint32_
 __device__ __forceinline__ void issue_update(uint32_t tS, uint32_t vq, uint32_t kdo) {
     constexpr uint32_t idesc = instr_desc_bf16(128, 128, true, true);
     const uint32_t al = smem_desc_lo(vq, 16384), bl = smem_desc_lo(kdo, 16384);
-#pragma unroll
+#pragma unroll 2
     for (int kk = 0; kk < kC / 16; ++kk) mma_ss_w(tS, al + kk * 128u, kDescHi, bl + kk * 128u, kDescHi, idesc, 1u);
 }
 
@@ -196,6 +196,9 @@ __device__ __forceinline__ void issue_update(uint32_t tS, uint32_t vq, uint32_t 
 //     dQ^ = dO S^T ,   dK^ = V R^T ,   dV' = K^ R ,
 // so the score products, the masks, the state update and the per-chunk state copies fall away;
 // loads, row norms, epilogues, stores and the dm sum are those of the causal walk.
+// Instruction caches: five roles run different code on one SM, so the product chains, the masks and the
+// epilogues are kept as rolled loops (the backward at B=4, H=16, N=4096: 96 us unrolled, 90 with
+// the product chains rolled, 89 with all; B=8, H=12, N=1024: 49.6 against 45.7).
 // SEG: a segment of a longer causal sequence (cott_bwd_stateful): the running states start from
 // the caller's, and dm is summed over the value rows.  An instance of its own, so that the plain
 // causal walk carries none of it.
@@ -603,30 +606,20 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 if (tid == 0) BSTAMP(3, c, 1);
                 uint8_t* tile = stage_g(c) + (hw == 0 ? L::kOffQ : L::kOffK);
                 uint4 w[8];
-                float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+                float2 s0 = make_float2(0.f, 0.f), s1 = s0;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) w[j] = *reinterpret_cast<const uint4*>(tile + swz(row, j));
 #pragma unroll
-                for (int j = 0; j < 8; j += 2) {
-                    const __nv_bfloat162* e0 = reinterpret_cast<const __nv_bfloat162*>(&w[j]);
-                    const __nv_bfloat162* e1 = reinterpret_cast<const __nv_bfloat162*>(&w[j + 1]);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float2 f0 = __bfloat1622float2(e0[i]), f1 = __bfloat1622float2(e1[i]);
-                        a0 = fmaf(f0.x, f0.x, a0); a1 = fmaf(f0.y, f0.y, a1);
-                        a2 = fmaf(f1.x, f1.x, a2); a3 = fmaf(f1.y, f1.y, a3);
-                    }
+                for (int j = 0; j < 32; j += 2) {
+                    const float2 f0 = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[j]);
+                    const float2 f1 = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[j + 1]);
+                    s0 = __ffma2_rn(f0, f0, s0); s1 = __ffma2_rn(f1, f1, s1);
                 }
-                const float nrm = sqrtf((a0 + a1) + (a2 + a3));
+                const float nrm = sqrtf((s0.x + s0.y) + (s1.x + s1.y));
                 float rn = 1.0f / fmaxf(nrm, kEps);
                 if (VARLEN && chunk_row(c) + row >= tok1) rn = 0.f;      // a row of the next sequence
-                // x * rn in packed bf16 arithmetic with the scale split in two bf16 terms
-                // (rn = hi + lo to 2^-17): round(x hi + round(x lo)) is x rn rounded once, up to a
-                // second rounding of the small term -- two instructions per pair of elements
-                // instead of unpacking, two multiplies and a conversion.
-                const __nv_bfloat16 hi = __float2bfloat16_rn(rn);
-                const __nv_bfloat16 lo = __float2bfloat16_rn(rn - __bfloat162float(hi));
-                const __nv_bfloat162 hi2 = __halves2bfloat162(hi, hi), lo2 = __halves2bfloat162(lo, lo);
+                const RowScale rs(rn);
+                const __nv_bfloat162 hi2 = rs.hi2, lo2 = rs.lo2;
                 // Bidirectional: what the rounding of x^ to bf16 drops, x rn - x^, goes to the
                 // (unused) score buffer as 7-bit fixed point, for the first-order correction of dm in
                 // the projection epilogue: units of 2^-15 (|x rn - x^| <= 2^-9 since |x^| <= 1),
@@ -647,7 +640,7 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const __nv_bfloat162 x = e[i];
-                        e[i] = __hfma2(x, hi2, __hmul2(x, lo2));
+                        e[i] = rs(x);
                         if (BIDIR) {
                             __nv_bfloat162 r = __hfma2(x, lo2s, __hfma2(x, hi2s, __hmul2(e[i], nsc)));
                             r = __hadd2(__hmin2(__hmax2(r, __hneg2(c63)), c63), c192);
@@ -683,7 +676,7 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 if (!wait(bar(B_P1FULL, c), par(c))) break;
                 BSTAMP(0, c, 1);
                 tc_fence_after();
-#pragma unroll
+#pragma unroll 1
                 for (int hb = 0; hb < 2; ++hb) {
                     const int cb = 2 * hw + hb;
                     uint8_t* gdst = gbase + L::kOffG + hw * 16384;
@@ -739,31 +732,29 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 tc_fence_after();
                 {
                     const uint32_t sib = bars + B_B1READ + 16 * q4 + 8 * (c & 1);
-                    if (hw == 1 && !wait(sib, par(c))) break;
-                    uint32_t pk[2][16];
-#pragma unroll
+#pragma unroll 1
                     for (int hb = 0; hb < 2; ++hb) {
                         const int cb = 2 * hw + hb;
+                        uint32_t r[32];
                         if (cb >= q4) {                  // warp-uniform
-                            uint32_t r[32];
                             tmem_ld32(tmem + lane_base + colP2 + cb * 32, r);
                             tmem_wait_ld();
                             if (cb == q4) {
 #pragma unroll
                                 for (int j = 0; j < 32; ++j) r[j] = (j >= lane) ? r[j] : 0u;
                             }
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) pk[hb][j] = pack_bf16(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
                         } else {
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) pk[hb][j] = 0u;
+                            for (int j = 0; j < 32; ++j) r[j] = 0u;
                         }
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) r[j] = pack_bf16(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+                        // blocks 2, 3 land in the columns of fp32 block 1, which the hw = 0 warp reads
+                        if (hb == 1 && hw == 0) { tc_fence_before(); mbar_arrive(sib); }
+                        if (hb == 0 && hw == 1) { if (!wait(sib, par(c))) break; tc_fence_after(); }
+                        tmem_st16(tmem + lane_base + colP2 + cb * 16, r);
                     }
-                    // (both fp32 blocks of this warp have been read -- or need not be: now the
-                    // sibling may write into block 1, and this warp into blocks 0 / 1)
-                    if (hw == 0) { tc_fence_before(); mbar_arrive(sib); }
-                    tmem_st16(tmem + lane_base + colP2 + hw * 32, pk[0]);
-                    tmem_st16(tmem + lane_base + colP2 + hw * 32 + 16, pk[1]);
+                    if (!alive) break;
                     tmem_wait_st();
                 }
                 tc_fence_before();
@@ -792,6 +783,18 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         } else {
             // -------------------------------------------------------------- group B
             const bool isq = hw == 0;
+            // 16 bytes (columns 8 j .. + 7) of this thread's row of output `which` (dq, dk, dv): into the
+            // staging tile; the rows of a ragged last chunk of a packed batch leave one by one.
+            auto put = [&](uint8_t* st_tile, int which, int c, int j, uint4 o) {
+                if (VARLEN && ragged_last && c == n_chunks - 1) {
+                    const long long grow = (long long)chunk_row(c) + row;
+                    if (grow < tok1 && j * 8 < p.out_w[which])
+                        *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out_rows[which]) + grow * p.out_sn[which] +
+                                                  (long long)h * p.out_sh[which] + j * 8) = o;
+                } else {
+                    *reinterpret_cast<uint4*>(st_tile + swz(row, j)) = o;
+                }
+            };
             const int off_tile = isq ? L::kOffQ : L::kOffK;
             const float2* rn_buf = isq ? rq_buf : rk_buf;
             uint8_t* out_tile = gbase + (isq ? L::kOffStQ : L::kOffStK);
@@ -809,50 +812,45 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 BSTAMP(1 + hw, c, 1);
                 tc_fence_after();
                 {
-                    // Two sweeps over the accumulator row: holding all of it next to the tile
-                    // chunks does not fit the register budget (and a single spilled value in this
-                    // loop costs more than the second round trip to tensor memory).
+                    // Two sweeps over the accumulator row, 16 columns at a time in rolled loops: holding all
+                    // of it next to the tile chunks does not fit the register budget (a single spilled
+                    // value in this loop costs more than the second round trip to tensor memory), and
+                    // short code is worth more than wide loads (see the note on instruction caches).
                     const uint32_t tacc = tmem + lane_base + colP1 + (c & 1) * 128 + (isq ? 0 : 64);
                     const uint8_t* tile = stage_g(c) + off_tile;
                     const float2 rn = rn_buf[(c & 1) * kC + row];
                     const uint8_t* res = gbase + L::kOffG + (c & 1) * 16384 + hw * 8192 + row * 64;
-                    float d0 = 0.f, d1 = 0.f;
+                    float2 d2 = make_float2(0.f, 0.f);
                     __nv_bfloat162 ec[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) ec[i] = __halves2bfloat162(__float2bfloat16_rn(0.f), __float2bfloat16_rn(0.f));
 #pragma unroll 1
-                    for (int hf = 0; hf < 2; ++hf) {
-                        uint32_t a[32];
-                        tmem_ld32(tacc + hf * 32, a);
+                    for (int pc = 0; pc < 4; ++pc) {
+                        float2 a[8];
+                        tmem_ld16(tacc + pc * 16, reinterpret_cast<uint32_t*>(a));
+                        uint4 w[2];
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) w[j] = *reinterpret_cast<const uint4*>(tile + swz(row, 2 * pc + j));
                         tmem_wait_ld();
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const uint4 w = *reinterpret_cast<const uint4*>(tile + swz(row, hf * 4 + j));
-                            const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&w);
+                        for (int i = 0; i < 8; ++i)
+                            d2 = __ffma2_rn(__bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[i]), a[i], d2);
+                        if (BIDIR) {
+                            // <x rn - x^, a>: the part of <x^, a> that the bf16 rounding of x^ lost,
+                            // in packed bf16 arithmetic (a correction: one percent of it is plenty).
+                            // Byte m of the residuals next to 0x43 is the bf16 number 128 + m.
+                            const uint4 rw = *reinterpret_cast<const uint4*>(res + (((pc ^ (row >> 1)) & 3) << 4));
+                            const __nv_bfloat162 c192 = __halves2bfloat162(__float2bfloat16_rn(192.f), __float2bfloat16_rn(192.f));
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const float2 f = __bfloat1622float2(e[i]);
-                                d0 = fmaf(f.x, __uint_as_float(a[8 * j + 2 * i]), d0);
-                                d1 = fmaf(f.y, __uint_as_float(a[8 * j + 2 * i + 1]), d1);
-                            }
-                            if (BIDIR) {
-                                // <x rn - x^, a>: the part of <x^, a> that the bf16 rounding of x^ lost,
-                                // in packed bf16 arithmetic (a correction: one percent of it is plenty).
-                                // Byte m of the residuals next to 0x43 is the bf16 number 128 + m.
-                                const uint2 rw = *reinterpret_cast<const uint2*>(res + ((((hf * 2 + (j >> 1)) ^ (row >> 1)) & 3) << 4) + (j & 1) * 8);
-                                const __nv_bfloat162 c192 = __halves2bfloat162(__float2bfloat16_rn(192.f), __float2bfloat16_rn(192.f));
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) {
-                                    const uint32_t word = i < 2 ? rw.x : rw.y;
-                                    const uint32_t pr = __byte_perm(word, 0x43434343u, (i & 1) ? 0x4342 : 0x4140);
-                                    const __nv_bfloat162 r = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&pr), c192);
-                                    const __nv_bfloat162 ab = __floats2bfloat162_rn(__uint_as_float(a[8 * j + 2 * i]), __uint_as_float(a[8 * j + 2 * i + 1]));
-                                    ec[i] = __hfma2(r, ab, ec[i]);
-                                }
+                            for (int i = 0; i < 8; ++i) {
+                                const uint32_t word = i < 2 ? rw.x : i < 4 ? rw.y : i < 6 ? rw.z : rw.w;
+                                const uint32_t pr = __byte_perm(word, 0x43434343u, (i & 1) ? 0x4342 : 0x4140);
+                                const __nv_bfloat162 r = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&pr), c192);
+                                ec[i & 3] = __hfma2(r, __floats2bfloat162_rn(a[i].x, a[i].y), ec[i & 3]);
                             }
                         }
                     }
-                    float dot = d0 + d1;
+                    float dot = d2.x + d2.y;
                     if (BIDIR) {
                         // dm = <S, R> (formed in the prologue) + sum_i <dq^_i, dQ^_i> + sum_j <dk^_j, dK^_j>,
                         // dx^ the rounding residuals: exact to second order in the bf16 roundings.
@@ -865,32 +863,23 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     }
                     // out = sc (a - coef x^), rounded to bf16 once
                     const float sc = cfac * rn.x, mc = -(dot * rn.y) * sc;
+                    const float2 sc2 = make_float2(sc, sc), mc2 = make_float2(mc, mc);
 #pragma unroll 1
-                    for (int hf = 0; hf < 2; ++hf) {
-                        uint32_t a[32];
-                        tmem_ld32(tacc + hf * 32, a);
+                    for (int pc = 0; pc < 4; ++pc) {
+                        float2 a[8];
+                        tmem_ld16(tacc + pc * 16, reinterpret_cast<uint32_t*>(a));
+                        uint4 w[2], o[2];
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) w[j] = *reinterpret_cast<const uint4*>(tile + swz(row, 2 * pc + j));
                         tmem_wait_ld();
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const uint4 w = *reinterpret_cast<const uint4*>(tile + swz(row, hf * 4 + j));
-                            const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&w);
-                            uint4 o;
-                            uint32_t* ow = reinterpret_cast<uint32_t*>(&o);
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const float2 f = __bfloat1622float2(e[i]);
-                                ow[i] = pack_bf16(fmaf(f.x, mc, __uint_as_float(a[8 * j + 2 * i]) * sc),
-                                                  fmaf(f.y, mc, __uint_as_float(a[8 * j + 2 * i + 1]) * sc));
-                            }
-                            if (VARLEN && ragged_last && c == n_chunks - 1) {
-                                const long long grow = (long long)chunk_row(c) + row;
-                                if (grow < tok1 && (hf * 4 + j) * 8 < p.out_w[hw])
-                                    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out_rows[hw]) + grow * p.out_sn[hw] +
-                                                              (long long)h * p.out_sh[hw] + (hf * 4 + j) * 8) = o;
-                            } else {
-                                *reinterpret_cast<uint4*>(out_tile + swz(row, hf * 4 + j)) = o;
-                            }
+                        for (int i = 0; i < 8; ++i) {
+                            const float2 v = __ffma2_rn(__bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[i]), mc2,
+                                                        __fmul2_rn(a[i], sc2));
+                            reinterpret_cast<uint32_t*>(o)[i] = pack_bf16(v.x, v.y);
                         }
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) put(out_tile, hw, c, 2 * pc + j, o[j]);
                     }
                 }
                 fence_proxy_async();
@@ -904,46 +893,35 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 if (!wait(bars + B_STQFREE, (uint32_t)(c & 1))) break;
                 tc_fence_after();
                 {
-                    uint32_t a[32];
-                    tmem_ld32(tmem + lane_base + colP2 + 64 + hw * 32, a);
-                    tmem_wait_ld();
-                    tc_fence_before();
-                    mbar_arrive(bar(B_OVFREE, c));     // the P columns may take the next chunk's scores
-                    uint8_t* tile = gbase + L::kOffStQ;
-                    if (SEG && (long long)chunk_row(c) + row < tok1) {
-                        // dm of a segment: <dV'_j, v_j> of the unscaled accumulator with the raw v row
-                        // (the copy thread keeps the v tile until this epilogue is done)
-                        const uint8_t* vt = stage_g(c) + L::kOffV;
-                        float t0 = 0.f, t1 = 0.f;
+                    const uint8_t* vt = stage_g(c) + L::kOffV;
+                    const bool vrow = SEG && (long long)chunk_row(c) + row < tok1;
+                    float2 t2 = make_float2(0.f, 0.f);
+                    const float2 cf2 = make_float2(cfac, cfac);
+#pragma unroll 1
+                    for (int pc = 0; pc < 2; ++pc) {
+                        float2 a[8];
+                        tmem_ld16(tmem + lane_base + colP2 + 64 + hw * 32 + pc * 16, reinterpret_cast<uint32_t*>(a));
+                        tmem_wait_ld();
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const uint4 w = *reinterpret_cast<const uint4*>(vt + swz(row, hw * 4 + j));
-                            const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&w);
+                        for (int j = 0; j < 2; ++j) {
+                            const int jj = hw * 4 + pc * 2 + j;
+                            if (SEG && vrow) {
+                                const uint4 w = *reinterpret_cast<const uint4*>(vt + swz(row, jj));
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) t2 = __ffma2_rn(__bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&w)[i]), a[4 * j + i], t2);
+                            }
+                            uint4 o;
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
-                                const float2 f = __bfloat1622float2(e[i]);
-                                t0 = fmaf(f.x, __uint_as_float(a[8 * j + 2 * i]), t0);
-                                t1 = fmaf(f.y, __uint_as_float(a[8 * j + 2 * i + 1]), t1);
+                                const float2 v = __fmul2_rn(a[4 * j + i], cf2);
+                                reinterpret_cast<uint32_t*>(&o)[i] = pack_bf16(v.x, v.y);
                             }
-                        }
-                        dm_acc += t0 + t1;
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        uint4 o;
-                        o.x = pack_bf16(__uint_as_float(a[8 * j]) * cfac, __uint_as_float(a[8 * j + 1]) * cfac);
-                        o.y = pack_bf16(__uint_as_float(a[8 * j + 2]) * cfac, __uint_as_float(a[8 * j + 3]) * cfac);
-                        o.z = pack_bf16(__uint_as_float(a[8 * j + 4]) * cfac, __uint_as_float(a[8 * j + 5]) * cfac);
-                        o.w = pack_bf16(__uint_as_float(a[8 * j + 6]) * cfac, __uint_as_float(a[8 * j + 7]) * cfac);
-                        if (VARLEN && ragged_last && c == n_chunks - 1) {
-                            const long long grow = (long long)chunk_row(c) + row;
-                            if (grow < tok1 && (hw * 4 + j) * 8 < p.out_w[2])
-                                *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out_rows[2]) + grow * p.out_sn[2] +
-                                                          (long long)h * p.out_sh[2] + (hw * 4 + j) * 8) = o;
-                        } else {
-                            *reinterpret_cast<uint4*>(tile + swz(row, hw * 4 + j)) = o;
+                            put(gbase + L::kOffStQ, 2, c, jj, o);
                         }
                     }
+                    tc_fence_before();
+                    mbar_arrive(bar(B_OVFREE, c));     // the P columns may take the next chunk's scores
+                    if (SEG) dm_acc += t2.x + t2.y;
                 }
                 fence_proxy_async();
                 mbar_arrive(bar(B_EVDONE, c));
