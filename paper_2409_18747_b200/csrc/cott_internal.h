@@ -200,8 +200,13 @@ cudaError_t launch_tc_short_fwd(const void* q, const void* k, const void* v, voi
                                 const float* seq_len, float seq_len_scalar, int B, int H, int N, int d, int dk, int dv,
                                 int causal, cudaStream_t st);
 
-// A block of at most 64 tokens per (b, h) on a caller's state (cott_tc_block.cu): o and the new
-// state in one launch, the only kernel of its call.
+// A block of at most 64 tokens per (b, h) on a caller's state, o and the new state in one launch, the
+// only kernel of its call.  launch_block_fwd (cott_block.cu): the state streams through registers, any
+// dk, dv up to 128.  launch_tc_block_fwd (cott_tc_block.cu): the state in tensor memory, d x d.
+cudaError_t launch_block_fwd(const void* q, const void* k, const void* v, void* o, const RowLayout& l_qk,
+                             const RowLayout& l_v, const RowLayout& l_o, const float* state_in, float* state_out,
+                             int* status, const float* m, const float* seq_len, float seq_len_scalar, int B, int H,
+                             int N, int dk, int dv, cudaStream_t st);
 cudaError_t launch_tc_block_fwd(const void* q, const void* k, const void* v, void* o, const RowLayout& l_qk,
                                 const RowLayout& l_v, const RowLayout& l_o, const float* state_in, float* state_out,
                                 int* status, const float* m, const float* seq_len, float seq_len_scalar, int B, int H,

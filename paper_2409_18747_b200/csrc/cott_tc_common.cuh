@@ -48,6 +48,23 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
     return wait_slow(bar, parity, abort_flag);
 }
 
+// The same with the limit checked between a test and a (suspending) try: for a kernel whose only wait is
+// shorter than one suspension, so that its bound is a bound there too.
+static __device__ __noinline__ bool wait_polling(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    const long long t0 = clock64();
+    for (;;) {
+        if (mbar_test_wait(bar, parity)) return true;
+        if (*abort_flag) return false;
+        if (clock64() - t0 > ((long long)abort_flag[3] << 10)) {
+            const uint32_t bars = (uint32_t)__cvta_generic_to_shared((const void*)abort_flag) - (uint32_t)kCtlAbort;
+            const uint32_t where = 0x80000000u | ((threadIdx.x >> 5) << 16) | (((bar - bars) & 0x3FFu) << 4) | (parity & 1u);
+            atomicCAS(const_cast<int*>(abort_flag), 0, (int)where);
+            return false;
+        }
+        if (mbar_try_wait(bar, parity)) return true;
+    }
+}
+
 __device__ __forceinline__ uint4 pack8(const uint32_t* r) {
     uint4 w;
     w.x = pack_bf16(__uint_as_float(r[0]), __uint_as_float(r[1]));

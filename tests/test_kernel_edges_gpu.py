@@ -68,3 +68,27 @@ def test_backward_d128_chunk_and_group_edges(N, group, dk, dv, causal, force_gro
         # over random shapes of this size for bf16 operands
         cond = dm_condition(rv, c["v"], c["m"], None)
         assert (abs(dm.double().cpu().numpy() - rm) <= 1e-3 * cond).all()
+
+
+@pytest.mark.parametrize("T", [1, 8, 15, 16, 17, 32, 48, 49, 64])
+@pytest.mark.parametrize("dk,dv", [(128, 128), (64, 64), (8, 8), (24, 104), (120, 72)])
+def test_token_block_edges(T, dk, dv):
+    """The token-block kernel (tiles of 16 tokens, strips of 32 value columns, steps of 16 key rows):
+    edges of each, with and without a state on either side."""
+    B, H = 2, 3
+    c = synth.make_qkv(B, H, T, dk, torch.bfloat16, 7500 + T + dk, row_lognormal=True, d_v=dv)
+    c["k"][1, 1, T // 2] = 0.0
+    s = 300.0
+    g = torch.Generator().manual_seed(3)
+    state = torch.randn((B, H, dk, dv), generator=g)
+    q, k, v, m = (dev(c[x]) for x in ("q", "k", "v", "m"))
+    for st in (state, torch.zeros(B, H, dk, dv)):
+        given = st is state
+        if not given and (dk != dv or T == 1):     # (one token alone: a row of a single term, four roundings deep)
+            continue
+        o, st_out = cott.fwd_stateful(q, k, v, m, s, state_in=dev(st) if given else None)
+        r_o, r_s = oracle.fwd_segment(c["q"], c["k"], c["v"], c["m"], st, torch.tensor([s] * B))
+        gate(o, r_o, torch.bfloat16)
+        assert norm_max_err(st_out, r_s) <= 1e-2
+    o2 = cott.fwd_stateful(q, k, v, m, s, state_in=dev(state), return_state=False)
+    assert torch.equal(o2, cott.fwd_stateful(q, k, v, m, s, state_in=dev(state))[0])
