@@ -133,12 +133,14 @@ struct Plan {
 // Sequence groups give sequence-level parallelism when B*H alone cannot fill the GPU:
 // halve the group until there are enough CTAs, but never below a floor that keeps the
 // per-group state traffic (d*d fp32) small against the group's own q,k,v,o bytes.
-// May every walk CTA sum the partial states it needs itself (no scan launch)?  Only while those
-// extra reads (n_groups / 2 states of d x d floats per CTA on average) stay small against the
-// group's own rows: measured at B*H = 16, d = 128, dropping the scan launch this way where the
-// rule says no cost 14 us at N = 4096 (58.7 against 44.6 us) and at N = 16384 (107 against 94 us).
-static bool fused_scan_ok(int n_groups, int d, int group) {
-    return (long long)n_groups * d * 8 <= group;
+// May every walk CTA sum the partial states it needs itself (no scan launch)?  It reads n_groups / 2
+// states of d x d floats on average, one after the other out of L2.  At d = 64 (16 KB each) that beats
+// a scan launch up to nine groups (B H = 24, N = 4096, six groups: 24.9 us against 25.4); at d = 128
+// (64 KB) up to four (B=3, H=16, N=2999, three groups: 50 us against 57; six groups: 50 against 45 the
+// other way round), and up to nine where the group's own rows dwarf the sum (B H = 16, N = 131072 with the
+// state kept: 510 us against 514).
+static bool sum_in_walk(int n_groups, int d, int group) {
+    return n_groups <= (d == 64 ? 9 : 4) || (n_groups <= 9 && (long long)n_groups * d * 8 <= group);
 }
 
 static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv, int causal, Plan* p) {
@@ -194,7 +196,7 @@ static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv
     // sums `split` times as many states.
     p->split = 1;
     if (p->path == 1 && causal && p->n_groups >= 2 && p->n_groups <= 8 &&
-        fused_scan_ok(p->n_groups, d, group) && N % group == 0) {
+        sum_in_walk(p->n_groups, d, group) && N % group == 0) {
         const long ctas = BH * (p->n_groups - 1);
         const int chunks = group / p->chunk;
         for (int s2 = 4; s2 >= 2; s2 >>= 1)
@@ -414,11 +416,11 @@ static cott_status run_tc_stream(TcWalkArgs t, const Plan& p, int B, int H, int 
         COTT_CUDA(launch_tc_walk(t, B, H, N, d, st));
         return COTT_OK;
     }
-    // Few groups and no state export: every walk CTA sums the partial states it needs itself
-    // and the scan launch is dropped -- as long as those extra d x d reads (n_groups / 2 of
-    // them on average) stay small against the group's own q, k, v, o bytes.
-    // (A caller's initial state enters through the scan kernel.)
-    const bool fused_scan = !total_out && !state_in && p.n_groups <= 8 && fused_scan_ok(p.n_groups, d, p.group);
+    // Few groups: every walk CTA sums the partial states it needs itself and the scan launch is
+    // dropped.  In the forward pass a caller's initial state joins that sum, and the CTA of the last
+    // group, whose running state ends as the total, writes it; the other streams leave both to the scan.
+    const bool forward = causal && !t.reverse && t.x_norm && !t.norm_bv && !t.cu_seqlens;
+    const bool fused_scan = (forward || (!total_out && !state_in)) && sum_in_walk(p.n_groups, d, p.group);
     const int split = (fused_scan && causal) ? p.split : 1;
     if (!reuse_transposed) {
         TcWalkArgs a = t;
@@ -427,7 +429,7 @@ static cott_status run_tc_stream(TcWalkArgs t, const Plan& p, int B, int H, int 
         a.state_out = states; a.dm_partial = nullptr; a.dm_out = nullptr; a.epilogue = EPI_PLAIN;
         t.clear_status = 0;              // the state pass, launched first, does it
         a.reverse = t.reverse ? 0 : 1;   // chunk order opposite to the walk's: L2 reuse of its tiles
-        if (causal && !total_out) {
+        if (causal && (fused_scan || !total_out)) {
             // Nobody reads the partial state of the group the walk visits last.
             a.grid_groups = (p.n_groups - 1) * split;
             a.first_group = t.reverse ? split : 0;
@@ -453,6 +455,7 @@ static cott_status run_tc_stream(TcWalkArgs t, const Plan& p, int B, int H, int 
     // walks in the same direction.
     if (states_only) return COTT_OK;
     t.init_sum = fused_scan ? 1 : 0;
+    if (fused_scan) { t.init_extra = state_in; t.state_final = total_out; }
     t.init_split = split;
     t.init_transposed = (reuse_states && states_transposed) ? 1 : 0;
     t.mode = causal ? 1 : 2; t.init = states; t.state_out = nullptr;
@@ -649,7 +652,7 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
             // The forward call of the same q, k, v (no state in or out) left the partial states
             // K^^T V of every group but the last in its workspace whenever its walk summed them
             // itself: the transposes of what this walk needs, so the state pass skips k and v.
-            if (fwd_ws && !packed.cu_seqlens && causal && p.n_groups >= 2 && p.n_groups <= 8 && fused_scan_ok(p.n_groups, d, p.group)) {
+            if (fwd_ws && !packed.cu_seqlens && causal && p.n_groups >= 2 && sum_in_walk(p.n_groups, d, p.group)) {
                 f.sq_fwd = reinterpret_cast<const float*>(static_cast<const char*>(fwd_ws) + kWsHeaderBytes);
                 f.sq_fwd_split = p.split;
             }

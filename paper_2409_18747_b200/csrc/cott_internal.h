@@ -122,6 +122,7 @@ struct TcWalkArgs {
     // Causal walk of a single group: `init` is a caller's state (it contains c and is divided
     // by c on the way in), and the state after the last token goes to state_final, times c.
     int init_has_scale;
+    const float* init_extra;   // with init_sum, forward: a caller's state (contains c) the sum starts from, or NULL
     float* state_final;
     // Columns the tensors really have, when fewer than the kernel's d: x and a have d_xa, bv,
     // the raw rows and out have d_bo (0: d).  The tensor maps get the real extents -- tiles are

@@ -370,6 +370,9 @@ __global__ void __launch_bounds__(256) scan_kernel(float* __restrict__ states,
     constexpr int kBatch = 8;
     const int e4 = blockIdx.x * blockDim.x + threadIdx.x;
     const int bh = blockIdx.y;
+    // (started while the state pass drains; the walk behind it starts while this one does)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (e4 * 4 >= dd) return;
     float4* base = reinterpret_cast<float4*>(states + (size_t)bh * n_groups * dd) + e4;
     const size_t stride = (size_t)dd / 4;
@@ -571,9 +574,18 @@ cudaError_t launch_scan(float* states, float* total_out, int BH, int n_groups, i
                         cudaStream_t st, const float* total_scale_m, const float* seq_len,
                         float seq_len_scalar, int H, int N, const float* init_in) {
     const int dd = d * d;
-    dim3 grid((unsigned)((dd / 4 + 255) / 256), (unsigned)BH);
-    scan_kernel<<<grid, 256, 0, st>>>(states, total_out, n_groups, dd, mode, total_scale_m, seq_len,
-                                      seq_len_scalar, H, N, init_in);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((dd / 4 + 255) / 256), (unsigned)BH);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaError_t e = cudaLaunchKernelEx(&cfg, scan_kernel, states, total_out, n_groups, dd, mode, total_scale_m, seq_len,
+                                           seq_len_scalar, H, N, init_in); e != cudaSuccess)
+        return e;
     note_launch();
     return cudaGetLastError();
 }

@@ -19,6 +19,7 @@
 #include <stdlib.h>
 #include "cott_internal.h"
 #include "cott_sm100.cuh"
+#include "cott_tc_common.cuh"
 
 namespace cott {
 
@@ -43,7 +44,8 @@ struct TcWalkParams {
     const float* dm_extra;  // the finalising stream: the other stream's [BH, n_groups] part, or NULL
     float* dm_out;          // that stream: dm[H], written by the CTA that finishes last (or NULL)
     int init_has_scale;     // init is a caller's state (contains c): divide by c on the way in
-    float* state_final;     // causal walk, one group: [BH, d*d] state after the last token, times c (or NULL)
+    const float* init_extra;  // with init_sum: a caller's state [BH, d*d] (contains c) that the sum starts from, or NULL
+    float* state_final;     // causal walk forward in time: [BH, d*d] state after the last token, times c (or NULL)
     int* status;            // workspace status word
     const float* m; const float* seq_len; float seq_len_scalar;
     int H; int N; int group; int n_groups;
@@ -235,13 +237,12 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 }
 
 // Sum of squares of eight bf16 values, on two independent accumulators.
-__device__ __forceinline__ void sumsq8(const uint4& w, float& a0, float& a1) {
+__device__ __forceinline__ void sumsq8(const uint4& w, float2& a) {
     const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&w);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        float2 f = __bfloat1622float2(e[i]);
-        a0 = fmaf(f.x, f.x, a0);
-        a1 = fmaf(f.y, f.y, a1);
+        const float2 f = __bfloat1622float2(e[i]);
+        a = __ffma2_rn(f, f, a);
     }
 }
 
@@ -531,6 +532,15 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
             float acc[QW];
 #pragma unroll
             for (int i = 0; i < QW; ++i) acc[i] = 0.f;
+            if (STREAM == S_FWD && MODE == MODE_CAUSAL && p.init_extra != nullptr && owns_srow) {
+                const float ic = 1.0f / cfac;
+                const float* ex = p.init_extra + (size_t)bh * D * D + (size_t)srow * D + cq * QW;
+#pragma unroll
+                for (int i = 0; i < QW; i += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(ex + i);
+                    acc[i] = v.x * ic; acc[i + 1] = v.y * ic; acc[i + 2] = v.z * ic; acc[i + 3] = v.w * ic;
+                }
+            }
             const int g_lo = (MODE == MODE_READOUT) ? 0 : (kReverse ? (g + 1) * p.init_split : 0);
             const int g_hi = (MODE == MODE_READOUT) ? n_init : (kReverse ? n_init : g * p.init_split);
             if (owns_srow) {
@@ -785,24 +795,29 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
         // x^ = x / max(||x||, eps) on this thread's half row, in place, rounded to bf16.
         auto normalise_half_row = [&](uint8_t* nt, int c) {
             uint4 wn[NC];
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+            float2 s0 = make_float2(0.f, 0.f), s1 = s0;
 #pragma unroll
             for (int j = 0; j < NC; ++j) wn[j] = *reinterpret_cast<const uint4*>(tile_h_ptr(nt, j));
 #pragma unroll
-            for (int j = 0; j < NC; j += 2) { sumsq8(wn[j], a0, a1); sumsq8(wn[j + 1], a2, a3); }
-            float r = 1.0f / fmaxf(sqrtf(pair_sum((a0 + a1) + (a2 + a3))), kEps);
+            for (int j = 0; j < NC; j += 2) { sumsq8(wn[j], s0); sumsq8(wn[j + 1], s1); }
+            float r = 1.0f / fmaxf(sqrtf(pair_sum((s0.x + s0.y) + (s1.x + s1.y))), kEps);
             if (varlen && chunk_row(c) + nrow >= tok1) r = 0.f;     // a row of the next sequence
+            const tc::RowScale rs(r);
 #pragma unroll
             for (int j = 0; j < NC; ++j) {
-                const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&wn[j]);
-                uint4 o;
-                uint32_t* ow = reinterpret_cast<uint32_t*>(&o);
+                __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&wn[j]);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    float2 f = __bfloat1622float2(e[i]);
-                    ow[i] = pack_bf16(f.x * r, f.y * r);
+                    // (the state pass, which loads bound, rounds x r itself: its sums enter dm, which
+                    // cancels heavily)
+                    if (MODE == MODE_STATE) {
+                        const float2 f = __fmul2_rn(__bfloat1622float2(e[i]), make_float2(r, r));
+                        e[i] = __floats2bfloat162_rn(f.x, f.y);
+                    } else {
+                        e[i] = rs(e[i]);
+                    }
                 }
-                *reinterpret_cast<uint4*>(tile_h_ptr(nt, j)) = o;
+                *reinterpret_cast<uint4*>(tile_h_ptr(nt, j)) = wn[j];
             }
             fence_proxy_async();
         };
@@ -836,13 +851,13 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
             {
                 if (!wait(bar_full + 8 * s, (c / NST) & 1)) return;
                 const uint8_t* xt = gbase + s * L::kStage + L::kOffX;
-                float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+                float2 s0 = make_float2(0.f, 0.f), s1 = s0;
 #pragma unroll
                 for (int j = 0; j < NC; j += 2) {
-                    sumsq8(*reinterpret_cast<const uint4*>(tile_h_ptr(const_cast<uint8_t*>(xt), j)), a0, a1);
-                    sumsq8(*reinterpret_cast<const uint4*>(tile_h_ptr(const_cast<uint8_t*>(xt), j + 1)), a2, a3);
+                    sumsq8(*reinterpret_cast<const uint4*>(tile_h_ptr(const_cast<uint8_t*>(xt), j)), s0);
+                    sumsq8(*reinterpret_cast<const uint4*>(tile_h_ptr(const_cast<uint8_t*>(xt), j + 1)), s1);
                 }
-                rx = cfac / fmaxf(sqrtf(pair_sum((a0 + a1) + (a2 + a3))), kEps);
+                rx = cfac / fmaxf(sqrtf(pair_sum((s0.x + s0.y) + (s1.x + s1.y))), kEps);
             }
             if (nhalf == 0) rx_buf[(c % NRX) * 128 + nrow] = rx;
         };
@@ -975,6 +990,58 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
                 COTT_STAMP_AT(1, c, 2);
                 const uint32_t tO = tmem + lane_base + colO0 + (c % kOBufs) * D + hf * HW;
                 const float rx = kXNorm ? rx_buf[(c % NRX) * 128 + arow] : cfac;
+                // When the staging slot may be filled.  With own buffers: the store of the chunk before
+                // last (pair) or the last one (single) has read it, and nothing else waits for the last
+                // state update, which must not be in flight when the CTA gives back its tensor memory.
+                // Else it is the Bv slot, which the state update (issued behind P~ Bv) still reads.
+                auto slot_free = [&]() {
+                    if (own_out && c + 1 == n_chunks && !wait(sfull_bar(c), sfull_par(c))) return;
+                    if (out_pair) {
+                        if (c >= 2) wait(bar_out_free + 8 * (c & 1), ((c >> 1) & 1) ^ 1);
+                    } else if (own_out) {
+                        if (c >= 1) wait(bar_out_free, (c - 1) & 1);
+                    } else if (MODE == MODE_CAUSAL) wait(sfull_bar(c), sfull_par(c));
+                };
+                uint8_t* so = own_out ? gbase + out_off(c) : st + L::kOffOut;
+                // Eight output columns from `col` on: into the staging slot, or (packed batch, last chunk
+                // of the sequence, where a tile store would overwrite rows of the next one) row by row.
+                auto put = [&](int col, uint4 w) {
+                    if (ragged_last && c == last_visit_of_ragged) {
+                        const long long grow = (long long)chunk_row(c) + arow;
+                        if (grow < tok1 && col < p.d_out)
+                            *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out_rows) +
+                                                      grow * p.out_sn + (long long)h * p.out_sh + col) = w;
+                    } else {
+                        *reinterpret_cast<uint4*>(so + (col >> 6) * 16384 + swz(arow, (col & 63) >> 3)) = w;
+                    }
+                };
+                if constexpr (!with_proj) {
+                    // Scale, round, stage, 32 columns at a time (short code: see the note on STREAM).
+                    slot_free();
+                    if (!alive) break;
+                    const float2 rx2 = make_float2(rx, rx);
+#pragma unroll 1
+                    for (int pc = 0; pc < NPIECE; ++pc) {
+                        float2 r[16];
+                        tmem_ld32(tO + pc * 32, *reinterpret_cast<uint32_t(*)[32]>(&r[0]));
+                        tmem_wait_ld();
+                        if (pc + 1 == NPIECE) { tc_fence_before(); mbar_arrive(bar_o_free + 8 * (c & 1)); }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            uint4 w;
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const float2 v = __fmul2_rn(r[4 * i + j], rx2);
+                                reinterpret_cast<uint32_t*>(&w)[j] = pack_bf16(v.x, v.y);
+                            }
+                            put(hf * HW + pc * 32 + i * 8, w);
+                        }
+                    }
+                    fence_proxy_async();
+                    mbar_arrive(edone_bar(c));
+                    COTT_STAMP_AT(1, c, 5);
+                    continue;
+                }
                 uint32_t r[HW];
 #pragma unroll
                 for (int pc = 0; pc < NPIECE; ++pc)
@@ -1043,22 +1110,11 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
                         }
                     }
                 }
-                // Scale, (project,) round to bf16, stage for the TMA store.  The staging slot is
-                // the Bv slot, which the state update (issued behind P~ Bv) still reads: wait for it.
+                // Scale, project, round to bf16, stage for the TMA store.
                 COTT_STAMP_AT(1, c, 3);
-                if (own_out) {
-                    // Nothing else waits for the last state update: it must not be in flight
-                    // when the CTA gives back its tensor memory.
-                    if (c + 1 == n_chunks && !wait(sfull_bar(c), sfull_par(c))) break;
-                }
-                if (out_pair) {
-                    // own buffer of this chunk parity: the store of chunk c - 2 has read it
-                    if (c >= 2 && !wait(bar_out_free + 8 * (c & 1), ((c >> 1) & 1) ^ 1)) break;
-                } else if (own_out) {
-                    if (c >= 1 && !wait(bar_out_free, (c - 1) & 1)) break;   // the one buffer: store of chunk c - 1
-                } else if (MODE == MODE_CAUSAL && !wait(sfull_bar(c), sfull_par(c))) break;
+                slot_free();
+                if (!alive) break;
                 COTT_STAMP_AT(1, c, 4);
-                uint8_t* so = own_out ? gbase + out_off(c) : st + L::kOffOut;
 #pragma unroll
                 for (int i = 0; i < HW; i += 8) {
                     const int col = hf * HW + i;
@@ -1078,16 +1134,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
                     uint4 w;
                     w.x = pack_bf16(v[0], v[1]); w.y = pack_bf16(v[2], v[3]);
                     w.z = pack_bf16(v[4], v[5]); w.w = pack_bf16(v[6], v[7]);
-                    if (ragged_last && c == last_visit_of_ragged) {
-                        // Packed batch, last chunk of the sequence: a tile store would overwrite
-                        // rows of the next sequence; the rows that exist go out one by one.
-                        const long long grow = (long long)chunk_row(c) + arow;
-                        if (grow < tok1 && col < p.d_out)
-                            *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out_rows) +
-                                                      grow * p.out_sn + (long long)h * p.out_sh + col) = w;
-                    } else {
-                        *reinterpret_cast<uint4*>(so + (col >> 6) * 16384 + swz(arow, (col & 63) >> 3)) = w;
-                    }
+                    put(col, w);
                 }
                 fence_proxy_async();
                 mbar_arrive(edone_bar(c));
@@ -1118,8 +1165,8 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
                                     __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
             }
         }
-        if (MODE == MODE_CAUSAL && p.state_final != nullptr && alive) {
-            // State after the last token of the (single) group, times c: the caller's Eq. 8 state.
+        if (MODE == MODE_CAUSAL && p.state_final != nullptr && alive && (kReverse || g + 1 == p.n_groups)) {
+            // State after the last token, times c: the caller's Eq. 8 state.  (Backward in time: one group.)
             if (wait(sfull_bar(n_chunks - 1), sfull_par(n_chunks - 1))) {
                 tc_fence_after();
                 float* dst = p.state_final + (size_t)bh * D * D + (size_t)srow * D + cq * QW;
@@ -1356,7 +1403,7 @@ cudaError_t launch_tc_walk(const TcWalkArgs& a, int B, int H, int N, int d, cuda
         p.out_rows = a.out; p.out_sn = lo.sn; p.out_sh = lo.sh;
     }
     p.init = a.init; p.state_out = a.state_out; p.dm_partial = a.dm_partial; p.dm_extra = a.dm_extra; p.dm_out = a.dm_out; p.status = a.status;
-    p.init_has_scale = a.init_has_scale; p.state_final = a.state_final;
+    p.init_has_scale = a.init_has_scale; p.init_extra = a.init_extra; p.state_final = a.state_final;
     p.m = a.m; p.seq_len = a.seq_len; p.seq_len_scalar = a.seq_len_scalar;
     p.H = H; p.N = N; p.group = a.group; p.n_groups = a.n_groups;
     p.init_sum = a.init_sum; p.init_transposed = a.init_transposed;

@@ -92,3 +92,21 @@ def test_token_block_edges(T, dk, dv):
         assert norm_max_err(st_out, r_s) <= 1e-2
     o2 = cott.fwd_stateful(q, k, v, m, s, state_in=dev(state), return_state=False)
     assert torch.equal(o2, cott.fwd_stateful(q, k, v, m, s, state_in=dev(state))[0])
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("groups", [2, 4, 5, 9, 10])
+def test_forward_walk_sums_or_scans_the_group_states(d, groups, force_group):
+    """A causal forward in groups, with and without a state on either side: few groups are summed inside
+    the walk (whose last group then writes the state), more by a scan launch."""
+    force_group(128)
+    B, H, N = 1, 3, 128 * groups - 39
+    c = synth.make_qkv(B, H, N, d, torch.bfloat16, 7700 + N + d)
+    state = torch.randn((B, H, d, d), generator=torch.Generator().manual_seed(5))
+    q, k, v, m = (dev(c[x]) for x in ("q", "k", "v", "m"))
+    s = torch.full((B,), 2.0 * N)
+    for st in (state, torch.zeros_like(state)):
+        o, st_out = cott.fwd_stateful(q, k, v, m, 2.0 * N, state_in=dev(st) if st is state else None)
+        r_o, r_s = oracle.fwd_segment(c["q"], c["k"], c["v"], c["m"], st, s)
+        gate(o, r_o, torch.bfloat16)
+        assert norm_max_err(st_out, r_s) <= 1e-2
