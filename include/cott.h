@@ -25,7 +25,7 @@
  * All calls are asynchronous on `stream` (a cudaStream_t passed as void*; NULL is
  * the legacy default stream).  The returned status covers argument validation and
  * launch errors only.  cott_fwd*, cott_bwd* and cott_decode_step* with caller-owned outputs
- * and workspaces put only kernel launches and memsets on the stream (and, where gradient streams
+ * and workspaces put only kernel launches on the stream (and, where gradient streams
  * run side by side, event-ordered work on the library's streams): once each kernel has been
  * launched at least once on the device, such calls can be captured in a CUDA graph and
  * replayed.  Calls are thread-safe as long as concurrent calls use
@@ -81,7 +81,9 @@ const char* cott_status_string(cott_status st);
 /* Text of the last CUDA error seen by this thread inside the library (static storage). */
 const char* cott_last_cuda_error(void);
 
-/* Number of kernels this process has launched through the library so far (all threads). */
+/* Number of kernels this process has launched through the library so far (all threads); the one-warp
+ * kernel that clears the status words in front of some backward calls, like the memset it stands
+ * for, is not counted. */
 unsigned long long cott_launch_count(void);
 
 /*

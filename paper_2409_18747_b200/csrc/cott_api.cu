@@ -353,9 +353,9 @@ static cott_status run_streams(const SimtStream* s, int n, const Plan& p, int BH
             wb.w[i].init_extra = s[i].state_in; wb.w[i].update = 1; wb.w[i].write_out = 1;
             wb.w[i].final_state = s[i].total_out;
         }
-        if (wants_dm) COTT_CUDA(cudaMemsetAsync(status, 0, kWsHeaderBytes, st));   // (the CTA counter of dm)
+        if (wants_dm) COTT_CUDA(launch_clear_status(status, st));   // (the CTA counter of dm)
         wb.clear_status = wants_dm ? 0 : 1;
-        COTT_CUDA(launch_walk_simt(wb, n, BH, d, dt, st, false));
+        COTT_CUDA(launch_walk_simt(wb, n, BH, d, dt, st, wants_dm));
         return COTT_OK;
     }
     // Every walk CTA sums the partial states before its group itself while they are few: at most
@@ -682,8 +682,7 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
             if (causal && !packed.cu_seqlens && p.n_groups == 1 && N <= 128) {
                 // One chunk per (b, h): no state is ever read, the walk is the only launch.
                 f.sq_part = nullptr; f.r_part = nullptr;
-                COTT_CUDA(cudaMemsetAsync(ws, 0, kWsHeaderBytes, st));      // status words and the dm counter
-                f.plain_launch = 1;
+                COTT_CUDA(launch_clear_status(status, st));      // status words and the dm counter
                 COTT_CUDA(launch_tc_bwd_fused(f, B, H, N, st));
                 return COTT_OK;
             }
@@ -692,7 +691,7 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
                 // dm in one launch (cott_tc_bidir_bwd.cu), nothing but q, k, v, dO read and dq, dk, dv
                 // written.  (A CTA walks its sequence twice with two tile pairs in flight: beyond
                 // eight chunks the two-launch form with its deeper rings is as fast or faster.)
-                COTT_CUDA(cudaMemsetAsync(ws, 0, kWsHeaderBytes, st));      // status words and the dm counter
+                COTT_CUDA(launch_clear_status(status, st));      // status words and the dm counter
                 COTT_CUDA(launch_tc_bidir_bwd(f, B, H, N, st));
                 return COTT_OK;
             }
@@ -826,9 +825,9 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
                 }
                 f.sq_part = st0; f.r_part = st1;
             } else {
-                COTT_CUDA(cudaMemsetAsync(ws, 0, kWsHeaderBytes, st));      // status words and the dm counter
+                COTT_CUDA(launch_clear_status(status, st));      // status words and the dm counter
             }
-            COTT_CUDA(launch_tc_bwd128(f, in_walk ? 1 : 0, dm_partial2, states ? 0 : 1, B, H, N, st));
+            COTT_CUDA(launch_tc_bwd128(f, in_walk ? 1 : 0, dm_partial2, B, H, N, st));
             return COTT_OK;
         }
         if (ss) {

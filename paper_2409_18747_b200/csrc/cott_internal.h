@@ -76,6 +76,7 @@ struct WalkBatch {
 cudaError_t launch_walk_simt(const WalkBatch& wb, int n, int BH, int d, cott_dtype dt, cudaStream_t st, bool dependent);
 // `total_scale_m` non-NULL: the total written to total_out is multiplied by the stabilisation
 // factor c[b,h] (the tensor-core path keeps its states unscaled).
+cudaError_t launch_clear_status(int* status, cudaStream_t st);
 cudaError_t launch_scan(float* states, float* total_out, int BH, int n_groups, int d, int mode,
                         cudaStream_t st, const float* total_scale_m = nullptr,
                         const float* seq_len = nullptr, float seq_len_scalar = 0.f, int H = 1,
@@ -167,9 +168,8 @@ cudaError_t launch_tc_bwd_fused(const TcBwdFusedArgs& a, int B, int H, int N, cu
 cudaError_t launch_tc_bidir_bwd(const TcBwdFusedArgs& a, int B, int H, int N, cudaStream_t st);
 // Backward at d = 128 in one launch of two kinds of walks (cott_tc_bwd128.cu): sq_part / r_part are the
 // groups' V^T K^ and dO^T Q^ (both NULL with one causal group), raw with init_sum, else scanned;
-// dm_k: [BH, n_groups] beside dm_partial; clear_status: no kernel of the call comes before it.
-cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, int init_sum, float* dm_k, int clear_status, int B, int H, int N,
-                             cudaStream_t st);
+// dm_k: [BH, n_groups] beside dm_partial.
+cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, int init_sum, float* dm_k, int B, int H, int N, cudaStream_t st);
 // Both partial states of every group in one launch (uses q, k, v, d_o, the layouts, group,
 // n_groups and status of `a`); clear_status: this is the first kernel of a library call.
 cudaError_t launch_tc_bwd_states(const TcBwdFusedArgs& a, float* sq_out, float* r_out, int clear_status, int B, int H,

@@ -270,21 +270,10 @@ tc_bidir_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             // c / max(||q||, eps): each of the two threads of a row sums the whole row (cheaper
             // than meeting through shared memory)
             const uint8_t* qt = gbase + (c & 3) * kTile;
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+            uint4 xr[8];
 #pragma unroll
-            for (int j = 0; j < 8; j += 2) {
-                const uint4 w0 = *reinterpret_cast<const uint4*>(qt + swz(row, j));
-                const uint4 w1 = *reinterpret_cast<const uint4*>(qt + swz(row, j + 1));
-                const __nv_bfloat162* e0 = reinterpret_cast<const __nv_bfloat162*>(&w0);
-                const __nv_bfloat162* e1 = reinterpret_cast<const __nv_bfloat162*>(&w1);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float2 f0 = __bfloat1622float2(e0[i]), f1 = __bfloat1622float2(e1[i]);
-                    a0 = fmaf(f0.x, f0.x, a0); a1 = fmaf(f0.y, f0.y, a1);
-                    a2 = fmaf(f1.x, f1.x, a2); a3 = fmaf(f1.y, f1.y, a3);
-                }
-            }
-            const float rx = cfac / fmaxf(sqrtf((a0 + a1) + (a2 + a3)), kEps);
+            for (int j = 0; j < 8; ++j) xr[j] = *reinterpret_cast<const uint4*>(qt + swz(row, j));
+            const float rx = cfac / fmaxf(sqrtf(sumsq_row64(xr)), kEps);
             mbar_arrive(bars + B_QREAD + 8 * (c & 3));
             // the product has read the q tile and filled the accumulator: drain it, then stage
             // the rows where q was

@@ -365,63 +365,60 @@ tc_bidir_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         // x^ = x rn in fp32 from the raw row: out = c rn (a - x^ <x^, a> [not clamped]), bf16, written
         // over the raw row.  Returns <x^ - bf16(x^), a>, bf16(x^) the operand phase 1 used.
         float dm_acc = 0.f;
+        // (sixteen bytes of a gradient row, columns 8 j .. + 7: over the raw row, or, in a ragged last
+        // chunk of a packed batch, straight to memory)
+        auto put = [&](uint8_t* tile, int j, int c, int which, uint4 o) {
+            if (VARLEN && ragged_last && c == n_chunks - 1) {
+                const long long grow = (long long)chunk_row(c) + row;
+                if (grow < tok1 && j * 8 < p.out_w[which])
+                    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out_rows[which]) + grow * p.out_sn[which] +
+                                              (long long)h * p.out_sh[which] + j * 8) = o;
+            } else {
+                *reinterpret_cast<uint4*>(tile + swz(row, j)) = o;
+            }
+        };
         auto project = [&](uint32_t tacc, uint8_t* tile, float rn, bool clamped, int c, int which) {
-            const __nv_bfloat16 hi = __float2bfloat16_rn(rn);
-            const __nv_bfloat16 lo = __float2bfloat16_rn(rn - __bfloat162float(hi));
-            const __nv_bfloat162 hi2 = __halves2bfloat162(hi, hi), lo2 = __halves2bfloat162(lo, lo);
-            float d0 = 0.f, d1 = 0.f, e0 = 0.f, e1 = 0.f;
+            const RowScale rs(rn);
+            float2 d2 = make_float2(0.f, 0.f), e2 = d2;
             // (two sweeps over the accumulator row, the raw row read from the tile chunk by chunk:
             // holding either next to the other does not fit the register budget)
 #pragma unroll 1
             for (int hf = 0; hf < 2; ++hf) {
-                uint32_t a[32];
-                tmem_ld32(tacc + hf * 32, a);
+                float2 a[16];
+                tmem_ld32(tacc + hf * 32, *reinterpret_cast<uint32_t(*)[32]>(&a[0]));
+                uint4 w[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const uint4*>(tile + swz(row, hf * 4 + j));
                 tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint4 wj = *reinterpret_cast<const uint4*>(tile + swz(row, hf * 4 + j));
-                    const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&wj);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        // <x, a> with the raw row (times rn afterwards) and <bf16(x^), a>
-                        const float2 x = __bfloat1622float2(e[i]);
-                        const float2 xh = __bfloat1622float2(__hfma2(e[i], hi2, __hmul2(e[i], lo2)));
-                        const float a0 = __uint_as_float(a[8 * j + 2 * i]), a1 = __uint_as_float(a[8 * j + 2 * i + 1]);
-                        d0 = fmaf(x.x, a0, d0); d1 = fmaf(x.y, a1, d1);
-                        e0 = fmaf(xh.x, a0, e0); e1 = fmaf(xh.y, a1, e1);
-                    }
+                for (int i = 0; i < 16; ++i) {
+                    // <x, a> with the raw row (times rn afterwards) and <bf16(x^), a>
+                    const __nv_bfloat162 x = reinterpret_cast<const __nv_bfloat162*>(w)[i];
+                    d2 = __ffma2_rn(__bfloat1622float2(x), a[i], d2);
+                    e2 = __ffma2_rn(__bfloat1622float2(rs(x)), a[i], e2);
                 }
             }
-            const float dot = (d0 + d1) * rn;                       // <x^, a>
+            const float dot = (d2.x + d2.y) * rn;                       // <x^, a>
             const float sc = cfac * rn, mc = (clamped ? 0.f : -dot * sc) * rn;   // (times rn: applied to the raw row)
+            const float2 sc2 = make_float2(sc, sc), mc2 = make_float2(mc, mc);
 #pragma unroll 1
             for (int hf = 0; hf < 2; ++hf) {
-                uint32_t a[32];
-                tmem_ld32(tacc + hf * 32, a);
+                float2 a[16];
+                tmem_ld32(tacc + hf * 32, *reinterpret_cast<uint32_t(*)[32]>(&a[0]));
+                uint4 w[4], o[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const uint4*>(tile + swz(row, hf * 4 + j));
                 tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint4 wj = *reinterpret_cast<const uint4*>(tile + swz(row, hf * 4 + j));
-                    const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&wj);
-                    uint4 o;
-                    uint32_t* ow = reinterpret_cast<uint32_t*>(&o);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float2 x = __bfloat1622float2(e[i]);
-                        ow[i] = pack_bf16(fmaf(x.x, mc, __uint_as_float(a[8 * j + 2 * i]) * sc),
-                                          fmaf(x.y, mc, __uint_as_float(a[8 * j + 2 * i + 1]) * sc));
-                    }
-                    if (VARLEN && ragged_last && c == n_chunks - 1) {
-                        const long long grow = (long long)chunk_row(c) + row;
-                        if (grow < tok1 && (hf * 4 + j) * 8 < p.out_w[which])
-                            *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out_rows[which]) + grow * p.out_sn[which] +
-                                                      (long long)h * p.out_sh[which] + (hf * 4 + j) * 8) = o;
-                    } else {
-                        *reinterpret_cast<uint4*>(tile + swz(row, hf * 4 + j)) = o;
-                    }
+                for (int i = 0; i < 16; ++i) {
+                    const float2 v = __ffma2_rn(__bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[i]), mc2,
+                                                __fmul2_rn(a[i], sc2));
+                    reinterpret_cast<uint32_t*>(o)[i] = pack_bf16(v.x, v.y);
                 }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) put(tile, hf * 4 + j, c, which, o[j]);
             }
-            return dot - (e0 + e1);                                 // <x^ - bf16(x^), a>
+            return dot - (e2.x + e2.y);                                 // <x^ - bf16(x^), a>
         };
         for (int g = n1; g < n_items && alive; ++g) {
             if (!wait(bars + B_FULL + 8 * stage_of(g), fpar(g))) break;
@@ -430,21 +427,10 @@ tc_bidir_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             const int c = (g - n1) >> 1;
             // the raw q (half 0) or k (half 1) row, its norm
             uint8_t* xt = gbase + stage_base(g) + kTile;
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+            uint4 xr[8];
 #pragma unroll
-            for (int j = 0; j < 8; j += 2) {
-                const uint4 w0 = *reinterpret_cast<const uint4*>(xt + swz(row, j));
-                const uint4 w1 = *reinterpret_cast<const uint4*>(xt + swz(row, j + 1));
-                const __nv_bfloat162* e0 = reinterpret_cast<const __nv_bfloat162*>(&w0);
-                const __nv_bfloat162* e1 = reinterpret_cast<const __nv_bfloat162*>(&w1);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float2 f0 = __bfloat1622float2(e0[i]), f1 = __bfloat1622float2(e1[i]);
-                    a0 = fmaf(f0.x, f0.x, a0); a1 = fmaf(f0.y, f0.y, a1);
-                    a2 = fmaf(f1.x, f1.x, a2); a3 = fmaf(f1.y, f1.y, a3);
-                }
-            }
-            const float nrm = sqrtf((a0 + a1) + (a2 + a3));
+            for (int j = 0; j < 8; ++j) xr[j] = *reinterpret_cast<const uint4*>(xt + swz(row, j));
+            const float nrm = sqrtf(sumsq_row64(xr));
             float rn = 1.0f / fmaxf(nrm, kEps);
             const bool clamped = !(nrm > kEps);
             if (VARLEN && chunk_row(c) + row >= tok1) rn = 0.f;      // a row of the next sequence: nothing to dm, never stored
@@ -465,27 +451,20 @@ tc_bidir_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 // products that read them are done)
                 uint8_t* vt = gbase + stage_base(g);
                 const float sc = cfac * rn;
+                const float2 sc2 = make_float2(sc, sc);
 #pragma unroll 1
                 for (int hf = 0; hf < 2; ++hf) {
-                    uint32_t a[32];
-                    tmem_ld32(tmem + lane_base + colV + hf * 32, a);
+                    float2 a[16];
+                    tmem_ld32(tmem + lane_base + colV + hf * 32, *reinterpret_cast<uint32_t(*)[32]>(&a[0]));
                     tmem_wait_ld();
+                    uint4 o[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        uint4 o;
-                        o.x = pack_bf16(__uint_as_float(a[8 * j]) * sc, __uint_as_float(a[8 * j + 1]) * sc);
-                        o.y = pack_bf16(__uint_as_float(a[8 * j + 2]) * sc, __uint_as_float(a[8 * j + 3]) * sc);
-                        o.z = pack_bf16(__uint_as_float(a[8 * j + 4]) * sc, __uint_as_float(a[8 * j + 5]) * sc);
-                        o.w = pack_bf16(__uint_as_float(a[8 * j + 6]) * sc, __uint_as_float(a[8 * j + 7]) * sc);
-                        if (VARLEN && ragged_last && c == n_chunks - 1) {
-                            const long long grow = (long long)chunk_row(c) + row;
-                            if (grow < tok1 && (hf * 4 + j) * 8 < p.out_w[2])
-                                *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out_rows[2]) + grow * p.out_sn[2] +
-                                                          (long long)h * p.out_sh[2] + (hf * 4 + j) * 8) = o;
-                        } else {
-                            *reinterpret_cast<uint4*>(vt + swz(row, hf * 4 + j)) = o;
-                        }
+                    for (int i = 0; i < 16; ++i) {
+                        const float2 v = __fmul2_rn(a[i], sc2);
+                        reinterpret_cast<uint32_t*>(o)[i] = pack_bf16(v.x, v.y);
                     }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) put(vt, hf * 4 + j, c, 2, o[j]);
                 }
                 tc_fence_before();
                 mbar_arrive(bars + B_KDRAIN);

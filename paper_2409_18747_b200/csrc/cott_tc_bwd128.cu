@@ -18,7 +18,7 @@
 // along the chain (tiles without a second slot land, scores, mask, products, slots free again).  The
 // two CTAs of a (b, h, group) start side by side, so one of them finds most tiles in L2.
 // Measured against the three role-swapped walks with their state passes and scans: B=4, H=16,
-// N=2048 93 us (207), B=3, H=16, N=2999 129 us (210), 32 packed sequences of 512 to 2048 tokens,
+// N=2048 93 us (207), B=3, H=16, N=2999 128 us (210), 32 packed sequences of 512 to 2048 tokens,
 // H=16, 390 us (622), bidirectional B=8, H=16, N=1024 107 us (124).
 #include "cott_internal.h"
 #include "cott_sm100.cuh"
@@ -64,7 +64,6 @@ struct Bwd128Params {
     float* dm_out; int* status;
     const float* m; const float* seq_len; float seq_len_scalar;
     int H; int N; int group; int n_groups;
-    int clear_status;                   // no kernel of the call comes before this one
     int wait_limit_kcycles;
     int head_first_mask;                // bit i: in tensor map i (q, k, v, dO, dq, dk, dv) the head index comes before the token index
     const int* cu_seqlens;              // packed batch (VARLEN instances)
@@ -226,8 +225,9 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
     auto load_a = [&](int c) { load(off_a(c), kw ? &tmDO : &tmV, kw ? 3 : 2, bar(B_FA, c), chunk_row(c)); };
     auto load_b = [&](int c) { load(off_b(c), kw ? &tmQ : &tmK, kw ? 0 : 1, bar(B_FB, c), chunk_row(c)); };
     auto load_p = [&](int c) { load(off_p(c), kw ? &tmK : &tmQ, kw ? 1 : 0, bar(B_FP, c), chunk_row(c)); };
-    auto first_loads = [&]() {
-        if (!is_copy || lane != 0 || n_chunks == 0) return;
+    // A kernel of the same call, which writes none of the tensors loaded here, comes before this one: the
+    // first tiles are requested before the wait for it.
+    if (is_copy && lane == 0 && n_chunks > 0) {
         if (!BIDIR) { load_b(0); load_a(0); }
         load_x(0);
         load_p(0);
@@ -236,13 +236,9 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
             else if (BIDIR) { load_x(1); load_p(1); }
             else { load_b(1); load_a(1); }
         }
-    };
-    // Behind a state pass of the same call (which writes none of the tensors loaded here) the first
-    // tiles are requested before the wait for it.
-    if (!p.clear_status) first_loads();
+    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (p.clear_status) first_loads();
 
     const float s_b = p.seq_len ? p.seq_len[bseq]
                                 : (p.seq_len_scalar > 0.f ? p.seq_len_scalar : (float)(VARLEN ? max(seq1 - seq0, 1) : p.N));
@@ -718,8 +714,7 @@ tc_bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 
 }  // namespace
 
-cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, int init_sum, float* dm_k, int clear_status, int B, int H, int N,
-                             cudaStream_t st) {
+cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, int init_sum, float* dm_k, int B, int H, int N, cudaStream_t st) {
     const void* ptrs[7] = {a.q, a.k, a.v, a.d_o, a.dq, a.dk, a.dv};
     const RowLayout lays[7] = {a.l_qkv, a.l_qkv, a.l_v, a.l_do, a.l_dqkv, a.l_dqkv, a.l_dv};
     const int wk = a.w_k > 0 ? a.w_k : kD, wv = a.w_v > 0 ? a.w_v : kD;
@@ -743,7 +738,6 @@ cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, int init_sum, float* dm_k,
     p.dm_q = a.dm_partial; p.dm_k = dm_k; p.dm_out = a.dm_out; p.status = a.status;
     p.m = a.m; p.seq_len = a.seq_len; p.seq_len_scalar = a.seq_len_scalar;
     p.H = H; p.N = N; p.group = a.group; p.n_groups = a.n_groups;
-    p.clear_status = clear_status;
     p.wait_limit_kcycles = wait_limit_kcycles();
     p.cu_seqlens = a.cu_seqlens;
     if (a.bidir && (!a.sq_part || !a.r_part)) return cudaErrorInvalidValue;
@@ -761,8 +755,8 @@ cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, int init_sum, float* dm_k,
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    // (a packed batch reads cu_seqlens before anything else; behind a memset there is nothing to overlap)
-    cfg.numAttrs = (a.plain_launch || a.cu_seqlens || clear_status) ? 0 : 1;
+    // (a packed batch reads cu_seqlens before anything else)
+    cfg.numAttrs = (a.plain_launch || a.cu_seqlens) ? 0 : 1;
     cudaError_t le = cudaLaunchKernelEx(&cfg, kern, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], p);
     profile_end_launch(prof, st);
     note_launch();

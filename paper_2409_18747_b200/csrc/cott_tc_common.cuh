@@ -49,8 +49,9 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
 }
 
 // The same with the limit checked between a test and a (suspending) try: for a kernel whose only wait is
-// shorter than one suspension, so that its bound is a bound there too.
-static __device__ __noinline__ bool wait_polling(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+// shorter than one suspension, so that its bound is a bound there too.  (Inlined: a call would first wait
+// for every load its caller has in flight.)
+__device__ __forceinline__ bool wait_polling(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
     const long long t0 = clock64();
     for (;;) {
         if (mbar_test_wait(bar, parity)) return true;
@@ -86,34 +87,27 @@ struct RowScale {
     __device__ __forceinline__ __nv_bfloat162 operator()(__nv_bfloat162 x) const { return __hfma2(x, hi2, __hmul2(x, lo2)); }
 };
 
-// x / max(||x||, eps) on one row of 64 bf16 values held in w[8] (eight 16-byte chunks), in
-// packed bf16 arithmetic with the scale split in two bf16 terms (rn = hi + lo to 2^-17):
-// round(x hi + round(x lo)) is x rn rounded once, up to a second rounding of the small term --
-// two instructions per pair of elements instead of unpacking, two multiplies and a conversion.
-// Returns the norm; *rn_out = 1 / max(norm, eps).
-__device__ __forceinline__ float normalise_row64(uint4 (&w)[8], float eps, float* rn_out) {
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+// Sum of squares of 64 bf16 values held in w[8] (eight 16-byte chunks), packed fp32 arithmetic.
+__device__ __forceinline__ float sumsq_row64(const uint4 (&w)[8]) {
+    float2 s0 = make_float2(0.f, 0.f), s1 = s0;
 #pragma unroll
-    for (int j = 0; j < 8; j += 2) {
-        const __nv_bfloat162* e0 = reinterpret_cast<const __nv_bfloat162*>(&w[j]);
-        const __nv_bfloat162* e1 = reinterpret_cast<const __nv_bfloat162*>(&w[j + 1]);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 f0 = __bfloat1622float2(e0[i]), f1 = __bfloat1622float2(e1[i]);
-            a0 = fmaf(f0.x, f0.x, a0); a1 = fmaf(f0.y, f0.y, a1);
-            a2 = fmaf(f1.x, f1.x, a2); a3 = fmaf(f1.y, f1.y, a3);
-        }
+    for (int j = 0; j < 32; j += 2) {
+        const float2 f0 = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[j]);
+        const float2 f1 = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[j + 1]);
+        s0 = __ffma2_rn(f0, f0, s0); s1 = __ffma2_rn(f1, f1, s1);
     }
-    const float nrm = sqrtf((a0 + a1) + (a2 + a3));
+    return (s0.x + s0.y) + (s1.x + s1.y);
+}
+
+// x / max(||x||, eps) on one row of 64 bf16 values held in w[8].  Returns the norm; *rn_out = 1 / max(norm, eps).
+__device__ __forceinline__ float normalise_row64(uint4 (&w)[8], float eps, float* rn_out) {
+    const float nrm = sqrtf(sumsq_row64(w));
     const float rn = 1.0f / fmaxf(nrm, eps);
-    const __nv_bfloat16 hi = __float2bfloat16_rn(rn);
-    const __nv_bfloat16 lo = __float2bfloat16_rn(rn - __bfloat162float(hi));
-    const __nv_bfloat162 hi2 = __halves2bfloat162(hi, hi), lo2 = __halves2bfloat162(lo, lo);
+    const RowScale rs(rn);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&w[j]);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) e[i] = __hfma2(e[i], hi2, __hmul2(e[i], lo2));
+    for (int j = 0; j < 32; ++j) {
+        __nv_bfloat162& e = reinterpret_cast<__nv_bfloat162*>(w)[j];
+        e = rs(e);
     }
     *rn_out = rn;
     return nrm;
