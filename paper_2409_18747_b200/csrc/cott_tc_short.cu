@@ -8,7 +8,9 @@
 // tile: a single score product P = Q K^^T (128 x 128), a block-diagonal mask -- a row keeps the
 // columns of its own sequence, up to and including its own position when causal --, a single
 // product O = P~ V, rows scaled by c / max(||q||, eps) (Eq. 2-4) and stored.  No state update,
-// no state copy, no second launch; B H / k CTAs instead of B H, two per SM.
+// no state copy, no second launch; B H / k CTAs instead of B H, four (d = 64) or two per SM.
+// Bound by the chain of one CTA (tiles, norms, scores, mask, product, rows out), hence by how many share
+// an SM: B=64, H=12, N=77, d=64 14.1 us (18.2 with two), B=256, H=12, N=100 45.6 (65).
 #include "cott_internal.h"
 #include "cott_sm100.cuh"
 #include "cott_tc_common.cuh"
@@ -29,7 +31,13 @@ struct SL {
     static constexpr int kTile = kRows * D * 2;       // D / 64 boxes of 128 rows x 64 columns
     static constexpr int kOffQ = 0, kOffK = kTile, kOffV = 2 * kTile;
     static constexpr int kOffCtl = 3 * kTile;
-    static constexpr int kDynBytes = kOffCtl + 1024 + 1024;
+    static constexpr int kOffRx = 1024;               // float [128]: 1 / max(||q||, eps), behind the barriers
+    static constexpr int kDynBytes = kOffCtl + kOffRx + 512 + 1024;
+    // D = 64: the masked scores are packed over the start of the scores and the output accumulator takes
+    // their second half: 128 tensor-memory columns, so that four CTAs share an SM; D = 128, whose shared
+    // memory allows two, keeps them apart.
+    static constexpr int kTmemCols = D == 64 ? 128 : 256;
+    static constexpr int kCtas = D == 64 ? 4 : 2;
 };
 
 struct ShortParams {
@@ -43,18 +51,19 @@ struct ShortParams {
 };
 
 template <int D>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, SL<D>::kCtas)
 tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, ShortParams p) {
     using L = SL<D>;
     constexpr int NH = D / 64;
-    // Tensor-memory columns: scores, later the output accumulator 0..127 | masked bf16 scores 128..191.
-    constexpr uint32_t colP = 0, colPt = 128;
+    // Tensor-memory columns, D = 128: scores, later the output accumulator 0..127 | masked bf16 scores 128..191.
+    // D = 64: scores 0..127, then masked bf16 scores 0..63 | output accumulator 64..127.
+    constexpr uint32_t colP = 0, colPt = D == 64 ? 0 : 128, colO = D == 64 ? 64 : 0;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* gbase = smem_raw + (base - smem_u32(smem_raw));
     const uint32_t bars = base + L::kOffCtl;
-    enum { B_FULL = 0, B_KREADY = 8, B_PFULL = 16, B_PTREADY = 24, B_OFULL = 32, B_EDONE = 40 };
+    enum { B_FULL = 0, B_KREADY = 8, B_PFULL = 16, B_PTREADY = 24, B_OFULL = 32, B_EDONE = 40, B_SIB = 48 /* [4 quadrants] */ };
     const uint32_t tmem_slot = bars + kCtlTmemSlot;
     volatile uint32_t* tmem_slot_g = reinterpret_cast<volatile uint32_t*>(gbase + L::kOffCtl + kCtlTmemSlot);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(gbase + L::kOffCtl + kCtlAbort);
@@ -65,7 +74,7 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const int row0 = (int)blockIdx.x * rows_used;             // first row of the tile in the list of B H N rows
 
     if (is_ctrl) {
-        tmem_alloc(tmem_slot, 256);
+        tmem_alloc(tmem_slot, L::kTmemCols);
         tmem_relinquish();
     }
     if (tid == 0) {
@@ -75,6 +84,7 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         mbar_init(bars + B_PTREADY, 256);
         mbar_init(bars + B_OFULL, 1);
         mbar_init(bars + B_EDONE, 256);
+        for (int i = 0; i < 4; ++i) mbar_init(bars + B_SIB + 8 * i, 32);
         *abort_flag = 0;
         abort_flag[3] = p.wait_limit_kcycles;
         mbar_fence_init();
@@ -119,13 +129,13 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             }
             if (ok) {
                 // O = P~ V: P~ from tensor memory (8 columns per K = 16), V MN-major; the
-                // accumulator takes the place of the scores, which every worker has read
+                // accumulator takes columns of the scores, which every worker has read
                 tc_fence_after();
                 constexpr uint32_t idesc = instr_desc_bf16(128, D, false, true);
                 const uint32_t bl = smem_desc_lo(base + L::kOffV, 16384);
 #pragma unroll
                 for (int kk = 0; kk < kRows / 16; ++kk)
-                    mma_ts_w(tmem + colP, tmem + colPt + kk * 8u, bl + kk * 128u, kDescHi, idesc, kk > 0);
+                    mma_ts_w(tmem + colO, tmem + colPt + kk * 8u, bl + kk * 128u, kDescHi, idesc, kk > 0);
                 tc_commit(bars + B_OFULL);
                 ok = wait_or_abort(bars + B_EDONE, 0u, abort_flag);
             }
@@ -149,11 +159,13 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
         const bool valid = row < rows_used;
         // rows the copies do not write: zero (a zero v row times a zero score must not be NaN)
-        if (!valid) {
+        // (two lanes, l and l ^ 16, share a row here and in the row norms, half of it each)
+        const int nrow = warp * 16 + (lane & 15), half = lane >> 4;
+        if (nrow >= rows_used) {
 #pragma unroll
             for (int j = 0; j < 4 * NH; ++j) {
-                const int ch = hf * 4 * NH + j;                       // 16-byte chunk of the row
-                const uint32_t off = (ch >> 3) * 16384u + swz(row, ch & 7);
+                const int ch = half * 4 * NH + j;                     // 16-byte chunk of the row
+                const uint32_t off = (ch >> 3) * 16384u + swz(nrow, ch & 7);
                 *reinterpret_cast<uint4*>(gbase + L::kOffQ + off) = make_uint4(0, 0, 0, 0);
                 *reinterpret_cast<uint4*>(gbase + L::kOffK + off) = make_uint4(0, 0, 0, 0);
                 *reinterpret_cast<uint4*>(gbase + L::kOffV + off) = make_uint4(0, 0, 0, 0);
@@ -170,37 +182,37 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             cfac = stab_factor(p.m[h], s_b);
         }
         const int lo = seq * p.N, hi = live ? (p.causal ? row : lo + p.N - 1) : -1;
-        float rx = 0.f;
+        float* rq_buf = reinterpret_cast<float*>(gbase + L::kOffCtl + L::kOffRx);
         if (wait(bars + B_FULL, 0u)) {
-            // ||q|| and ||k|| over the whole row (each of the row's two threads sums all of it);
-            // k is normalised in place, each thread its half of the columns
-            float sq = 0.f, sk = 0.f;
-#pragma unroll
-            for (int ch = 0; ch < 8 * NH; ++ch) {
-                const uint32_t off = (ch >> 3) * 16384u + swz(row, ch & 7);
-                const uint4 wq = *reinterpret_cast<const uint4*>(gbase + L::kOffQ + off);
-                const uint4 wk = *reinterpret_cast<const uint4*>(gbase + L::kOffK + off);
-                const __nv_bfloat162* eq = reinterpret_cast<const __nv_bfloat162*>(&wq);
-                const __nv_bfloat162* ek = reinterpret_cast<const __nv_bfloat162*>(&wk);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float2 fq = __bfloat1622float2(eq[i]), fk = __bfloat1622float2(ek[i]);
-                    sq = fmaf(fq.x, fq.x, sq); sq = fmaf(fq.y, fq.y, sq);
-                    sk = fmaf(fk.x, fk.x, sk); sk = fmaf(fk.y, fk.y, sk);
-                }
-            }
-            rx = cfac / fmaxf(sqrtf(sq), kEps);
-            const float rk = 1.0f / fmaxf(sqrtf(sk), kEps);
+            // ||q|| and ||k||; k is normalised in place
+            float2 sq = make_float2(0.f, 0.f), sk = sq;
 #pragma unroll
             for (int j = 0; j < 4 * NH; ++j) {
-                const int ch = hf * 4 * NH + j;
-                uint4* pk = reinterpret_cast<uint4*>(gbase + L::kOffK + (ch >> 3) * 16384u + swz(row, ch & 7));
-                uint4 w = *pk;
-                __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&w);
+                const int ch = half * 4 * NH + j;
+                const uint32_t off = (ch >> 3) * 16384u + swz(nrow, ch & 7);
+                const uint4 wq = *reinterpret_cast<const uint4*>(gbase + L::kOffQ + off);
+                const uint4 wk = *reinterpret_cast<const uint4*>(gbase + L::kOffK + off);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const float2 f = __bfloat1622float2(e[i]);
-                    e[i] = __floats2bfloat162_rn(f.x * rk, f.y * rk);
+                    const float2 fq = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&wq)[i]);
+                    const float2 fk = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&wk)[i]);
+                    sq = __ffma2_rn(fq, fq, sq); sk = __ffma2_rn(fk, fk, sk);
+                }
+            }
+            float nq = sq.x + sq.y, nk = sk.x + sk.y;
+            nq += __shfl_xor_sync(0xffffffffu, nq, 16);
+            nk += __shfl_xor_sync(0xffffffffu, nk, 16);
+            if (half == 0) rq_buf[nrow] = 1.0f / fmaxf(sqrtf(nq), kEps);
+            const RowScale rk(1.0f / fmaxf(sqrtf(nk), kEps));
+#pragma unroll
+            for (int j = 0; j < 4 * NH; ++j) {
+                const int ch = half * 4 * NH + j;
+                uint4* pk = reinterpret_cast<uint4*>(gbase + L::kOffK + (ch >> 3) * 16384u + swz(nrow, ch & 7));
+                uint4 w = *pk;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    __nv_bfloat162& e = reinterpret_cast<__nv_bfloat162*>(&w)[i];
+                    e = rk(e);
                 }
                 *pk = w;
             }
@@ -224,6 +236,9 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     const float b2 = (jb >= lo && jb <= hi) ? __uint_as_float(r[2 * j + 1]) : 0.f;
                     pk[j] = pack_bf16(a, b2);
                 }
+                // (D = 64: columns 32-63, which the hf = 1 warp writes, hold scores of the hf = 0 warp)
+                if (D == 64 && hf == 0 && pc == 1) { tc_fence_before(); mbar_arrive(bars + B_SIB + 8 * q4); }
+                if (D == 64 && hf == 1 && pc == 0) { if (!wait(bars + B_SIB + 8 * q4, 0u)) break; tc_fence_after(); }
                 tmem_st16(tmem + lane_base + colPt + (c0 >> 1), pk);
             }
             tmem_wait_st();
@@ -233,11 +248,12 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         if (wait(bars + B_OFULL, 0u)) {
             // this thread's D / 2 accumulator columns: scale, round, stage where q was
             tc_fence_after();
+            const float rx = cfac * rq_buf[row];
 #pragma unroll 1
             for (int pc = 0; pc < D / 64; ++pc) {
                 const int c0 = hf * (D / 2) + pc * 32;
                 uint32_t a[32];
-                tmem_ld32(tmem + lane_base + colP + c0, a);
+                tmem_ld32(tmem + lane_base + colO + c0, a);
                 tmem_wait_ld();
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -266,7 +282,7 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             p.status[2] = (int)blockIdx.x | (6 << 24);
         }
     }
-    if (is_ctrl) tmem_dealloc(tmem, 256);
+    if (is_ctrl) tmem_dealloc(tmem, L::kTmemCols);
 }
 
 template <int D>
