@@ -6,7 +6,6 @@ allocated here with torch because the library itself never allocates.
 """
 from __future__ import annotations
 
-import contextlib
 import ctypes
 import functools
 import os
@@ -137,20 +136,22 @@ def _on_call_stream(fn):
     kernels run on: the caching allocator then cannot hand such a block to work on another
     stream while libcott kernels still use it."""
     @functools.wraps(fn)
-    def wrapped(*args, **kwargs):
-        stream = kwargs.get("stream")
-        ctx = torch.cuda.stream(stream) if stream is not None else contextlib.nullcontext()
-        with ctx:
+    def wrapped(*args, stream=None, **kwargs):
+        if stream is None:
             return fn(*args, **kwargs)
+        with torch.cuda.stream(stream):
+            return fn(*args, stream=stream, **kwargs)
     return wrapped
 
 
+_DTYPES = {torch.float32: F32, torch.bfloat16: BF16}
+
+
 def _dt(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return F32
-    if t.dtype == torch.bfloat16:
-        return BF16
-    raise TypeError(f"libcott supports float32 and bfloat16 I/O, got {t.dtype}")
+    dt = _DTYPES.get(t.dtype)
+    if dt is None:
+        raise TypeError(f"libcott supports float32 and bfloat16 I/O, got {t.dtype}")
+    return dt
 
 
 def _check_dev(*ts):
@@ -167,41 +168,36 @@ class _Strides(ctypes.Structure):
     _fields_ = [("batch", ctypes.c_longlong), ("head", ctypes.c_longlong), ("token", ctypes.c_longlong)]
 
 
-def _check_rows(*ts):
-    """[B,H,N,d] CUDA tensors with contiguous rows; any strides over batch, head and token."""
+def _layout(*ts):
+    """Checks a group of [B,H,N,d] CUDA tensors with contiguous rows that share their strides over batch,
+    head and token; returns these as a ctypes reference (None when they are dense [B,H,N,d])."""
+    first = ts[0].stride()
+    dense = True
     for t in ts:
         if not t.is_cuda:
             raise RuntimeError("libcott needs CUDA tensors (there is no CPU path)")
-        if t.dim() != 4 or (t.shape[3] > 1 and t.stride(3) != 1):
+        st = t.stride()
+        if len(st) != 4 or (st[3] != 1 and t.shape[3] > 1):
             raise ValueError("libcott needs [B,H,N,d] tensors whose last dimension is contiguous")
-
-
-def _strides_of(*ts):
-    """ctypes strides shared by the given tensors (None when they are dense [B,H,N,d])."""
-    st = tuple(ts[0].stride()[:3])
-    for t in ts[1:]:
-        if tuple(t.stride()[:3]) != st:
+        if st[:3] != first[:3]:
             raise ValueError("tensors of one group (q,k,v / dq,dk,dv) must share their strides")
-    if all(t.is_contiguous() for t in ts):
-        return None
-    return _Strides(st[0], st[1], st[2])
-
-
-def _ref(s):
-    return ctypes.byref(s) if s is not None else None
+        if dense and not t.is_contiguous():
+            dense = False
+    return None if dense else ctypes.byref(_Strides(first[0], first[1], first[2]))
 
 
 def _stream_ptr(stream) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return int(s.cuda_stream)
+    if stream is None:      # (the raw handle of torch's current stream: a Stream object costs 3 us to build)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return int(stream.cuda_stream)
 
 
 def _scale(m: torch.Tensor, seq_len, scalar: float = 0.0) -> _ScaleParams:
-    sp = _ScaleParams()
-    sp.m = m.data_ptr()
-    sp.seq_len = seq_len.data_ptr() if isinstance(seq_len, torch.Tensor) else None
-    sp.seq_len_scalar = float(seq_len) if (seq_len is not None and not isinstance(seq_len, torch.Tensor)) else scalar
-    return sp
+    if seq_len is None:
+        return _ScaleParams(m.data_ptr(), None, scalar)
+    if isinstance(seq_len, torch.Tensor):
+        return _ScaleParams(m.data_ptr(), seq_len.data_ptr(), scalar)
+    return _ScaleParams(m.data_ptr(), None, float(seq_len))
 
 
 def fwd_noalloc_status(stream=None) -> int:
@@ -220,6 +216,7 @@ def shutdown() -> None:
 def set_option(name: str, value: int) -> None:
     """cott_set_option: a process-wide switch for tests and measurements (see ``cott.h``)."""
     rc = _load().cott_set_option(name.encode(), int(value))
+    _bytes.cache_clear()
     if rc != 0:
         raise CottError(rc, f"cott_set_option({name})")
 
@@ -228,11 +225,17 @@ def get_option(name: str) -> int:
     return int(_load().cott_get_option(name.encode()))
 
 
-def workspace_bytes(op: int, dt: int, B: int, H: int, N: int, d: int, causal: bool) -> int:
-    n = _load().cott_workspace_bytes(op, dt, B, H, N, d, int(bool(causal)))
+@functools.lru_cache(maxsize=256)
+def _bytes(op, dt, B, H, N, d_k, d_v, causal) -> int:
+    """The size query of a problem (it depends on the arguments and the options only)."""
+    n = _load().cott_workspace_bytes_dkdv(op, dt, B, H, N, d_k, d_v, int(causal))
     if n == _SIZE_MAX:
         raise CottError(-2, "cott_workspace_bytes")
     return int(n)
+
+
+def workspace_bytes(op: int, dt: int, B: int, H: int, N: int, d: int, causal: bool) -> int:
+    return _bytes(op, dt, B, H, N, d, d, bool(causal))
 
 
 def query_plan(op: int, dt: int, B: int, H: int, N: int, d: int, causal: bool) -> dict:
@@ -245,10 +248,7 @@ def query_plan(op: int, dt: int, B: int, H: int, N: int, d: int, causal: bool) -
 
 
 def workspace_bytes_dkdv(op: int, dt: int, B: int, H: int, N: int, d_k: int, d_v: int, causal: bool) -> int:
-    n = _load().cott_workspace_bytes_dkdv(op, dt, B, H, N, d_k, d_v, int(bool(causal)))
-    if n == _SIZE_MAX:
-        raise CottError(-2, "cott_workspace_bytes_dkdv")
-    return int(n)
+    return _bytes(op, dt, B, H, N, d_k, d_v, bool(causal))
 
 
 def query_plan_dkdv(op: int, dt: int, B: int, H: int, N: int, d_k: int, d_v: int, causal: bool) -> dict:
@@ -262,35 +262,32 @@ def query_plan_dkdv(op: int, dt: int, B: int, H: int, N: int, d_k: int, d_v: int
 
 def _fwd_dkdv(q, k, v, m, seq_len, causal, state_in, return_state, out, workspace, stream):
     """cott_fwd_dkdv: q, k ``[B,H,N,d_k]``, v ``[B,H,N,d_v]``; states ``[B,H,d_k,d_v]``."""
-    _check_rows(q, k, v)
     _check_dev(m, state_in, seq_len if isinstance(seq_len, torch.Tensor) else None)
     B, H, N, dk = q.shape
     dv = v.shape[3]
     dt = _dt(q)
-    if state_in is not None and (state_in.dtype != torch.float32 or tuple(state_in.shape) != (B, H, dk, dv)):
+    if state_in is not None and (state_in.dtype != torch.float32 or state_in.shape != (B, H, dk, dv)):
         raise ValueError("state_in must be float32 [B,H,d_k,d_v]")
     o = torch.empty_like(v) if out is None else out
-    _check_rows(o)
-    s_qk, s_v, s_o = _strides_of(q, k), _strides_of(v), _strides_of(o)
+    s_qk, s_v, s_o = _layout(q, k), _layout(v), _layout(o)
     state = torch.empty((B, H, dk, dv), dtype=torch.float32, device=q.device) if return_state else None
-    need = workspace_bytes_dkdv(OP_FWD, dt, B, H, N, dk, dv, causal)
-    ws = torch.empty(max(need, 256), dtype=torch.uint8, device=q.device) if workspace is None else workspace
+    ws = _workspace(OP_FWD, dt, B, H, N, dk, dv, causal, q, workspace)
     sp = _scale(m, seq_len)
     rc = _load().cott_fwd_dkdv(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(),
                                state_in.data_ptr() if state_in is not None else None,
                                state.data_ptr() if state is not None else None, B, H, N, dk, dv,
-                               int(bool(causal)), dt, _ref(s_qk), _ref(s_v), _ref(s_o), ctypes.byref(sp),
+                               int(bool(causal)), dt, s_qk, s_v, s_o, ctypes.byref(sp),
                                ws.data_ptr(), ws.numel(), _stream_ptr(stream))
     if rc != 0:
         raise CottError(rc, "cott_fwd_dkdv")
     return (o, state) if return_state else o
 
 
-def _workspace(op, dt, B, H, N, d, causal, device, workspace):
-    need = workspace_bytes(op, dt, B, H, N, d, causal)
+def _workspace(op, dt, B, H, N, d_k, d_v, causal, like, workspace):
+    """The caller's workspace or a new one on the device of ``like``."""
     if workspace is None:
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=device)
-    return workspace, workspace.numel()
+        return like.new_empty(max(_bytes(op, dt, B, H, N, d_k, d_v, bool(causal)), 256), dtype=torch.uint8)
+    return workspace
 
 
 def workspace_bytes_varlen(op, dt, B, H, total_tokens, max_seqlen, d, causal=True) -> int:
@@ -319,20 +316,18 @@ def fwd(q, k, v, m, seq_len=None, causal=True, return_state=False, out=None, wor
     memory, else dense ``[B,H,N,d]``; or ``out``) or ``(o, state[B,H,d,d] fp32)``."""
     if v.shape[-1] != q.shape[-1]:      # different key and value sizes
         return _fwd_dkdv(q, k, v, m, seq_len, causal, None, return_state, out, workspace, stream)
-    _check_rows(q, k, v)
     _check_dev(m, seq_len if isinstance(seq_len, torch.Tensor) else None)
     B, H, N, d = q.shape
     dt = _dt(q)
     o = torch.empty_like(q) if out is None else out
-    _check_rows(o)
-    s_qkv, s_o = _strides_of(q, k, v), _strides_of(o)
+    s_qkv, s_o = _layout(q, k, v), _layout(o)
     state = torch.empty((B, H, d, d), dtype=torch.float32, device=q.device) if return_state else None
-    ws, ws_bytes = _workspace(OP_FWD, dt, B, H, N, d, causal, q.device, workspace)
+    ws = _workspace(OP_FWD, dt, B, H, N, d, d, causal, q, workspace)
     sp = _scale(m, seq_len)
     rc = _load().cott_fwd_strided(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(),
                                   state.data_ptr() if state is not None else None, B, H, N, d,
-                                  int(bool(causal)), dt, _ref(s_qkv), _ref(s_o), ctypes.byref(sp),
-                                  ws.data_ptr(), ws_bytes, _stream_ptr(stream))
+                                  int(bool(causal)), dt, s_qkv, s_o, ctypes.byref(sp),
+                                  ws.data_ptr(), ws.numel(), _stream_ptr(stream))
     if rc != 0:
         raise CottError(rc, "cott_fwd_strided")
     return (o, state) if return_state else o
@@ -345,7 +340,6 @@ def fwd_stateful(q, k, v, m, seq_len, state_in=None, return_state=True, out=None
     (fp32 ``[B,H,d,d]`` or None) is the state the previous segment (or a decode step) left;
     ``seq_len`` (a float >= 1 or a float32 ``[B]`` CUDA tensor) is the scaling base of the WHOLE
     sequence and must be the same for all its segments.  Returns ``(o, state)`` or ``o``."""
-    _check_rows(q, k, v)
     _check_dev(m, state_in, seq_len if isinstance(seq_len, torch.Tensor) else None)
     if seq_len is None:
         raise ValueError("fwd_stateful needs the scaling base of the whole sequence")
@@ -355,18 +349,17 @@ def fwd_stateful(q, k, v, m, seq_len, state_in=None, return_state=True, out=None
         return _fwd_dkdv(q, k, v, m, seq_len, True, state_in, return_state, out, workspace, stream)
     B, H, N, d = q.shape
     dt = _dt(q)
-    if state_in is not None and (state_in.dtype != torch.float32 or tuple(state_in.shape) != (B, H, d, d)):
+    if state_in is not None and (state_in.dtype != torch.float32 or state_in.shape != (B, H, d, d)):
         raise ValueError("state_in must be float32 [B,H,d,d]")
     o = torch.empty_like(q) if out is None else out
     state = torch.empty((B, H, d, d), dtype=torch.float32, device=q.device) if return_state else None
-    _check_rows(o)
-    s_qkv, s_o = _strides_of(q, k, v), _strides_of(o)
-    ws, ws_bytes = _workspace(OP_FWD, dt, B, H, N, d, True, q.device, workspace)
+    s_qkv, s_o = _layout(q, k, v), _layout(o)
+    ws = _workspace(OP_FWD, dt, B, H, N, d, d, True, q, workspace)
     sp = _scale(m, seq_len)
     rc = _load().cott_fwd_stateful_strided(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(),
                                            state_in.data_ptr() if state_in is not None else None,
                                            state.data_ptr() if state is not None else None, B, H, N, d, dt,
-                                           _ref(s_qkv), _ref(s_o), ctypes.byref(sp), ws.data_ptr(), ws_bytes,
+                                           s_qkv, s_o, ctypes.byref(sp), ws.data_ptr(), ws.numel(),
                                            _stream_ptr(stream))
     if rc != 0:
         raise CottError(rc, "cott_fwd_stateful_strided")
@@ -395,45 +388,41 @@ def bwd(q, k, v, d_o, m, seq_len=None, causal=True, workspace=None, stream=None,
     left there.  q, k, v (common strides) and d_o as for ``fwd``; ``out``:
     optional ``(dq, dk, dv)`` tensors with common strides (e.g. the slices of a fused gradient
     buffer), else they are allocated like q.  Returns ``(dq, dk, dv, dm[H] fp32)``."""
-    _check_rows(q, k, v, d_o)
     _check_dev(m, seq_len if isinstance(seq_len, torch.Tensor) else None)
     B, H, N, d = q.shape
     dt = _dt(q)
     if v.shape[-1] != d:                # different key and value sizes: cott_bwd_dkdv
         d_v = v.shape[-1]
         dq, dk, dv = (torch.empty_like(q), torch.empty_like(k), torch.empty_like(v)) if out is None else out
-        _check_rows(dq, dk, dv)
-        dm = torch.empty((H,), dtype=torch.float32, device=q.device)
-        need = workspace_bytes_dkdv(OP_BWD, dt, B, H, N, d, d_v, causal)
-        ws = torch.empty(max(need, 256), dtype=torch.uint8, device=q.device) if workspace is None else workspace
+        dm = q.new_empty((H,), dtype=torch.float32)
+        ws = _workspace(OP_BWD, dt, B, H, N, d, d_v, causal, q, workspace)
         sp = _scale(m, seq_len)
-        st = [_strides_of(q, k), _strides_of(v), _strides_of(d_o), _strides_of(dq, dk), _strides_of(dv)]
+        st = [_layout(q, k), _layout(v), _layout(d_o), _layout(dq, dk), _layout(dv)]
         rc = _load().cott_bwd_dkdv(q.data_ptr(), k.data_ptr(), v.data_ptr(), d_o.data_ptr(), dq.data_ptr(),
                                    dk.data_ptr(), dv.data_ptr(), dm.data_ptr(), B, H, N, d, d_v,
-                                   int(bool(causal)), dt, *[_ref(x) for x in st], ctypes.byref(sp),
+                                   int(bool(causal)), dt, *st, ctypes.byref(sp),
                                    ws.data_ptr(), ws.numel(), _stream_ptr(stream))
         if rc != 0:
             raise CottError(rc, "cott_bwd_dkdv")
         return dq, dk, dv, dm
     dq, dk, dv = (torch.empty_like(q), torch.empty_like(q), torch.empty_like(q)) if out is None else out
-    _check_rows(dq, dk, dv)
-    s_qkv, s_do, s_dqkv = _strides_of(q, k, v), _strides_of(d_o), _strides_of(dq, dk, dv)
-    dm = torch.empty((H,), dtype=torch.float32, device=q.device)
-    ws, ws_bytes = _workspace(OP_BWD, dt, B, H, N, d, causal, q.device, workspace)
+    s_qkv, s_do, s_dqkv = _layout(q, k, v), _layout(d_o), _layout(dq, dk, dv)
+    dm = q.new_empty((H,), dtype=torch.float32)
+    ws = _workspace(OP_BWD, dt, B, H, N, d, d, causal, q, workspace)
     sp = _scale(m, seq_len)
     if fwd_workspace is not None:
         rc = _load().cott_bwd_after_fwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), d_o.data_ptr(),
                                         dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), dm.data_ptr(), B, H, N,
-                                        d, int(bool(causal)), dt, _ref(s_qkv), _ref(s_do), _ref(s_dqkv),
-                                        ctypes.byref(sp), fwd_workspace.data_ptr(), ws.data_ptr(), ws_bytes,
+                                        d, int(bool(causal)), dt, s_qkv, s_do, s_dqkv,
+                                        ctypes.byref(sp), fwd_workspace.data_ptr(), ws.data_ptr(), ws.numel(),
                                         _stream_ptr(stream))
         if rc != 0:
             raise CottError(rc, "cott_bwd_after_fwd")
         return dq, dk, dv, dm
     rc = _load().cott_bwd_strided(q.data_ptr(), k.data_ptr(), v.data_ptr(), d_o.data_ptr(),
                                   dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), dm.data_ptr(), B, H, N,
-                                  d, int(bool(causal)), dt, _ref(s_qkv), _ref(s_do), _ref(s_dqkv),
-                                  ctypes.byref(sp), ws.data_ptr(), ws_bytes, _stream_ptr(stream))
+                                  d, int(bool(causal)), dt, s_qkv, s_do, s_dqkv,
+                                  ctypes.byref(sp), ws.data_ptr(), ws.numel(), _stream_ptr(stream))
     if rc != 0:
         raise CottError(rc, "cott_bwd_strided")
     return dq, dk, dv, dm
@@ -479,7 +468,7 @@ def bwd_varlen(q, k, v, d_o, m, cu_seqlens, max_seqlen, seq_len=None, causal=Tru
     B = cu_seqlens.numel() - 1
     dt = _dt(q)
     dq, dk, dv = torch.empty_like(q), torch.empty_like(q), torch.empty_like(q)
-    dm = torch.empty((H,), dtype=torch.float32, device=q.device)
+    dm = q.new_empty((H,), dtype=torch.float32)
     ws, ws_bytes = _workspace_varlen(OP_BWD, dt, B, H, T, int(max_seqlen), d, causal, q.device, workspace)
     sp = _scale(m, seq_len)
     rc = _load().cott_bwd_varlen(q.data_ptr(), k.data_ptr(), v.data_ptr(), d_o.data_ptr(), dq.data_ptr(),
@@ -500,7 +489,6 @@ def bwd_stateful(q, k, v, d_o, m, seq_len, state_in=None, d_state_out=None, retu
     ``d_state_in`` of the next segment's backward); ``seq_len`` as for ``fwd_stateful``; tensors and
     ``out`` as for ``bwd`` (strides are picked up).  Returns ``(dq, dk, dv, d_state_in, dm)``
     (``d_state_in`` is None when not asked for)."""
-    _check_rows(q, k, v, d_o)
     _check_dev(m, state_in, d_state_out, seq_len if isinstance(seq_len, torch.Tensor) else None)
     B, H, N, d = q.shape
     d_v = v.shape[-1]
@@ -509,19 +497,17 @@ def bwd_stateful(q, k, v, d_o, m, seq_len, state_in=None, d_state_out=None, retu
         if t is not None and (t.dtype != torch.float32 or tuple(t.shape) != (B, H, d, d_v) or not t.is_contiguous()):
             raise ValueError("states must be contiguous float32 [B,H,d_k,d_v]")
     dq, dk, dv = (torch.empty_like(q), torch.empty_like(k), torch.empty_like(v)) if out is None else out
-    _check_rows(dq, dk, dv)
     same = d == d_v
-    st = [_strides_of(q, k, v) if same else _strides_of(q, k), None if same else _strides_of(v), _strides_of(d_o),
-          _strides_of(dq, dk, dv) if same else _strides_of(dq, dk), None if same else _strides_of(dv)]
-    dm = torch.empty((H,), dtype=torch.float32, device=q.device)
+    st = [_layout(q, k, v) if same else _layout(q, k), None if same else _layout(v), _layout(d_o),
+          _layout(dq, dk, dv) if same else _layout(dq, dk), None if same else _layout(dv)]
+    dm = q.new_empty((H,), dtype=torch.float32)
     d_state_in = torch.empty((B, H, d, d_v), dtype=torch.float32, device=q.device) if return_d_state else None
-    need = workspace_bytes_dkdv(OP_BWD, dt, B, H, N, d, d_v, True)
-    ws = torch.empty(max(need, 256), dtype=torch.uint8, device=q.device) if workspace is None else workspace
+    ws = _workspace(OP_BWD, dt, B, H, N, d, d_v, True, q, workspace)
     sp = _scale(m, seq_len)
     ptr = lambda t: 0 if t is None else t.data_ptr()
     rc = _load().cott_bwd_stateful_strided(q.data_ptr(), k.data_ptr(), v.data_ptr(), d_o.data_ptr(), ptr(state_in),
                                            ptr(d_state_out), dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), ptr(d_state_in),
-                                           dm.data_ptr(), B, H, N, d, d_v, dt, *[_ref(x) for x in st], ctypes.byref(sp),
+                                           dm.data_ptr(), B, H, N, d, d_v, dt, *st, ctypes.byref(sp),
                                            ws.data_ptr(), ws.numel(), _stream_ptr(stream))
     if rc != 0:
         raise CottError(rc, "cott_bwd_stateful_strided")
@@ -535,7 +521,7 @@ def decode_step(q, k, v, state, m, seq_len, out=None, stream=None):
     _check_dev(q, k, v, state, m, seq_len if isinstance(seq_len, torch.Tensor) else None)
     B, H, d = q.shape
     d_v = v.shape[-1]
-    if state.dtype != torch.float32 or tuple(state.shape) != (B, H, d, d_v):
+    if state.dtype != torch.float32 or state.shape != (B, H, d, d_v):
         raise ValueError("state must be float32 [B,H,d_k,d_v]")
     o = torch.empty_like(v) if out is None else out
     sp = _scale(m, seq_len)
