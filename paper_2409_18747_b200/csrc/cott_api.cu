@@ -182,9 +182,11 @@ static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv
         group = 1024;
         while (group > 128 && BH * ((N + group - 1) / group) < 4 * 148) group >>= 1;
         // Short sequences of few heads: groups down to one chunk, as long as they do not yet give two
-        // CTAs per SM and the group states stay small (2 MiB).
+        // CTAs per SM and the group states stay small: 2 MiB, or 8 MiB at d = 128, where a chunk is four
+        // times the work (B=2, H=8, N=509: d = 64 backward 43 us with 2 MiB, 59 with 8; d = 128 forward 72
+        // with 2, 43 with 8).
         while (group > 32 && BH * ((N + group - 1) / group) < 2 * 148 &&
-               BH * ((N + group / 2 - 1) / (group / 2)) * d * d * 4 <= (2L << 20)) group >>= 1;
+               BH * ((N + group / 2 - 1) / (group / 2)) * d * d * 4 <= (d == 128 ? 8L << 20 : 2L << 20)) group >>= 1;
     }
     if (forced > 0) group = (forced + p->chunk - 1) / p->chunk * p->chunk;
     if (group >= N) group = (N + p->chunk - 1) / p->chunk * p->chunk;

@@ -55,7 +55,10 @@ __device__ __forceinline__ float dot4(float4 a, float4 b) {
     return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w)));
 }
 __device__ __forceinline__ void axpy4(float4& y, float a, float4 x) {
-    y.x = fmaf(a, x.x, y.x); y.y = fmaf(a, x.y, y.y); y.z = fmaf(a, x.z, y.z); y.w = fmaf(a, x.w, y.w);
+    const float2 a2 = make_float2(a, a);
+    const float2 lo = __ffma2_rn(a2, make_float2(x.x, x.y), make_float2(y.x, y.y));
+    const float2 hi = __ffma2_rn(a2, make_float2(x.z, x.w), make_float2(y.z, y.w));
+    y = make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
 // Shared memory of the walk: three chunk tiles (rows padded by four words: threads that read 16
@@ -70,26 +73,32 @@ template <int D> struct WalkSmem {
 
 // One pass of the running-sum walk (WalkArgs) over one sequence group, 32 tokens at a time:
 //     P = X A^T, masked to the pairs the running sum holds (Eq. 6) ;  Out = P Bv + X S ;  S += A^T Bv
-// in fp32 multiply-adds throughout.  What bounds it is the multiply-add rate (per token 2 * 32 * d
+// in fp32 multiply-adds (packed in pairs) throughout.  What bounds it is the multiply-add rate (per token 2 * 32 * d
 // for the scores side, 2 d^2 for the state side), and for the small problems this path serves the
 // chain of launches and the fill of the SMs; the token-by-token recurrence it replaces was one
 // serial chain (0.35 us a token) on the same SMs.  32 tokens a chunk: a 64-token chunk does 1.3
 // times the multiply-adds at d = 64 and halves the number of CTAs a short sequence gives.
 // Measured, forward and backward at B=2, H=8, N=509, d=64: 303 us and 13 launches with the
-// recurrence, 88 us and 4 launches (state pass and walk each way) here.
+// recurrence, 68 us and 4 launches (state pass and walk each way) here.
 // Thread (ty, tx) owns columns 4 tx .. + 3 everywhere: rows ty, ty + TY, .. of the chunk (it loads,
 // normalises and produces them; the TX threads of a row sit in one warp, so row sums are
 // shuffles) and rows SR ty .. + SR - 1 of the state, which stays in its registers and is copied
 // to shared memory once per chunk.  The next chunk's rows are loaded while this one is computed.
 // blockIdx.y picks one of up to three streams (the three gradients of a backward call).
+// Threads of a CTA: few, so that each has a tile of four rows (d = 64; 32: two) and shared memory feeds
+// twice as many multiply-adds per load; three or four CTAs share an SM.  (Backward at B=2, H=8, N=509, d = 64:
+// 43 us against 56 with 256 threads, B=32, H=12, N=100, d = 32: 57 against 90; 170 registers, 128 spill.)
+template <int D> struct WalkThreads { static constexpr int n = D == 128 ? 256 : 128, ctas = D == 128 ? 1 : (D == 64 ? 3 : 4); };
+
 template <int D, typename T>
-__global__ void __launch_bounds__(kThreads) walk_kernel(const __grid_constant__ WalkBatch batch) {
+__global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_kernel(const __grid_constant__ WalkBatch batch) {
     using M = WalkSmem<D>;
-    constexpr int TX = D / 4, TY = kThreads / TX;
+    constexpr int NT = WalkThreads<D>::n;
+    constexpr int TX = D / 4, TY = NT / TX;
     constexpr int RPT = kChunk / TY;      // chunk rows per thread
     constexpr int SR = D / TY;            // state rows per thread
     extern __shared__ __align__(16) float sm[];
-    __shared__ float dm_red[kThreads / 32];
+    __shared__ float dm_red[NT / 32];
     __shared__ int last_flag;
     const WalkArgs& w = batch.w[blockIdx.y];
 
@@ -153,9 +162,21 @@ __global__ void __launch_bounds__(kThreads) walk_kernel(const __grid_constant__ 
             }
         } else {
             const float* s0 = src + (size_t)(tx * 4) * D + ty * SR;
+            if constexpr (SR >= 4) {
 #pragma unroll
-            for (int r = 0; r < SR; ++r) {
-                S[r].x += s0[r]; S[r].y += s0[D + r]; S[r].z += s0[2 * D + r]; S[r].w += s0[3 * D + r];
+                for (int r = 0; r < SR; r += 4) {
+                    const float4 v0 = *reinterpret_cast<const float4*>(s0 + r), v1 = *reinterpret_cast<const float4*>(s0 + D + r);
+                    const float4 v2 = *reinterpret_cast<const float4*>(s0 + 2 * D + r), v3 = *reinterpret_cast<const float4*>(s0 + 3 * D + r);
+                    S[r].x += v0.x; S[r].y += v1.x; S[r].z += v2.x; S[r].w += v3.x;
+                    S[r + 1].x += v0.y; S[r + 1].y += v1.y; S[r + 1].z += v2.y; S[r + 1].w += v3.y;
+                    S[r + 2].x += v0.z; S[r + 2].y += v1.z; S[r + 2].z += v2.z; S[r + 2].w += v3.z;
+                    S[r + 3].x += v0.w; S[r + 3].y += v1.w; S[r + 3].z += v2.w; S[r + 3].w += v3.w;
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < SR; ++r) {
+                    S[r].x += s0[r]; S[r].y += s0[D + r]; S[r].z += s0[2 * D + r]; S[r].w += s0[3 * D + r];
+                }
             }
         }
     };
@@ -208,31 +229,32 @@ __global__ void __launch_bounds__(kThreads) walk_kernel(const __grid_constant__ 
         float4 out[RPT];
         if (write_out) {
             if (update) {
-                // scores: rows pi, pi + 16 against keys pj, pj + 16
+                // scores: SU rows pi + PY u against keys pj, pj + 16
+                constexpr int PY = NT / 16, SU = kChunk / PY;
                 const int pi = tid >> 4, pj = tid & 15;
-                float4 acc[2][2];
+                float2 acc[SU][2];
 #pragma unroll
-                for (int u = 0; u < 2; ++u) { acc[u][0] = zero4; acc[u][1] = zero4; }
+                for (int u = 0; u < SU; ++u) { acc[u][0] = make_float2(0.f, 0.f); acc[u][1] = acc[u][0]; }
 #pragma unroll 4
                 for (int k = 0; k < D; k += 4) {
-                    const float4 x0 = *reinterpret_cast<const float4*>(sm + M::kX + pi * M::kRow + k);
-                    const float4 x1 = *reinterpret_cast<const float4*>(sm + M::kX + (pi + 16) * M::kRow + k);
                     const float4 a0 = *reinterpret_cast<const float4*>(sm + M::kA + pj * M::kRow + k);
                     const float4 a1 = *reinterpret_cast<const float4*>(sm + M::kA + (pj + 16) * M::kRow + k);
-                    auto fma4 = [](float4& d, float4 p, float4 q) {
-                        d.x = fmaf(p.x, q.x, d.x); d.y = fmaf(p.y, q.y, d.y);
-                        d.z = fmaf(p.z, q.z, d.z); d.w = fmaf(p.w, q.w, d.w);
-                    };
-                    fma4(acc[0][0], x0, a0); fma4(acc[0][1], x0, a1); fma4(acc[1][0], x1, a0); fma4(acc[1][1], x1, a1);
+#pragma unroll
+                    for (int u = 0; u < SU; ++u) {
+                        const float4 x = *reinterpret_cast<const float4*>(sm + M::kX + (pi + PY * u) * M::kRow + k);
+                        acc[u][0] = __ffma2_rn(make_float2(x.x, x.y), make_float2(a0.x, a0.y), acc[u][0]);
+                        acc[u][1] = __ffma2_rn(make_float2(x.x, x.y), make_float2(a1.x, a1.y), acc[u][1]);
+                        acc[u][0] = __ffma2_rn(make_float2(x.z, x.w), make_float2(a0.z, a0.w), acc[u][0]);
+                        acc[u][1] = __ffma2_rn(make_float2(x.z, x.w), make_float2(a1.z, a1.w), acc[u][1]);
+                    }
                 }
 #pragma unroll
-                for (int u = 0; u < 2; ++u)
+                for (int u = 0; u < SU; ++u)
 #pragma unroll
                     for (int v = 0; v < 2; ++v) {
-                        const int i = pi + 16 * u, j = pj + 16 * v;
+                        const int i = pi + PY * u, j = pj + 16 * v;
                         const bool keep = w.reverse ? j >= i : j <= i;
-                        const float4 s = acc[u][v];
-                        sm[M::kP + i * M::kScoreRow + j] = keep ? (s.x + s.y) + (s.z + s.w) : 0.f;
+                        sm[M::kP + i * M::kScoreRow + j] = keep ? acc[u][v].x + acc[u][v].y : 0.f;
                     }
             }
 #pragma unroll
@@ -329,7 +351,7 @@ __global__ void __launch_bounds__(kThreads) walk_kernel(const __grid_constant__ 
         __syncthreads();
         if (tid == 0) {
             float t = 0.f;
-            for (int i = 0; i < kThreads / 32; ++i) t += dm_red[i];
+            for (int i = 0; i < NT / 32; ++i) t += dm_red[i];
             w.dm_partial[(size_t)bh * w.n_groups + g] = t;
             __threadfence();
             last_flag = atomicAdd(&batch.status[4], 1) == (int)gridDim.x - 1;
@@ -340,7 +362,7 @@ __global__ void __launch_bounds__(kThreads) walk_kernel(const __grid_constant__ 
             // Fixed summation order (deterministic); one warp per head.
             __threadfence();
             const int n_b = (int)gridDim.x / (w.n_groups * w.H), per = n_b * w.n_groups;
-            for (int hh = warp; hh < w.H; hh += kThreads / 32) {
+            for (int hh = warp; hh < w.H; hh += NT / 32) {
                 const float sg = 1.0f / (1.0f + expf(-w.m[hh]));
                 float sum = 0.f;
                 for (int i = lane; i < per; i += 32) {
@@ -518,7 +540,7 @@ cudaError_t launch_walk_dt(const WalkBatch& wb, int n, int BH, cudaStream_t st, 
         return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(BH * wb.w[0].n_groups), (unsigned)n);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(WalkThreads<D>::n);
     cfg.dynamicSmemBytes = WalkSmem<D>::kBytes;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
