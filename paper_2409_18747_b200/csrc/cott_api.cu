@@ -1,5 +1,6 @@
 // C-ABI entry points of libcott: argument validation, execution plan, workspace layout and
 // the launch sequences.  All arithmetic of the method runs in the kernels.
+#include <algorithm>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -603,6 +604,58 @@ static SideStreams* side_streams() {
     return &ss;
 }
 
+// Groups of the two walks of the d = 128 backward.
+static Bwd128Groups bwd128_groups(const Plan& p, int BH, int N, int causal, bool packed) {
+    Bwd128Groups g;
+    g.parts = 1;
+    if (!causal || packed || option_force_group() > 0 || p.n_groups < 2) {
+        // Bidirectional: the plan's groups, every walk starts from the totals.  Packed batches: half as many,
+        // since two CTAs take each.
+        int n = p.n_groups, group = p.group;
+        if (causal && n > 1 && option_force_group() <= 0) {
+            n = n / 2;
+            group = ((N + n - 1) / n + 127) / 128 * 128;
+            n = (N + group - 1) / group;
+        }
+        g.group_q = g.group_k = group; g.n_q = g.n_k = n;
+        g.init_sum = n <= 4;     // (up to four states of 64 KB each out of L2 per CTA, else a scan launch)
+        return g;
+    }
+    // Causal: as many groups for either walk as make the slower one short, within one wave of CTAs.  Per
+    // chunk of 128 tokens a K walk takes 4.6 us and a Q walk 3.5; a walk cut in groups costs a state pass of
+    // about 5 us and 0.9 us per chunk of its parts.  A single later group of the K walk leaves SMs idle in
+    // its state pass: that pass is cut into up to four parts.  (Against half the plan's groups for both:
+    // B=3, H=16, N=2999 113 us / 127, B=1, H=40, N=4096 143 / 165, B=1, H=16, N=16384 224 / 254.)
+    const int chunks = (N + 127) / 128, slots = 148 / BH;
+    double best = 1e30;
+    for (int n_q = 1; n_q < slots; ++n_q)
+        for (int n_k = 1; n_q + n_k <= slots; ++n_k) {
+            if (n_q > chunks || n_k > chunks || n_q > p.n_groups || n_k > p.n_groups) continue;
+            const int n_max = n_q > n_k ? n_q : n_k;
+            int parts = 1;
+            if (n_max > 1)
+                for (int s = 2; s <= 4; ++s)
+                    if (s * (n_max - 1) <= 4 && BH * (n_max - 1) * s <= 148 && n_q * s <= p.n_groups * p.split &&
+                        n_k * s <= 2 * p.n_groups * p.split && chunks >= 2 * n_max * s) parts = s;
+            auto len = [&](int n) { return n == 1 ? chunks : (chunks + n * parts - 1) / (n * parts) * parts; };
+            const double cost = std::max(3.5 * len(n_q), 4.6 * len(n_k)) + (n_q > 1 ? 5 + 0.9 * len(n_q) / parts : 0) +
+                                (n_k > 1 ? 5 + 0.9 * len(n_k) / parts : 0) +
+                                ((n_max - 1) * parts > 4 ? (4.0 + 0.15 * n_max) * ((n_q > 1) + (n_k > 1)) : 0);   // (scan launches)
+            if (cost < best - 1e-9) {
+                best = cost;
+                g.parts = parts;
+                g.group_q = len(n_q) * 128; g.n_q = (chunks + len(n_q) - 1) / len(n_q);
+                g.group_k = len(n_k) * 128; g.n_k = (chunks + len(n_k) - 1) / len(n_k);
+            }
+        }
+    if (best > 1e29) {      // (no room for two CTAs per (b, h) in one wave)
+        g.group_q = g.group_k = chunks * 128; g.n_q = g.n_k = 1;
+    }
+    g.init_sum = (std::max(g.n_q, g.n_k) - 1) * g.parts <= 4;
+    if (!g.init_sum && g.parts > 1) g.init_sum = 1;
+    return g;
+}
+
 static cott_status bwd_impl(const void* q, const void* k, const void* v, const void* d_o, void* dq,
                             void* dk, void* dv, float* dm, int B, int H, int N, int d, int causal,
                             cott_dtype dt, const cott_scale_params* sp, void* ws, const Plan& p,
@@ -658,6 +711,7 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
                 f.sq_fwd = reinterpret_cast<const float*>(static_cast<const char*>(fwd_ws) + kWsHeaderBytes);
                 f.sq_fwd_split = p.split;
             }
+            if (causal && !packed.cu_seqlens && p.n_groups == 1) f.sq_part = nullptr;     // (not computed: nothing precedes the group)
             if (seg.on) {
                 // A segment: the states enter and leave through copies of the kernels' size behind
                 // the other regions of the workspace (zero where the caller passed none).
@@ -786,15 +840,8 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
             return COTT_OK;
         }
         if (d == 128 && option_fused_bwd() != 0) {
-            // Two kinds of walks in one launch (cott_tc_bwd128.cu), each over half as many groups as the
-            // plan has (it counts one CTA per group, here there are two); with one group no partial
-            // state is needed.  (Bidirectional: the plan's groups, every walk starts from the totals.)
-            int n = p.n_groups, group = p.group;
-            if (causal && n > 1 && option_force_group() <= 0) {
-                n = n / 2;
-                group = ((N + n - 1) / n + 127) / 128 * 128;
-                n = (N + group - 1) / group;
-            }
+            // Two kinds of walks in one launch (cott_tc_bwd128.cu).
+            const Bwd128Groups gr = bwd128_groups(p, BH, N, causal, packed.cu_seqlens != nullptr);
             TcBwdFusedArgs f;
             memset(&f, 0, sizeof(f));
             f.q = q; f.k = k; f.v = v; f.d_o = d_o; f.dq = dq; f.dk = dk; f.dv = dv;
@@ -802,34 +849,33 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
             f.l_v = lay.of(v); f.l_dv = lay.of(dv); f.w_k = p.dk; f.w_v = p.dv;
             f.dm_partial = dm_partial; f.dm_out = dm; f.status = status;
             f.m = sp->m; f.seq_len = sp->seq_len; f.seq_len_scalar = sp->seq_len_scalar;
-            f.group = group; f.n_groups = n; f.bidir = causal ? 0 : 1;
+            f.bidir = causal ? 0 : 1;
             f.cu_seqlens = packed.cu_seqlens; f.total_tokens = packed.total_tokens;
-            const bool states = !causal || n > 1;
-            // Up to four partial states are summed by the walks themselves (64 KB each out of L2 per CTA).
-            const bool in_walk = n <= 4;
-            if (states) {
-                auto state_pass = [&](TcWalkArgs a, float* out, int clear) {
-                    a.mode = 0; a.x = nullptr; a.proj = nullptr; a.out = nullptr; a.init = nullptr;
-                    a.state_out = out; a.dm_partial = nullptr; a.dm_out = nullptr; a.epilogue = EPI_PLAIN;
-                    a.status = status; a.clear_status = clear;
-                    a.m = sp->m; a.seq_len = sp->seq_len; a.seq_len_scalar = sp->seq_len_scalar;
-                    a.group = group; a.n_groups = n;
-                    // Nobody reads the state of the group a causal walk visits last.
-                    if (causal) { a.first_group = a.reverse ? 1 : 0; a.grid_groups = n - 1; }
-                    a.reverse = a.reverse ? 0 : 1;       // chunk order opposite to the walk's: L2 reuse of its tiles
-                    return launch_tc_walk(a, B, H, N, d, st);
-                };
-                COTT_CUDA(state_pass(tq, st0, 1));
-                COTT_CUDA(state_pass(tk, st1, 0));
-                if (!in_walk) {
-                    COTT_CUDA(launch_scan(st0, nullptr, BH, n, d, causal ? SCAN_PREFIX : SCAN_TOTAL, st));
-                    COTT_CUDA(launch_scan(st1, nullptr, BH, n, d, causal ? SCAN_SUFFIX : SCAN_TOTAL, st));
-                }
-                f.sq_part = st0; f.r_part = st1;
-            } else {
-                COTT_CUDA(launch_clear_status(status, st));      // status words and the dm counter
+            // (the dQ^ stream's state pass gives V^T K^, the dK^ stream's dO^T Q^; nobody reads the state of
+            // the group a causal walk visits last)
+            const bool need_q = !causal || gr.n_q > 1, need_k = !causal || gr.n_k > 1;
+            auto state_pass = [&](TcWalkArgs a, float* out, int group, int n, int clear) {
+                a.mode = 0; a.x = nullptr; a.proj = nullptr; a.out = nullptr; a.init = nullptr;
+                a.state_out = out; a.dm_partial = nullptr; a.dm_out = nullptr; a.epilogue = EPI_PLAIN;
+                a.status = status; a.clear_status = clear;
+                a.m = sp->m; a.seq_len = sp->seq_len; a.seq_len_scalar = sp->seq_len_scalar;
+                a.group = group / gr.parts; a.n_groups = n * gr.parts;
+                if (causal) { a.first_group = a.reverse ? gr.parts : 0; a.grid_groups = (n - 1) * gr.parts; }
+                a.reverse = a.reverse ? 0 : 1;       // chunk order opposite to the walk's: L2 reuse of its tiles
+                return launch_tc_walk(a, B, H, N, d, st);
+            };
+            if (need_q) {
+                COTT_CUDA(state_pass(tq, st0, gr.group_q, gr.n_q, 1));
+                f.sq_part = st0;
             }
-            COTT_CUDA(launch_tc_bwd128(f, in_walk ? 1 : 0, dm_partial2, B, H, N, st));
+            if (need_k) {
+                COTT_CUDA(state_pass(tk, st1, gr.group_k, gr.n_k, need_q ? 0 : 1));
+                f.r_part = st1;
+            }
+            if (!need_q && !need_k) COTT_CUDA(launch_clear_status(status, st));      // status words and the dm counter
+            if (!gr.init_sum && need_q) COTT_CUDA(launch_scan(st0, nullptr, BH, gr.n_q, d, causal ? SCAN_PREFIX : SCAN_TOTAL, st));
+            if (!gr.init_sum && need_k) COTT_CUDA(launch_scan(st1, nullptr, BH, gr.n_k, d, causal ? SCAN_SUFFIX : SCAN_TOTAL, st));
+            COTT_CUDA(launch_tc_bwd128(f, gr, dm_partial2, B, H, N, st));
             return COTT_OK;
         }
         if (ss) {

@@ -166,10 +166,15 @@ cudaError_t launch_tc_bwd_fused(const TcBwdFusedArgs& a, int B, int H, int N, cu
 // d <= 64 in one launch (cott_tc_bidir_bwd.cu): uses the tensors, layouts, widths, dm_partial
 // ([B * H] floats), dm_out, status (words 0-7 zero at launch), m, seq_len and cu_seqlens of `a`.
 cudaError_t launch_tc_bidir_bwd(const TcBwdFusedArgs& a, int B, int H, int N, cudaStream_t st);
-// Backward at d = 128 in one launch of two kinds of walks (cott_tc_bwd128.cu): sq_part / r_part are the
-// groups' V^T K^ and dO^T Q^ (both NULL with one causal group), raw with init_sum, else scanned;
-// dm_k: [BH, n_groups] beside dm_partial.
-cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, int init_sum, float* dm_k, int B, int H, int N, cudaStream_t st);
+// Backward at d = 128 in one launch of two kinds of walks (cott_tc_bwd128.cu), each over groups of its own;
+// sq_part / r_part are the V^T K^ of the Q walk's groups and the dO^T Q^ of the K walk's (NULL with one
+// causal group), raw with init_sum (`parts` entries per group), else scanned; dm_k: [BH, n_k] beside
+// dm_partial ([BH, n_q]).
+struct Bwd128Groups {
+    int group_q, n_q, group_k, n_k;
+    int parts, init_sum;
+};
+cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, const Bwd128Groups& g, float* dm_k, int B, int H, int N, cudaStream_t st);
 // Both partial states of every group in one launch (uses q, k, v, d_o, the layouts, group,
 // n_groups and status of `a`); clear_status: this is the first kernel of a library call.
 cudaError_t launch_tc_bwd_states(const TcBwdFusedArgs& a, float* sq_out, float* r_out, int clear_status, int B, int H,

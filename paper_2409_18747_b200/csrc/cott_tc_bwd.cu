@@ -1288,7 +1288,8 @@ cudaError_t launch_tc_bwd_states(const TcBwdFusedArgs& a, float* sq_out, float* 
     p.H = H; p.N = N; p.group = a.group; p.n_groups = a.n_groups;
     p.clear_status = clear_status;
     p.all_sq = a.bidir;
-    p.no_sq = (!a.bidir && a.sq_fwd != nullptr) ? 1 : 0;
+    // V^T K^: in the forward call's workspace, or (one group) read by nobody
+    p.no_sq = (!a.bidir && (a.sq_fwd != nullptr || a.n_groups == 1)) ? 1 : 0;
     p.grid_groups = a.n_groups;
     p.wait_limit_kcycles = wait_limit_kcycles();
     static_assert(kStStages * L::kStage <= L::kOffCtl && kStStagesR * 2 * kTile <= L::kOffCtl, "the stage ring overlaps the control block");

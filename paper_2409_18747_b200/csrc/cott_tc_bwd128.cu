@@ -18,7 +18,7 @@
 // along the chain (tiles without a second slot land, scores, mask, products, slots free again).  The
 // two CTAs of a (b, h, group) start side by side, so one of them finds most tiles in L2.
 // Measured against the three role-swapped walks with their state passes and scans: B=4, H=16,
-// N=2048 93 us (207), B=3, H=16, N=2999 128 us (210), 32 packed sequences of 512 to 2048 tokens,
+// N=2048 93 us (207), B=3, H=16, N=2999 113 us (210), 32 packed sequences of 512 to 2048 tokens,
 // H=16, 390 us (622), bidirectional B=8, H=16, N=1024 107 us (124).
 #include "cott_internal.h"
 #include "cott_sm100.cuh"
@@ -56,14 +56,15 @@ struct L {
 };
 
 struct Bwd128Params {
-    // partial states of the groups, fp32 [BH, n_groups, 128 * 128]: V^T K^ and dO^T Q^ (or NULL: one
-    // group, nothing precedes it), raw (init_sum: summed here over the groups before, after, or all)
-    // or already scanned
-    const float* sq; const float* rt; int init_sum;
-    float* dm_q; float* dm_k;           // [BH, n_groups]: parts of the dm sum of the two walks
+    // partial states of the groups, fp32 [BH, n * parts, 128 * 128]: V^T K^ of the Q walk's groups and
+    // dO^T Q^ of the K walk's (or NULL: one group, nothing precedes it), raw (init_sum: summed here over
+    // the groups before, after, or all, `parts` entries each) or already scanned
+    const float* sq; const float* rt; int init_sum; int parts;
+    float* dm_q; float* dm_k;           // [BH, n]: parts of the dm sum of the two walks
     float* dm_out; int* status;
     const float* m; const float* seq_len; float seq_len_scalar;
-    int H; int N; int group; int n_groups;
+    int H; int N;
+    int group_q, n_q, group_k, n_k;     // tokens per group and groups of the two walks
     int wait_limit_kcycles;
     int head_first_mask;                // bit i: in tensor map i (q, k, v, dO, dq, dk, dv) the head index comes before the token index
     const int* cu_seqlens;              // packed batch (VARLEN instances)
@@ -164,13 +165,13 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
         }
         return;
     }
-    const int item = blockIdx.x >> 1;
-    const int g = item % p.n_groups, bh = item / p.n_groups;
+    const int n_groups = kw ? p.n_k : p.n_q, group = kw ? p.group_k : p.group_q;
+    const int bh = blockIdx.x / (p.n_q + p.n_k), g = blockIdx.x % (p.n_q + p.n_k) - (kw ? 0 : p.n_k);
     const int bseq = bh / p.H, h = bh % p.H;
     const int b = VARLEN ? 0 : bseq;                   // batch coordinate of the tensor maps
     const int seq0 = VARLEN ? p.cu_seqlens[bseq] : 0, seq1 = VARLEN ? p.cu_seqlens[bseq + 1] : p.N;
-    const int tok0 = seq0 + g * p.group;
-    const int tok1 = min(seq1, tok0 + p.group);
+    const int tok0 = seq0 + g * group;
+    const int tok1 = min(seq1, tok0 + group);
     const int n_chunks = tok1 > tok0 ? (tok1 - tok0 + kC - 1) / kC : 0;
     // (a packed batch: the last chunk of a sequence may hold rows of the next one; they are normalised
     // to zero in Bv, which silences them in every product, and that chunk's rows are stored one by one)
@@ -261,12 +262,13 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
     if (init_state && warp < kWorkerWarps) {
         // The state before the group's first chunk: row `row`, columns 32 (warp / 4) .. + 31.
         const int cq = warp >> 2;
-        const float* src = part + (size_t)bh * p.n_groups * kD * kD + (size_t)row * kD + cq * 32;
+        const int entries = n_groups * p.parts;
+        const float* src = part + (size_t)bh * entries * kD * kD + (size_t)row * kD + cq * 32;
         float acc[32];
 #pragma unroll
         for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-        const int g_lo = !p.init_sum ? g : (BIDIR ? 0 : (kw ? g + 1 : 0));
-        const int g_hi = !p.init_sum ? g + 1 : (BIDIR ? p.n_groups : (kw ? p.n_groups : g));
+        const int g_lo = !p.init_sum ? g : (BIDIR ? 0 : (kw ? (g + 1) * p.parts : 0));
+        const int g_hi = !p.init_sum ? g + 1 : (BIDIR ? entries : (kw ? entries : g * p.parts));
         for (int gg = g_lo; gg < g_hi; ++gg) {
 #pragma unroll
             for (int i = 0; i < 32; i += 4) {
@@ -658,7 +660,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
         int* last_flag = reinterpret_cast<int*>(&dm_red[8]);
         if (tid == 0) {
             if (!*abort_flag)
-                (kw ? p.dm_k : p.dm_q)[(size_t)bh * p.n_groups + g] = ((dm_red[0] + dm_red[1]) + (dm_red[2] + dm_red[3])) +
+                (kw ? p.dm_k : p.dm_q)[(size_t)bh * n_groups + g] = ((dm_red[0] + dm_red[1]) + (dm_red[2] + dm_red[3])) +
                                                                    ((dm_red[4] + dm_red[5]) + (dm_red[6] + dm_red[7]));
             __threadfence();
             *last_flag = atomicAdd(&p.status[4], 1) == (int)gridDim.x - 1;
@@ -669,18 +671,19 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
             // over rows of <q^, dQ^> plus the rounding term, dc/dm = -ln(s_b) sigma(m_h) (1 - sigma(m_h))
             // c_{b,h}; fixed order, so deterministic.  One warp per head.
             __threadfence();
-            const int per = (int)gridDim.x / (2 * p.H);
+            const int per_q = p.n_q + p.n_k, per = (int)gridDim.x / p.H;
             for (int hh = warp; hh < p.H; hh += kThreads / 32) {
                 const float sg = 1.0f / (1.0f + expf(-p.m[hh]));
                 float sum = 0.f;
                 for (int i = lane; i < per; i += 32) {
-                    const int bb = i / p.n_groups, gg = i - bb * p.n_groups;
+                    const int bb = i / per_q, gg = i - bb * per_q;
                     const float sb2 = p.seq_len ? p.seq_len[bb]
                                                 : (p.seq_len_scalar > 0.f ? p.seq_len_scalar
                                                    : (float)(VARLEN ? max(p.cu_seqlens[bb + 1] - p.cu_seqlens[bb], 1) : p.N));
                     const float ls = logf(sb2);
-                    const size_t idx = ((size_t)bb * p.H + hh) * p.n_groups + gg;
-                    sum += (__ldcg(&p.dm_q[idx]) + __ldcg(&p.dm_k[idx])) * (-ls * sg * (1.0f - sg) * expf(-sg * ls));
+                    const size_t bh2 = (size_t)bb * p.H + hh;
+                    const float part_sum = gg < p.n_q ? __ldcg(&p.dm_q[bh2 * p.n_q + gg]) : __ldcg(&p.dm_k[bh2 * p.n_k + gg - p.n_q]);
+                    sum += part_sum * (-ls * sg * (1.0f - sg) * expf(-sg * ls));
                 }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -707,14 +710,14 @@ tc_bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmDO,
                  const __grid_constant__ CUtensorMap tmDQ, const __grid_constant__ CUtensorMap tmDK,
                  const __grid_constant__ CUtensorMap tmDV, const __grid_constant__ Bwd128Params p) {
-    // The two walks of a (b, h, group) are neighbours in the grid; the longer one, K, first.
-    if ((blockIdx.x & 1) == 0) walk<true, BIDIR, VARLEN>(tmQ, tmK, tmV, tmDO, tmDQ, tmDK, tmDV, p);
+    // The walks of a (b, h) are neighbours in the grid; the longer ones, K, first.
+    if ((int)(blockIdx.x % (p.n_q + p.n_k)) < p.n_k) walk<true, BIDIR, VARLEN>(tmQ, tmK, tmV, tmDO, tmDQ, tmDK, tmDV, p);
     else walk<false, BIDIR, VARLEN>(tmQ, tmK, tmV, tmDO, tmDQ, tmDK, tmDV, p);
 }
 
 }  // namespace
 
-cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, int init_sum, float* dm_k, int B, int H, int N, cudaStream_t st) {
+cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, const Bwd128Groups& g, float* dm_k, int B, int H, int N, cudaStream_t st) {
     const void* ptrs[7] = {a.q, a.k, a.v, a.d_o, a.dq, a.dk, a.dv};
     const RowLayout lays[7] = {a.l_qkv, a.l_qkv, a.l_v, a.l_do, a.l_dqkv, a.l_dqkv, a.l_dv};
     const int wk = a.w_k > 0 ? a.w_k : kD, wv = a.w_v > 0 ? a.w_v : kD;
@@ -734,10 +737,11 @@ cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, int init_sum, float* dm_k,
         const RowLayout lo = resolve_layout(lays[4 + i], H, map_N, dims[4 + i]);
         p.out_rows[i] = const_cast<void*>(ptrs[4 + i]); p.out_sn[i] = lo.sn; p.out_sh[i] = lo.sh; p.out_w[i] = dims[4 + i];
     }
-    p.sq = a.sq_part; p.rt = a.r_part; p.init_sum = init_sum;
+    p.sq = a.sq_part; p.rt = a.r_part; p.init_sum = g.init_sum; p.parts = g.parts;
     p.dm_q = a.dm_partial; p.dm_k = dm_k; p.dm_out = a.dm_out; p.status = a.status;
     p.m = a.m; p.seq_len = a.seq_len; p.seq_len_scalar = a.seq_len_scalar;
-    p.H = H; p.N = N; p.group = a.group; p.n_groups = a.n_groups;
+    p.H = H; p.N = N;
+    p.group_q = g.group_q; p.n_q = g.n_q; p.group_k = g.group_k; p.n_k = g.n_k;
     p.wait_limit_kcycles = wait_limit_kcycles();
     p.cu_seqlens = a.cu_seqlens;
     if (a.bidir && (!a.sq_part || !a.r_part)) return cudaErrorInvalidValue;
@@ -747,7 +751,7 @@ cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, int init_sum, float* dm_k,
         return e;
     const int prof = profile_begin_launch(3, st);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * B * H * a.n_groups));
+    cfg.gridDim = dim3((unsigned)(B * H * (g.n_q + g.n_k)));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = L::kDynBytes;
     cfg.stream = st;

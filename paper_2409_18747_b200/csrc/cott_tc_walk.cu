@@ -1145,8 +1145,8 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
             }
         }
 
-        if (MODE == MODE_STATE && varlen && n_chunks == 0 && p.state_out != nullptr) {
-            // A group behind the end of its sequence: its partial state is zero.
+        if (MODE == MODE_STATE && n_chunks == 0 && p.state_out != nullptr) {
+            // A group (or part of one) behind the end of its sequence: its partial state is zero.
             float4* dst = reinterpret_cast<float4*>(p.state_out + ((size_t)bh * p.n_groups + g) * D * D);
             for (int i = tid; i < D * D / 4; i += 16 * 32) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }

@@ -110,3 +110,16 @@ def test_forward_walk_sums_or_scans_the_group_states(d, groups, force_group):
         r_o, r_s = oracle.fwd_segment(c["q"], c["k"], c["v"], c["m"], st, s)
         gate(o, r_o, torch.bfloat16)
         assert norm_max_err(st_out, r_s) <= 1e-2
+
+
+@pytest.mark.parametrize("B,H,N", [(3, 16, 700), (3, 8, 1000), (1, 12, 900), (2, 20, 1300), (1, 40, 1100), (5, 15, 300)])
+def test_backward_d128_groups_of_the_two_walks(B, H, N):
+    """The d = 128 backward with the library's own choice of groups: the dK, dV walk cut finer than the
+    dQ walk, both cut, state passes in parts, neither cut; ragged last chunks and groups."""
+    c = synth.make_qkv(B, H, N, 128, torch.bfloat16, 7900 + N, with_do=True)
+    q, k, v, d_o, m = (dev(c[x]) for x in ("q", "k", "v", "d_o", "m"))
+    dq, dk, dv, dm = cott.bwd(q, k, v, d_o, m, causal=True)
+    rq, rk, rv, rm = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, True)
+    gate(dq, rq, torch.bfloat16); gate(dk, rk, torch.bfloat16); gate(dv, rv, torch.bfloat16)
+    # (as in the edge test above)
+    assert (abs(dm.double().cpu().numpy() - rm) <= 1e-3 * dm_condition(rv, c["v"], c["m"], None)).all()
