@@ -105,7 +105,11 @@ block_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     if (blockIdx.x == 0 && tid < 8) p.status[tid] = 0;
     if (tid == 0) {
         const int nk = p.dk > 64 ? 2 : 1, nv = p.dv > 64 ? 2 : 1;
+        // (the bound of the wait for these tiles counts from here: a bound of zero runs out whenever the
+        // other warps get to their wait)
+        const long long t0 = clock64();
         mbar_expect_tx(full, (uint32_t)((2 * nk + nv) * L::kBox));
+        wait_expired(full, 0u, t0, abort_flag);
         auto load = [&](uint32_t dst, const CUtensorMap* tm, int which, int n) {
             const bool hf = (p.head_first_mask >> which) & 1;
             for (int hh = 0; hh < n; ++hh) tma_load_4d(dst + hh * L::kBox, tm, full, hh * 64, hf ? h : 0, hf ? 0 : h, b);

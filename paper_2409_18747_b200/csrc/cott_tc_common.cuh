@@ -51,17 +51,19 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
 // The same with the limit checked between a test and a (suspending) try: for a kernel whose only wait is
 // shorter than one suspension, so that its bound is a bound there too.  (Inlined: a call would first wait
 // for every load its caller has in flight.)
+// (wait_expired: one poll of such a wait that began at t0.)
+__device__ __forceinline__ bool wait_expired(uint32_t bar, uint32_t parity, long long t0, volatile int* abort_flag) {
+    if (mbar_test_wait(bar, parity) || clock64() - t0 <= ((long long)abort_flag[3] << 10)) return false;
+    const uint32_t bars = (uint32_t)__cvta_generic_to_shared((const void*)abort_flag) - (uint32_t)kCtlAbort;
+    const uint32_t where = 0x80000000u | ((threadIdx.x >> 5) << 16) | (((bar - bars) & 0x3FFu) << 4) | (parity & 1u);
+    atomicCAS(const_cast<int*>(abort_flag), 0, (int)where);
+    return true;
+}
 __device__ __forceinline__ bool wait_polling(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
     const long long t0 = clock64();
     for (;;) {
         if (mbar_test_wait(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (clock64() - t0 > ((long long)abort_flag[3] << 10)) {
-            const uint32_t bars = (uint32_t)__cvta_generic_to_shared((const void*)abort_flag) - (uint32_t)kCtlAbort;
-            const uint32_t where = 0x80000000u | ((threadIdx.x >> 5) << 16) | (((bar - bars) & 0x3FFu) << 4) | (parity & 1u);
-            atomicCAS(const_cast<int*>(abort_flag), 0, (int)where);
-            return false;
-        }
+        if (*abort_flag || wait_expired(bar, parity, t0, abort_flag)) return false;
         if (mbar_try_wait(bar, parity)) return true;
     }
 }
