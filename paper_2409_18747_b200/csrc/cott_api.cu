@@ -742,11 +742,14 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
                 COTT_CUDA(launch_tc_bwd_fused(f, B, H, N, st));
                 return COTT_OK;
             }
-            if (!causal && p.n_groups == 1 && N <= 1024 && option_bidir_bwd() != 0) {
-                // One group per (b, h) of at most 1024 tokens: both state totals, the three gradients and
-                // dm in one launch (cott_tc_bidir_bwd.cu), nothing but q, k, v, dO read and dq, dk, dv
-                // written.  (A CTA walks its sequence twice with two tile pairs in flight: beyond
-                // eight chunks the two-launch form with its deeper rings is as fast or faster.)
+            if (!causal && p.n_groups == 1 && option_bidir_bwd() != 0) {
+                // One group per (b, h): both state totals, the three gradients and dm in one launch
+                // (cott_tc_bidir_bwd.cu), nothing but q, k, v, dO read and dq, dk, dv written.  At every
+                // length: its second reading comes from L2 or not, two CTAs share an SM, and the two
+                // launches of one CTA per SM pay for every wave twice (B H = 96, N = 2048 78 us against
+                // 85, B H = 256 132 / 168, B H = 256, N = 8192 491 / 607).  Where the plan cuts a
+                // sequence in groups, too few (b, h) for the SMs, the two launches are the faster form
+                // (B H = 64, N = 4096 90 us against 138, B H = 12, N = 1024 24 / 35).
                 COTT_CUDA(launch_clear_status(status, st));      // status words and the dm counter
                 COTT_CUDA(launch_tc_bidir_bwd(f, B, H, N, st));
                 return COTT_OK;

@@ -7,7 +7,7 @@ import torch
 import oracle
 import paper_2409_18747_b200 as cott
 from paper_2409_18747_b200 import synth
-from test_parity_gpu import (DM_COND_F32, TOL_STATE_F32, dev, dm_condition, force_group, gate, gate_dm, option)  # noqa: F401
+from test_parity_gpu import (DM_COND_BF16, DM_COND_F32, TOL_STATE_F32, dev, dm_condition, force_group, gate, gate_dm, option)  # noqa: F401
 from _metrics import norm_max_err
 
 pytestmark = pytest.mark.gpu
@@ -123,3 +123,30 @@ def test_backward_d128_groups_of_the_two_walks(B, H, N):
     gate(dq, rq, torch.bfloat16); gate(dk, rk, torch.bfloat16); gate(dv, rv, torch.bfloat16)
     # (as in the edge test above)
     assert (abs(dm.double().cpu().numpy() - rm) <= 1e-3 * dm_condition(rv, c["v"], c["m"], None)).all()
+
+
+@pytest.mark.parametrize("N", [1025, 1152, 2175])
+@pytest.mark.parametrize("packed", [False, True])
+def test_bidirectional_backward_in_one_launch_beyond_eight_chunks(N, packed, force_group):
+    """The one-launch bidirectional backward with nine, exactly nine and seventeen chunks (its ring has
+    three stages), dense and as a packed batch with short neighbours."""
+    force_group(4096)
+    H, d = 2, 64
+    lens = [N, 1, 130] if packed else [N]
+    cs = [synth.make_qkv(1, H, n, d, torch.bfloat16, 7900 + n + H, with_do=True) for n in lens]
+    m = dev(cs[0]["m"])
+    n0 = cott.cott.launch_count()
+    if packed:
+        q, k, v, d_o = (torch.cat([dev(c[x])[0].permute(1, 0, 2) for c in cs]).contiguous() for x in ("q", "k", "v", "d_o"))
+        cu = torch.tensor([0, N, N + 1, N + 131], dtype=torch.int32, device="cuda")
+        *grads, dm = cott.bwd_varlen(q, k, v, d_o, m, cu, N, causal=False)
+        grads = [x[:N].permute(1, 0, 2)[None] for x in grads]
+    else:
+        *grads, dm = cott.bwd(*(dev(cs[0][x]) for x in ("q", "k", "v", "d_o")), m, causal=False)
+    assert cott.cott.launch_count() - n0 == 1
+    c = cs[0]
+    *refs, rm = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, False)
+    for x, r in zip(grads, refs):
+        gate(x.contiguous(), r, torch.bfloat16)
+    if not packed:
+        gate_dm(dm, rm, 1e-2, dm_condition(refs[2], c["v"], c["m"], None), DM_COND_BF16)
