@@ -209,19 +209,25 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
         if (mode != ROW_RAW) { v.x *= s; v.y *= s; v.z *= s; v.w *= s; }
     };
     auto put_rows = [&](float4 (&r)[RPT], int off, int mode) {
+        bool finite = true;
 #pragma unroll
         for (int u = 0; u < RPT; ++u) {
             treat(r[u], mode);
             *reinterpret_cast<float4*>(sm + off + (ty + TY * u) * M::kRow + tx * 4) = r[u];
+            finite = finite && dot4(r[u], zero4) == 0.f;      // (infinity and NaN times zero are NaN)
         }
+        return finite;
     };
 
     float dm_acc = 0.f;
     for (int it = 0; it < n_chunks; ++it) {
         const int t0 = chunk_row(it);
         if (write_out) put_rows(rx, M::kX, w.mode_x);
-        if (update) { put_rows(ra, M::kA, w.mode_a); put_rows(rb, M::kB, w.mode_b); }
-        __syncthreads();
+        bool finite = true;
+        if (update) { put_rows(ra, M::kA, w.mode_a); finite = put_rows(rb, M::kB, w.mode_b); }
+        // A masked score is zero, and zero times an infinity or a NaN is not: with one in a Bv row of this
+        // chunk the masked pairs are left out of P Bv, not multiplied by zero.
+        const bool skip_masked = __syncthreads_or(!finite);
         float4 rp[RPT];
         if (w.epilogue != EPI_PLAIN) load_rows(rp, P, w.lproj.sn, t0);
         if (it + 1 < n_chunks) load_chunk(chunk_row(it + 1));
@@ -276,6 +282,17 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
             }
             if (update) {
                 __syncthreads();
+                if (skip_masked) {
+#pragma unroll 1
+                    for (int k = 0; k < kChunk; ++k) {
+                        const float4 v = *reinterpret_cast<const float4*>(sm + M::kB + k * M::kRow + tx * 4);
+#pragma unroll
+                        for (int u = 0; u < RPT; ++u) {
+                            const int i = ty + TY * u;
+                            if (w.reverse ? k >= i : k <= i) axpy4(out[u], sm[M::kP + i * M::kScoreRow + k], v);
+                        }
+                    }
+                } else
 #pragma unroll 2
                 for (int k = 0; k < kChunk; k += 4) {
                     float4 x[RPT];

@@ -150,3 +150,34 @@ def test_bidirectional_backward_in_one_launch_beyond_eight_chunks(N, packed, for
         gate(x.contiguous(), r, torch.bfloat16)
     if not packed:
         gate_dm(dm, rm, 1e-2, dm_condition(refs[2], c["v"], c["m"], None), DM_COND_BF16)
+
+
+@pytest.mark.parametrize("d", [32, 64, 128])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("t", [0, 5, 31, 40, 69])
+def test_fp32_causal_rows_do_not_see_infinities_of_masked_tokens(d, bad, t):
+    """One token of v, k or dO is not finite: what does not depend on it stays what it is without it.  The
+    walk masks pairs inside a chunk of 32 tokens, and a masked score of zero times infinity would be NaN."""
+    B, H, N = 1, 2, 70
+    c = synth.make_qkv(B, H, N, d, torch.float32, 8100 + d + t, with_do=True)
+    m = dev(c["m"])
+    clean = {x: dev(c[x]) for x in ("q", "k", "v", "d_o")}
+    ref_o = oracle.fwd_quadratic(c["q"], c["k"], c["v"], c["m"], None, True)
+    refs = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, True)
+    for name in ("v", "k", "d_o"):
+        x = {**clean, name: clean[name].clone()}
+        x[name][0, 0, t] = bad
+        o = cott.fwd(x["q"], x["k"], x["v"], m, causal=True)
+        dq, dk, dv, _ = cott.bwd(x["q"], x["k"], x["v"], x["d_o"], m, causal=True)
+        ok = torch.ones(B, H, N, dtype=torch.bool)
+        if name == "d_o":                     # dk, dv of a token sum over the tokens from it on
+            ok[0, 0, :t + 1] = False
+            pairs = ((dk, refs[1]), (dv, refs[2]))
+        else:                                 # o, dq of a token over the tokens up to it
+            ok[0, 0, t:] = False
+            pairs = ((o, ref_o), (dq, refs[0]))
+        for got, r in pairs:
+            got = got.cpu()
+            assert got[ok].isfinite().all() and not got[~ok].isfinite().all()
+            r = torch.from_numpy(r)
+            assert (got[ok].double() - r[ok]).abs().max() <= 1e-5 * r.abs().max()
