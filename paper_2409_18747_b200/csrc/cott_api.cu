@@ -381,9 +381,8 @@ static cott_status run_streams(const SimtStream* s, int n, const Plan& p, int BH
         for (int i = 0; i < n; ++i) {
             if (s[i].sibling >= 0) continue;
             const int mode = !causal ? SCAN_TOTAL : (s[i].w.reverse ? SCAN_SUFFIX : SCAN_PREFIX);
-            // (these states contain c, like a caller's initial state, which the scan starts from)
-            COTT_CUDA(launch_scan(s[i].states, s[i].total_out, BH, p.n_groups, d, mode, st, nullptr, nullptr, 0.f, 1, 1,
-                                  s[i].state_in));
+            // (a caller's state joins in the walks, which add it to the sums and not the partial states to it)
+            COTT_CUDA(launch_scan(s[i].states, s[i].total_out, BH, p.n_groups, d, mode, st));
         }
     for (int i = 0; i < n; ++i) {
         WalkArgs w = s[i].w;
@@ -391,8 +390,8 @@ static cott_status run_streams(const SimtStream* s, int n, const Plan& p, int BH
         w.init = s[i].sibling >= 0 ? s[s[i].sibling].states : s[i].states;
         w.init_transposed = s[i].sibling >= 0 ? 1 : 0;
         w.init_sum = in_walk ? 1 : 0;
-        w.init_extra = in_walk ? s[i].state_in : nullptr;
-        w.final_state = in_walk ? s[i].total_out : nullptr;
+        w.init_extra = s[i].state_in;
+        w.final_state = (in_walk || s[i].state_in) ? s[i].total_out : nullptr;
         wb.w[i] = w;
     }
     COTT_CUDA(launch_walk_simt(wb, n, BH, d, dt, st, in_walk));

@@ -61,6 +61,17 @@ __device__ __forceinline__ void axpy4(float4& y, float a, float4 x) {
     y = make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
+// y += a.x x0 + a.y x1 + a.z x2 + a.w x3, the four products summed among themselves first: a chain of D
+// multiply-adds onto one accumulator rounds at the size of the whole sum D times, this D / 4 times.
+__device__ __forceinline__ void axpy4x4(float4& y, float4 a, float4 x0, float4 x1, float4 x2, float4 x3) {
+    float2 lo = __fmul2_rn(make_float2(a.x, a.x), make_float2(x0.x, x0.y)), hi = __fmul2_rn(make_float2(a.x, a.x), make_float2(x0.z, x0.w));
+    lo = __ffma2_rn(make_float2(a.y, a.y), make_float2(x1.x, x1.y), lo); hi = __ffma2_rn(make_float2(a.y, a.y), make_float2(x1.z, x1.w), hi);
+    lo = __ffma2_rn(make_float2(a.z, a.z), make_float2(x2.x, x2.y), lo); hi = __ffma2_rn(make_float2(a.z, a.z), make_float2(x2.z, x2.w), hi);
+    lo = __ffma2_rn(make_float2(a.w, a.w), make_float2(x3.x, x3.y), lo); hi = __ffma2_rn(make_float2(a.w, a.w), make_float2(x3.z, x3.w), hi);
+    lo = __fadd2_rn(make_float2(y.x, y.y), lo); hi = __fadd2_rn(make_float2(y.z, y.w), hi);
+    y = make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+
 // Shared memory of the walk: three chunk tiles (rows padded by four words: threads that read 16
 // consecutive rows at the same column then hit different banks), the chunk's masked scores and
 // the state.
@@ -180,7 +191,9 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
             }
         }
     };
-    if (w.init_extra) add_state(w.init_extra + (size_t)bh * D * D, false);
+    // A caller's state is added to the sum of the partial states, not they to it one by one; a single group
+    // keeps it apart altogether, and the two meet where the state is read.
+    const float* base = (w.init_extra && !w.init) ? w.init_extra + (size_t)bh * D * D : nullptr;
     if (w.init) {
         const float* part = w.init + (size_t)bh * w.n_groups * D * D;
         if (w.init_sum) {
@@ -189,10 +202,35 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
         } else {
             add_state(part + (size_t)g * D * D, w.init_transposed);
         }
+        if (w.init_extra) add_state(w.init_extra + (size_t)bh * D * D, false);
     }
-    auto put_state = [&]() {
+    if (base) have_state = true;
+    // The total of several groups is what comes before the last one plus its partial state: the former goes
+    // to its place now, the latter is added at the end (this walk's rows accumulate onto the whole sum).
+    // Where a scan launch has left the sum of the partial states there, the caller's state is added.
+    const bool total = w.init && w.final_state && update && g == (w.reverse ? 0 : w.n_groups - 1);
+    auto final_row = [&](int r) {
+        return reinterpret_cast<float4*>(w.final_state + (w.final_grouped ? ((size_t)bh * w.n_groups + g) : (size_t)bh) * D * D +
+                                         (size_t)(ty * SR + r) * D + tx * 4);
+    };
+    if (total && w.init_sum) {
 #pragma unroll
-        for (int r = 0; r < SR; ++r) *reinterpret_cast<float4*>(sm + M::kS + (ty * SR + r) * D + tx * 4) = S[r];
+        for (int r = 0; r < SR; ++r) *final_row(r) = S[r];
+    }
+    auto add = [](float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); };
+    auto state_row = [&](int r) {
+        return base ? add(*reinterpret_cast<const float4*>(base + (size_t)(ty * SR + r) * D + tx * 4), S[r]) : S[r];
+    };
+    auto put_state = [&]() {
+        constexpr int RB = SR < 4 ? SR : 4;
+#pragma unroll
+        for (int r0 = 0; r0 < SR; r0 += RB) {
+            float4 v[RB];
+#pragma unroll
+            for (int r = 0; r < RB; ++r) v[r] = state_row(r0 + r);
+#pragma unroll
+            for (int r = 0; r < RB; ++r) *reinterpret_cast<float4*>(sm + M::kS + (ty * SR + r0 + r) * D + tx * 4) = v[r];
+        }
     };
     if (write_out && have_state) put_state();
 
@@ -219,6 +257,7 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
         return finite;
     };
 
+    const bool keep_state = w.final_state && (w.final_grouped || w.n_groups == 1);
     float dm_acc = 0.f;
     for (int it = 0; it < n_chunks; ++it) {
         const int t0 = chunk_row(it);
@@ -241,17 +280,24 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
                 float2 acc[SU][2];
 #pragma unroll
                 for (int u = 0; u < SU; ++u) { acc[u][0] = make_float2(0.f, 0.f); acc[u][1] = acc[u][0]; }
-#pragma unroll 4
-                for (int k = 0; k < D; k += 4) {
-                    const float4 a0 = *reinterpret_cast<const float4*>(sm + M::kA + pj * M::kRow + k);
-                    const float4 a1 = *reinterpret_cast<const float4*>(sm + M::kA + (pj + 16) * M::kRow + k);
+#pragma unroll 2
+                for (int k = 0; k < D; k += 8) {       // (eight products are summed among themselves first, as in axpy4x4)
+                    const float4 a00 = *reinterpret_cast<const float4*>(sm + M::kA + pj * M::kRow + k);
+                    const float4 a01 = *reinterpret_cast<const float4*>(sm + M::kA + pj * M::kRow + k + 4);
+                    const float4 a10 = *reinterpret_cast<const float4*>(sm + M::kA + (pj + 16) * M::kRow + k);
+                    const float4 a11 = *reinterpret_cast<const float4*>(sm + M::kA + (pj + 16) * M::kRow + k + 4);
+                    auto part = [](float4 x0, float4 x1, float4 y0, float4 y1) {
+                        float2 t = __fmul2_rn(make_float2(x0.x, x0.y), make_float2(y0.x, y0.y));
+                        t = __ffma2_rn(make_float2(x0.z, x0.w), make_float2(y0.z, y0.w), t);
+                        t = __ffma2_rn(make_float2(x1.x, x1.y), make_float2(y1.x, y1.y), t);
+                        return __ffma2_rn(make_float2(x1.z, x1.w), make_float2(y1.z, y1.w), t);
+                    };
 #pragma unroll
                     for (int u = 0; u < SU; ++u) {
-                        const float4 x = *reinterpret_cast<const float4*>(sm + M::kX + (pi + PY * u) * M::kRow + k);
-                        acc[u][0] = __ffma2_rn(make_float2(x.x, x.y), make_float2(a0.x, a0.y), acc[u][0]);
-                        acc[u][1] = __ffma2_rn(make_float2(x.x, x.y), make_float2(a1.x, a1.y), acc[u][1]);
-                        acc[u][0] = __ffma2_rn(make_float2(x.z, x.w), make_float2(a0.z, a0.w), acc[u][0]);
-                        acc[u][1] = __ffma2_rn(make_float2(x.z, x.w), make_float2(a1.z, a1.w), acc[u][1]);
+                        const float4 x0 = *reinterpret_cast<const float4*>(sm + M::kX + (pi + PY * u) * M::kRow + k);
+                        const float4 x1 = *reinterpret_cast<const float4*>(sm + M::kX + (pi + PY * u) * M::kRow + k + 4);
+                        acc[u][0] = __fadd2_rn(acc[u][0], part(x0, x1, a00, a01));
+                        acc[u][1] = __fadd2_rn(acc[u][1], part(x0, x1, a10, a11));
                     }
                 }
 #pragma unroll
@@ -275,9 +321,7 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
                     const float4 v0 = *reinterpret_cast<const float4*>(s0), v1 = *reinterpret_cast<const float4*>(s0 + D);
                     const float4 v2 = *reinterpret_cast<const float4*>(s0 + 2 * D), v3 = *reinterpret_cast<const float4*>(s0 + 3 * D);
 #pragma unroll
-                    for (int u = 0; u < RPT; ++u) {
-                        axpy4(out[u], x[u].x, v0); axpy4(out[u], x[u].y, v1); axpy4(out[u], x[u].z, v2); axpy4(out[u], x[u].w, v3);
-                    }
+                    for (int u = 0; u < RPT; ++u) axpy4x4(out[u], x[u], v0, v1, v2, v3);
                 }
             }
             if (update) {
@@ -303,9 +347,7 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
                     const float4 v0 = *reinterpret_cast<const float4*>(b0), v1 = *reinterpret_cast<const float4*>(b0 + M::kRow);
                     const float4 v2 = *reinterpret_cast<const float4*>(b0 + 2 * M::kRow), v3 = *reinterpret_cast<const float4*>(b0 + 3 * M::kRow);
 #pragma unroll
-                    for (int u = 0; u < RPT; ++u) {
-                        axpy4(out[u], x[u].x, v0); axpy4(out[u], x[u].y, v1); axpy4(out[u], x[u].z, v2); axpy4(out[u], x[u].w, v3);
-                    }
+                    for (int u = 0; u < RPT; ++u) axpy4x4(out[u], x[u], v0, v1, v2, v3);
                 }
             }
 #pragma unroll
@@ -354,13 +396,20 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
         __syncthreads();
     }
 
-    // The group's partial state, or the total where this group is the last one the walk visits.
-    if (w.final_state && (w.final_grouped || w.n_groups == 1 || !update || g == (w.reverse ? 0 : w.n_groups - 1))) {
-        float* dst = w.final_state + (w.final_grouped ? ((size_t)bh * w.n_groups + g) : (size_t)bh) * D * D;
-        if (w.final_grouped || update || g == 0) {
+    // The group's partial state, or the total: of a single group, or of all where the mask is all ones.
+    if (total) {
+        const float* rest = (w.init_sum ? w.init + ((size_t)bh * w.n_groups + g) * D * D : w.init_extra + (size_t)bh * D * D) +
+                            (size_t)ty * SR * D + tx * 4;
+        // (all loads before the first store: the compiler has to keep their order)
 #pragma unroll
-            for (int r = 0; r < SR; ++r) *reinterpret_cast<float4*>(dst + (size_t)(ty * SR + r) * D + tx * 4) = S[r];
-        }
+        for (int r = 0; r < SR; ++r) S[r] = add(*final_row(r), *reinterpret_cast<const float4*>(rest + r * D));
+#pragma unroll
+        for (int r = 0; r < SR; ++r) *final_row(r) = S[r];
+    } else if (keep_state || (w.final_state && !update && g == 0)) {
+#pragma unroll
+        for (int r = 0; r < SR; ++r) S[r] = state_row(r);
+#pragma unroll
+        for (int r = 0; r < SR; ++r) *final_row(r) = S[r];
     }
     if (w.dm_partial) {
         dm_acc = warp_sum(dm_acc);
