@@ -257,10 +257,12 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
         return finite;
     };
 
+    // (the state after the last chunk is read by nobody unless it is a partial state or a single group's total)
     const bool keep_state = w.final_state && (w.final_grouped || w.n_groups == 1);
     float dm_acc = 0.f;
     for (int it = 0; it < n_chunks; ++it) {
         const int t0 = chunk_row(it);
+        const int n_rows = min(kChunk, hi - t0);     // (rows behind it are zero: the loops over tokens leave them out)
         if (write_out) put_rows(rx, M::kX, w.mode_x);
         bool finite = true;
         if (update) { put_rows(ra, M::kA, w.mode_a); finite = put_rows(rb, M::kB, w.mode_b); }
@@ -338,7 +340,7 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
                     }
                 } else
 #pragma unroll 2
-                for (int k = 0; k < kChunk; k += 4) {
+                for (int k = 0; k < n_rows; k += 4) {
                     float4 x[RPT];
 #pragma unroll
                     for (int u = 0; u < RPT; ++u)
@@ -373,10 +375,10 @@ __global__ void __launch_bounds__(WalkThreads<D>::n, WalkThreads<D>::ctas) walk_
                 if (t < hi) store4<T>(O + (long long)t * w.lout.sn + tx * 4, out[u]);
             }
         }
-        if (update) {
+        if (update && (it + 1 < n_chunks || keep_state)) {
             have_state = true;
 #pragma unroll 4
-            for (int k = 0; k < kChunk; ++k) {
+            for (int k = 0; k < n_rows; ++k) {
                 const float4 v = *reinterpret_cast<const float4*>(sm + M::kB + k * M::kRow + tx * 4);
                 const float* ap = sm + M::kA + k * M::kRow + ty * SR;
                 if constexpr (SR >= 4) {
