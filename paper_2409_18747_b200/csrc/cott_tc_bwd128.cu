@@ -459,8 +459,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
                 tmem_wait_st();
                 tc_fence_before();
             };
-            // x^ = x / max(||x||, eps) on half a row of Bv, in place (lanes l and l ^ 16 share a row),
-            // scaled in packed bf16 arithmetic with the scale split in two terms (see normalise_row64).
+            // x^ = x / max(||x||, eps) on half a row of Bv, in place (lanes l and l ^ 16 share a row).
             auto normalise = [&](int c) {
                 if (!wait(bar(B_FB, c), par(c))) return;
                 const int nrow = w8 * 16 + (lane & 15), half = lane >> 4;
@@ -480,13 +479,12 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
                 ss += __shfl_xor_sync(0xffffffffu, ss, 16);
                 float rn = 1.0f / fmaxf(sqrtf(ss), kEps);
                 if (VARLEN && chunk_row(c) + nrow >= tok1) rn = 0.f;      // a row of the next sequence
-                const RowScale sc(rn);
 #pragma unroll 2
                 for (int j = 0; j < 8; ++j) {
                     uint4 w = *reinterpret_cast<const uint4*>(tile + ((j ^ (nrow & 7)) << 4));
                     __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&w);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) e[i] = sc(e[i]);
+                    for (int i = 0; i < 4; ++i) e[i] = scale_round(e[i], rn);
                     *reinterpret_cast<uint4*>(tile + ((j ^ (nrow & 7)) << 4)) = w;
                 }
                 fence_proxy_async();
@@ -597,7 +595,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
                 const bool by_rows = is_ragged(c);
                 const float sc = cfac * rp, mc = nrm > kEps ? -dp * cfac * rp * rp * rp : 0.f;
                 const float2 sc2 = make_float2(sc, sc), mc2 = make_float2(mc, mc);
-                const RowScale ks(use ? rp : 0.f);
+                const float ks = use ? rp : 0.f;
                 float2 k2 = make_float2(0.f, 0.f);
 #pragma unroll 1
                 for (int pc = 0; pc < 4; ++pc) {
@@ -611,7 +609,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const __nv_bfloat162 e = reinterpret_cast<const __nv_bfloat162*>(w)[i];
-                        if (kw) k2 = __ffma2_rn(__bfloat1622float2(ks(e)), r[i], k2);
+                        if (kw) k2 = __ffma2_rn(__bfloat1622float2(scale_round(e, ks)), r[i], k2);
                         const float2 v = __ffma2_rn(__bfloat1622float2(e), mc2, __fmul2_rn(r[i], sc2));
                         reinterpret_cast<uint32_t*>(o)[i] = pack_bf16(v.x, v.y);
                     }

@@ -77,6 +77,12 @@ __device__ __forceinline__ uint4 pack8(const uint32_t* r) {
     return w;
 }
 
+// x * rn in fp32, rounded to bf16 once.
+__device__ __forceinline__ __nv_bfloat162 scale_round(__nv_bfloat162 x, float rn) {
+    const float2 f = __fmul2_rn(__bfloat1622float2(x), make_float2(rn, rn));
+    return __floats2bfloat162_rn(f.x, f.y);
+}
+
 // x * rn in packed bf16 arithmetic with the scale split in two bf16 terms (rn = hi + lo to 2^-17):
 // round(x hi + round(x lo)) is x rn rounded once, up to a second rounding of the small term.
 struct RowScale {

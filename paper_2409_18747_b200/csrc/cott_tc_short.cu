@@ -203,7 +203,7 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             nq += __shfl_xor_sync(0xffffffffu, nq, 16);
             nk += __shfl_xor_sync(0xffffffffu, nk, 16);
             if (half == 0) rq_buf[nrow] = 1.0f / fmaxf(sqrtf(nq), kEps);
-            const RowScale rk(1.0f / fmaxf(sqrtf(nk), kEps));
+            const float rk = 1.0f / fmaxf(sqrtf(nk), kEps);
 #pragma unroll
             for (int j = 0; j < 4 * NH; ++j) {
                 const int ch = half * 4 * NH + j;
@@ -212,7 +212,7 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     __nv_bfloat162& e = reinterpret_cast<__nv_bfloat162*>(&w)[i];
-                    e = rk(e);
+                    e = scale_round(e, rk);
                 }
                 *pk = w;
             }

@@ -802,21 +802,11 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
             for (int j = 0; j < NC; j += 2) { sumsq8(wn[j], s0); sumsq8(wn[j + 1], s1); }
             float r = 1.0f / fmaxf(sqrtf(pair_sum((s0.x + s0.y) + (s1.x + s1.y))), kEps);
             if (varlen && chunk_row(c) + nrow >= tok1) r = 0.f;     // a row of the next sequence
-            const tc::RowScale rs(r);
 #pragma unroll
             for (int j = 0; j < NC; ++j) {
                 __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&wn[j]);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    // (the state pass, which loads bound, rounds x r itself: its sums enter dm, which
-                    // cancels heavily)
-                    if (MODE == MODE_STATE) {
-                        const float2 f = __fmul2_rn(__bfloat1622float2(e[i]), make_float2(r, r));
-                        e[i] = __floats2bfloat162_rn(f.x, f.y);
-                    } else {
-                        e[i] = rs(e[i]);
-                    }
-                }
+                for (int i = 0; i < 4; ++i) e[i] = tc::scale_round(e[i], r);
                 *reinterpret_cast<uint4*>(tile_h_ptr(nt, j)) = wn[j];
             }
             fence_proxy_async();

@@ -226,3 +226,30 @@ def test_fp32_rows_are_summed_in_short_chains(N, causal):
     m = torch.randn(H, generator=g)
     o = cott.fwd(*(dev(x) for x in (q, k, v, m)), causal=causal)
     assert _rel(o, oracle.fwd_quadratic(q, k, v, m, None, causal)) <= 2.7 * U32
+
+
+@pytest.mark.parametrize("path", ["walk", "short64", "short128", "backward128"])
+def test_normalised_rows_are_rounded_once(path):
+    """x / ||x|| as the tensor cores get it is bf16, rounded once from fp32: only elements whose exact quotient
+    is within 3 u of the middle between two bf16 numbers may end on the other side, 3 u / 2^-9 = one in ten
+    thousand; the gate is three times that.  (Products with a scale split in two bf16 terms measure 5 to 8.)
+    Unit vectors as the other operands, with c = 1/2, make the call return the rows."""
+    d = 64 if path == "short64" else 128
+    B, H = 2, 3
+    g = torch.Generator().manual_seed(11)
+    x = torch.randn((B, H, d, d), generator=g).to(torch.bfloat16)
+    eye = torch.eye(d, dtype=torch.bfloat16).expand(B, H, d, d).contiguous()
+    m, s = torch.zeros(H), torch.full((B,), 4.0)               # 4^-sigma(0) = 1/2
+    xd, ed = dev(x), dev(eye)
+    if path == "walk":                                         # state = c sum_j x^_j e_j^T
+        got = cott.fwd(ed, xd, ed, dev(m), dev(s), causal=True, return_state=True)[1].transpose(-1, -2)
+    elif path == "backward128":                                # dk_j = c q^_j without its part along k_j = e_{d-1}
+        k = torch.zeros_like(ed)
+        k[..., d - 1] = 1
+        got = cott.bwd(xd, k, ed, ed, dev(m), dev(s), causal=True)[1]
+    else:                                                      # o_i = c sum_j <e_i, x^_j> e_j
+        got = cott.fwd(ed, xd, ed, dev(m), dev(s), causal=False).transpose(-1, -2)
+    want = (x.double() / x.double().norm(dim=-1, keepdim=True)).float().to(torch.bfloat16)
+    got = (2.0 * got.float().cpu()).to(torch.bfloat16)
+    cols = slice(0, d - 1) if path == "backward128" else slice(None)
+    assert (got != want)[..., cols].double().mean().item() <= 3e-4
