@@ -131,19 +131,23 @@ struct Plan {
     bool padded;
 };
 
+// May every walk CTA sum the partial states it needs itself (no scan launch)?  `reads`: how many states of
+// d x d floats the last CTA adds up, one after the other out of L2 (a caller's state among them).
+// d = 64 (16 KB each): the sum is 0.5 to 4 us ahead of a scan launch up to six groups and level with it at seven
+// and eight; more only where a group's own rows dwarf the states.
+// d = 128 (64 KB, about 2.4 us each): a scan launch costs more the more heads there are, so one read
+// always pays (B H = 1 to 73, two groups: 2.4 to 19 us), two from about 20 heads on (B H = 8: 0.6 to 1.8 us
+// slower than a scan, 24: level, 32: 1 to 1.6 us faster), three from 40 on (B H = 48, N = 2999, a caller's
+// state, three groups: 50 us against 57 with the scan; 32 heads: up to 3 us slower), four up to 11 us
+// slower except for groups as long as the last clause asks for (B H = 16, N = 131072: 510 us against 514).
+static bool sum_in_walk(int n_groups, int reads, long BH, int d, int group) {
+    if (n_groups <= 9 && (long long)n_groups * d * 8 <= group) return true;
+    return d == 64 ? n_groups <= 7 : reads <= (BH >= 40 ? 3 : BH >= 20 ? 2 : 1);
+}
+
 // Sequence groups give sequence-level parallelism when B*H alone cannot fill the GPU:
 // halve the group until there are enough CTAs, but never below a floor that keeps the
 // per-group state traffic (d*d fp32) small against the group's own q,k,v,o bytes.
-// May every walk CTA sum the partial states it needs itself (no scan launch)?  It reads n_groups / 2
-// states of d x d floats on average, one after the other out of L2.  At d = 64 (16 KB each) that beats
-// a scan launch up to nine groups (B H = 24, N = 4096, six groups: 24.9 us against 25.4); at d = 128
-// (64 KB) up to four (B=3, H=16, N=2999, three groups: 50 us against 57; six groups: 50 against 45 the
-// other way round), and up to nine where the group's own rows dwarf the sum (B H = 16, N = 131072 with the
-// state kept: 510 us against 514).
-static bool sum_in_walk(int n_groups, int d, int group) {
-    return n_groups <= (d == 64 ? 9 : 4) || (n_groups <= 9 && (long long)n_groups * d * 8 <= group);
-}
-
 static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv, int causal, Plan* p) {
     if (B < 1 || H < 1 || N < 1) return false;
     if (dt != COTT_F32 && dt != COTT_BF16) return false;
@@ -199,7 +203,7 @@ static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv
     // sums `split` times as many states.
     p->split = 1;
     if (p->path == 1 && causal && p->n_groups >= 2 && p->n_groups <= 8 &&
-        sum_in_walk(p->n_groups, d, group) && N % group == 0) {
+        sum_in_walk(p->n_groups, p->n_groups - 1, BH, d, group) && N % group == 0) {
         const long ctas = BH * (p->n_groups - 1);
         const int chunks = group / p->chunk;
         for (int s2 = 4; s2 >= 2; s2 >>= 1)
@@ -422,7 +426,10 @@ static cott_status run_tc_stream(TcWalkArgs t, const Plan& p, int B, int H, int 
     // dropped.  In the forward pass a caller's initial state joins that sum, and the CTA of the last
     // group, whose running state ends as the total, writes it; the other streams leave both to the scan.
     const bool forward = causal && !t.reverse && t.x_norm && !t.norm_bv && !t.cu_seqlens;
-    const bool fused_scan = (forward || (!total_out && !state_in)) && sum_in_walk(p.n_groups, d, p.group);
+    const int reads = causal ? p.n_groups - 1 + (state_in ? 1 : 0) : p.n_groups;
+    // (a packed batch has more groups than fit one wave, and with an all-ones mask every CTA reads all of a
+    // sequence's states: 6 sequences of up to 900 tokens, H = 4, d = 64, seven groups: 23 us against 19 with a scan)
+    const bool fused_scan = (forward || (!total_out && !state_in)) && !(t.cu_seqlens && !causal && reads > 3) && sum_in_walk(p.n_groups, reads, (long)B * H, d, p.group);
     const int split = (fused_scan && causal) ? p.split : 1;
     if (!reuse_transposed) {
         TcWalkArgs a = t;
@@ -706,7 +713,7 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
             // The forward call of the same q, k, v (no state in or out) left the partial states
             // K^^T V of every group but the last in its workspace whenever its walk summed them
             // itself: the transposes of what this walk needs, so the state pass skips k and v.
-            if (fwd_ws && !packed.cu_seqlens && causal && p.n_groups >= 2 && sum_in_walk(p.n_groups, d, p.group)) {
+            if (fwd_ws && !packed.cu_seqlens && causal && p.n_groups >= 2 && sum_in_walk(p.n_groups, p.n_groups - 1, BH, d, p.group)) {
                 f.sq_fwd = reinterpret_cast<const float*>(static_cast<const char*>(fwd_ws) + kWsHeaderBytes);
                 f.sq_fwd_split = p.split;
             }

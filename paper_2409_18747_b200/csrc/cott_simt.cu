@@ -695,7 +695,10 @@ cudaError_t launch_scan(float* states, float* total_out, int BH, int n_groups, i
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    // Started while the state pass drains only where that pass leaves most SMs free (1 us): else the scan's CTAs
+    // crowd onto the few that are (d = 128, 32 groups, B H = 4, N = 4096: 28 us a forward against 25 started
+    // behind the pass; a readout 26 against 19).
+    cfg.numAttrs = (long)BH * (n_groups - 1) <= 40 ? 1 : 0;
     if (cudaError_t e = cudaLaunchKernelEx(&cfg, scan_kernel, states, total_out, n_groups, dd, mode, total_scale_m, seq_len,
                                            seq_len_scalar, H, N, init_in); e != cudaSuccess)
         return e;

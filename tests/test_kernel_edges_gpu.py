@@ -112,6 +112,26 @@ def test_forward_walk_sums_or_scans_the_group_states(d, groups, force_group):
         assert norm_max_err(st_out, r_s) <= 1e-2
 
 
+@pytest.mark.parametrize("BH,d,groups,given,summed", [
+    (3, 64, 6, True, True), (3, 64, 8, True, False), (3, 128, 2, False, True), (3, 128, 2, True, False),
+    (3, 128, 3, False, False), (20, 128, 3, False, True), (20, 128, 3, True, False), (40, 128, 3, True, True),
+    (40, 128, 4, True, False)])
+def test_forward_walk_sums_states_where_that_is_faster(BH, d, groups, given, summed, force_group):
+    """The rule that picks between the sum inside the walk (two launches) and a scan launch (three): by the
+    number of states a CTA would read and, at d = 128, the number of heads."""
+    force_group(128)
+    B, H, N = 1, BH, 128 * groups - 5
+    c = synth.make_qkv(B, H, N, d, torch.bfloat16, 8600 + BH + groups)
+    state = torch.randn((B, H, d, d), generator=torch.Generator().manual_seed(6)) if given else torch.zeros(B, H, d, d)
+    q, k, v, m = (dev(c[x]) for x in ("q", "k", "v", "m"))
+    n0 = cott.cott.launch_count()
+    o, st_out = cott.fwd_stateful(q, k, v, m, 2.0 * N, state_in=dev(state) if given else None)
+    assert cott.cott.launch_count() - n0 == (2 if summed else 3)
+    r_o, r_s = oracle.fwd_segment(c["q"], c["k"], c["v"], c["m"], state, torch.full((B,), 2.0 * N))
+    gate(o, r_o, torch.bfloat16)
+    assert norm_max_err(st_out, r_s) <= 1e-2
+
+
 @pytest.mark.parametrize("B,H,N", [(3, 16, 700), (3, 8, 1000), (1, 12, 900), (2, 20, 1300), (1, 40, 1100), (5, 15, 300)])
 def test_backward_d128_groups_of_the_two_walks(B, H, N):
     """The d = 128 backward with the library's own choice of groups: the dK, dV walk cut finer than the
