@@ -618,9 +618,13 @@ static Bwd128Groups bwd128_groups(const Plan& p, int BH, int N, int causal, bool
         // Bidirectional: the plan's groups, every walk starts from the totals.  Packed batches: half as many,
         // since two CTAs take each.
         int n = p.n_groups, group = p.group;
-        if (causal && n > 1 && option_force_group() <= 0) {
-            n = n / 2;
-            group = ((N + n - 1) / n + 127) / 128 * 128;
+        int fewer = causal ? n / 2 : n;
+        // (two CTAs a group: where they exceed one wave and a group has no more than four chunks, half a wave of
+        // groups is 1 to 20 us faster -- B H = 24, N = 512 32 us against 54, B H = 64, N = 512 38 / 51, B H = 16,
+        // N = 3000 58.7 / 60.1 -- and beyond that slower: B H = 16, N = 6000 95 / 92)
+        if (!causal && !packed && 2 * BH * n > 148 && group <= 512) fewer = 74 / BH;
+        if (fewer >= 1 && fewer < n && option_force_group() <= 0) {
+            group = ((N + fewer - 1) / fewer + 127) / 128 * 128;
             n = (N + group - 1) / group;
         }
         g.group_q = g.group_k = group; g.n_q = g.n_k = n;

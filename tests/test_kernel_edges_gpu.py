@@ -132,6 +132,17 @@ def test_forward_walk_sums_states_where_that_is_faster(BH, d, groups, given, sum
     assert norm_max_err(st_out, r_s) <= 1e-2
 
 
+@pytest.mark.parametrize("B,H,N", [(2, 12, 500), (4, 16, 260), (1, 18, 1000), (1, 74, 200)])
+def test_bidirectional_backward_d128_in_one_wave(B, H, N):
+    """Where the plan's groups would give the two walks more CTAs than SMs: as many groups as fit."""
+    c = synth.make_qkv(B, H, N, 128, torch.bfloat16, 8700 + N, with_do=True)
+    q, k, v, d_o, m = (dev(c[x]) for x in ("q", "k", "v", "d_o", "m"))
+    dq, dk, dv, dm = cott.bwd(q, k, v, d_o, m, causal=False)
+    rq, rk, rv, rm = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, False)
+    gate(dq, rq, torch.bfloat16); gate(dk, rk, torch.bfloat16); gate(dv, rv, torch.bfloat16)
+    gate_dm(dm, rm, 1e-2, dm_condition(rv, c["v"], c["m"], None), DM_COND_BF16)
+
+
 @pytest.mark.parametrize("B,H,N", [(3, 16, 700), (3, 8, 1000), (1, 12, 900), (2, 20, 1300), (1, 40, 1100), (5, 15, 300)])
 def test_backward_d128_groups_of_the_two_walks(B, H, N):
     """The d = 128 backward with the library's own choice of groups: the dK, dV walk cut finer than the
