@@ -502,8 +502,10 @@ static cott_status fwd_impl(const void* q, const void* k, const void* v, void* o
         // tokens, and wherever the states would have to be padded, they stream through registers
         // (cott_block.cu); beyond, the scores of a block outweigh that and the tensor-memory form is
         // faster.  Measured, B H = 1024, d = 128: 16 tokens 31 us against 56, 32 tokens 37 against 58, 64
-        // tokens 63 against 61; B H = 768, d = 64, 64 tokens: 21.5 against 17.
-        if (N <= 32 || p.padded)
+        // tokens 63 against 61; B H = 768, d = 64, 64 tokens: 21.5 against 17.  At d = 64 a second tile of
+        // tokens costs more than it gives while there is no more than one CTA per SM (17 to 32 tokens,
+        // B H = 144: 6.9 against 5.6; 160: 7.1 against 7.3).
+        if (p.padded || N <= 16 || (N <= 32 && (d == 128 || (long)B * H > 148)))
             COTT_CUDA(launch_block_fwd(q, k, v, o, lay.qkv, lay.of(v), lay.o, state_in, state_out, static_cast<int*>(ws),
                                        sp->m, sp->seq_len, sp->seq_len_scalar, B, H, N, p.dk, p.dv, st));
         else

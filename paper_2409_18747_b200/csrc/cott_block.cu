@@ -349,7 +349,9 @@ cudaError_t launch_t(const CUtensorMap* tm, const BlockParams& p, int BH, cudaSt
     const int prof = profile_begin_launch(6, st);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)BH);
-    cfg.blockDim = dim3(32u * (unsigned)((p.dv + 31) / 32));
+    // (two warps at least: a second one without value columns shares the row passes; d_k = d_v = 32, 33 tokens,
+    // 12 (b, h): 11 us with one)
+    cfg.blockDim = dim3(32u * (unsigned)(p.dv > 64 ? (p.dv + 31) / 32 : 2));
     cfg.dynamicSmemBytes = BL<TT>::kDynBytes;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];

@@ -143,6 +143,30 @@ def test_bidirectional_backward_d128_in_one_wave(B, H, N):
     gate_dm(dm, rm, 1e-2, dm_condition(rv, c["v"], c["m"], None), DM_COND_BF16)
 
 
+@pytest.mark.parametrize("B,H,T,d", [(64, 16, 16, 128), (64, 16, 20, 128), (72, 16, 40, 120), (37, 4, 17, 64), (15, 10, 17, 64), (15, 10, 32, 64)])
+def test_token_blocks_of_many_heads(B, H, T, d):
+    """States of more than the L2 (1024 heads of 64 KB and more) take the instances that mark them for early
+    eviction, d = 64 with more than 148 (b, h) those of 32 tokens: as the same rows in calls on a quarter of
+    the batch, bit for bit where the kernel is the same, and two heads against the definition."""
+    g = torch.Generator(device="cuda").manual_seed(B + T)
+    q, k, v = ((torch.randn((B, H, T, d), generator=g, device="cuda") + 0.2).to(torch.bfloat16) for _ in range(3))
+    m, state = torch.randn(H, generator=g, device="cuda"), torch.randn((B, H, d, d), generator=g, device="cuda")
+    o, st = cott.fwd_stateful(q, k, v, m, 300.0, state_in=state)
+    for b0 in range(0, B, B // 4):
+        sl = slice(b0, b0 + B // 4)
+        o1, st1 = cott.fwd_stateful(q[sl].contiguous(), k[sl].contiguous(), v[sl].contiguous(), m, 300.0, state_in=state[sl].contiguous())
+        if d != 64:
+            assert torch.equal(o[sl], o1) and torch.equal(st[sl], st1)
+        else:
+            gate(o[sl], o1.double().cpu().numpy(), torch.bfloat16)
+            assert norm_max_err(st[sl], st1) <= 1e-2
+    for b in (0, B - 1):
+        x = [t[b:b + 1, :2].contiguous().cpu() for t in (q, k, v)]
+        r_o, r_s = oracle.fwd_segment(*x, m[:2].cpu(), state[b:b + 1, :2].cpu(), torch.tensor([300.0]))
+        gate(o[b:b + 1, :2], r_o, torch.bfloat16)
+        assert norm_max_err(st[b:b + 1, :2], r_s) <= 1e-2
+
+
 @pytest.mark.parametrize("B,H,N", [(3, 16, 700), (3, 8, 1000), (1, 12, 900), (2, 20, 1300), (1, 40, 1100), (5, 15, 300)])
 def test_backward_d128_groups_of_the_two_walks(B, H, N):
     """The d = 128 backward with the library's own choice of groups: the dK, dV walk cut finer than the
