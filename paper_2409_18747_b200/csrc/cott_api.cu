@@ -640,31 +640,40 @@ static Bwd128Groups bwd128_groups(const Plan& p, int BH, int N, int causal, bool
     // B=3, H=16, N=2999 113 us / 127, B=1, H=40, N=4096 143 / 165, B=1, H=16, N=16384 224 / 254.)
     const int chunks = (N + 127) / 128, slots = 148 / BH;
     double best = 1e30;
-    for (int n_q = 1; n_q < slots; ++n_q)
-        for (int n_k = 1; n_q + n_k <= slots; ++n_k) {
-            if (n_q > chunks || n_k > chunks || n_q > p.n_groups || n_k > p.n_groups) continue;
-            const int n_max = n_q > n_k ? n_q : n_k;
-            int parts = 1;
-            if (n_max > 1)
+    // Of the numbers of groups with walks of one length only the least is looked at (others have the same walks
+    // and more of them; below four groups, where parts depend on the number, all): 1 to 10 us on the host.
+    int n_of[148], l_of[148], n_cand = 0;
+    const int most = std::min({slots - 1, chunks, p.n_groups});
+    for (int n = 1; n <= most; ++n) {
+        const int l = (chunks + n - 1) / n;
+        if (n > 3 && l == l_of[n_cand - 1]) continue;
+        n_of[n_cand] = n; l_of[n_cand++] = l;
+    }
+    for (int iq = 0; iq < n_cand; ++iq)
+        for (int ik = 0; ik < n_cand && n_of[iq] + n_of[ik] <= slots; ++ik) {
+            const int n_q = n_of[iq], n_k = n_of[ik], n_max = n_q > n_k ? n_q : n_k;
+            int parts = 1, l_q = l_of[iq], l_k = l_of[ik];
+            if (n_max == 2 || n_max == 3) {
                 for (int s = 2; s <= 4; ++s)
                     if (s * (n_max - 1) <= 4 && BH * (n_max - 1) * s <= 148 && n_q * s <= p.n_groups * p.split &&
                         n_k * s <= 2 * p.n_groups * p.split && chunks >= 2 * n_max * s) parts = s;
-            auto len = [&](int n) { return n == 1 ? chunks : (chunks + n * parts - 1) / (n * parts) * parts; };
-            const double cost = std::max(3.5 * len(n_q), 4.6 * len(n_k)) + (n_q > 1 ? 5 + 0.9 * len(n_q) / parts : 0) +
-                                (n_k > 1 ? 5 + 0.9 * len(n_k) / parts : 0) +
+                if (n_q > 1) l_q = (chunks + n_q * parts - 1) / (n_q * parts) * parts;
+                if (n_k > 1) l_k = (chunks + n_k * parts - 1) / (n_k * parts) * parts;
+            }
+            const double cost = std::max(3.5 * l_q, 4.6 * l_k) + (n_q > 1 ? 5 + 0.9 * l_q / parts : 0) +
+                                (n_k > 1 ? 5 + 0.9 * l_k / parts : 0) +
                                 ((n_max - 1) * parts > 4 ? (4.0 + 0.15 * n_max) * ((n_q > 1) + (n_k > 1)) : 0);   // (scan launches)
             if (cost < best - 1e-9) {
                 best = cost;
                 g.parts = parts;
-                g.group_q = len(n_q) * 128; g.n_q = (chunks + len(n_q) - 1) / len(n_q);
-                g.group_k = len(n_k) * 128; g.n_k = (chunks + len(n_k) - 1) / len(n_k);
+                g.group_q = l_q * 128; g.n_q = (chunks + l_q - 1) / l_q;
+                g.group_k = l_k * 128; g.n_k = (chunks + l_k - 1) / l_k;
             }
         }
     if (best > 1e29) {      // (no room for two CTAs per (b, h) in one wave)
         g.group_q = g.group_k = chunks * 128; g.n_q = g.n_k = 1;
     }
     g.init_sum = (std::max(g.n_q, g.n_k) - 1) * g.parts <= 4;
-    if (!g.init_sum && g.parts > 1) g.init_sum = 1;
     return g;
 }
 
