@@ -44,6 +44,18 @@ def test_fp32_walk_chunk_and_group_edges(d, N, group, causal, force_group):
         assert (abs(x.double().cpu().numpy() - r) <= u * bound).all()
 
 
+def one_token_bounds(got, refs, c):
+    """Gradients of a sequence of one token (c = 1), where the relative error of a row has no bound: the rows
+    are one product of unit rows with raw rows, and dq, dk lose their part along q or k.  With u = 2^-9 (bf16
+    rounding): dV' = (q^ . k^) dO has the roundings of q^, k^, the score and the result, 4 u |dO|; dq^ and dk^
+    have two (score, unit row) of |dO| |v|, which the projection can double, and the result's."""
+    nq, nk, nv, nd = (c[x].double().norm(dim=-1, keepdim=True).numpy() for x in ("q", "k", "v", "d_o"))
+    nq, nk = nq.clip(1e-12), nk.clip(1e-12)
+    u = 2.0 ** -9
+    for x, r, bound in zip(got, refs, (6 * nd * nv / nq, 6 * nd * nv / nk, 4 * nd)):
+        assert (abs(x.double().cpu().numpy() - r) <= u * bound).all()
+
+
 @pytest.mark.parametrize("N,group", [(1, 0), (127, 0), (128, 0), (129, 0), (257, 0), (400, 128), (900, 256), (700, 128)])
 @pytest.mark.parametrize("dk,dv", [(128, 128), (72, 128), (96, 40)])
 @pytest.mark.parametrize("causal", [True, False])
@@ -57,17 +69,21 @@ def test_backward_d128_chunk_and_group_edges(N, group, dk, dv, causal, force_gro
     args = [dev(c[x]) for x in ("q", "k", "v", "d_o", "m")]
     dq, dk_, dv_, dm = cott.bwd(*args, causal=causal)
     rq, rk, rv, rm = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, causal)
-    if N > 1:      # (one token: see the note on single-term rows in test_parity_gpu's gates)
-        # the zero key row's gradient is that of the clamped formula, 1e12 times larger: gated on its own
-        z = (0, 1, N // 2)
-        assert norm_max_err(dk_[z], rk[z]) <= 1e-2
-        dk_[z] = 0.0
-        rk[z] = 0.0
-        gate(dq, rq, torch.bfloat16); gate(dk_, rk, torch.bfloat16); gate(dv_, rv, torch.bfloat16)
-        # dm's error scales with the sum of its absolute terms (see dm_condition): 3e-4 of it at worst
-        # over random shapes of this size for bf16 operands
-        cond = dm_condition(rv, c["v"], c["m"], None)
-        assert (abs(dm.double().cpu().numpy() - rm) <= 1e-3 * cond).all()
+    if N == 1:
+        one_token_bounds((dq, dk_, dv_), (rq, rk, rv), c)
+        assert (dm == 0).all() and (rm == 0).all()         # (c = 1: ln 1 = 0)
+        return
+    # the zero key row's gradient is that of the clamped formula, 1e12 times larger: gated on its own
+    z = (0, 1, N // 2)
+    assert norm_max_err(dk_[z], rk[z]) <= 1e-2
+    dk_[z] = 0.0
+    rk[z] = 0.0
+    gate(dq, rq, torch.bfloat16); gate(dk_, rk, torch.bfloat16); gate(dv_, rv, torch.bfloat16)
+    # dm's error scales with the sum of its absolute terms (see dm_condition): 3e-4 of it at worst
+    # over random shapes of this size for bf16 operands
+    cond = dm_condition(rv, c["v"], c["m"], None)
+    assert (abs(dm.double().cpu().numpy() - rm) <= 1e-3 * cond).all()
+    gate_dm(dm, rm, 1e-2, cond, DM_COND_BF16)
 
 
 @pytest.mark.parametrize("T", [1, 8, 15, 16, 17, 32, 48, 49, 64])
@@ -176,8 +192,9 @@ def test_backward_d128_groups_of_the_two_walks(B, H, N):
     dq, dk, dv, dm = cott.bwd(q, k, v, d_o, m, causal=True)
     rq, rk, rv, rm = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, True)
     gate(dq, rq, torch.bfloat16); gate(dk, rk, torch.bfloat16); gate(dv, rv, torch.bfloat16)
-    # (as in the edge test above)
-    assert (abs(dm.double().cpu().numpy() - rm) <= 1e-3 * dm_condition(rv, c["v"], c["m"], None)).all()
+    cond = dm_condition(rv, c["v"], c["m"], None)       # (as in the edge test above)
+    assert (abs(dm.double().cpu().numpy() - rm) <= 1e-3 * cond).all()
+    gate_dm(dm, rm, 1e-2, cond, DM_COND_BF16)
 
 
 @pytest.mark.parametrize("N", [1025, 1152, 2175])
@@ -195,16 +212,21 @@ def test_bidirectional_backward_in_one_launch_beyond_eight_chunks(N, packed, for
         q, k, v, d_o = (torch.cat([dev(c[x])[0].permute(1, 0, 2) for c in cs]).contiguous() for x in ("q", "k", "v", "d_o"))
         cu = torch.tensor([0, N, N + 1, N + 131], dtype=torch.int32, device="cuda")
         *grads, dm = cott.bwd_varlen(q, k, v, d_o, m, cu, N, causal=False)
-        grads = [x[:N].permute(1, 0, 2)[None] for x in grads]
     else:
         *grads, dm = cott.bwd(*(dev(cs[0][x]) for x in ("q", "k", "v", "d_o")), m, causal=False)
     assert cott.cott.launch_count() - n0 == 1
-    c = cs[0]
-    *refs, rm = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, False)
-    for x, r in zip(grads, refs):
-        gate(x.contiguous(), r, torch.bfloat16)
-    if not packed:
-        gate_dm(dm, rm, 1e-2, dm_condition(refs[2], c["v"], c["m"], None), DM_COND_BF16)
+    rm = cond = 0.0
+    for i, (n, c) in enumerate(zip(lens, cs)):
+        c["m"] = cs[0]["m"]
+        own = [x[sum(lens[:i]):sum(lens[:i + 1])].permute(1, 0, 2)[None] for x in grads] if packed else grads
+        *refs, r = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, False)
+        rm, cond = rm + r, cond + dm_condition(refs[2], c["v"], c["m"], None)
+        if n == 1:
+            one_token_bounds(own, refs, c)
+        else:
+            for x, ref in zip(own, refs):
+                gate(x.contiguous(), ref, torch.bfloat16)
+    gate_dm(dm, rm, 1e-2, cond, DM_COND_BF16)
 
 
 @pytest.mark.parametrize("d", [32, 64, 128])
