@@ -104,10 +104,13 @@ unsigned long long cott_launch_count(void);
  *   "wait_limit_kcycles" (COTT_WAIT_LIMIT_KCYCLES, -1) the same bound in units of 1024 SM cycles; negative = use the millisecond
  *                        value; 0 = every wait that is not met within a few polls gives up (the timeout test)
  * cott_set_option returns COTT_ERR_INVALID_ARG for an unknown name; cott_get_option returns -1.
+ * cott_option_changes counts the calls that set an option: a program that keeps the answers of size and
+ * plan queries, which depend on the options, asks again when it has changed.
  * No paper passage: library plumbing.
  */
 cott_status cott_set_option(const char* name, long long value);
 long long cott_get_option(const char* name);
+extern volatile unsigned cott_option_changes;
 
 /*
  * Per-launch timing of the tensor-core walk kernels, for benchmarks.  cott_profile_enable(n)

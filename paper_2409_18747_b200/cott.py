@@ -126,6 +126,7 @@ def _load():
     lib.cott_set_option.argtypes = [ctypes.c_char_p, ctypes.c_longlong]
     lib.cott_get_option.restype = ctypes.c_longlong
     lib.cott_get_option.argtypes = [ctypes.c_char_p]
+    lib.option_changes = ctypes.c_uint.in_dll(lib, "cott_option_changes")
     _lib = lib
     return lib
 
@@ -216,7 +217,6 @@ def shutdown() -> None:
 def set_option(name: str, value: int) -> None:
     """cott_set_option: a process-wide switch for tests and measurements (see ``cott.h``)."""
     rc = _load().cott_set_option(name.encode(), int(value))
-    _bytes.cache_clear()
     if rc != 0:
         raise CottError(rc, f"cott_set_option({name})")
 
@@ -226,12 +226,17 @@ def get_option(name: str) -> int:
 
 
 @functools.lru_cache(maxsize=256)
-def _bytes(op, dt, B, H, N, d_k, d_v, causal) -> int:
-    """The size query of a problem (it depends on the arguments and the options only)."""
+def _bytes_at(_changes, op, dt, B, H, N, d_k, d_v, causal) -> int:
     n = _load().cott_workspace_bytes_dkdv(op, dt, B, H, N, d_k, d_v, int(causal))
     if n == _SIZE_MAX:
         raise CottError(-2, "cott_workspace_bytes")
     return int(n)
+
+
+def _bytes(op, dt, B, H, N, d_k, d_v, causal) -> int:
+    """The size query of a problem: it depends on the arguments and the options only, so answers are kept
+    for as long as no option has been set, through this module or past it."""
+    return _bytes_at(_load().option_changes.value, op, dt, B, H, N, d_k, d_v, causal)
 
 
 def workspace_bytes(op: int, dt: int, B: int, H: int, N: int, d: int, causal: bool) -> int:

@@ -66,7 +66,7 @@ struct Option {
         });
         return value.load(std::memory_order_relaxed);
     }
-    void set(long long v) { get(); value.store(v, std::memory_order_relaxed); }
+    void set(long long v) { get(); value.store(v, std::memory_order_relaxed); __atomic_fetch_add(&cott_option_changes, 1u, __ATOMIC_RELEASE); }
 };
 static Option g_opt_force_group("force_group", "COTT_FORCE_GROUP", 0);     // tokens per sequence group (0: the plan's)
 static Option g_opt_force_path("force_path", "COTT_FORCE_PATH", 1);        // 0: bf16 d=64/128 through the fp32-accumulating SIMT kernels
@@ -1006,6 +1006,8 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
 using namespace cott;
 
 extern "C" {
+
+volatile unsigned cott_option_changes = 0;
 
 int cott_version(void) { return 100; }
 

@@ -228,3 +228,17 @@ def test_cpu_tensors_are_rejected():
         assert "CUDA" in str(e)
     else:
         raise AssertionError("CPU tensors must be rejected")
+
+
+def test_size_queries_follow_options_set_past_the_binding():
+    """The binding keeps the answers of size queries; one that an option set directly through the library
+    has made stale must not come back (the library would refuse the workspace)."""
+    lib = cott._load()
+    args = (cott.OP_FWD, cott.BF16, 1, 2, 1024, 64, True)
+    before = cott.workspace_bytes(*args)
+    try:
+        assert lib.cott_set_option(b"force_group", 256) == 0
+        assert cott.workspace_bytes(*args) == lib.cott_workspace_bytes(*args) != before
+    finally:
+        assert lib.cott_set_option(b"force_group", 0) == 0
+    assert cott.workspace_bytes(*args) == before
