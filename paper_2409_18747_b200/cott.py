@@ -187,9 +187,13 @@ def _layout(*ts):
     return None if dense else ctypes.byref(_Strides(first[0], first[1], first[2]))
 
 
+# (the raw handle of torch's current stream, where this torch has the call: a Stream object costs 3 us to build)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda dev: torch.cuda.current_stream(dev).cuda_stream)
+
+
 def _stream_ptr(stream) -> int:
-    if stream is None:      # (the raw handle of torch's current stream: a Stream object costs 3 us to build)
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if stream is None:
+        return _raw_stream(torch.cuda.current_device())
     return int(stream.cuda_stream)
 
 
