@@ -1044,6 +1044,8 @@ tc_bwd_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const int g = blockIdx.x % p.grid_groups, bh = blockIdx.x / p.grid_groups;
     const int bseq = bh / p.H, h = bh % p.H;
     const int b = VARLEN ? 0 : bseq;                   // batch coordinate of the tensor maps
+    // (a packed batch reads cu_seqlens, which the kernel before this call may have written)
+    if (VARLEN) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int tok0 = (VARLEN ? p.cu_seqlens[bseq] : 0) + g * p.group;
     const int tok1 = min(VARLEN ? p.cu_seqlens[bseq + 1] : p.N, tok0 + p.group);
     const int n_chunks = tok1 > tok0 ? (tok1 - tok0 + kC - 1) / kC : 0;
