@@ -71,7 +71,7 @@ struct Option {
 static Option g_opt_force_group("force_group", "COTT_FORCE_GROUP", 0);     // tokens per sequence group (0: the plan's)
 static Option g_opt_force_path("force_path", "COTT_FORCE_PATH", 1);        // 0: bf16 d=64/128 through the fp32-accumulating SIMT kernels
 static Option g_opt_pair("pair", "COTT_PAIR", 1);                          // 0: gradient streams one after the other
-static Option g_opt_fused_bwd("fused_bwd", "COTT_FUSED_BWD", 1);           // 0: causal d=64 backward through the three role-swapped walks
+static Option g_opt_fused_bwd("fused_bwd", "COTT_FUSED_BWD", 1);           // 0: backward through the three role-swapped walks (d = 64 and 128)
 static Option g_opt_fused_bidir("fused_bidir", "COTT_FUSED_BIDIR", 1);     // 0: bidirectional d=64 forward as state pass + read-out
 static Option g_opt_bidir_bwd("bidir_bwd", "COTT_BIDIR_BWD", 1);           // 0: bidirectional d=64 backward of one group per (b, h) as state pass + walk
 static Option g_opt_short_fwd("short_fwd", "COTT_SHORT_FWD", 1);           // 0: sequences of <= 128 tokens through the generic walk
@@ -183,7 +183,7 @@ static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv
             if (g8 <= 4096 && (N + g8 - 1) / g8 == 8) group = g8;
         }
     } else {
-        p->chunk = 32;
+        p->chunk = kSimtChunk;
         group = 1024;
         while (group > 128 && BH * ((N + group - 1) / group) < 4 * 148) group >>= 1;
         // Short sequences of few heads: groups down to one chunk, as long as they do not yet give two
@@ -510,7 +510,7 @@ static cott_status fwd_impl(const void* q, const void* k, const void* v, void* o
                                        sp->m, sp->seq_len, sp->seq_len_scalar, B, H, N, p.dk, p.dv, st));
         else
             COTT_CUDA(launch_tc_block_fwd(q, k, v, o, lay.qkv, lay.of(v), lay.o, state_in, state_out, static_cast<int*>(ws),
-                                          sp->m, sp->seq_len, sp->seq_len_scalar, B, H, N, d, p.dk, p.dv, st));
+                                          sp->m, sp->seq_len, sp->seq_len_scalar, B, H, N, d, st));
         return COTT_OK;
     }
     float* states = reinterpret_cast<float*>(static_cast<char*>(ws) + kWsHeaderBytes);
@@ -757,7 +757,7 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
                 return COTT_OK;
             }
             if (causal && !packed.cu_seqlens && p.n_groups == 1 && N <= 128) {
-                // One chunk per (b, h): no state is ever read, the walk is the only launch.
+                // One chunk per (b, h): no state is ever read, the walk needs none before it.
                 f.sq_part = nullptr; f.r_part = nullptr;
                 COTT_CUDA(launch_clear_status(status, st));      // status words and the dm counter
                 COTT_CUDA(launch_tc_bwd_fused(f, B, H, N, st));
@@ -1256,7 +1256,7 @@ static cott_status bwd_entry(const void* q, const void* k, const void* v, const 
         const bool tc_walks = p.path == 1 && p.d == 128;
         if (p.path == 1 && !tc_fused && !tc_walks) {
             if (!(d_k == d_v && (d_k == 32 || d_k == 64 || d_k == 128))) return COTT_ERR_UNSUPPORTED;
-            p.path = 0; p.chunk = 16; p.d = d_k; p.padded = false; p.split = 1;
+            p.path = 0; p.chunk = kSimtChunk; p.d = d_k; p.padded = false; p.split = 1;
         }
         if ((seg.state_in && !aligned16(seg.state_in)) || (seg.d_state_out && !aligned16(seg.d_state_out)) ||
             (seg.d_state_in && !aligned16(seg.d_state_in)))
@@ -1338,7 +1338,7 @@ static bool varlen_plan(int op, cott_dtype dt, int B, int H, int total_tokens, i
     const bool simt_ok = (dt == COTT_F32 || dt == COTT_BF16) && (d == 32 || d == 64 || d == 128);
     if (!tc_ok && !simt_ok) return false;
     p->path = (tc_ok && (option_force_path() != 0 || !simt_ok)) ? 1 : 0;
-    p->chunk = p->path == 1 ? 128 : 16;
+    p->chunk = p->path == 1 ? 128 : kSimtChunk;
     p->group = (max_seqlen + p->chunk - 1) / p->chunk * p->chunk; p->n_groups = 1; p->split = 1;
     p->dk = p->dv = d; p->d = p->path == 1 ? (d <= 64 ? 64 : 128) : d; p->padded = p->d != d;
     if (p->path == 1) {

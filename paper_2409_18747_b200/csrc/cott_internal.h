@@ -11,6 +11,8 @@ namespace cott {
 constexpr float kEps = 1e-12f;        // denominator floor of the row normalisation (Eq. 2/3)
 constexpr int kWsHeaderBytes = 256;   // workspace header: word 0 = asynchronous status
 
+constexpr int kSimtChunk = 32;        // tokens per chunk of the fp32-accumulating walk
+
 // Row treatment applied to a tile row when it is staged in shared memory.
 enum RowMode : int {
     ROW_RAW = 0,    // use as is (dO)
@@ -74,9 +76,10 @@ struct WalkBatch {
 // `dependent`: may start while the previous kernel of the stream drains (it reads nothing before
 // that one has finished).
 cudaError_t launch_walk_simt(const WalkBatch& wb, int n, int BH, int d, cott_dtype dt, cudaStream_t st, bool dependent);
+// Zeroes the status words and the dm counter of a workspace, in front of a kernel that needs them zero.
+cudaError_t launch_clear_status(int* status, cudaStream_t st);
 // `total_scale_m` non-NULL: the total written to total_out is multiplied by the stabilisation
 // factor c[b,h] (the tensor-core path keeps its states unscaled).
-cudaError_t launch_clear_status(int* status, cudaStream_t st);
 cudaError_t launch_scan(float* states, float* total_out, int BH, int n_groups, int d, int mode,
                         cudaStream_t st, const float* total_scale_m = nullptr,
                         const float* seq_len = nullptr, float seq_len_scalar = 0.f, int H = 1,
@@ -146,7 +149,6 @@ struct TcBwdFusedArgs {
     float* dm_partial; float* dm_out; int* status;
     const float* m; const float* seq_len; float seq_len_scalar;
     int group; int n_groups;
-    int plain_launch;
     // Causal walk: the partial states K^^T V the forward call of the same q, k, v left in its
     // workspace ([BH, n_groups * sq_fwd_split, 64 * 64], unscaled; every group but the last): read
     // transposed instead of sq_part, which the state pass then does not compute.  NULL: none.
@@ -216,7 +218,7 @@ cudaError_t launch_block_fwd(const void* q, const void* k, const void* v, void* 
 cudaError_t launch_tc_block_fwd(const void* q, const void* k, const void* v, void* o, const RowLayout& l_qk,
                                 const RowLayout& l_v, const RowLayout& l_o, const float* state_in, float* state_out,
                                 int* status, const float* m, const float* seq_len, float seq_len_scalar, int B, int H,
-                                int N, int d, int dk, int dv, cudaStream_t st);
+                                int N, int d, cudaStream_t st);
 
 // Opt-in to `bytes` of dynamic shared memory for a kernel, once per (kernel, device).
 cudaError_t configure_smem_once(const void* func, int bytes);

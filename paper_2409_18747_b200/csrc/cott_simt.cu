@@ -10,7 +10,7 @@ namespace cott {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kChunk = 32;  // tokens per chunk of the walk
+constexpr int kChunk = kSimtChunk;
 
 template <typename T> __device__ __forceinline__ float4 load4(const T* p);
 template <> __device__ __forceinline__ float4 load4<float>(const float* p) {

@@ -44,7 +44,6 @@ struct BlockParams {
     int* status;
     const float* m; const float* seq_len; float seq_len_scalar;
     int H; int N;            // N <= 64 tokens
-    int d_out;               // columns o really has
     int wait_limit_kcycles;
     int head_first_mask;     // bit i: in tensor map i (q, k, v, o) the head index comes before the token index
 };
@@ -160,7 +159,7 @@ tc_block_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 const bool hfo = (p.head_first_mask >> 3) & 1;
 #pragma unroll
                 for (int hh = 0; hh < NH; ++hh)
-                    if (hh * 64 < p.d_out) tma_store_4d(&tmO, base + L::kOffQ + hh * kBox, hh * 64, hfo ? h : 0, hfo ? 0 : h, b);
+                    tma_store_4d(&tmO, base + L::kOffQ + hh * kBox, hh * 64, hfo ? h : 0, hfo ? 0 : h, b);
                 tma_store_commit();
                 tma_store_wait_all0();
             }
@@ -349,21 +348,20 @@ cudaError_t launch_d(const CUtensorMap* tm, const BlockParams& p, int BH, cudaSt
 cudaError_t launch_tc_block_fwd(const void* q, const void* k, const void* v, void* o, const RowLayout& l_qk,
                                 const RowLayout& l_v, const RowLayout& l_o, const float* state_in, float* state_out,
                                 int* status, const float* m, const float* seq_len, float seq_len_scalar, int B, int H,
-                                int N, int d, int dk, int dv, cudaStream_t st) {
-    if (N < 1 || N > kT || (d != 64 && d != 128) || dk > d || dv > d) return cudaErrorInvalidValue;
+                                int N, int d, cudaStream_t st) {
+    if (N < 1 || N > kT || (d != 64 && d != 128)) return cudaErrorInvalidValue;
     BlockParams p;
     p.state_in = state_in; p.state_out = state_out; p.status = status;
     p.m = m; p.seq_len = seq_len; p.seq_len_scalar = seq_len_scalar;
-    p.H = H; p.N = N; p.d_out = dv;
+    p.H = H; p.N = N;
     p.wait_limit_kcycles = wait_limit_kcycles();
     const void* ptrs[4] = {q, k, v, o};
     const RowLayout lays[4] = {l_qk, l_qk, l_v, l_o};
-    const int widths[4] = {dk, dk, dv, dv};
     CUtensorMap tm[4];
     p.head_first_mask = 0;
     for (int i = 0; i < 4; ++i) {
         bool hf = false;
-        if (!make_tile_map(&tm[i], ptrs[i], B, H, N, widths[i], lays[i], &hf, kT)) return cudaErrorInvalidValue;
+        if (!make_tile_map(&tm[i], ptrs[i], B, H, N, d, lays[i], &hf, kT)) return cudaErrorInvalidValue;
         p.head_first_mask |= (hf ? 1 : 0) << i;
     }
     return d == 64 ? launch_d<64>(tm, p, B * H, st) : launch_d<128>(tm, p, B * H, st);

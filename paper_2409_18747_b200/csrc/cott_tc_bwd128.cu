@@ -758,7 +758,7 @@ cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, const Bwd128Groups& g, flo
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     // (a packed batch reads cu_seqlens before anything else)
-    cfg.numAttrs = (a.plain_launch || a.cu_seqlens) ? 0 : 1;
+    cfg.numAttrs = a.cu_seqlens ? 0 : 1;
     cudaError_t le = cudaLaunchKernelEx(&cfg, kern, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], p);
     profile_end_launch(prof, st);
     note_launch();

@@ -236,7 +236,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// Sum of squares of eight bf16 values, on two independent accumulators.
+// Sum of squares of eight bf16 values, even and odd columns in one accumulator each.
 __device__ __forceinline__ void sumsq8(const uint4& w, float2& a) {
     const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&w);
 #pragma unroll

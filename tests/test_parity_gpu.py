@@ -295,9 +295,12 @@ def test_forward_backward_small(dtype, d, causal, force_group):
     gate_dm(dm, rm, 1e-4 if f32 else 1e-2, dm_condition(rv, c["v"], c["m"], s), DM_COND_F32 if f32 else DM_COND_BF16)
 
 
-def test_backward_d128_several_chunks_per_group(force_group):
-    """d = 128 gradient streams with groups of several chunks and a ragged tail: the two-stage
-    ring, the projection tile in the A slot and the separate Bv barrier all cycle."""
+@pytest.mark.parametrize("fused", [1, 0])
+def test_backward_d128_several_chunks_per_group(fused, force_group, option):
+    """d = 128 gradient streams with groups of several chunks and a ragged tail: in the two walks of one
+    launch, and in the three walks that segments take, whose two-stage ring, projection tile in the A
+    slot and separate Bv barrier all cycle."""
+    option("fused_bwd", fused)
     force_group(512)
     B, H, N, d = 1, 2, 1061, 128
     c = synth.make_qkv(B, H, N, d, torch.bfloat16, 4500, with_do=True)
