@@ -137,9 +137,10 @@ struct Plan {
 // and eight; more only where a group's own rows dwarf the states.
 // d = 128 (64 KB, about 2.4 us each): a scan launch costs more the more heads there are, so one read
 // always pays (B H = 1 to 73, two groups: 2.4 to 19 us), two from about 20 heads on (B H = 8: 0.6 to 1.8 us
-// slower than a scan, 24: level, 32: 1 to 1.6 us faster), three from 40 on (B H = 48, N = 2999, a caller's
-// state, three groups: 50 us against 57 with the scan; 32 heads: up to 3 us slower), four up to 11 us
-// slower except for groups as long as the last clause asks for (B H = 16, N = 131072: 510 us against 514).
+// slower than a scan, 24: level, 32: 1 to 1.6 us faster), three from 40 on (B H = 48, three groups on a
+// caller's state: level up to N = 1536, 0.8 to 16 us faster from 2048 on; 32 heads: up to 3 us slower), four
+// up to 11 us slower except for groups as long as the first clause asks for (B H = 16, N = 131072: 510 us
+// against 514).
 static bool sum_in_walk(int n_groups, int reads, long BH, int d, int group) {
     if (n_groups <= 9 && (long long)n_groups * d * 8 <= group) return true;
     return d == 64 ? n_groups <= 7 : reads <= (BH >= 40 ? 3 : BH >= 20 ? 2 : 1);
@@ -189,7 +190,10 @@ static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv
         // Short sequences of few heads: groups down to one chunk, as long as they do not yet give two
         // CTAs per SM and the group states stay small: 2 MiB, or 8 MiB at d = 128, where a chunk is four
         // times the work (B=2, H=8, N=509: d = 64 backward 43 us with 2 MiB, 59 with 8; d = 128 forward 72
-        // with 2, 43 with 8).
+        // with 2, 43 with 8).  Over 396 calls a size (B H = 1 to 96, N = 64 to 2048), mean distance from the
+        // best of limits from 1 to 16 MiB: d = 128 2.8 % with 8 MiB (4: 7.2 %, 16: 6.6 %); d = 64
+        // 2.4 % in the backward and 10 % in the forward with 2 MiB (8: 7 % and 1 %); d = 32 2.6 % whatever
+        // the limit.
         while (group > 32 && BH * ((N + group - 1) / group) < 2 * 148 &&
                BH * ((N + group / 2 - 1) / (group / 2)) * d * d * 4 <= (d == 128 ? 8L << 20 : 2L << 20)) group >>= 1;
     }

@@ -90,7 +90,7 @@ template <int D> struct WalkSmem {
 // serial chain (0.35 us a token) on the same SMs.  32 tokens a chunk: a 64-token chunk does 1.3
 // times the multiply-adds at d = 64 and halves the number of CTAs a short sequence gives.
 // Measured, forward and backward at B=2, H=8, N=509, d=64: 303 us and 13 launches with the
-// recurrence, 68 us and 4 launches (state pass and walk each way) here.
+// recurrence, 70 us and 4 launches (state pass and walk each way) here.
 // Thread (ty, tx) owns columns 4 tx .. + 3 everywhere: rows ty, ty + TY, .. of the chunk (it loads,
 // normalises and produces them; the TX threads of a row sit in one warp, so row sums are
 // shuffles) and rows SR ty .. + SR - 1 of the state, which stays in its registers and is copied
@@ -98,7 +98,7 @@ template <int D> struct WalkSmem {
 // blockIdx.y picks one of up to three streams (the three gradients of a backward call).
 // Threads of a CTA: few, so that each has a tile of four rows (d = 64; 32: two) and shared memory feeds
 // twice as many multiply-adds per load; three or four CTAs share an SM.  (Backward at B=2, H=8, N=509, d = 64:
-// 43 us against 56 with 256 threads, B=32, H=12, N=100, d = 32: 57 against 90; 170 registers, 128 spill.)
+// 43 us against 56 with 256 threads, B=32, H=12, N=100, d = 32: 57 against 90; 168 registers, 128 spill.)
 template <int D> struct WalkThreads { static constexpr int n = D == 128 ? 256 : 128, ctas = D == 128 ? 1 : (D == 64 ? 3 : 4); };
 
 template <int D, typename T>
