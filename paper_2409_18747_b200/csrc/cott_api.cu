@@ -1,6 +1,7 @@
 // C-ABI entry points of libcott: argument validation, execution plan, workspace layout and
 // the launch sequences.  All arithmetic of the method runs in the kernels.
 #include <algorithm>
+#include <limits.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -131,6 +132,27 @@ struct Plan {
     bool padded;
 };
 
+static size_t states_bytes(const Plan& p, int B, int H, int d) {
+    return align_up((size_t)B * H * p.n_groups * p.split * d * d * sizeof(float), 256);
+}
+
+// (padded head sizes: room for a caller's initial and final state in the kernels' size)
+static size_t padded_state_bytes(const Plan& p, int B, int H) {
+    return p.padded ? align_up((size_t)B * H * p.d * p.d * sizeof(float), 256) : 0;
+}
+
+// (backward of a segment: the caller's two states and the one it gets back, in the kernels' size)
+static size_t segment_state_bytes(int B, int H, int d) { return align_up((size_t)B * H * d * d * sizeof(float), 256); }
+
+static size_t workspace_bytes_impl(int op, const Plan& p, int B, int H, int d) {
+    size_t total = kWsHeaderBytes;
+    if (op == COTT_OP_FWD) total += states_bytes(p, B, H, d) + 2 * padded_state_bytes(p, B, H);
+    else if (op == COTT_OP_BWD)
+        total += 3 * states_bytes(p, B, H, d) + 2 * align_up((size_t)B * H * p.n_groups * 4, 256) +
+                 (p.padded ? 6 : 3) * segment_state_bytes(B, H, d);
+    return total;
+}
+
 // May every walk CTA sum the partial states it needs itself (no scan launch)?  `reads`: how many states of
 // d x d floats the last CTA adds up, one after the other out of L2 (a caller's state among them).
 // d = 64 (16 KB each): the sum is 0.5 to 4 us ahead of a scan launch up to six groups and level with it at seven
@@ -149,7 +171,10 @@ static bool sum_in_walk(int n_groups, int reads, long BH, int d, int group) {
 // Sequence groups give sequence-level parallelism when B*H alone cannot fill the GPU:
 // halve the group until there are enough CTAs, but never below a floor that keeps the
 // per-group state traffic (d*d fp32) small against the group's own q,k,v,o bytes.
-static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv, int causal, Plan* p) {
+// `room`: the workspace there is, for a caller that cannot bring a larger one.  The finer partitions that only
+// make a call faster (short groups in fp32, a split state pass) are left out where they do not fit.
+static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv, int causal, Plan* p,
+                      size_t room = (size_t)-1) {
     if (B < 1 || H < 1 || N < 1) return false;
     if (dt != COTT_F32 && dt != COTT_BF16) return false;
     const long BH = (long)B * H;
@@ -194,7 +219,8 @@ static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv
         // best of limits from 1 to 16 MiB: d = 128 2.8 % with 8 MiB (4: 7.2 %, 16: 6.6 %); d = 64
         // 2.4 % in the backward and 10 % in the forward with 2 MiB (8: 7 % and 1 %); d = 32 2.6 % whatever
         // the limit.
-        while (group > 32 && BH * ((N + group - 1) / group) < 2 * 148 &&
+        const long room_states = room == (size_t)-1 ? LONG_MAX : (long)((room - kWsHeaderBytes) / ((size_t)d * d * 4));
+        while (group > 32 && BH * ((N + group - 1) / group) < 2 * 148 && BH * ((N + group / 2 - 1) / (group / 2)) <= room_states &&
                BH * ((N + group / 2 - 1) / (group / 2)) * d * d * 4 <= (d == 128 ? 8L << 20 : 2L << 20)) group >>= 1;
     }
     if (forced > 0) group = (forced + p->chunk - 1) / p->chunk * p->chunk;
@@ -212,29 +238,9 @@ static bool make_plan(int op, cott_dtype dt, int B, int H, int N, int dk, int dv
         const int chunks = group / p->chunk;
         for (int s2 = 4; s2 >= 2; s2 >>= 1)
             if (ctas * s2 <= 148 && chunks % s2 == 0 && chunks / s2 >= 4) { p->split = s2; break; }
+        if (workspace_bytes_impl(op, *p, B, H, d) > room) p->split = 1;
     }
     return true;
-}
-
-static size_t states_bytes(const Plan& p, int B, int H, int d) {
-    return align_up((size_t)B * H * p.n_groups * p.split * d * d * sizeof(float), 256);
-}
-
-// (padded head sizes: room for a caller's initial and final state in the kernels' size)
-static size_t padded_state_bytes(const Plan& p, int B, int H) {
-    return p.padded ? align_up((size_t)B * H * p.d * p.d * sizeof(float), 256) : 0;
-}
-
-// (backward of a segment: the caller's two states and the one it gets back, in the kernels' size)
-static size_t segment_state_bytes(int B, int H, int d) { return align_up((size_t)B * H * d * d * sizeof(float), 256); }
-
-static size_t workspace_bytes_impl(int op, const Plan& p, int B, int H, int d) {
-    size_t total = kWsHeaderBytes;
-    if (op == COTT_OP_FWD) total += states_bytes(p, B, H, d) + 2 * padded_state_bytes(p, B, H);
-    else if (op == COTT_OP_BWD)
-        total += 3 * states_bytes(p, B, H, d) + 2 * align_up((size_t)B * H * p.n_groups * 4, 256) +
-                 (p.padded ? 6 : 3) * segment_state_bytes(B, H, d);
-    return total;
 }
 
 static cott_status check_scale(const cott_scale_params* sp) {
@@ -1130,7 +1136,7 @@ static cott_status fwd_entry(const void* q, const void* k, const void* v, void* 
                              float* state_out, int B, int H, int N, int d_k, int d_v, int causal, bool stateful,
                              cott_dtype dt, const cott_strides* qk_strides, const cott_strides* v_strides,
                              const cott_strides* o_strides, const cott_scale_params* sp, void* workspace,
-                             size_t workspace_bytes, void* stream) {
+                             size_t workspace_bytes, void* stream, size_t room = (size_t)-1) {
     if (!q || !k || !v || !o || B < 1 || H < 1 || N < 1 || d_k < 1 || d_v < 1) return COTT_ERR_INVALID_ARG;
     const cott_strides* vs = v_strides ? v_strides : (d_k == d_v ? qk_strides : nullptr);
     if (!layout_ok(qk_strides, d_k, dt) || !layout_ok(vs, d_v, dt) || !layout_ok(o_strides, d_v, dt))
@@ -1150,7 +1156,7 @@ static cott_status fwd_entry(const void* q, const void* k, const void* v, void* 
         if (!sp->seq_len && sp->seq_len_scalar > 0.f && sp->seq_len_scalar < 1.f) return COTT_ERR_INVALID_ARG;
     }
     Plan p;
-    if (!make_plan(COTT_OP_FWD, dt, B, H, N, d_k, d_v, causal, &p)) return COTT_ERR_UNSUPPORTED;
+    if (!make_plan(COTT_OP_FWD, dt, B, H, N, d_k, d_v, causal, &p, room)) return COTT_ERR_UNSUPPORTED;
     if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o) ||
         (state_in && !aligned16(state_in)) || (state_out && !aligned16(state_out)))
         return COTT_ERR_UNSUPPORTED;
@@ -1161,6 +1167,22 @@ static cott_status fwd_entry(const void* q, const void* k, const void* v, void* 
                     static_cast<cudaStream_t>(stream), state_in, qk_strides, o_strides, Packed(),
                     (d_k != d_v || v_strides) ? vs : nullptr);
 }
+
+}  // extern "C"
+
+namespace cott {
+cott_status fwd_in_room(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d, int causal,
+                        cott_dtype dt, const cott_scale_params* sp, void* workspace, size_t room, void* stream) {
+    Plan p;
+    if (!make_plan(COTT_OP_FWD, dt, B, H, N, d, d, causal, &p, room)) return COTT_ERR_UNSUPPORTED;
+    if (workspace_bytes_impl(COTT_OP_FWD, p, B, H, p.d) > room) return COTT_ERR_WORKSPACE;
+    if (!workspace) return COTT_OK;
+    return fwd_entry(q, k, v, o, nullptr, nullptr, B, H, N, d, d, causal, false, dt, nullptr, nullptr, nullptr, sp, workspace, room,
+                     stream, room);
+}
+}  // namespace cott
+
+extern "C" {
 
 cott_status cott_fwd(const void* q, const void* k, const void* v, void* o, float* state_out,
                      int B, int H, int N, int d, int causal, cott_dtype dt,

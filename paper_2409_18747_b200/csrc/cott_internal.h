@@ -220,6 +220,11 @@ cudaError_t launch_tc_block_fwd(const void* q, const void* k, const void* v, voi
                                 int* status, const float* m, const float* seq_len, float seq_len_scalar, int B, int H,
                                 int N, int d, cudaStream_t st);
 
+// A dense forward without a state on a workspace of `room` bytes, by a plan that fits it where there is one;
+// workspace NULL: only the check (COTT_OK, COTT_ERR_UNSUPPORTED or COTT_ERR_WORKSPACE).
+cott_status fwd_in_room(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d, int causal,
+                        cott_dtype dt, const cott_scale_params* sp, void* workspace, size_t room, void* stream);
+
 // Opt-in to `bytes` of dynamic shared memory for a kernel, once per (kernel, device).
 cudaError_t configure_smem_once(const void* func, int bytes);
 

@@ -47,15 +47,14 @@ size_t cott_fwd_noalloc_max_bytes(void) { return kScratchBytes; }
 cott_status cott_fwd_noalloc(const void* q, const void* k, const void* v, void* o, int B, int H,
                              int N, int d, int causal, cott_dtype dt, const cott_scale_params* sp,
                              void* stream) {
-    const size_t need = cott_workspace_bytes(COTT_OP_FWD, dt, B, H, N, d, causal);
-    if (need == (size_t)-1) return COTT_ERR_UNSUPPORTED;
-    if (need > kScratchBytes) return COTT_ERR_WORKSPACE;   // problem too large for the built-in scratch
     void* ws = nullptr;
+    // (a problem too large for the built-in scratch is refused before anything else is looked at)
+    if (cott_status rc = cott::fwd_in_room(q, k, v, o, B, H, N, d, causal, dt, sp, ws, kScratchBytes, stream); rc != COTT_OK) return rc;
     if (scratch_address(&ws) != cudaSuccess) return COTT_ERR_CUDA;
-    // Same kernels as cott_fwd; the status word is cleared on the stream at the start of the
+    // Same kernels as cott_fwd (with coarser groups where those of cott_fwd do not fit); the status word is cleared on the stream at the start of the
     // call and every partial state is written before it is read, so what an earlier call left
     // in the array does not matter.
-    return cott_fwd(q, k, v, o, nullptr, B, H, N, d, causal, dt, sp, ws, kScratchBytes, stream);
+    return cott::fwd_in_room(q, k, v, o, B, H, N, d, causal, dt, sp, ws, kScratchBytes, stream);
 }
 
 cott_status cott_fwd_noalloc_status(void* stream) {

@@ -242,3 +242,17 @@ def test_size_queries_follow_options_set_past_the_binding():
     finally:
         assert lib.cott_set_option(b"force_group", 0) == 0
     assert cott.workspace_bytes(*args) == before
+
+
+def test_noalloc_is_not_refused_for_the_finer_groups_of_a_plan():
+    """d = 128 problems whose group states fit the built-in scratch, but not in the finer partition that the
+    plan of cott_fwd picks for speed: not a workspace error (what comes next needs a GPU)."""
+    lib = cott._load()
+    sp = cott._ScaleParams()
+    sp.m, sp.seq_len, sp.seq_len_scalar = 256, None, 0.0
+    a, far = 1 << 20, 1 << 40
+    for dt, BH, N in ((cott.F32, 4, 1024), (cott.F32, 16, 509), (cott.BF16, 50, 2048)):
+        assert cott.workspace_bytes(cott.OP_FWD, dt, 1, BH, N, 128, True) > lib.cott_fwd_noalloc_max_bytes()
+        if not os.path.exists("/dev/nvidia0"):
+            assert lib.cott_fwd_noalloc(a, a, a, far, 1, BH, N, 128, 1, dt, ctypes.byref(sp), None) != -3
+    assert lib.cott_fwd_noalloc(a, a, a, far, 64, 16, 8192, 128, 1, cott.BF16, ctypes.byref(sp), None) == -3

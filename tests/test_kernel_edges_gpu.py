@@ -330,3 +330,20 @@ def test_normalised_rows_are_rounded_once(path):
     got = (2.0 * got.float().cpu()).to(torch.bfloat16)
     cols = slice(0, d - 1) if path == "backward128" else slice(None)
     assert (got != want)[..., cols].double().mean().item() <= 3e-4
+
+
+@pytest.mark.parametrize("dtype,BH,N", [(torch.float32, 4, 1024), (torch.float32, 16, 509), (torch.bfloat16, 50, 2048)])
+@pytest.mark.parametrize("causal", [True, False])
+def test_noalloc_takes_coarser_groups_where_the_finer_ones_do_not_fit(dtype, BH, N, causal):
+    """cott_fwd's own plan for these d = 128 problems needs a little more or much more than the 8 MiB of the
+    built-in scratch, a coarser one fits: the call is taken, and its rows are those of cott_fwd to rounding."""
+    g = torch.Generator(device="cuda").manual_seed(N)
+    q, k, v = (torch.randn((1, BH, N, 128), generator=g, device="cuda").to(dtype) for _ in range(3))
+    m = torch.randn(BH, generator=g, device="cuda")
+    lib = cott.cott
+    dt = lib.F32 if dtype == torch.float32 else lib.BF16
+    if causal or dt == lib.F32:
+        assert cott.workspace_bytes(lib.OP_FWD, dt, 1, BH, N, 128, causal) > 8 << 20
+    got, want = cott.fwd_noalloc(q, k, v, m, causal=causal), cott.fwd(q, k, v, m, causal=causal)
+    gate(got, want.double().cpu().numpy(), dtype)
+    assert lib.fwd_noalloc_status() == 0
