@@ -347,3 +347,35 @@ def test_noalloc_takes_coarser_groups_where_the_finer_ones_do_not_fit(dtype, BH,
     got, want = cott.fwd_noalloc(q, k, v, m, causal=causal), cott.fwd(q, k, v, m, causal=causal)
     gate(got, want.double().cpu().numpy(), dtype)
     assert lib.fwd_noalloc_status() == 0
+
+
+@pytest.mark.parametrize("kind", ["head first", "token first", "wide rows", "every other token"])
+@pytest.mark.parametrize("call", ["block", "backward128", "segment128", "fp32"])
+def test_memory_orders_match_dense(call, kind):
+    """Tensors stored [H,B,N,d] or [N,B,H,d], as columns of wider rows or as every other token of a longer tensor:
+    the kernels that calls of these shapes take give the bits they give on dense tensors."""
+    B, H, N, d, dtype = {"block": (2, 3, 16, 128, torch.bfloat16), "backward128": (2, 3, 300, 128, torch.bfloat16),
+                         "segment128": (2, 3, 300, 128, torch.bfloat16), "fp32": (2, 3, 150, 64, torch.float32)}[call]
+
+    def stored(x):
+        if kind == "head first":
+            return x.permute(1, 0, 2, 3).contiguous().permute(1, 0, 2, 3)
+        if kind == "token first":
+            return x.permute(2, 0, 1, 3).contiguous().permute(1, 2, 0, 3)
+        if kind == "wide rows":
+            y = torch.full((B, H, N, d + 24), 7.0, dtype=dtype, device="cuda")
+            y[..., 8:8 + d] = x
+            return y[..., 8:8 + d]
+        y = torch.full((B, H, 2 * N + 1, d), 7.0, dtype=dtype, device="cuda")
+        y[:, :, 1::2] = x
+        return y[:, :, 1::2]
+
+    g = torch.Generator(device="cuda").manual_seed(17)
+    q, k, v, d_o = (torch.randn((B, H, N, d), generator=g, device="cuda").to(dtype) for _ in range(4))
+    m = torch.randn(H, generator=g, device="cuda")
+    st, ds = (torch.randn((B, H, d, d), generator=g, device="cuda") for _ in range(2))
+    run = {"block": lambda *x: cott.fwd_stateful(*x[:3], m, 99.0, state_in=st),
+           "backward128": lambda *x: cott.bwd(*x, m, causal=True), "fp32": lambda *x: (cott.fwd(*x[:3], m), *cott.bwd(*x, m)),
+           "segment128": lambda *x: cott.bwd_stateful(*x, m, 999.0, state_in=st, d_state_out=ds)}[call]
+    for got, want in zip(run(*(stored(x) for x in (q, k, v, d_o))), run(q, k, v, d_o)):
+        assert torch.equal(got, want)
