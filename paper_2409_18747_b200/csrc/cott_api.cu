@@ -155,17 +155,19 @@ static size_t workspace_bytes_impl(int op, const Plan& p, int B, int H, int d) {
 
 // May every walk CTA sum the partial states it needs itself (no scan launch)?  `reads`: how many states of
 // d x d floats the last CTA adds up, one after the other out of L2 (a caller's state among them).
-// d = 64 (16 KB each): the sum is 0.5 to 4 us ahead of a scan launch up to six groups and level with it at seven
-// and eight; more only where a group's own rows dwarf the states.
+// A launch less is also 2.5 us less on the host, which is what a small call waits for.
+// d = 64 (16 KB each): the sum is 0.5 to 4 us ahead of a scan launch up to six groups, level at seven and at
+// most 1 us behind with eight and nine (B=1, H=8, N=952 on a caller's state, through the binding: 21.7 us
+// against 24.6 with the scan).
 // d = 128 (64 KB, about 2.4 us each): a scan launch costs more the more heads there are, so one read
-// always pays (B H = 1 to 73, two groups: 2.4 to 19 us), two from about 20 heads on (B H = 8: 0.6 to 1.8 us
-// slower than a scan, 24: level, 32: 1 to 1.6 us faster), three from 40 on (B H = 48, three groups on a
-// caller's state: level up to N = 1536, 0.8 to 16 us faster from 2048 on; 32 heads: up to 3 us slower), four
+// always pays (B H = 1 to 73, two groups: 2.4 to 19 us), two from about 16 heads on (B H = 8: 0.6 to 1.8 us
+// slower than a scan, 16: 0 to 0.9, 24: level, 32: 1 to 1.6 us faster), three from 40 on (B H = 48, three groups on
+// a caller's state: level up to N = 1536, 0.8 to 16 us faster from 2048 on; 32 heads: up to 3 us slower), four
 // up to 11 us slower except for groups as long as the first clause asks for (B H = 16, N = 131072: 510 us
 // against 514).
 static bool sum_in_walk(int n_groups, int reads, long BH, int d, int group) {
     if (n_groups <= 9 && (long long)n_groups * d * 8 <= group) return true;
-    return d == 64 ? n_groups <= 7 : reads <= (BH >= 40 ? 3 : BH >= 20 ? 2 : 1);
+    return d == 64 ? n_groups <= 9 : reads <= (BH >= 40 ? 3 : BH >= 16 ? 2 : 1);
 }
 
 // Sequence groups give sequence-level parallelism when B*H alone cannot fill the GPU:

@@ -129,8 +129,8 @@ def test_forward_walk_sums_or_scans_the_group_states(d, groups, force_group):
 
 
 @pytest.mark.parametrize("BH,d,groups,given,summed", [
-    (3, 64, 6, True, True), (3, 64, 8, True, False), (3, 128, 2, False, True), (3, 128, 2, True, False),
-    (3, 128, 3, False, False), (20, 128, 3, False, True), (20, 128, 3, True, False), (40, 128, 3, True, True),
+    (3, 64, 9, True, True), (3, 64, 10, True, False), (3, 128, 2, False, True), (3, 128, 2, True, False),
+    (3, 128, 3, False, False), (16, 128, 3, False, True), (16, 128, 2, True, True), (16, 128, 3, True, False), (40, 128, 3, True, True),
     (40, 128, 4, True, False)])
 def test_forward_walk_sums_states_where_that_is_faster(BH, d, groups, given, summed, force_group):
     """The rule that picks between the sum inside the walk (two launches) and a scan launch (three): by the
