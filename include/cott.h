@@ -429,8 +429,9 @@ cott_status cott_fwd_bwd_host(const void* q_host, const void* k_host, const void
  * that loads the library gives up that much memory until the process exits.  The call itself
  * allocates and frees nothing.
  *   - Arguments as for cott_fwd (no state export); inputs and outputs are still the caller's.
- *   - Returns COTT_ERR_WORKSPACE when cott_workspace_bytes(COTT_OP_FWD, ...) for this problem
- *     exceeds the 8 MiB; use cott_fwd with your own workspace then.
+ *   - Returns COTT_ERR_WORKSPACE when the group states of this problem do not fit the 8 MiB; use
+ *     cott_fwd with your own workspace then.  (Where cott_workspace_bytes(COTT_OP_FWD, ...) exceeds
+ *     them only for partitions that make cott_fwd faster, the call runs without those.)
  *   - The first call on each device looks up the array's device address (a host-side set-up
  *     step); make that first call before starting any stream capture.
  *   - All calls on a device share the one array: two calls whose kernels may overlap on the
