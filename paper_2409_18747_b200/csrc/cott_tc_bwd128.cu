@@ -11,15 +11,14 @@
 // tiles in flight at this head size, so dQ, whose sum runs the other way, has CTAs of its own.  With
 // an all-ones mask (BIDIR) both sums are totals and only the products with them remain.
 //
-// What bounds it: shared memory and the chain of one chunk.  A 128 x 128 x 16 product reads 8 KB of
-// operands in the 64 cycles it takes at full rate, all the bandwidth shared memory has, so the K
-// walk's seven products, its tiles coming in and going out and the worker warps' passes over them are
-// about 6600 cycles of shared-memory time a chunk (Q walk: 4900); 8800 pass, the rest being waits
-// along the chain (tiles without a second slot land, scores, mask, products, slots free again).  The
-// two CTAs of a (b, h, group) start side by side, so one of them finds most tiles in L2.
-// Measured against the three role-swapped walks with their state passes and scans: B=4, H=16,
-// N=2048 93 us (207), B=3, H=16, N=2999 113 us (210), 32 packed sequences of 512 to 2048 tokens,
-// H=16, 390 us (622), bidirectional B=8, H=16, N=1024 107 us (124).
+// What bounds it: the chain of one chunk (scores, mask, products, epilogue, state copy) on one SM, not
+// memory: two (b, h) on an idle GPU take as long a chunk as 64.  A K chunk takes 8400 cycles and a Q chunk
+// 5400; the products alone would keep the tensor core busy for 3600 and 2100, and shared memory (operands
+// of the products, tiles in and out, the workers' passes) for 6600 and 4900.
+// Measured, L2 cold: B=4, H=16, N=2048 99 us; B=3, H=16, N=2999 112 us; 32 packed sequences of 512 to
+// 2048 tokens, H=16, 378 us; B=10, H=12, N=5349, d=96 411 us.  With one slot for P in the Q walk and three
+// pairs of slots that took turns in the K walk, where every chunk waited for rows on their way out, and
+// with eight warps for the masks: 103, 126, 400 and 441 us.
 #include "cott_internal.h"
 #include "cott_sm100.cuh"
 #include "cott_tc_common.cuh"
@@ -35,17 +34,19 @@ constexpr int kC = 128;
 constexpr int kD = 128;
 constexpr int kTile = kC * kD * 2;      // one 128 x 128 bf16 tile: two 64-column halves 16 KB apart
 constexpr int kHalf = kTile / 2;
-constexpr int kWorkerWarps = 16;
-constexpr int kGroup = kWorkerWarps / 2 * 32;       // threads of a worker group
+constexpr int kWarpsA = 16, kWarpsB = 8, kWorkerWarps = kWarpsA + kWarpsB;
+constexpr int kGroupA = kWarpsA * 32, kGroupB = kWarpsB * 32;       // threads of the worker groups
 constexpr int kThreads = (kWorkerWarps + 4) * 32;   // + score, product, state-update and copy threads
 
 // Six tile slots, the bf16 copy of the state and the control block are all of the 227 KB.
 // A walk has four tiles a chunk: X and A (scores X A^T), Bv (normalised in place) and the raw rows P
-// that the projection needs.  Q walk: X = dO, A = V, Bv = K, P = Q; X and A have two slots, so the
-// scores of the next chunk do not wait for this one; dq is staged over P.  K walk: X = V, A = dO,
-// Bv = Q, P = K, in three pairs of slots that take turns: (A, Bv) of chunk c + 1 wait in one, landed
-// and normalised, while chunk c has the other two; (X, P) of chunk c + 1 go where (A, Bv) of chunk c
-// were as soon as its products are done; dv and dk are staged over (X, P).
+// that the projection needs.  Q walk: X = dO, A = V, Bv = K, P = Q.  K walk: X = V, A = dO, Bv = Q, P = K.
+// A slot is asked for again when the last product or epilogue that reads it is done, and a slot that the
+// chunk needs to its end, or that output rows are staged in, has a second one, so that no chunk waits for
+// rows on their way out.  X is done first (scores and X State): one slot.  P is read by the epilogue, which
+// stages its rows (dq, dk) over it: two.  Q walk: A is done with the state update, which goes ahead of the
+// scores because Bv has two slots: one.  K walk: A is read by the chunk's last product, and dv is staged
+// over it: two; Bv by its first: one.  (With an all-ones mask there is no A and no Bv; X has two, dv over X.)
 struct L {
     static constexpr int kOffSb = 6 * kTile;
     static constexpr int kOffCtl = kOffSb + kTile;
@@ -77,7 +78,7 @@ struct Bwd128Params {
 __device__ long long g_b128_stamps[2 * 6 * 16 * 8];
 #define STAMP(role, c, slot)                                                                                 \
     do {                                                                                                     \
-        if (blockIdx.x < 2 && (c) < 16 && ((role) > 1 || threadIdx.x == (role) * 256))                       \
+        if (blockIdx.x < 2 && (c) < 16 && ((role) > 1 || threadIdx.x == ((role) ? kGroupA : 96)))                       \
             g_b128_stamps[((blockIdx.x * 6 + (role)) * 16 + (c)) * 8 + (slot)] = clock64();                  \
     } while (0)
 #else
@@ -117,12 +118,13 @@ __device__ __forceinline__ void issue_update(uint32_t tS, uint32_t a, uint32_t b
     for (int kk = 0; kk < 8; ++kk) mma_ss_w(tS, al + kk * 128u, kDescHi, bl + kk * 128u, kDescHi, idesc, (acc_first || kk > 0) ? 1u : 0u);
 }
 
-// Thread roles.  Warps 0-15 are row workers (warp w owns tensor-memory lanes / tile rows
-// 32 (w % 4) .. + 31 and one half of the columns) in two groups of eight:
-//   group A: masks of the scores, row norms of Bv, bf16 copy of the state;
-//   group B: epilogues.
-// Lane 0 of warp 16 issues the scores, of warp 17 the output products, of warp 18 the state update,
-// of warp 19 every TMA load and store.  The roles meet only through mbarriers, every wait bounded.
+// Thread roles.  Warps 0-23 are row workers (warp w owns tensor-memory lanes / tile rows
+// 32 (w % 4) .. + 31 and a part of the columns):
+//   group A (16 warps, a quarter of the columns each): masks of the scores, row norms of Bv, bf16 copy
+//           of the state -- one after the other the longest chain of a chunk, hence the larger group;
+//   group B (8 warps, half of the columns each): epilogues.
+// Lane 0 of warp 24 issues the scores, of warp 25 the output products, of warp 26 the state update,
+// of warp 27 every TMA load and store.  The roles meet only through mbarriers, every wait bounded.
 // Every barrier is a pair indexed by chunk parity; no role can be two chunks behind another: each
 // chunk's tiles are requested only after the products (and, where a tile is staged over, the stores)
 // of the chunk that held the slot before.
@@ -149,7 +151,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
            B_S1 = 80, B_S2 = 112 /* scores done */, B_M1 = 96, B_M2 = 128 /* masked scores in tensor memory */,
            B_U = 144 /* state updated */, B_CP = 160 /* bf16 state copy written */, B_O1 = 176, B_O2 = 192 /* accumulators complete */,
            B_D1 = 208, B_D2 = 224 /* accumulators drained */, B_E1 = 240, B_E2 = 256 /* output rows staged */,
-           B_XCH = 272, B_SIB = 288 /* [4 quadrants][2] */, B_SIB2 = 352 };
+           B_XCH = 272, B_RD = 288 /* [4 quadrants][2] first scores read */, B_XF = 352 /* X State done */ };
     auto bar = [&](int which, int c) { return bars + which + 8 * (c & 1); };
     auto par = [&](int c) { return (uint32_t)((c >> 1) & 1); };
     const uint32_t tmem_slot = bars + kCtlTmemSlot;
@@ -188,9 +190,10 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
             const int o = 8 * i;
-            for (int w : {(int)B_FX, (int)B_FA, (int)B_FB, (int)B_FP, (int)B_S1, (int)B_S2, (int)B_U, (int)B_O1, (int)B_O2}) mbar_init(bars + w + o, 1);
-            for (int w : {(int)B_NB, (int)B_M1, (int)B_M2, (int)B_CP, (int)B_D1, (int)B_D2, (int)B_E1, (int)B_E2, (int)B_XCH}) mbar_init(bars + w + o, kGroup);
-            for (int qq = 0; qq < 4; ++qq) { mbar_init(bars + B_SIB + 16 * qq + o, 32); mbar_init(bars + B_SIB2 + 16 * qq + o, 32); }
+            for (int w : {(int)B_FX, (int)B_FA, (int)B_FB, (int)B_FP, (int)B_S1, (int)B_S2, (int)B_U, (int)B_O1, (int)B_O2, (int)B_XF}) mbar_init(bars + w + o, 1);
+            for (int w : {(int)B_NB, (int)B_M1, (int)B_M2, (int)B_CP}) mbar_init(bars + w + o, kGroupA);
+            for (int w : {(int)B_D1, (int)B_D2, (int)B_E1, (int)B_E2, (int)B_XCH}) mbar_init(bars + w + o, kGroupB);
+            for (int qq = 0; qq < 4; ++qq) mbar_init(bars + B_RD + 16 * qq + o, kGroupA / 4);
         }
         *abort_flag = 0;
         abort_flag[3] = p.wait_limit_kcycles;
@@ -208,14 +211,12 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
     tc_fence_after();
     const uint32_t tmem = *tmem_slot_g;
 
-    // Slots of the four tiles of chunk c (see L).  K walk: (A, Bv) in pair 2 c mod 3, (X, P) in pair
-    // 2 c + 1 mod 3 = the pair of (A, Bv) of chunk c - 1 (bidirectional: no A, Bv; pairs by parity).
-    auto pair_xp = [&](int c) { return BIDIR ? (c & 1) : (2 * c + 1) % 3; };
-    auto pair_ab = [&](int c) { return (2 * c) % 3; };
-    auto off_x = [&](int c) { return kw ? pair_xp(c) * 2 * kTile : (c & 1) * kTile; };
-    auto off_a = [&](int c) { return kw ? pair_ab(c) * 2 * kTile : (2 + (c & 1)) * kTile; };
-    auto off_b = [&](int c) { return kw ? pair_ab(c) * 2 * kTile + kTile : 4 * kTile; };
-    auto off_p = [&](int c) { return kw ? pair_xp(c) * 2 * kTile + kTile : 5 * kTile; };
+    // Slots of the four tiles of chunk c (see L).
+    auto off_x = [&](int c) { return BIDIR ? (c & 1) * kTile : 0; };
+    auto off_a = [&](int c) { return kw ? (1 + (c & 1)) * kTile : kTile; };
+    auto off_b = [&](int c) { return kw ? 3 * kTile : (2 + (c & 1)) * kTile; };
+    auto off_p = [&](int c) { return (4 + (c & 1)) * kTile; };
+    auto off_dv = [&](int c) { return BIDIR ? off_x(c) : off_a(c); };
     auto load = [&](int off, const CUtensorMap* tm, int which, uint32_t fb, int row) {
         const bool hf = (p.head_first_mask >> which) & 1;
         mbar_expect_tx(fb, kTile);
@@ -233,9 +234,8 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
         load_x(0);
         load_p(0);
         if (n_chunks > 1) {
-            if (!kw) { load_x(1); if (!BIDIR) load_a(1); }
-            else if (BIDIR) { load_x(1); load_p(1); }
-            else { load_b(1); load_a(1); }
+            if (BIDIR) load_x(1); else if (kw) load_a(1); else load_b(1);
+            load_p(1);
         }
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -259,7 +259,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
             *reinterpret_cast<uint4*>(gbase + L::kOffSb + (col >> 6) * kHalf + swz(row, (col & 63) >> 3)) = pack8(&r[i]);
         }
     };
-    if (init_state && warp < kWorkerWarps) {
+    if (init_state && warp < kWarpsA) {
         // The state before the group's first chunk: row `row`, columns 32 (warp / 4) .. + 31.
         const int cq = warp >> 2;
         const int entries = n_groups * p.parts;
@@ -297,47 +297,48 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
                 for (int hh = 0; hh < 2; ++hh)
                     if (hh * 64 < p.out_w[which - 4]) tma_store_4d(tm, base + off + hh * kHalf, hh * 64, hf ? h : r0, hf ? r0 : h, b);
             };
+            auto done = [&](int which, int c) { return wait_or_abort(bar(which, c), par(c), abort_flag); };
             for (int c = 0; c < n_chunks; ++c) {
                 const bool by_rows = is_ragged(c);      // the workers stored this chunk's rows themselves
-                if (c + 1 < n_chunks) {
-                    if (!wait_or_abort(bar(B_O1, c), par(c), abort_flag)) break;
-                    if (kw && !wait_or_abort(bar(B_O2, c), par(c), abort_flag)) break;
+                // What chunk c + 1 lacks, in the order in which the slots come free.
+                if (!BIDIR && c + 1 < n_chunks) {
+                    if (!done(B_S1, c) || !done(B_XF, c)) break;
                     STAMP(5, c, 0);
-                    if (!BIDIR && !wait_or_abort(bar(B_U, c), par(c), abort_flag)) break;
+                    load_x(c + 1);
                     if (!kw) {
-                        if (!BIDIR) load_b(c + 1);
-                        if (c + 2 < n_chunks) {
-                            load_x(c + 2);
-                            if (!BIDIR) load_a(c + 2);
-                        }
-                    } else if (!BIDIR) {
-                        load_x(c + 1);
-                        load_p(c + 1);
+                        if (!done(B_U, c)) break;
+                        load_a(c + 1);
                     }
                     STAMP(5, c, 1);
                 }
-                if (!wait_or_abort(bar(B_E1, c), par(c), abort_flag)) break;
-                STAMP(5, c, 2);
-                if (!by_rows) store(kw ? &tmDK : &tmDQ, kw ? 5 : 4, off_p(c), chunk_row(c));
-                tma_store_commit();
-                if (kw) {
-                    if (!wait_or_abort(bar(B_E2, c), par(c), abort_flag)) break;
-                    STAMP(5, c, 3);
-                    if (!by_rows) store(&tmDV, 6, off_x(c), chunk_row(c));
-                    tma_store_commit();
-                    if (c + 2 < n_chunks) {
-                        // (the P slot, whose store is the older one, takes Bv or P; the X slot A or X)
+                // The rows staged a chunk ago have left their slots.
+                if (c >= 1 && c + 1 < n_chunks) {
+                    if (kw) {
                         tma_store_wait_read1();
-                        if (BIDIR) load_p(c + 2); else load_b(c + 2);
-                        tma_store_wait_read0();
-                        if (BIDIR) load_x(c + 2); else load_a(c + 2);
-                        STAMP(5, c, 4);
+                        if (BIDIR) load_x(c + 1); else load_a(c + 1);
                     }
-                } else if (c + 1 < n_chunks) {
                     tma_store_wait_read0();
                     load_p(c + 1);
-                    STAMP(5, c, 4);
                 }
+                STAMP(5, c, 2);
+                if (!BIDIR && c + 1 < n_chunks) {
+                    if (kw && (!done(B_U, c) || !done(B_S2, c))) break;
+                    if (!done(B_O1, c)) break;
+                    if (kw) load_b(c + 1); else if (c + 2 < n_chunks) load_b(c + 2);
+                } else if (BIDIR && !kw && c + 2 < n_chunks) {
+                    if (!done(B_O1, c)) break;
+                    load_x(c + 2);
+                }
+                STAMP(5, c, 3);
+                if (kw) {
+                    if (!done(B_E2, c)) break;
+                    if (!by_rows) store(&tmDV, 6, off_dv(c), chunk_row(c));
+                    tma_store_commit();
+                }
+                if (!done(B_E1, c)) break;
+                STAMP(5, c, 4);
+                if (!by_rows) store(kw ? &tmDK : &tmDQ, kw ? 5 : 4, off_p(c), chunk_row(c));
+                tma_store_commit();
             }
             tma_store_wait_all0();
         }
@@ -397,6 +398,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
                 tc_fence_after();
                 if (acc) issue_x_state(tO, base + off_x(c), sb);
                 if (!BIDIR) {
+                    tc_commit(bar(B_XF, c));
                     if (!wait_or_abort(bar(B_M1, c), par(c), abort_flag)) break;
                     STAMP(3, c, 2);
                     if (!wait_or_abort(bar(B_NB, c), par(c), abort_flag)) break;
@@ -425,93 +427,89 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
             if (alive && !wait_or_abort(bar_, parity, abort_flag)) alive = false;
             return alive;
         };
-        if (warp < 8) {
+        if (warp < kWarpsA) {
             // -------------------------------------------------------------- group A
-            // Two 32 x 32 score blocks of this warp (row block q4, column blocks 2 hw, 2 hw + 1),
-            // masked (Q walk: columns up to the row, K walk: from the row on; diagonal kept, Eq. 6)
-            // and packed to bf16, two per column, to the columns from tdst on.  Per block the mask is
-            // all-keep, all-zero or a triangle; the first two are warp-uniform.  `guard`: a barrier
-            // to wait for before the first store (0: none).
-            auto mask = [&](uint32_t tsc, uint32_t tdst, uint32_t guard, uint32_t gpar) {
-#pragma unroll 1
-                for (int hb = 0; hb < 2; ++hb) {
-                    const int cb = 2 * hw + hb;
-                    uint32_t r[32];
-                    if (kw ? cb >= q4 : cb <= q4) {
-                        tmem_ld32(tsc + lane_base + cb * 32, r);
-                        tmem_wait_ld();
-                        if (cb == q4) {
+            const int cb = warp >> 2;                  // this warp's 32 columns
+            // One 32 x 32 score block a warp (row block q4, column block cb), masked (Q walk: columns up
+            // to the row, K walk: from the row on; diagonal kept, Eq. 6) and packed to bf16, two per
+            // column, to the columns from tdst on.  The mask of a block is all-keep, all-zero or a
+            // triangle; the first two are warp-uniform.  The packed scores go over the start of the
+            // first fp32 ones: `rd` is the barrier on which the four warps of a row block meet when they
+            // have read theirs (0: no need, they have).
+            auto mask = [&](uint32_t tsc, uint32_t tdst, uint32_t rd, uint32_t rpar) {
+                uint32_t r[32];
+                if (kw ? cb >= q4 : cb <= q4) {
+                    tmem_ld32(tsc + lane_base + cb * 32, r);
+                    tmem_wait_ld();
+                    if (cb == q4) {
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) r[j] = (kw ? j >= lane : j <= lane) ? r[j] : 0u;
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) r[j] = 0u;
+                        for (int j = 0; j < 32; ++j) r[j] = (kw ? j >= lane : j <= lane) ? r[j] : 0u;
                     }
+                } else {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) r[j] = pack_bf16(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
-                    if (hb == 0 && guard) {
-                        if (!wait(guard, gpar)) return;
-                        tc_fence_after();
-                    }
-                    tmem_st16(tdst + lane_base + cb * 16, r);
+                    for (int j = 0; j < 32; ++j) r[j] = 0u;
                 }
+                if (rd) { tc_fence_before(); mbar_arrive(rd); }
+#pragma unroll
+                for (int j = 0; j < 16; ++j) r[j] = pack_bf16(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+                if (rd) {
+                    if (!wait(rd, rpar)) return;
+                    tc_fence_after();
+                }
+                tmem_st16(tdst + lane_base + cb * 16, r);
                 tmem_wait_st();
                 tc_fence_before();
             };
-            // x^ = x / max(||x||, eps) on half a row of Bv, in place (lanes l and l ^ 16 share a row).
+            // x^ = x / max(||x||, eps) on a quarter of a row of Bv, in place (lanes l, l ^ 8, l ^ 16, l ^ 24
+            // share a row).
             auto normalise = [&](int c) {
                 if (!wait(bar(B_FB, c), par(c))) return;
-                const int nrow = w8 * 16 + (lane & 15), half = lane >> 4;
-                uint8_t* tile = gbase + off_b(c) + half * kHalf + nrow * 128;
-                float2 s0 = make_float2(0.f, 0.f), s1 = s0;
-#pragma unroll 2
-                for (int j = 0; j < 8; ++j) {
-                    const uint4 w = *reinterpret_cast<const uint4*>(tile + ((j ^ (nrow & 7)) << 4));
-                    const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&w);
+                const int nrow = warp * 8 + (lane & 7), part = lane >> 3;
+                uint8_t* tile = gbase + off_b(c) + (part >> 1) * kHalf;
+                uint4 w[4];
 #pragma unroll
-                    for (int i = 0; i < 4; i += 2) {
-                        const float2 f0 = __bfloat1622float2(e[i]), f1 = __bfloat1622float2(e[i + 1]);
-                        s0 = __ffma2_rn(f0, f0, s0); s1 = __ffma2_rn(f1, f1, s1);
-                    }
+                for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const uint4*>(tile + swz(nrow, (part & 1) * 4 + j));
+                float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+#pragma unroll
+                for (int i = 0; i < 16; i += 2) {
+                    const float2 f0 = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[i]);
+                    const float2 f1 = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[i + 1]);
+                    s0 = __ffma2_rn(f0, f0, s0); s1 = __ffma2_rn(f1, f1, s1);
                 }
                 float ss = (s0.x + s0.y) + (s1.x + s1.y);
+                ss += __shfl_xor_sync(0xffffffffu, ss, 8);
                 ss += __shfl_xor_sync(0xffffffffu, ss, 16);
                 float rn = 1.0f / fmaxf(sqrtf(ss), kEps);
                 if (VARLEN && chunk_row(c) + nrow >= tok1) rn = 0.f;      // a row of the next sequence
-#pragma unroll 2
-                for (int j = 0; j < 8; ++j) {
-                    uint4 w = *reinterpret_cast<const uint4*>(tile + ((j ^ (nrow & 7)) << 4));
-                    __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&w);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&w[j]);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) e[i] = scale_round(e[i], rn);
-                    *reinterpret_cast<uint4*>(tile + ((j ^ (nrow & 7)) << 4)) = w;
+                    *reinterpret_cast<uint4*>(tile + swz(nrow, (part & 1) * 4 + j)) = w[j];
                 }
                 fence_proxy_async();
                 mbar_arrive(bar(B_NB, c));
             };
+            if (!BIDIR && !kw) normalise(0);
             for (int c = 0; !BIDIR && c < n_chunks && alive; ++c) {
-                // K walk: Bv of this chunk landed during the chunk before.  Q walk: it lands last.
+                // K walk: Bv of this chunk was asked for during the chunk before.  Q walk: Bv of the next
+                // chunk has been there for a while; its norms fill the wait for this chunk's products.
                 STAMP(0, c, 0);
                 if (kw) { normalise(c); if (!alive) break; }
                 STAMP(0, c, 1);
-                // The packed scores go over the start of the fp32 ones: blocks 2, 3 of a row land in
-                // the columns of fp32 block 1, which the sibling warp (hw = 0) reads first; the second
-                // scores of the K walk go to columns 64-127 of SC1, which the hw = 1 warp has read by then.
-                const uint32_t sib = bars + B_SIB + 16 * q4 + 8 * (c & 1), sib2 = sib + (B_SIB2 - B_SIB);
+                // (the second scores of the K walk are packed into columns 64-127 of SC1)
 #pragma unroll 1
                 for (int it = 0; it < (kw ? 2 : 1) && alive; ++it) {
                     if (!wait(bar(it ? B_S2 : B_S1, c), par(c))) break;
                     STAMP(0, c, 2 + 2 * it);
                     tc_fence_after();
-                    const uint32_t guard = it == 0 ? (hw == 1 ? sib : 0u) : (hw == 0 ? sib2 : 0u);
-                    mask(tmem + (it ? colSC2 : colSC1), tmem + colSC1 + it * 64, guard, par(c));
+                    mask(tmem + (it ? colSC2 : colSC1), tmem + colSC1 + it * 64, it ? 0u : bars + B_RD + 16 * q4 + 8 * (c & 1), par(c));
                     if (!alive) break;
                     mbar_arrive(bar(it ? B_M2 : B_M1, c));
-                    if (it == 0) mbar_arrive(hw == 0 ? sib : sib2);
                     STAMP(0, c, 3 + 2 * it);
                 }
-                if (!kw && alive) normalise(c);
+                if (!kw && alive && c + 1 < n_chunks) normalise(c + 1);
                 if (!alive) break;
                 // bf16 copy of the updated state for the next chunk, once this chunk's products
                 // have read the previous copy.
@@ -521,12 +519,11 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
                     if (kw && !wait(bar(B_O2, c), par(c))) break;
                     STAMP(0, c, 6);
                     tc_fence_after();
-#pragma unroll 1
-                    for (int pc = 0; pc < 2; ++pc) {
+                    {
                         uint32_t r[32];
-                        tmem_ld32(tmem + lane_base + colS + hw * 64 + pc * 32, r);
+                        tmem_ld32(tmem + lane_base + colS + cb * 32, r);
                         tmem_wait_ld();
-                        write_sb(r, hw * 64 + pc * 32);
+                        write_sb(r, cb * 32);
                     }
                     fence_proxy_async();
                     tc_fence_before();
@@ -589,12 +586,38 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
                 // sum_j <k^_j - bf16(k^_j), dK^_j>, and the K walk has both factors.
                 const bool use = valid && (!kw || nrm > kEps);
                 if (use && hw == 0) dm_acc += dp * rp;
-                // out = (c acc - x coef) / max(||x||, eps) over the raw rows (K walk: which K Rt^T has read by then)
-                if (kw && !wait(bar(B_O2, c), par(c))) break;
-                STAMP(1, c, 3);
                 const bool by_rows = is_ragged(c);
                 const float sc = cfac * rp, mc = nrm > kEps ? -dp * cfac * rp * rp * rp : 0.f;
                 const float2 sc2 = make_float2(sc, sc), mc2 = make_float2(mc, mc);
+                if (kw) {
+                    // ---- dV = (c / max(||k||, eps)) dV', ahead of the rows of dk: the next chunk's second
+                    // scores wait for this accumulator.  (Its products and the state update are the last to read A.)
+                    if (!wait(bar(B_O2, c), par(c))) break;
+                    if (!BIDIR && c + 1 < n_chunks && !wait(bar(B_U, c), par(c))) break;
+                    tc_fence_after();
+                    STAMP(1, c, 3);
+                    uint8_t* vt = gbase + off_dv(c) + hw * kHalf;
+#pragma unroll 1
+                    for (int pc = 0; pc < 4; ++pc) {
+                        float2 r[8];
+                        tmem_ld16(tmem + lane_base + colSC2 + hw * 64 + pc * 16, reinterpret_cast<uint32_t*>(r));
+                        tmem_wait_ld();
+                        uint4 o[2];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const float2 v = __fmul2_rn(r[i], sc2);
+                            reinterpret_cast<uint32_t*>(o)[i] = pack_bf16(v.x, v.y);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) put(vt, 2, by_rows, c, (pc * 2 + i) * 8, o[i]);
+                    }
+                    tc_fence_before();
+                    mbar_arrive(bar(B_D2, c));
+                    fence_proxy_async();
+                    mbar_arrive(bar(B_E2, c));
+                }
+                STAMP(1, c, 4);
+                // ---- out = (c acc - x coef) / max(||x||, eps) over the raw rows
                 const float ks = use ? rp : 0.f;
                 float2 k2 = make_float2(0.f, 0.f);
 #pragma unroll 1
@@ -621,30 +644,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
                 mbar_arrive(bar(B_D1, c));
                 fence_proxy_async();
                 mbar_arrive(bar(B_E1, c));
-                STAMP(1, c, 4);
-                if (kw) {
-                    // ---- dV = (c / max(||k||, eps)) dV', over the v rows
-                    uint8_t* vt = gbase + off_x(c) + hw * kHalf;
-#pragma unroll 1
-                    for (int pc = 0; pc < 4; ++pc) {
-                        float2 r[8];
-                        tmem_ld16(tmem + lane_base + colSC2 + hw * 64 + pc * 16, reinterpret_cast<uint32_t*>(r));
-                        tmem_wait_ld();
-                        uint4 o[2];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const float2 v = __fmul2_rn(r[i], sc2);
-                            reinterpret_cast<uint32_t*>(o)[i] = pack_bf16(v.x, v.y);
-                        }
-#pragma unroll
-                        for (int i = 0; i < 2; ++i) put(vt, 2, by_rows, c, (pc * 2 + i) * 8, o[i]);
-                    }
-                    tc_fence_before();
-                    mbar_arrive(bar(B_D2, c));
-                    fence_proxy_async();
-                    mbar_arrive(bar(B_E2, c));
-                    STAMP(1, c, 5);
-                }
+                STAMP(1, c, 5);
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) dm_acc += __shfl_xor_sync(0xffffffffu, dm_acc, o);
