@@ -99,6 +99,7 @@ unsigned long long cott_launch_count(void);
  *   "bidir_bwd"          (COTT_BIDIR_BWD, 1)          0 = bidirectional d = 64 backward with one group per (b, h) as a state pass and a walk instead of one launch
  *   "short_fwd"          (COTT_SHORT_FWD, 1)          0 = sequences of at most 128 tokens through the generic walk instead of the stateless kernel
  *   "block_fwd"          (COTT_BLOCK_FWD, 1)          0 = blocks of at most 64 tokens on a state through the generic walk instead of the block kernel
+ *   "short_bwd"          (COTT_SHORT_BWD, 1)          0 = backward of at most 128 tokens through the kernels for longer sequences
  *   "host_slices"        (COTT_HOST_SLICES, 8)        most slices cott_fwd_bwd_host cuts a batch into (1 .. 16)
  *   "wait_limit_ms"      (COTT_WAIT_LIMIT_MS, 2000)   bound of every device-side wait
  *   "wait_limit_kcycles" (COTT_WAIT_LIMIT_KCYCLES, -1) the same bound in units of 1024 SM cycles; negative = use the millisecond

@@ -76,12 +76,13 @@ static Option g_opt_fused_bwd("fused_bwd", "COTT_FUSED_BWD", 1);           // 0:
 static Option g_opt_fused_bidir("fused_bidir", "COTT_FUSED_BIDIR", 1);     // 0: bidirectional d=64 forward as state pass + read-out
 static Option g_opt_bidir_bwd("bidir_bwd", "COTT_BIDIR_BWD", 1);           // 0: bidirectional d=64 backward of one group per (b, h) as state pass + walk
 static Option g_opt_short_fwd("short_fwd", "COTT_SHORT_FWD", 1);           // 0: sequences of <= 128 tokens through the generic walk
+static Option g_opt_short_bwd("short_bwd", "COTT_SHORT_BWD", 1);           // 0: backward of <= 128 tokens through the kernels for longer ones
 static Option g_opt_block_fwd("block_fwd", "COTT_BLOCK_FWD", 1);           // 0: blocks of <= 64 tokens on a state through the generic walk
 static Option g_opt_wait_ms("wait_limit_ms", "COTT_WAIT_LIMIT_MS", 2000);  // bound of every device-side wait
 static Option g_opt_wait_kc("wait_limit_kcycles", "COTT_WAIT_LIMIT_KCYCLES", -1);  // the same in units of 1024 SM cycles (< 0: use the ms value)
 static Option g_opt_host_slices("host_slices", "COTT_HOST_SLICES", 8);     // slices of the host-buffer step (1 .. 16)
 static Option* const g_options[] = {&g_opt_force_group, &g_opt_force_path, &g_opt_pair, &g_opt_fused_bwd,
-                                    &g_opt_wait_ms, &g_opt_wait_kc, &g_opt_host_slices, &g_opt_fused_bidir, &g_opt_short_fwd, &g_opt_block_fwd, &g_opt_bidir_bwd};
+                                    &g_opt_wait_ms, &g_opt_wait_kc, &g_opt_host_slices, &g_opt_fused_bidir, &g_opt_short_fwd, &g_opt_block_fwd, &g_opt_bidir_bwd, &g_opt_short_bwd};
 
 int option_force_group() { return (int)g_opt_force_group.get(); }
 int option_force_path() { return (int)g_opt_force_path.get(); }
@@ -90,6 +91,7 @@ int option_fused_bwd() { return (int)g_opt_fused_bwd.get(); }
 int option_fused_bidir() { return (int)g_opt_fused_bidir.get(); }
 int option_bidir_bwd() { return (int)g_opt_bidir_bwd.get(); }
 int option_short_fwd() { return (int)g_opt_short_fwd.get(); }
+int option_short_bwd() { return (int)g_opt_short_bwd.get(); }
 int option_block_fwd() { return (int)g_opt_block_fwd.get(); }
 int wait_limit_kcycles() {
     const long long kc = g_opt_wait_kc.get();
@@ -720,6 +722,27 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
         // over the whole sequence as a single group (no partial-state pass, no scan), with the
         // dQ^ stream's partial-state pass filling the SMs that are left; the dQ^ walk follows on
         // the whole GPU.  Each side stream then carries one tensor-core kernel per call.
+        // Short sequences: the quadratic form, several sequences per tile, one launch (cott_tc_short_bwd.cu), where
+        // the kernels for longer ones, a CTA or two per (b, h), need more than a wave.  One call behind the
+        // other, BH x N: causal d = 64 (one CTA a (b, h) and SM) 140 x 100 13.2 us against their 11.6, 228 x 79
+        // 15.2 / 19.1, 468 x 18 13.3 / 34.2, 1024 x 100 49.6 / 61.9; bidirectional (two an SM) 264 x 128 15.6 / 13.4,
+        // 468 x 18 13.3 / 21.8, and with one sequence a tile 1024 x 100 50 / 43; causal d = 128 (two CTAs a (b, h))
+        // 16 x 48 14.3 / 11.6, 112 x 26 15.2 / 21.7, 1024 x 100 103 / 136; bidirectional (state passes as well)
+        // 16 x 48 14.3 / 23.5, 468 x 18 16.5 / 119.
+        const bool short_pays = d == 128 ? !causal || BH > 74 : causal ? BH > 148 : BH > 296 && N <= 64;
+        if (N <= 128 && short_pays && !packed.cu_seqlens && !seg.on && option_short_bwd() != 0) {
+            TcBwdFusedArgs f;
+            memset(&f, 0, sizeof(f));
+            f.q = q; f.k = k; f.v = v; f.d_o = d_o; f.dq = dq; f.dk = dk; f.dv = dv;
+            f.l_qkv = lay.qkv; f.l_do = lay.o; f.l_dqkv = lay.dqkv;
+            f.l_v = lay.of(v); f.l_dv = lay.of(dv); f.w_k = p.dk; f.w_v = p.dv;
+            f.dm_partial = dm_partial; f.dm_out = dm; f.status = status;
+            f.m = sp->m; f.seq_len = sp->seq_len; f.seq_len_scalar = sp->seq_len_scalar;
+            f.bidir = causal ? 0 : 1;
+            COTT_CUDA(launch_clear_status(status, st));      // status words and the dm counter
+            COTT_CUDA(launch_tc_short_bwd(f, B, H, N, d, st));
+            return COTT_OK;
+        }
         if (d == 64 && option_fused_bwd() != 0) {
             // One walk forward in time gives all three gradients and the dm sum (cott_tc_bwd.cu).
             // It keeps two running states: Sq = V^T K^ over earlier tokens, accumulated chunk by

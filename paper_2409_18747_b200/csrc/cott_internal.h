@@ -208,6 +208,10 @@ cudaError_t launch_tc_short_fwd(const void* q, const void* k, const void* v, voi
                                 const float* seq_len, float seq_len_scalar, int B, int H, int N, int d, int dk, int dv,
                                 int causal, cudaStream_t st);
 
+// Backward for sequences of at most 128 tokens, any layout (cott_tc_short_bwd.cu): the quadratic form,
+// several sequences per 128-row tile; the only kernel of its call behind the one that clears the status words.
+cudaError_t launch_tc_short_bwd(const TcBwdFusedArgs& a, int B, int H, int N, int d, cudaStream_t st);
+
 // A block of at most 64 tokens per (b, h) on a caller's state, o and the new state in one launch, the
 // only kernel of its call.  launch_block_fwd (cott_block.cu): the state streams through registers, any
 // dk, dv up to 128.  launch_tc_block_fwd (cott_tc_block.cu): the state in tensor memory, d x d.
@@ -236,6 +240,7 @@ int option_fused_bwd();
 int option_fused_bidir();
 int option_bidir_bwd();
 int option_short_fwd();
+int option_short_bwd();
 int option_block_fwd();
 int wait_limit_kcycles();      // bound of every device-side wait, in units of 1024 SM cycles
 

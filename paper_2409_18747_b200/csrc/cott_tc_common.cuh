@@ -1,7 +1,7 @@
 // Helpers shared by the warp-specialised tensor-core kernels of cott_tc_bwd.cu and
 // cott_tc_bidir.cu: the bounded mbarrier wait with its abort protocol, and a few small device
 // functions.  Every kernel that uses them lays out its control block the same way: mbarriers in
-// the first 512 bytes, then the tensor-memory slot (offset 512), the abort flag (516) and, three
+// the first 448 bytes, then the tensor-memory slot (offset 448), the abort flag (452) and, three
 // words behind it, the wait limit in units of 1024 SM cycles.
 #pragma once
 #include "cott_sm100.cuh"
@@ -11,7 +11,7 @@ namespace tc {
 
 using namespace sm100;
 
-constexpr int kCtlTmemSlot = 512, kCtlAbort = 516;
+constexpr int kCtlTmemSlot = 448, kCtlAbort = 452;
 constexpr uint32_t kDescHi = smem_desc_hi(1024);
 #ifndef COTT_WAIT_HINT_NS
 #define COTT_WAIT_HINT_NS 1000

@@ -379,3 +379,73 @@ def test_memory_orders_match_dense(call, kind):
            "segment128": lambda *x: cott.bwd_stateful(*x, m, 999.0, state_in=st, d_state_out=ds)}[call]
     for got, want in zip(run(*(stored(x) for x in (q, k, v, d_o))), run(q, k, v, d_o)):
         assert torch.equal(got, want)
+
+
+def _laid_out(x, layout):
+    """x [B,H,N,d] on the GPU in another memory order: [B,N,H,d], or slices of a fused [B,N,3,H,d] buffer."""
+    x = dev(x)
+    if layout == "dense":
+        return x
+    B, H, N, d = x.shape
+    if layout == "bnhd":
+        return x.permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3)
+    buf = torch.full((B, N, 3, H, d), float("nan"), dtype=x.dtype, device=x.device)
+    buf[:, :, 1] = x.permute(0, 2, 1, 3)
+    return buf[:, :, 1].permute(0, 2, 1, 3)
+
+
+@pytest.mark.parametrize("N", [1, 2, 7, 8, 9, 24, 31, 64, 65, 100, 127, 128])
+@pytest.mark.parametrize("dk,dv", [(64, 64), (128, 128), (32, 32), (96, 40), (64, 128)])
+@pytest.mark.parametrize("causal", [True, False])
+def test_short_backward_tiles(N, dk, dv, causal):
+    """The backward of at most 128 tokens: one to sixteen sequences a tile, places of whole eights of rows
+    with and without rows to spare, a last tile that is not full, padded rows, every memory order."""
+    B, H = 13, 23                                          # (enough for the rule to take this kernel)
+    if max(dk, dv) <= 64 and not causal and N > 64:
+        pytest.skip("two CTAs an SM of the one-launch bidirectional kernel are faster with one sequence a tile")
+    layout = ("dense", "bnhd", "fused")[N % 3]
+    c = synth.make_qkv(B, H, N, dk, torch.bfloat16, 8100 + N + dk, row_lognormal=True, with_do=True, d_v=dv)
+    c["k"][0, 1, N // 2] = 0.0
+    args = [_laid_out(c[x], layout) for x in ("q", "k", "v", "d_o")]
+    before = cott.cott.launch_count()
+    dq, dk_, dv_, dm = cott.bwd(*args, dev(c["m"]), causal=causal)
+    assert cott.cott.launch_count() - before == 1
+    rq, rk, rv, rm = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, causal)
+    if N == 1:
+        one_token_bounds((dq, dk_, dv_), (rq, rk, rv), c)
+        assert (dm == 0).all() and (rm == 0).all()
+        return
+    z = (0, 1, N // 2)                                     # (the clamped formula's gradient, gated on its own)
+    assert norm_max_err(dk_[z], rk[z]) <= 1e-2
+    dk_[z] = 0.0
+    rk[z] = 0.0
+    gate(dq, rq, torch.bfloat16); gate(dk_, rk, torch.bfloat16); gate(dv_, rv, torch.bfloat16)
+    # dm: products of fp32 scores of the rows as they were given, summed in fp32: N terms a row in four
+    # chains, each with a few roundings of 2^-24
+    cond = dm_condition(rv, c["v"], c["m"], None)
+    assert (abs(dm.double().cpu().numpy() - rm) <= 1e-5 * cond).all()
+    again = cott.bwd(*args, dev(c["m"]), causal=causal)
+    dk2 = again[1].clone(); dk2[z] = 0.0
+    for x, y in zip((dq, dk_, dv_, dm), (again[0], dk2, again[2], again[3])):
+        assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), 3.0e38])
+@pytest.mark.parametrize("which", ["q", "k", "v", "d_o"])
+def test_short_backward_keeps_sequences_apart(d, bad, which):
+    """A row that is not finite (or whose scores overflow) in one sequence: the sequences that share its tile
+    get the bits that they get without it."""
+    B, H, N = 60, 5, 20                                    # five sequences a tile of 24 rows each
+    c = synth.make_qkv(B, H, N, d, torch.bfloat16, 8300 + d, with_do=True)
+    m = dev(c["m"])
+    ref = cott.bwd(*(dev(c[x]) for x in ("q", "k", "v", "d_o")), m)
+    c[which][0, 2, 3] = bad
+    got = cott.bwd(*(dev(c[x]) for x in ("q", "k", "v", "d_o")), m)
+    keep = torch.ones(B, H, dtype=torch.bool)
+    keep[0, 2] = False
+    for x, y in zip(got[:3], ref[:3]):
+        assert torch.equal(x[keep], y[keep])
+    assert torch.equal(got[3][[0, 1, 3, 4]], ref[3][[0, 1, 3, 4]])
+    if not bad < 1e38:
+        assert not all(torch.isfinite(x[0, 2].float()).all() for x in got[:3])
