@@ -2,7 +2,7 @@
 
 Every ``csrc/*.cu`` is compiled to an object of its own (in parallel; an object is rebuilt only
 when its source, a header or the flags changed) and the objects are linked into one shared
-library."""
+library; ``csrc/cott_torch.cpp``, the native half of the Python binding, becomes a module next to it."""
 from __future__ import annotations
 
 import concurrent.futures
@@ -10,12 +10,14 @@ import glob
 import hashlib
 import os
 import subprocess
+import sysconfig
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
 CSRC = os.path.join(_PKG, "csrc")
 OBJ = os.path.join(_PKG, "build")
 LIB = os.path.join(_PKG, "libcott.so")
+BINDING = os.path.join(_PKG, "_cott_torch.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -74,7 +76,32 @@ def build(force: bool = False, verbose: bool = False, lib: str | None = None) ->
             print(res.stderr)
         if res.returncode != 0:
             raise RuntimeError("nvcc failed linking libcott.so")
+    if lib == LIB:
+        build_binding(force, verbose)
     return lib
+
+
+def build_binding(force: bool = False, verbose: bool = False) -> str:
+    """Compile ``csrc/cott_torch.cpp``, the native half of the Python binding, against torch and libcott.so."""
+    src = os.path.join(CSRC, "cott_torch.cpp")
+    if not force and not _stale(BINDING, [src, os.path.join(_ROOT, "include", "cott.h")]):
+        return BINDING
+    import torch
+    t = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           *("-I" + p for p in (os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
+                                sysconfig.get_paths()["include"], os.path.join(cuda, "include"), os.path.join(_ROOT, "include"))),
+           src, "-o", BINDING, "-L" + os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python",
+           "-L" + _PKG, "-l:libcott.so", "-Wl,-rpath,$ORIGIN"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or res.returncode != 0:
+        print(res.stdout)
+        print(res.stderr)
+    if res.returncode != 0:
+        raise RuntimeError("the C++ compiler failed on cott_torch.cpp")
+    return BINDING
 
 
 if __name__ == "__main__":

@@ -1,4 +1,5 @@
-"""ctypes binding of the libcott C ABI: argument marshalling only.
+"""Binding of the libcott C ABI: argument marshalling only, through a native module where a call has a plain form
+and through ctypes otherwise.
 
 Function names and argument order follow ``include/cott.h``.  Tensors are torch CUDA
 tensors (contiguous ``[B,H,N,d]``, float32 or bfloat16); outputs and the workspace are
@@ -8,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import functools
+import importlib.util
 import os
 
 import torch
@@ -129,6 +131,29 @@ def _load():
     lib.option_changes = ctypes.c_uint.in_dll(lib, "cott_option_changes")
     _lib = lib
     return lib
+
+
+_native = None
+_NATIVE_PATH = os.path.join(_PKG, "_cott_torch.so")
+
+
+def _load_native():
+    """The native module with the plain forms of the calls below (``csrc/cott_torch.cpp``): each of its functions
+    returns None, having done nothing, for a call that is the Python code's, and an int for an error status."""
+    global _native
+    if _native is None:
+        _load()
+        if not os.path.exists(_NATIVE_PATH):
+            raise RuntimeError(f"{_NATIVE_PATH} is missing: build it with `python -m paper_2409_18747_b200._build`")
+        spec = importlib.util.spec_from_file_location("_cott_torch", _NATIVE_PATH)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _native = module
+    return _native
+
+
+def _checked(status, where):
+    raise CottError(status, where)
 
 
 def _on_call_stream(fn):
@@ -315,7 +340,6 @@ def _workspace_varlen(op, dt, B, H, T, max_seqlen, d, causal, device, workspace)
     return workspace, workspace.numel()
 
 
-@_on_call_stream
 def fwd(q, k, v, m, seq_len=None, causal=True, return_state=False, out=None, workspace=None,
         stream=None):
     """cott_fwd / cott_fwd_strided.  q, k, v: ``[B,H,N,d]`` tensors with contiguous rows and
@@ -323,6 +347,16 @@ def fwd(q, k, v, m, seq_len=None, causal=True, return_state=False, out=None, wor
     slices of a fused projection output; no copy is made.  ``seq_len``: None (s_b = N), a float,
     or a float32 ``[B]`` CUDA tensor.  Returns ``o`` (laid out like q when q is dense in
     memory, else dense ``[B,H,N,d]``; or ``out``) or ``(o, state[B,H,d,d] fp32)``."""
+    if stream is None:
+        done = (_native or _load_native()).fwd(q, k, v, m, seq_len, causal, return_state, out, workspace)
+        if done is not None:
+            return _checked(done, "cott_fwd_strided") if type(done) is int else done
+    return _fwd_any(q, k, v, m, seq_len=seq_len, causal=causal, return_state=return_state, out=out, workspace=workspace, stream=stream)
+
+
+@_on_call_stream
+def _fwd_any(q, k, v, m, seq_len=None, causal=True, return_state=False, out=None, workspace=None,
+        stream=None):
     if v.shape[-1] != q.shape[-1]:      # different key and value sizes
         return _fwd_dkdv(q, k, v, m, seq_len, causal, None, return_state, out, workspace, stream)
     _check_dev(m, seq_len if isinstance(seq_len, torch.Tensor) else None)
@@ -342,13 +376,22 @@ def fwd(q, k, v, m, seq_len=None, causal=True, return_state=False, out=None, wor
     return (o, state) if return_state else o
 
 
-@_on_call_stream
 def fwd_stateful(q, k, v, m, seq_len, state_in=None, return_state=True, out=None, workspace=None,
                  stream=None):
     """cott_fwd_stateful: causal forward over one segment of a longer sequence.  ``state_in``
     (fp32 ``[B,H,d,d]`` or None) is the state the previous segment (or a decode step) left;
     ``seq_len`` (a float >= 1 or a float32 ``[B]`` CUDA tensor) is the scaling base of the WHOLE
     sequence and must be the same for all its segments.  Returns ``(o, state)`` or ``o``."""
+    if stream is None:
+        done = (_native or _load_native()).fwd_stateful(q, k, v, m, seq_len, state_in, return_state, out, workspace)
+        if done is not None:
+            return _checked(done, "cott_fwd_stateful_strided") if type(done) is int else done
+    return _fwd_stateful_any(q, k, v, m, seq_len, state_in=state_in, return_state=return_state, out=out, workspace=workspace, stream=stream)
+
+
+@_on_call_stream
+def _fwd_stateful_any(q, k, v, m, seq_len, state_in=None, return_state=True, out=None, workspace=None,
+                 stream=None):
     _check_dev(m, state_in, seq_len if isinstance(seq_len, torch.Tensor) else None)
     if seq_len is None:
         raise ValueError("fwd_stateful needs the scaling base of the whole sequence")
@@ -390,13 +433,21 @@ def fwd_noalloc(q, k, v, m, seq_len=None, causal=True, out=None, stream=None):
     return o
 
 
-@_on_call_stream
 def bwd(q, k, v, d_o, m, seq_len=None, causal=True, workspace=None, stream=None, out=None, fwd_workspace=None):
     """cott_bwd / cott_bwd_strided; with ``fwd_workspace`` (the workspace tensor the forward call
     on the same q, k, v used, untouched since) cott_bwd_after_fwd, which reuses what that call
     left there.  q, k, v (common strides) and d_o as for ``fwd``; ``out``:
     optional ``(dq, dk, dv)`` tensors with common strides (e.g. the slices of a fused gradient
     buffer), else they are allocated like q.  Returns ``(dq, dk, dv, dm[H] fp32)``."""
+    if stream is None:
+        done = (_native or _load_native()).bwd(q, k, v, d_o, m, seq_len, causal, workspace, out, fwd_workspace)
+        if done is not None:
+            return _checked(done, "cott_bwd_strided" if fwd_workspace is None else "cott_bwd_after_fwd") if type(done) is int else done
+    return _bwd_any(q, k, v, d_o, m, seq_len=seq_len, causal=causal, workspace=workspace, stream=stream, out=out, fwd_workspace=fwd_workspace)
+
+
+@_on_call_stream
+def _bwd_any(q, k, v, d_o, m, seq_len=None, causal=True, workspace=None, stream=None, out=None, fwd_workspace=None):
     _check_dev(m, seq_len if isinstance(seq_len, torch.Tensor) else None)
     B, H, N, d = q.shape
     dt = _dt(q)
@@ -446,11 +497,20 @@ def _check_packed(cu_seqlens, *ts):
             raise ValueError("packed tensors must all be [total_tokens, H, d]")
 
 
-@_on_call_stream
 def fwd_varlen(q, k, v, m, cu_seqlens, max_seqlen, seq_len=None, causal=True, out=None, workspace=None,
                stream=None):
     """cott_fwd_varlen: q, k, v ``[total_tokens, H, d]`` (bf16, d a multiple of 8 up to 128), the sequences of the
     batch back to back; ``cu_seqlens`` int32 ``[B+1]`` CUDA tensor of row offsets.  Returns ``o``."""
+    if stream is None:
+        done = (_native or _load_native()).fwd_varlen(q, k, v, m, cu_seqlens, max_seqlen, seq_len, causal, out, workspace)
+        if done is not None:
+            return _checked(done, "cott_fwd_varlen") if type(done) is int else done
+    return _fwd_varlen_any(q, k, v, m, cu_seqlens, max_seqlen, seq_len=seq_len, causal=causal, out=out, workspace=workspace, stream=stream)
+
+
+@_on_call_stream
+def _fwd_varlen_any(q, k, v, m, cu_seqlens, max_seqlen, seq_len=None, causal=True, out=None, workspace=None,
+               stream=None):
     _check_packed(cu_seqlens, q, k, v)
     _check_dev(m, seq_len if isinstance(seq_len, torch.Tensor) else None)
     T, H, d = q.shape
@@ -467,10 +527,19 @@ def fwd_varlen(q, k, v, m, cu_seqlens, max_seqlen, seq_len=None, causal=True, ou
     return o
 
 
-@_on_call_stream
 def bwd_varlen(q, k, v, d_o, m, cu_seqlens, max_seqlen, seq_len=None, causal=True, workspace=None,
                stream=None):
     """cott_bwd_varlen.  Returns ``(dq, dk, dv, dm[H] fp32)`` for packed ``[total_tokens, H, d]`` inputs."""
+    if stream is None:
+        done = (_native or _load_native()).bwd_varlen(q, k, v, d_o, m, cu_seqlens, max_seqlen, seq_len, causal, workspace)
+        if done is not None:
+            return _checked(done, "cott_bwd_varlen") if type(done) is int else done
+    return _bwd_varlen_any(q, k, v, d_o, m, cu_seqlens, max_seqlen, seq_len=seq_len, causal=causal, workspace=workspace, stream=stream)
+
+
+@_on_call_stream
+def _bwd_varlen_any(q, k, v, d_o, m, cu_seqlens, max_seqlen, seq_len=None, causal=True, workspace=None,
+               stream=None):
     _check_packed(cu_seqlens, q, k, v, d_o)
     _check_dev(m, seq_len if isinstance(seq_len, torch.Tensor) else None)
     T, H, d = q.shape
@@ -489,7 +558,6 @@ def bwd_varlen(q, k, v, d_o, m, cu_seqlens, max_seqlen, seq_len=None, causal=Tru
     return dq, dk, dv, dm
 
 
-@_on_call_stream
 def bwd_stateful(q, k, v, d_o, m, seq_len, state_in=None, d_state_out=None, return_d_state=True,
                  workspace=None, stream=None, out=None):
     """cott_bwd_stateful: the backward of one segment of a longer causal sequence.  ``state_in``
@@ -498,6 +566,16 @@ def bwd_stateful(q, k, v, d_o, m, seq_len, state_in=None, d_state_out=None, retu
     ``d_state_in`` of the next segment's backward); ``seq_len`` as for ``fwd_stateful``; tensors and
     ``out`` as for ``bwd`` (strides are picked up).  Returns ``(dq, dk, dv, d_state_in, dm)``
     (``d_state_in`` is None when not asked for)."""
+    if stream is None:
+        done = (_native or _load_native()).bwd_stateful(q, k, v, d_o, m, seq_len, state_in, d_state_out, return_d_state, workspace, out)
+        if done is not None:
+            return _checked(done, "cott_bwd_stateful_strided") if type(done) is int else done
+    return _bwd_stateful_any(q, k, v, d_o, m, seq_len, state_in=state_in, d_state_out=d_state_out, return_d_state=return_d_state, workspace=workspace, stream=stream, out=out)
+
+
+@_on_call_stream
+def _bwd_stateful_any(q, k, v, d_o, m, seq_len, state_in=None, d_state_out=None, return_d_state=True,
+                 workspace=None, stream=None, out=None):
     _check_dev(m, state_in, d_state_out, seq_len if isinstance(seq_len, torch.Tensor) else None)
     B, H, N, d = q.shape
     d_v = v.shape[-1]
@@ -523,10 +601,18 @@ def bwd_stateful(q, k, v, d_o, m, seq_len, state_in=None, d_state_out=None, retu
     return dq, dk, dv, d_state_in, dm
 
 
-@_on_call_stream
 def decode_step(q, k, v, state, m, seq_len, out=None, stream=None):
     """cott_decode_step.  q,k,v ``[B,H,d]``; ``state`` fp32 ``[B,H,d,d]`` updated in place;
     ``seq_len`` a float (>= 1) or a float32 ``[B]`` CUDA tensor.  Returns ``o [B,H,d]``."""
+    if stream is None:
+        done = (_native or _load_native()).decode_step(q, k, v, state, m, seq_len, out)
+        if done is not None:
+            return _checked(done, "cott_decode_step") if type(done) is int else done
+    return _decode_step_any(q, k, v, state, m, seq_len, out=out, stream=stream)
+
+
+@_on_call_stream
+def _decode_step_any(q, k, v, state, m, seq_len, out=None, stream=None):
     _check_dev(q, k, v, state, m, seq_len if isinstance(seq_len, torch.Tensor) else None)
     B, H, d = q.shape
     d_v = v.shape[-1]

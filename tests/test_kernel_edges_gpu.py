@@ -449,3 +449,64 @@ def test_short_backward_keeps_sequences_apart(d, bad, which):
     assert torch.equal(got[3][[0, 1, 3, 4]], ref[3][[0, 1, 3, 4]])
     if not bad < 1e38:
         assert not all(torch.isfinite(x[0, 2].float()).all() for x in got[:3])
+
+
+@pytest.mark.parametrize("form", ["plain", "orders", "given", "per item", "subclass", "unequal"])
+def test_native_and_python_bindings_agree(form):
+    """The native half of the binding and the Python code behind it, which takes what the native half leaves:
+    the same bits, the same strides, the tensors that were given handed back, the same refusals."""
+    B, H, N, d = 2, 3, 70, 64
+    d_v = 96 if form == "unequal" else d
+    order = (lambda x: _laid_out(x, "fused")) if form == "orders" else dev
+    c = synth.make_qkv(B, H, N, d, torch.bfloat16, 8500, with_do=True, d_v=d_v)
+    q, k, v, d_o = (order(c[x]) for x in ("q", "k", "v", "d_o"))
+    m = dev(c["m"])
+    if form == "subclass":
+        class Tagged(torch.Tensor):
+            pass
+        q = q.as_subclass(Tagged)
+    s = torch.tensor([100.0, 300.0], device="cuda") if form == "per item" else 300.0
+    state = 0.1 * torch.randn(B, H, d, d_v, device="cuda")
+    give = form == "given"
+    new = torch.empty_like
+    ws = torch.empty(1 << 24, dtype=torch.uint8, device="cuda") if give else None
+
+    def flat(x):
+        return [y for z in x for y in flat(z)] if isinstance(x, (tuple, list)) else [x]
+
+    calls = [
+        ("fwd", (q, k, v, m, s), dict(causal=False, out=new(v) if give else None, workspace=ws)),
+        ("fwd", (q, k, v, m), dict(return_state=True)),
+        ("fwd_stateful", (q, k, v, m, s), dict(state_in=state, out=new(v) if give else None, workspace=ws)),
+        ("bwd", (q, k, v, d_o, m, s), dict(out=(new(q), new(k), new(v)) if give else None, workspace=ws)),
+        ("bwd_stateful", (q, k, v, d_o, m, s), dict(state_in=state, d_state_out=state, out=[new(q), new(k), new(v)] if give else None)),
+    ]
+    if form != "unequal":
+        cu = torch.tensor([0, 50, 70], dtype=torch.int32, device="cuda")
+        rows = [x.permute(0, 2, 1, 3)[0].contiguous() for x in (q, k, v, d_o)]
+        calls += [("fwd_varlen", (*rows[:3], m, cu, 50), dict(causal=False)), ("bwd_varlen", (*rows, m, cu, 50), {})]
+    for name, args, kw in calls:
+        a = flat(getattr(cott, name)(*args, **kw))
+        a = [x.clone(memory_format=torch.preserve_format) for x in a]
+        b = flat(getattr(cott.cott, f"_{name}_any")(*args, **kw))
+        assert len(a) == len(b)
+        for x, y in zip(a, b):
+            assert torch.equal(x, y) and x.stride() == y.stride() and x.dtype == y.dtype, name
+    if give:
+        got = cott.bwd(q, k, v, d_o, m, out=calls[3][2]["out"])
+        assert all(x is y for x, y in zip(got, calls[3][2]["out"]))
+    rows = [x[:, :, 0].contiguous() for x in (q, k, v)]
+    s1, s2 = state.clone(), state.clone()
+    o1, o2 = cott.decode_step(*rows, s1, m, s), cott.cott._decode_step_any(*rows, s2, m, s)
+    assert torch.equal(o1, o2) and torch.equal(s1, s2)
+    for bad in (lambda f: f(q, k.transpose(2, 3), v, m), lambda f: f(q.half(), k, v, m), lambda f: f(q.cpu(), k, v, m),
+                lambda f: f(q, k, v, m.cpu()), lambda f: f(q[0], k[0], v[0], m), lambda f: f(q, k, v, m, -1.0),
+                lambda f: f(q, k, v, m, workspace=torch.empty(16, dtype=torch.uint8, device="cuda"))):
+        said = []
+        for f in (cott.fwd, cott.cott._fwd_any):
+            try:
+                bad(f)
+                said.append(None)
+            except Exception as e:
+                said.append((type(e), str(e)))
+        assert said[0] == said[1]
