@@ -545,12 +545,19 @@ static cott_status fwd_impl(const void* q, const void* k, const void* v, void* o
             COTT_CUDA(launch_unpad_state(state_out, user_state_out, B * H, p.dk, p.dv, d, st));
         return COTT_OK;
     };
-    if (p.path == 1 && N <= 128 && !packed.cu_seqlens && !state_in && !state_out && !s_qkv && !s_o && !s_v &&
-        option_short_fwd() != 0) {
-        // Short sequences in dense tensors: the quadratic side of Eq. 5, several sequences per
-        // tile, no running state (cott_tc_short.cu).
-        COTT_CUDA(launch_tc_short_fwd(q, k, v, o, static_cast<int*>(ws), sp->m, sp->seq_len, sp->seq_len_scalar, B, H, N,
-                                      d, p.dk, p.dv, causal, st));
+    // In memory orders that are not dense every sequence of a tile is a copy of its own, and the kernels with a CTA
+    // per (b, h) stay ahead while those are one wave: BH x N, causal d = 64 140 x 100 5.9 us against their 5.2,
+    // 228 x 79 7.2 / 9.7, 468 x 18 5.9 / 18.1; bidirectional (two a SM) 264 x 128 7.5 / 7.0, 468 x 18 5.9 / 10.1, and with
+    // one sequence a tile 1024 x 100 17.2 / 16.7; causal d = 128 140 x 100 7.2 / 6.7, 468 x 18 7.5 / 22.7, 1024 x 100
+    // 34.8 / 47.2; bidirectional (a state pass as well) 16 x 48 6.5 / 12.7, 468 x 18 7.4 / 50.6.
+    const bool dense = !s_qkv && !s_o && !s_v;
+    const long BH = (long)B * H;
+    const bool short_pays = dense || (d == 128 ? !causal || BH > 148 : causal ? BH > 148 : BH > 296 && N <= 64);
+    if (p.path == 1 && N <= 128 && short_pays && !packed.cu_seqlens && !state_in && !state_out && option_short_fwd() != 0) {
+        // Short sequences: the quadratic side of Eq. 5, several sequences per tile, no running state
+        // (cott_tc_short.cu).
+        COTT_CUDA(launch_tc_short_fwd(q, k, v, o, lay.qkv, lay.of(v), lay.o, dense, static_cast<int*>(ws), sp->m,
+                                      sp->seq_len, sp->seq_len_scalar, B, H, N, d, p.dk, p.dv, causal, st));
         return COTT_OK;
     }
     if (p.path == 1 && !causal && d == 64 && p.n_groups == 1 && !(packed.cu_seqlens && state_out) && !state_in &&

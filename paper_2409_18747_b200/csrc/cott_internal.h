@@ -202,11 +202,11 @@ bool make_tile_map(CUtensorMap* map, const void* ptr, int B, int H, int N, int d
 
 bool make_rows_map(CUtensorMap* map, const void* ptr, long long rows, int d, int box_rows);
 
-// Forward for sequences of at most 128 tokens in dense [B,H,N,d] tensors (cott_tc_short.cu): the
-// quadratic form, several sequences per 128-row tile, no state; the only kernel of its call.
-cudaError_t launch_tc_short_fwd(const void* q, const void* k, const void* v, void* o, int* status, const float* m,
-                                const float* seq_len, float seq_len_scalar, int B, int H, int N, int d, int dk, int dv,
-                                int causal, cudaStream_t st);
+// Forward for sequences of at most 128 tokens (cott_tc_short.cu): the quadratic form, several sequences per
+// 128-row tile, no state; the only kernel of its call.  `dense`: all tensors are dense [B,H,N,d].
+cudaError_t launch_tc_short_fwd(const void* q, const void* k, const void* v, void* o, const RowLayout& l_qk, const RowLayout& l_v,
+                                const RowLayout& l_o, bool dense, int* status, const float* m, const float* seq_len,
+                                float seq_len_scalar, int B, int H, int N, int d, int dk, int dv, int causal, cudaStream_t st);
 
 // Backward for sequences of at most 128 tokens, any layout (cott_tc_short_bwd.cu): the quadratic form,
 // several sequences per 128-row tile; the only kernel of its call behind the one that clears the status words.

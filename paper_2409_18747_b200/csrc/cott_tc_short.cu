@@ -4,13 +4,16 @@
 // threshold is the 128-token tile of the tensor core.
 //
 // The rows of all (b, h) pairs of a dense [B,H,N,d] tensor are one long list of B H N rows, so a
-// tile of 128 rows holds k = floor(128 / N) whole sequences of consecutive pairs.  One CTA per
-// tile: a single score product P = Q K^^T (128 x 128), a block-diagonal mask -- a row keeps the
+// tile of 128 rows holds k = floor(128 / N) whole sequences of consecutive pairs.  In other memory
+// orders (SLOTS) a sequence is a copy of its own, in a place of N rows rounded up to eight (the
+// swizzle pattern's period).  One CTA per tile: a single score product P = Q K^^T (128 x 128), a block-diagonal mask -- a row keeps the
 // columns of its own sequence, up to and including its own position when causal --, a single
 // product O = P~ V, rows scaled by c / max(||q||, eps) (Eq. 2-4) and stored.  No state update,
 // no state copy, no second launch; B H / k CTAs instead of B H, four (d = 64) or two per SM.
 // Bound by the chain of one CTA (tiles, norms, scores, mask, product, rows out), hence by how many share
 // an SM: B=64, H=12, N=77, d=64 14.1 us (18.2 with two), B=256, H=12, N=100 45.6 (65).
+// In [B,N,H,d] storage, against a CTA per (b, h): 39 x 12 sequences of 18 tokens, d = 128, bidirectional 50.6 ->
+// 7.4 us, causal 22.7 -> 7.5; d = 64 18.1 -> 5.9.
 #include "cott_internal.h"
 #include "cott_sm100.cuh"
 #include "cott_tc_common.cuh"
@@ -45,12 +48,14 @@ struct ShortParams {
     const float* m; const float* seq_len; float seq_len_scalar;
     int H; int N; int BH;
     int seqs_per_tile;       // k
+    int slot;                // rows of a sequence's place in a tile
+    int head_first_mask;     // SLOTS: bit i: in tensor map i (q, k, v, o) the head index comes before the token index
     int causal;
     int d_out;               // columns o really has
     int wait_limit_kcycles;
 };
 
-template <int D>
+template <int D, bool SLOTS>
 __global__ void __launch_bounds__(kThreads, SL<D>::kCtas)
 tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, ShortParams p) {
@@ -64,14 +69,16 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     uint8_t* gbase = smem_raw + (base - smem_u32(smem_raw));
     const uint32_t bars = base + L::kOffCtl;
     enum { B_FULL = 0, B_KREADY = 8, B_PFULL = 16, B_PTREADY = 24, B_OFULL = 32, B_EDONE = 40, B_SIB = 48 /* [4 quadrants] */ };
+    volatile int* bad_flag = reinterpret_cast<volatile int*>(gbase + L::kOffCtl + 480);
     const uint32_t tmem_slot = bars + kCtlTmemSlot;
     volatile uint32_t* tmem_slot_g = reinterpret_cast<volatile uint32_t*>(gbase + L::kOffCtl + kCtlTmemSlot);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(gbase + L::kOffCtl + kCtlAbort);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool is_ctrl = warp == kWorkerWarps;
-    const int rows_used = p.seqs_per_tile * p.N;              // rows of this tile that hold sequences
-    const int row0 = (int)blockIdx.x * rows_used;             // first row of the tile in the list of B H N rows
+    const int row0 = (int)blockIdx.x * p.seqs_per_tile * p.N; // dense: first row of the tile in the list of B H N rows
+    const int pair0 = (int)blockIdx.x * p.seqs_per_tile;
+    const int n_seq = SLOTS ? min(p.seqs_per_tile, p.BH - pair0) : p.seqs_per_tile;
 
     if (is_ctrl) {
         tmem_alloc(tmem_slot, L::kTmemCols);
@@ -86,6 +93,7 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         mbar_init(bars + B_EDONE, 256);
         for (int i = 0; i < 4; ++i) mbar_init(bars + B_SIB + 8 * i, 32);
         *abort_flag = 0;
+        *bad_flag = 0;
         abort_flag[3] = p.wait_limit_kcycles;
         mbar_fence_init();
         fence_proxy_async();
@@ -102,18 +110,41 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (blockIdx.x == 0 && tid < 8) p.status[tid] = 0;
 
+    // SLOTS: a pass takes the sequences s0 .. s1 - 1 of the tile: all of them, once.  Sequences that share a tile
+    // meet in the second product as zeros times each other's v rows, which is no zero where a row is not finite:
+    // then (some output is not finite) the first pass is not stored and every sequence gets a pass of its own.
+    // (Dense tensors: one pass, as the rows of all sequences are one copy.)
+    int n_pass = 1;
+    for (int pass = 0; pass < n_pass; ++pass) {
+    const uint32_t par = (uint32_t)(pass & 1);
+    const int s0 = pass == 0 ? 0 : pass - 1, s1 = pass == 0 ? n_seq : pass;
     if (is_ctrl) {
-        if (lane == 0) {
-            // The copies bring rows_used rows per box; the rows below them are zeroed by the workers.
-            const uint32_t fb = bars + B_FULL;
-            mbar_expect_tx(fb, 3u * NH * (uint32_t)rows_used * 128u);
-#pragma unroll
-            for (int hh = 0; hh < NH; ++hh) {
-                tma_load_4d(base + L::kOffQ + hh * 16384, &tmQ, fb, hh * 64, row0, 0, 0);
-                tma_load_4d(base + L::kOffK + hh * 16384, &tmK, fb, hh * 64, row0, 0, 0);
-                tma_load_4d(base + L::kOffV + hh * 16384, &tmV, fb, hh * 64, row0, 0, 0);
+        bool go = true;
+        if (SLOTS) {
+            // One copy per sequence, tensor and half tile, over the lanes (rows past N read as zero).
+            if (lane == 0) mbar_expect_tx(bars + B_FULL, (uint32_t)((s1 - s0) * p.slot) * 128u * 3u * NH);
+            __syncwarp();
+            for (int i = lane; i < (s1 - s0) * 3 * NH; i += 32) {
+                const int sq = s0 + i / (3 * NH), r = i % (3 * NH), t = r / NH, hh = r % NH, pair = pair0 + sq;
+                const int b = pair / p.H, h = pair - b * p.H;
+                const bool hf = (p.head_first_mask >> t) & 1;
+                tma_load_4d(base + t * L::kTile + hh * 16384 + sq * p.slot * 128, t == 0 ? &tmQ : t == 1 ? &tmK : &tmV, bars + B_FULL,
+                            hh * 64, hf ? h : 0, hf ? 0 : h, b);
             }
-            bool ok = wait_or_abort(bars + B_KREADY, 0u, abort_flag);
+        }
+        if (lane == 0) {
+            if (!SLOTS) {
+                // The copies bring the rows of all sequences per box; the rows below them are zeroed by the workers.
+                const uint32_t fb = bars + B_FULL;
+                mbar_expect_tx(fb, 3u * NH * (uint32_t)(p.seqs_per_tile * p.N) * 128u);
+#pragma unroll
+                for (int hh = 0; hh < NH; ++hh) {
+                    tma_load_4d(base + L::kOffQ + hh * 16384, &tmQ, fb, hh * 64, row0, 0, 0);
+                    tma_load_4d(base + L::kOffK + hh * 16384, &tmK, fb, hh * 64, row0, 0, 0);
+                    tma_load_4d(base + L::kOffV + hh * 16384, &tmV, fb, hh * 64, row0, 0, 0);
+                }
+            }
+            bool ok = wait_or_abort(bars + B_KREADY, par, abort_flag);
             if (ok) {
                 // P = Q K^^T: both operands K-major
                 tc_fence_after();
@@ -125,7 +156,7 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     mma_ss_w(tmem + colP, xl + off, kDescHi, al + off, kDescHi, idesc, kk > 0);
                 }
                 tc_commit(bars + B_PFULL);
-                ok = wait_or_abort(bars + B_PTREADY, 0u, abort_flag);
+                ok = wait_or_abort(bars + B_PTREADY, par, abort_flag);
             }
             if (ok) {
                 // O = P~ V: P~ from tensor memory (8 columns per K = 16), V MN-major; the
@@ -137,15 +168,33 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 for (int kk = 0; kk < kRows / 16; ++kk)
                     mma_ts_w(tmem + colO, tmem + colPt + kk * 8u, bl + kk * 128u, kDescHi, idesc, kk > 0);
                 tc_commit(bars + B_OFULL);
-                ok = wait_or_abort(bars + B_EDONE, 0u, abort_flag);
+                ok = wait_or_abort(bars + B_EDONE, par, abort_flag);
             }
-            if (ok) {
+            if (ok && !SLOTS) {
 #pragma unroll
                 for (int hh = 0; hh < NH; ++hh)
                     if (hh * 64 < p.d_out) tma_store_4d(&tmO, base + L::kOffQ + hh * 16384, hh * 64, row0, 0, 0);
                 tma_store_commit();
                 tma_store_wait_all0();
             }
+            go = ok;
+        }
+        if (SLOTS) {
+            if (!__shfl_sync(0xffffffffu, go ? 1 : 0, 0)) break;
+            if (pass == 0 && n_seq > 1 && *bad_flag) {
+                n_pass = 1 + n_seq;
+            } else {
+                for (int i = lane; i < (s1 - s0) * NH; i += 32) {
+                    const int sq = s0 + i / NH, hh = i % NH, pair = pair0 + sq;
+                    const int b = pair / p.H, h = pair - b * p.H;
+                    const bool hf = (p.head_first_mask >> 3) & 1;
+                    if (hh * 64 < p.d_out)
+                        tma_store_4d(&tmO, base + L::kOffQ + hh * 16384 + sq * p.slot * 128, hh * 64, hf ? h : 0, hf ? 0 : h, b);
+                }
+                tma_store_commit();
+                tma_store_wait_read0();
+            }
+            __syncwarp();
         }
     } else {
         // ------------------------------------------------------------------ row workers
@@ -157,11 +206,11 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         };
         const int q4 = warp & 3, hf = warp >> 2, row = q4 * 32 + lane;
         const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
-        const bool valid = row < rows_used;
         // rows the copies do not write: zero (a zero v row times a zero score must not be NaN)
         // (two lanes, l and l ^ 16, share a row here and in the row norms, half of it each)
         const int nrow = warp * 16 + (lane & 15), half = lane >> 4;
-        if (nrow >= rows_used) {
+        if (pass > 0 && !wait(bars + B_FULL, par)) break;     // (behind which the rows of the pass before have left)
+        if (nrow < s0 * p.slot || nrow >= s1 * p.slot) {
 #pragma unroll
             for (int j = 0; j < 4 * NH; ++j) {
                 const int ch = half * 4 * NH + j;                     // 16-byte chunk of the row
@@ -172,18 +221,17 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             }
         }
         // the row's sequence: pair index, scaling factor, first row of the sequence in the tile
-        const int seq = row / p.N;
-        const int pair = (int)blockIdx.x * p.seqs_per_tile + seq;
-        const bool live = valid && pair < p.BH;
+        const int seq = row / p.slot, pair = pair0 + seq;
+        const bool live = seq >= s0 && seq < s1 && row - seq * p.slot < p.N && pair < p.BH;
         float cfac = 0.f;
         if (live) {
             const int b = pair / p.H, h = pair % p.H;
             const float s_b = p.seq_len ? p.seq_len[b] : (p.seq_len_scalar > 0.f ? p.seq_len_scalar : (float)p.N);
             cfac = stab_factor(p.m[h], s_b);
         }
-        const int lo = seq * p.N, hi = live ? (p.causal ? row : lo + p.N - 1) : -1;
+        const int lo = seq * p.slot, hi = live ? (p.causal ? row : lo + p.N - 1) : -1;
         float* rq_buf = reinterpret_cast<float*>(gbase + L::kOffCtl + L::kOffRx);
-        if (wait(bars + B_FULL, 0u)) {
+        if (wait(bars + B_FULL, par)) {
             // ||q|| and ||k||; k is normalised in place
             float2 sq = make_float2(0.f, 0.f), sk = sq;
 #pragma unroll
@@ -219,7 +267,7 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             fence_proxy_async();
             mbar_arrive(bars + B_KREADY);
         }
-        if (wait(bars + B_PFULL, 0u)) {
+        if (wait(bars + B_PFULL, par)) {
             // block-diagonal (causal) mask on this thread's 64 columns, packed to bf16 pairs
             tc_fence_after();
 #pragma unroll 1
@@ -238,23 +286,28 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 }
                 // (D = 64: columns 32-63, which the hf = 1 warp writes, hold scores of the hf = 0 warp)
                 if (D == 64 && hf == 0 && pc == 1) { tc_fence_before(); mbar_arrive(bars + B_SIB + 8 * q4); }
-                if (D == 64 && hf == 1 && pc == 0) { if (!wait(bars + B_SIB + 8 * q4, 0u)) break; tc_fence_after(); }
+                if (D == 64 && hf == 1 && pc == 0) { if (!wait(bars + B_SIB + 8 * q4, par)) break; tc_fence_after(); }
                 tmem_st16(tmem + lane_base + colPt + (c0 >> 1), pk);
             }
             tmem_wait_st();
             tc_fence_before();
             mbar_arrive(bars + B_PTREADY);
         }
-        if (wait(bars + B_OFULL, 0u)) {
+        if (wait(bars + B_OFULL, par)) {
             // this thread's D / 2 accumulator columns: scale, round, stage where q was
             tc_fence_after();
             const float rx = cfac * rq_buf[row];
+            float finite = 0.f;
 #pragma unroll 1
             for (int pc = 0; pc < D / 64; ++pc) {
                 const int c0 = hf * (D / 2) + pc * 32;
                 uint32_t a[32];
                 tmem_ld32(tmem + lane_base + colO + c0, a);
                 tmem_wait_ld();
+                if (SLOTS) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) finite = fmaf(__uint_as_float(a[j]), 0.f, finite);
+                }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     uint4 o;
@@ -266,11 +319,18 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     *reinterpret_cast<uint4*>(gbase + L::kOffQ + (ch >> 3) * 16384u + swz(row, ch & 7)) = o;
                 }
             }
+            if (SLOTS && !(finite == 0.f)) *bad_flag = 1;
             fence_proxy_async();
             tc_fence_before();
             mbar_arrive(bars + B_EDONE);
         }
+        if (SLOTS && n_seq > 1) {
+            if (!wait(bars + B_EDONE, par)) break;
+            if (pass == 0 && *bad_flag) n_pass = 1 + n_seq;
+        }
     }
+    }
+    if (SLOTS && is_ctrl) tma_store_wait_all0();
     tc_fence_before();
     __syncthreads();
     if (*abort_flag) {
@@ -285,9 +345,9 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     if (is_ctrl) tmem_dealloc(tmem, L::kTmemCols);
 }
 
-template <int D>
+template <int D, bool SLOTS>
 cudaError_t launch_d(const CUtensorMap* tm, const ShortParams& p, int tiles, cudaStream_t st) {
-    auto kern = tc_short_fwd_kernel<D>;
+    auto kern = tc_short_fwd_kernel<D, SLOTS>;
     if (cudaError_t e = configure_smem_once(reinterpret_cast<const void*>(kern), SL<D>::kDynBytes); e != cudaSuccess)
         return e;
     const int prof = profile_begin_launch(5, st);
@@ -309,25 +369,31 @@ cudaError_t launch_d(const CUtensorMap* tm, const ShortParams& p, int tiles, cud
 
 }  // namespace
 
-cudaError_t launch_tc_short_fwd(const void* q, const void* k, const void* v, void* o, int* status, const float* m,
-                                const float* seq_len, float seq_len_scalar, int B, int H, int N, int d, int dk, int dv,
-                                int causal, cudaStream_t st) {
+cudaError_t launch_tc_short_fwd(const void* q, const void* k, const void* v, void* o, const RowLayout& l_qk, const RowLayout& l_v,
+                                const RowLayout& l_o, bool dense, int* status, const float* m, const float* seq_len,
+                                float seq_len_scalar, int B, int H, int N, int d, int dk, int dv, int causal, cudaStream_t st) {
     if (N < 1 || N > kRows || (d != 64 && d != 128) || dk > d || dv > d) return cudaErrorInvalidValue;
     ShortParams p;
     p.status = status; p.m = m; p.seq_len = seq_len; p.seq_len_scalar = seq_len_scalar;
     p.H = H; p.N = N; p.BH = B * H;
-    p.seqs_per_tile = kRows / N;
+    p.slot = dense ? N : (N + 7) / 8 * 8;
+    p.seqs_per_tile = kRows / p.slot;
     p.causal = causal; p.d_out = dv;
+    p.head_first_mask = 0;
     p.wait_limit_kcycles = wait_limit_kcycles();
-    const int rows_used = p.seqs_per_tile * N;
-    const long long rows = (long long)B * H * N;
     const void* ptrs[4] = {q, k, v, o};
     const int widths[4] = {dk, dk, dv, dv};
+    const RowLayout lays[4] = {l_qk, l_qk, l_v, l_o};
     CUtensorMap tm[4];
-    for (int i = 0; i < 4; ++i)
-        if (!make_rows_map(&tm[i], ptrs[i], rows, widths[i], rows_used)) return cudaErrorInvalidValue;
+    for (int i = 0; i < 4; ++i) {
+        bool hf = false;
+        if (dense ? !make_rows_map(&tm[i], ptrs[i], (long long)B * H * N, widths[i], p.seqs_per_tile * N)
+                  : !make_tile_map(&tm[i], ptrs[i], B, H, N, widths[i], lays[i], &hf, p.slot)) return cudaErrorInvalidValue;
+        p.head_first_mask |= (hf ? 1 : 0) << i;
+    }
     const int tiles = (p.BH + p.seqs_per_tile - 1) / p.seqs_per_tile;
-    return d == 64 ? launch_d<64>(tm, p, tiles, st) : launch_d<128>(tm, p, tiles, st);
+    if (d == 64) return dense ? launch_d<64, false>(tm, p, tiles, st) : launch_d<64, true>(tm, p, tiles, st);
+    return dense ? launch_d<128, false>(tm, p, tiles, st) : launch_d<128, true>(tm, p, tiles, st);
 }
 
 }  // namespace cott

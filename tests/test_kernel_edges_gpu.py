@@ -510,3 +510,44 @@ def test_native_and_python_bindings_agree(form):
             except Exception as e:
                 said.append((type(e), str(e)))
         assert said[0] == said[1]
+
+
+@pytest.mark.parametrize("N", [1, 2, 7, 8, 9, 31, 64, 65, 100, 128])
+@pytest.mark.parametrize("dk,dv", [(64, 64), (128, 128), (32, 32), (96, 40), (64, 128)])
+@pytest.mark.parametrize("causal", [True, False])
+def test_short_forward_memory_orders(N, dk, dv, causal):
+    """The forward of at most 128 tokens in memory orders that are not dense: places of whole eights of rows,
+    a last tile that is not full; against the dense tensors' kernel, whose tiles hold the same rows (the
+    scores and the sums over a row's own columns do not depend on where in a tile a sequence lies)."""
+    B, H = 13, 23                                          # (enough for the rule to take this kernel)
+    if max(dk, dv) <= 64 and not causal and N > 64:
+        pytest.skip("the one-launch bidirectional kernel is faster with one sequence a tile")
+    c = synth.make_qkv(B, H, N, dk, torch.bfloat16, 8700 + N + dk, row_lognormal=True, d_v=dv)
+    c["k"][0, 1, N // 2] = 0.0
+    m = dev(c["m"])
+    o = cott.fwd(*(dev(c[x]) for x in ("q", "k", "v")), m, causal=causal)
+    if N > 1:
+        gate(o, oracle.fwd_quadratic(c["q"], c["k"], c["v"], c["m"], None, causal), torch.bfloat16)
+    for layout in ("bnhd", "fused"):
+        out = torch.full((B, N, H, dv), 7.0, dtype=torch.bfloat16, device="cuda").permute(0, 2, 1, 3)
+        before = cott.cott.launch_count()
+        cott.fwd(*(_laid_out(c[x], layout) for x in ("q", "k", "v")), m, causal=causal, out=out)
+        assert cott.cott.launch_count() - before == 1
+        assert norm_max_err(out, o) <= 2.0 ** -8           # (one rounding of the output)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("which", ["q", "k", "v"])
+def test_short_forward_keeps_sequences_apart(d, bad, which):
+    """A row that is not finite in one sequence of a tile of five: the others get the bits that they get without it."""
+    B, H, N = 60, 5, 20
+    c = synth.make_qkv(B, H, N, d, torch.bfloat16, 8800 + d)
+    m = dev(c["m"])
+    ref = cott.fwd(*(_laid_out(c[x], "bnhd") for x in ("q", "k", "v")), m)
+    c[which][0, 2, 3] = bad
+    got = cott.fwd(*(_laid_out(c[x], "bnhd") for x in ("q", "k", "v")), m)
+    keep = torch.ones(B, H, dtype=torch.bool)
+    keep[0, 2] = False
+    assert torch.equal(got[keep], ref[keep])
+    assert not torch.isfinite(got[0, 2].float()).all()
