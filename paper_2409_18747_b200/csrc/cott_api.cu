@@ -658,7 +658,9 @@ static Bwd128Groups bwd128_groups(const Plan& p, int BH, int N, int causal, bool
     // chunk of 128 tokens a K walk takes 4.6 us and a Q walk 3.5; a walk cut in groups costs a state pass of
     // about 5 us and 0.9 us per chunk of its parts.  A single later group of the K walk leaves SMs idle in
     // its state pass: that pass is cut into up to four parts.  (Against half the plan's groups for both:
-    // B=3, H=16, N=2999 113 us / 127, B=1, H=40, N=4096 143 / 165, B=1, H=16, N=16384 224 / 254.)
+    // B=3, H=16, N=2999 113 us / 127, B=1, H=40, N=4096 143 / 165, B=1, H=16, N=16384 224 / 254.  The chunks
+    // have since become 4.4 and 2.9 us, those calls 101, 121 and 214; with these figures in the sum below ten
+    // shapes from B H = 8 to 64 take the same time.)
     const int chunks = (N + 127) / 128, slots = 148 / BH;
     double best = 1e30;
     // Of the numbers of groups with walks of one length only the least is looked at (others have the same walks

@@ -57,7 +57,7 @@ struct L {
     static constexpr int kOffStQ = kOffEb + 2 * kStateTile;  // staging of the dq rows of a chunk
     static constexpr int kOffStK = kOffStQ + kTile;          // staging of the dk rows
     static constexpr int kOffCtl = kOffStK + kTile;
-    // control block: mbarriers (first 512 bytes), tensor-memory slot, abort flag and wait
+    // control block: mbarriers (first 448 bytes), tensor-memory slot, abort flag and wait
     // limit, reciprocal row norms of the two stages, dm scratch
     static constexpr int kOffTmemSlot = kCtlTmemSlot, kOffAbort = kCtlAbort;
     static constexpr int kOffRq = 1024;                      // float2 [2][128]: 1 / max(||q||, eps), 1 if not clamped
