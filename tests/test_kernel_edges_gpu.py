@@ -447,8 +447,35 @@ def test_short_backward_keeps_sequences_apart(d, bad, which):
     for x, y in zip(got[:3], ref[:3]):
         assert torch.equal(x[keep], y[keep])
     assert torch.equal(got[3][[0, 1, 3, 4]], ref[3][[0, 1, 3, 4]])
-    if not bad < 1e38:
+    if bad == 3.0e38 and which in "qk":                    # (too long for fp32, but finite: a unit row of zeros)
+        assert all(torch.isfinite(x[0, 2].float()).all() for x in got[:3])
+    else:
         assert not all(torch.isfinite(x[0, 2].float()).all() for x in got[:3])
+
+
+@pytest.mark.parametrize("dk,dv,N,causal", [(64, 64, 20, True), (64, 64, 20, False), (64, 64, 128, True), (128, 128, 20, True),
+                                            (128, 128, 20, False), (128, 128, 128, True), (128, 128, 128, False), (96, 40, 20, True)])
+@pytest.mark.parametrize("value", [3.0e38, 1.0e25, "one"])
+@pytest.mark.parametrize("which", ["q", "k"])
+def test_short_backward_rows_too_long_for_fp32(which, value, causal, N, dk, dv):
+    """Finite rows of q or k whose squared norm overflows fp32 (1 / norm = 0), one sequence a tile and five: the
+    same as a row of zeros there for everybody else, as in the kernels that normalise the rows first, and a
+    gradient of zeros for the row itself."""
+    B, H, z = (30, 11, (0, 2, 3)) if N == 20 else (14, 11, (0, 2, 77))
+    c = synth.make_qkv(B, H, N, dk, torch.bfloat16, 8400 + N + dk, with_do=True, d_v=dv)
+    args = {x: dev(c[x]) for x in ("q", "k", "v", "d_o", "m")}
+    args[which][z] = 0.0
+    want = cott.bwd(*args.values(), causal=causal)
+    if value == "one":
+        args[which][z][5] = 3.0e38
+    else:
+        args[which][z] = value
+    got = cott.bwd(*args.values(), causal=causal)
+    own = 0 if which == "q" else 1
+    assert (got[own][z] == 0).all()
+    want[own][z] = 0.0                                     # (the zero row's is that of the clamped formula)
+    for x, y in zip(got, want):
+        assert torch.equal(x, y)
 
 
 @pytest.mark.parametrize("form", ["plain", "orders", "given", "per item", "subclass", "unequal"])
