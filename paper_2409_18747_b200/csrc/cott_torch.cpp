@@ -11,6 +11,7 @@
 #include <torch/csrc/utils/python_arg_parser.h>
 #include <ATen/ATen.h>
 #include <ATen/PythonTorchFunctionTLS.h>
+#include <c10/core/impl/LocalDispatchKeySet.h>
 #include <c10/core/impl/TorchDispatchModeTLS.h>
 #include <c10/cuda/CUDAStream.h>
 #include <algorithm>
@@ -99,7 +100,9 @@ PyObject* wrap(const at::Tensor& t) { return THPVariable_Wrap(t); }
 // Runs f with the argument count checked and everything that is not a plain call handed back as None.
 template <class F> PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F f) {
     if (n != want) { PyErr_SetString(PyExc_TypeError, "wrong number of arguments"); return nullptr; }
-    if (at::impl::torch_function_mode_enabled() || c10::impl::TorchDispatchModeTLS::any_modes_set()) Py_RETURN_NONE;
+    // (inside a level of torch.func.grad or jvp even a tensor made from plain ones is a wrapper without storage)
+    if (at::impl::torch_function_mode_enabled() || c10::impl::TorchDispatchModeTLS::any_modes_set() ||
+        c10::impl::tls_is_dispatch_key_included(c10::DispatchKey::FuncTorchDynamicLayerFrontMode)) Py_RETURN_NONE;
     try {
         return f();
     } catch (const Other&) {
@@ -112,12 +115,14 @@ template <class F> PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F f) {
         Py_RETURN_NONE;
     }
 }
+// The interpreter lock released while f runs and taken again however it ends: asking for a data pointer may throw.
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
 template <class F> cott_status without_gil(F f) {
-    cott_status rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = f();
-    Py_END_ALLOW_THREADS
-    return rc;
+    Unlocked unlocked;
+    return f();
 }
 PyObject* given_or_new(PyObject* given, const at::Tensor& t) {
     if (none(given)) return wrap(t);

@@ -3,6 +3,7 @@ tiles, remainders, the smallest and the largest of its range.  Oracle, metrics a
 of test_parity_gpu.py."""
 import pytest
 import torch
+from torch.utils._python_dispatch import TorchDispatchMode
 
 import oracle
 import paper_2409_18747_b200 as cott
@@ -537,6 +538,86 @@ def test_native_and_python_bindings_agree(form):
             except Exception as e:
                 said.append((type(e), str(e)))
         assert said[0] == said[1]
+
+
+def _native_and_python_calls(B=2, H=3, N=70, d=64):
+    """(name, arguments) of every call that has a native form."""
+    c = synth.make_qkv(B, H, N, d, torch.bfloat16, 8600, with_do=True)
+    q, k, v, d_o, m = (dev(c[x]) for x in ("q", "k", "v", "d_o", "m"))
+    state = 0.1 * torch.randn(B, H, d, d, device="cuda")
+    cu = torch.tensor([0, 50, 70], dtype=torch.int32, device="cuda")
+    rows = [x.permute(0, 2, 1, 3)[0].contiguous() for x in (q, k, v, d_o)]
+    one = [x[:, :, 0].contiguous() for x in (q, k, v)]
+    return [("fwd", (q, k, v, m, None, True, False, None, None)),
+            ("fwd_stateful", (q, k, v, m, 300.0, state, True, None, None)),
+            ("bwd", (q, k, v, d_o, m, None, True, None, None, None)),
+            ("bwd_stateful", (q, k, v, d_o, m, 300.0, state, state, True, None, None)),
+            ("fwd_varlen", (*rows[:3], m, cu, 50, None, True, None, None)),
+            ("bwd_varlen", (*rows, m, cu, 50, None, True, None)),
+            ("decode_step", (*one, state, m, 300.0, None))]
+
+
+class _PassThrough(TorchDispatchMode):
+    def __torch_dispatch__(self, func, types, args=(), kwargs=None):
+        return func(*args, **(kwargs or {}))
+
+
+@pytest.mark.parametrize("inside", ["grad", "jvp", "vmap", "dispatch mode", "function mode"])
+def test_native_binding_leaves_transforms_and_modes_to_python(inside):
+    """Tensors that a transform only captures look plain, but what is allocated inside a level of grad or jvp has
+    no storage: the native half hands every call back, and the Python code answers as it does by itself."""
+    native = cott.cott._load_native()
+
+    def within(f):
+        got = []
+        body = lambda x: (got.append(f()), x.sum())[1]
+        x = torch.ones(2, 2, device="cuda")
+        if inside == "grad":
+            torch.func.grad(body)(x)
+        elif inside == "jvp":
+            torch.func.jvp(body, (x,), (x,))
+        elif inside == "vmap":
+            torch.func.vmap(body)(x)
+        elif inside == "dispatch mode":
+            with _PassThrough():
+                body(x)
+        else:
+            with torch.overrides.BaseTorchFunctionMode():
+                body(x)
+        return got[0]
+
+    def said(f):
+        try:
+            return within(f)
+        except Exception as e:
+            return type(e), str(e)
+
+    for name, args in _native_and_python_calls():
+        assert within(lambda: getattr(native, name)(*args)) is None, name
+        again = [x.clone() if i == 3 and name == "decode_step" else x for i, x in enumerate(args)]
+        a, b = said(lambda: getattr(cott, name)(*args)), said(lambda: getattr(cott.cott, f"_{name}_any")(*again))
+        assert type(a) is type(b)
+        if isinstance(a, tuple) and isinstance(a[0], type):
+            assert a == b, name
+        else:
+            for x, y in zip(a if isinstance(a, tuple) else [a], b if isinstance(b, tuple) else [b]):
+                assert torch.equal(x, y), name
+        assert getattr(native, name)(*args) is not None, name     # (and it takes the call outside)
+
+
+def test_native_binding_holds_the_lock_after_a_refused_pointer():
+    """torch refuses the data pointer of a workspace while the native half has the interpreter lock released: the
+    lock is taken again and the Python code reports the refusal."""
+    for name, args in _native_and_python_calls():
+        if name == "decode_step":
+            continue                                       # (no workspace)
+        at = {"bwd": 7, "bwd_varlen": 9, "bwd_stateful": 9, "fwd_varlen": 9}.get(name, 8)
+        ws = torch.empty(1 << 24, dtype=torch.uint8, device="cuda")
+        assert getattr(cott.cott._load_native(), name)(*args[:at], ws, *args[at + 1:]) is not None
+        torch._C._set_throw_on_mutable_data_ptr(ws)
+        with pytest.raises(RuntimeError):
+            getattr(cott, name)(*args[:at], workspace=ws)
+        assert getattr(cott.cott._load_native(), name)(*args) is not None
 
 
 @pytest.mark.parametrize("N", [1, 2, 7, 8, 9, 31, 64, 65, 100, 128])
