@@ -95,6 +95,7 @@ void* ptr(const at::Tensor& t) { return t.data_ptr(); }
 float* fptr(const at::Tensor& t) { return static_cast<float*>(t.data_ptr()); }
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
+// (a tensor that came in as an argument goes out as the object that it came in as)
 PyObject* wrap(const at::Tensor& t) { return THPVariable_Wrap(t); }
 
 // Runs f with the argument count checked and everything that is not a plain call handed back as None.
@@ -124,16 +125,12 @@ template <class F> cott_status without_gil(F f) {
     Unlocked unlocked;
     return f();
 }
-PyObject* given_or_new(PyObject* given, const at::Tensor& t) {
-    if (none(given)) return wrap(t);
-    Py_INCREF(given);
-    return given;
-}
-void three(PyObject* out, PyObject* (&o)[3]) {
+// The tensors of a tuple or list, held as tensors: another thread may change a list while the lock is released.
+void three(PyObject* out, at::Tensor (&o)[3]) {
     if (PyTuple_CheckExact(out) && PyTuple_GET_SIZE(out) == 3) {
-        for (int i = 0; i < 3; ++i) o[i] = PyTuple_GET_ITEM(out, i);
+        for (int i = 0; i < 3; ++i) o[i] = plain(PyTuple_GET_ITEM(out, i));
     } else if (PyList_CheckExact(out) && PyList_GET_SIZE(out) == 3) {
-        for (int i = 0; i < 3; ++i) o[i] = PyList_GET_ITEM(out, i);
+        for (int i = 0; i < 3; ++i) o[i] = plain(PyList_GET_ITEM(out, i));
     } else throw Other();
 }
 
@@ -162,8 +159,7 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
                                     lo.get(), &sp, ptr(ws), (size_t)ws.numel(), st);
         });
         if (rc != COTT_OK) return PyLong_FromLong(rc);
-        PyObject* po = given_or_new(a[7], o);
-        return want_state ? Py_BuildValue("(NN)", po, wrap(state)) : po;
+        return want_state ? Py_BuildValue("(NN)", wrap(o), wrap(state)) : wrap(o);
     });
 }
 
@@ -195,8 +191,7 @@ PyObject* fwd_stateful(PyObject*, PyObject* const* a, Py_ssize_t n) {
                                              (size_t)ws.numel(), st);
         });
         if (rc != COTT_OK) return PyLong_FromLong(rc);
-        PyObject* po = given_or_new(a[7], o);
-        return want_state ? Py_BuildValue("(NN)", po, wrap(state)) : po;
+        return want_state ? Py_BuildValue("(NN)", wrap(o), wrap(state)) : wrap(o);
     });
 }
 
@@ -212,11 +207,9 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const Layout lq = layout(q, k, v), ld = layout(d_o);
         at::Tensor ws = none(a[7]) ? at::Tensor() : plain(a[7]);
         const bool given = !none(a[8]);
-        PyObject* po[3] = {nullptr, nullptr, nullptr};
         at::Tensor g[3];
         if (given) {
-            three(a[8], po);
-            for (int i = 0; i < 3; ++i) g[i] = plain(po[i]);
+            three(a[8], g);
             layout(g[0], g[1], g[2]);
         }
         at::Tensor fws = none(a[9]) ? at::Tensor() : plain(a[9]);
@@ -235,8 +228,7 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
                                    lq.get(), ld.get(), lg.get(), &sp, ptr(ws), (size_t)ws.numel(), st);
         });
         if (rc != COTT_OK) return PyLong_FromLong(rc);
-        return Py_BuildValue("(NNNN)", given_or_new(given ? po[0] : Py_None, g[0]), given_or_new(given ? po[1] : Py_None, g[1]),
-                             given_or_new(given ? po[2] : Py_None, g[2]), wrap(dm));
+        return Py_BuildValue("(NNNN)", wrap(g[0]), wrap(g[1]), wrap(g[2]), wrap(dm));
     });
 }
 
@@ -258,11 +250,9 @@ PyObject* bwd_stateful(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const Layout lq = layout(q, k, v), ld = layout(d_o);
         at::Tensor ws = none(a[9]) ? at::Tensor() : plain(a[9]);
         const bool given = !none(a[10]);
-        PyObject* po[3] = {nullptr, nullptr, nullptr};
         at::Tensor g[3];
         if (given) {
-            three(a[10], po);
-            for (int i = 0; i < 3; ++i) g[i] = plain(po[i]);
+            three(a[10], g);
             layout(g[0], g[1], g[2]);
         }
         const size_t need = ws.defined() ? 0 : cott_workspace_bytes_dkdv(COTT_OP_BWD, dt, B, H, N, d, d, 1);
@@ -282,8 +272,7 @@ PyObject* bwd_stateful(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (rc != COTT_OK) return PyLong_FromLong(rc);
         PyObject* pd = Py_None;
         if (want) pd = wrap(ds); else Py_INCREF(Py_None);
-        return Py_BuildValue("(NNNNN)", given_or_new(given ? po[0] : Py_None, g[0]), given_or_new(given ? po[1] : Py_None, g[1]),
-                             given_or_new(given ? po[2] : Py_None, g[2]), pd, wrap(dm));
+        return Py_BuildValue("(NNNNN)", wrap(g[0]), wrap(g[1]), wrap(g[2]), pd, wrap(dm));
     });
 }
 
@@ -328,7 +317,7 @@ PyObject* fwd_varlen(PyObject*, PyObject* const* a, Py_ssize_t n) {
                                    c.dt, &c.sp, ptr(ws), (size_t)ws.numel(), st);
         });
         if (rc != COTT_OK) return PyLong_FromLong(rc);
-        return given_or_new(a[8], o);
+        return wrap(o);
     });
 }
 
@@ -365,7 +354,7 @@ PyObject* decode_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const cott_dtype dt = dtype_of(q);
         const cott_scale_params sp = scale(a[4], a[5]);
         at::Tensor o = none(a[6]) ? at::empty_like(v) : plain(a[6]);
-        PyObject* po = given_or_new(a[6], o);      // (before the state is updated: nothing may fail after that)
+        PyObject* po = wrap(o);      // (before the state is updated: nothing may fail after that)
         void* st = stream();
         const cott_status rc = without_gil([&] { return cott_decode_step(ptr(q), ptr(k), ptr(v), fptr(s), ptr(o), B, H, d, dt, &sp, st); });
         if (rc == COTT_OK) return po;

@@ -1,6 +1,8 @@
 """GPU parity at the sizes where a kernel or a branch of its dispatch can go wrong: edges of its
 tiles, remainders, the smallest and the largest of its range.  Oracle, metrics and gates are those
 of test_parity_gpu.py."""
+import threading
+
 import pytest
 import torch
 from torch.utils._python_dispatch import TorchDispatchMode
@@ -618,6 +620,30 @@ def test_native_binding_holds_the_lock_after_a_refused_pointer():
         with pytest.raises(RuntimeError):
             getattr(cott, name)(*args[:at], workspace=ws)
         assert getattr(cott.cott._load_native(), name)(*args) is not None
+
+
+@pytest.mark.parametrize("name", ["bwd", "bwd_stateful"])
+def test_native_binding_while_another_thread_changes_the_list(name):
+    """`out` given as a list whose items another thread replaces during the call, which runs without the
+    interpreter lock: the tensors that the gradients went to come back, whole."""
+    args = dict(_native_and_python_calls())[name][:4 + 2 * (name == "bwd_stateful") + 1]
+    want = getattr(cott, name)(*args)
+    new = lambda: [torch.empty_like(x) for x in args[:3]]
+    out, stop = new(), threading.Event()
+
+    def replace():
+        while not stop.is_set():
+            out[:] = new()
+
+    t = threading.Thread(target=replace)
+    t.start()
+    try:
+        for _ in range(300):
+            for x, y in zip(getattr(cott, name)(*args, out=out), want):
+                assert torch.equal(x, y)
+    finally:
+        stop.set()
+        t.join()
 
 
 @pytest.mark.parametrize("N", [1, 2, 7, 8, 9, 31, 64, 65, 100, 128])
