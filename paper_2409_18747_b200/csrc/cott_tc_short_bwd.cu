@@ -205,6 +205,8 @@ tc_short_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 }
                 wait(B_ED, par);
             }
+            // (lane 0 alone has waited for the staged rows and for the flag: the barrier shows them to the lanes that store)
+            __syncwarp();
             alive = __shfl_sync(0xffffffffu, alive ? 1 : 0, 0) != 0;
             if (!alive) break;
             const bool skip = pass == 0 && n_seq > 1 && *bad_flag;
@@ -346,7 +348,8 @@ tc_short_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 fence_proxy_async();
                 mbar_arrive(bars + B_R2);
             }
-            if (wait(B_OF, par)) {
+            // (the flag and the sums of the other parts of a row are there with B_R1, which is long complete)
+            if (wait(B_OF, par) && wait(B_R1, par)) {
                 const bool skip = pass == 0 && n_seq > 1 && *bad_flag;
                 if (skip) {
                     n_pass = 1 + n_seq;
