@@ -256,7 +256,7 @@ tc_short_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 const int nrow = L::kHalves == 1 ? w0 * 32 + lane : w0 * 16 + (lane & 15);
                 constexpr int kCh = D / 8 / L::kHalves;
                 const int ch0 = L::kHalves == 1 ? 0 : (lane >> 4) * kCh;
-                const uint8_t* tile = gbase + (isk ? L::kOffK : L::kOffQ);
+                uint8_t* tile = gbase + (isk ? L::kOffK : L::kOffQ);
                 float2 a0 = make_float2(0.f, 0.f), a1 = a0;
 #pragma unroll 1
                 for (int j = ch0; j < ch0 + kCh; j += 4) {
@@ -272,19 +272,22 @@ tc_short_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 }
                 float ss = (a0.x + a0.y) + (a1.x + a1.y);
                 if (L::kHalves > 1) ss += __shfl_xor_sync(0xffffffffu, ss, 16);
-                const float nrm = sqrtf(ss);
-                float r = 1.0f / fmaxf(nrm, kEps);
-                if (!(ss <= 3.4028235e38f)) {
-                    // A row too long for fp32 has r = 0 and gives and gets zeros, as if normalised in bf16 (0 in every
-                    // column); a row that is not finite has r = NaN.
+                const float nrm = sqrtf(ss), r = 1.0f / fmaxf(nrm, kEps);
+                // A row too long for fp32 has r = 0, that is a unit row of zeros, and its scores may be infinite: it
+                // becomes zeros here, so that they are 0 as well.  (A row that is not finite stays.)
+                const uint32_t too_long = __ballot_sync(0xffffffffu, !(ss <= 3.4028235e38f));
+                if (too_long >> lane & 1) {
                     bool finite = true;
 #pragma unroll 1
-                    for (int j = 0; j < D / 8; ++j) {
+                    for (int j = ch0; j < ch0 + kCh; ++j) {
                         const uint4 w = *reinterpret_cast<const uint4*>(tile + (j >> 3) * 16384 + swz(nrow, j & 7));
                         for (uint32_t x : {w.x, w.y, w.z, w.w})
                             finite = finite && (x & 0x7f80u) != 0x7f80u && (x & 0x7f800000u) != 0x7f800000u;
                     }
-                    r = finite ? 0.f : __int_as_float(0x7fc00000);
+                    if (L::kHalves > 1) finite = __shfl_xor_sync(too_long, finite ? 1 : 0, 16) && finite;
+#pragma unroll 1
+                    for (int j = ch0; j < ch0 + kCh && finite; ++j)
+                        *reinterpret_cast<uint4*>(tile + (j >> 3) * 16384 + swz(nrow, j & 7)) = make_uint4(0, 0, 0, 0);
                 }
                 if (ch0 == 0) (isk ? rk_buf : rq_buf)[nrow] = nrm > kEps ? r : -r;
                 fence_proxy_async();
@@ -314,8 +317,7 @@ tc_short_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                         const float2 rk = *reinterpret_cast<const float2*>(&rk_buf[ja]);
                         const float sa = rq * fabsf(rk.x), sb = rq * fabsf(rk.y);
                         const bool ka = ja >= lo && ja <= hi, kb = jb >= lo && jb <= hi;
-                        // (a scale of 0 is that of a row too long for fp32, whose score may be infinite)
-                        const float pa = ka && sa != 0.f ? x[i].x * sa : 0.f, pb = kb && sb != 0.f ? x[i].y * sb : 0.f;
+                        const float pa = ka ? x[i].x * sa : 0.f, pb = kb ? x[i].y * sb : 0.f;
                         const float ga = ka ? g[i].x : 0.f, gb = kb ? g[i].y : 0.f;
                         t_sum = fmaf(pa, ga, t_sum);
                         t_sum = fmaf(pb, gb, t_sum);
