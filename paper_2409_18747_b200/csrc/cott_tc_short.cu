@@ -180,9 +180,9 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             go = ok;
         }
         if (SLOTS) {
-            // (lane 0 alone has waited for the staged rows and for the flag: the barrier shows them to the lanes that store)
-            __syncwarp();
             if (!__shfl_sync(0xffffffffu, go ? 1 : 0, 0)) break;
+            // (long complete: the staged rows and the flag, which lane 0 alone has waited for, are shown to the lanes that store)
+            if (!wait_or_abort(bars + B_EDONE, par, abort_flag)) break;
             if (pass == 0 && n_seq > 1 && *bad_flag) {
                 n_pass = 1 + n_seq;
             } else {

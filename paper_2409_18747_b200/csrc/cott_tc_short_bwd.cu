@@ -205,10 +205,9 @@ tc_short_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 }
                 wait(B_ED, par);
             }
-            // (lane 0 alone has waited for the staged rows and for the flag: the barrier shows them to the lanes that store)
-            __syncwarp();
             alive = __shfl_sync(0xffffffffu, alive ? 1 : 0, 0) != 0;
-            if (!alive) break;
+            // (long complete: the staged rows and the flag, which lane 0 alone has waited for, are shown to the lanes that store)
+            if (!alive || !wait(B_ED, par)) break;
             const bool skip = pass == 0 && n_seq > 1 && *bad_flag;
             if (skip) {
                 n_pass = 1 + n_seq;
