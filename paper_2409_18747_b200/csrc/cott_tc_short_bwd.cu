@@ -228,15 +228,22 @@ tc_short_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             // -------------------------------------------------------------- row workers
             const int q4 = warp & 3, part = warp >> 2, row = q4 * 32 + lane;
             const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
-            // Rows that no copy writes are zeroed, the four tiles by the threads of the row.
+            // norms: the first half of the warps the rows of q, the second those of k, kHalves threads (lanes l and
+            // l ^ 16) a row
+            const int w0 = warp % (NW / 2), isk = warp / (NW / 2);
+            const int nrow = L::kHalves == 1 ? w0 * 32 + lane : w0 * 16 + (lane & 15);
+            constexpr int kCh = D / 8 / L::kHalves;
+            const int ch0 = L::kHalves == 1 ? 0 : (lane >> 4) * kCh;
+            // Rows that no copy writes are zeroed: in q or k by the threads that take their norm, which so read what they
+            // wrote themselves, and in v or dO alike.
             // (After the first pass: once the copies are on their way, behind which the rows before them have left.)
             if (pass > 0 && !wait(B_FULL, par)) break;
-            if (row < s0 * p.slot || row >= s1 * p.slot) {
+            if (nrow < s0 * p.slot || nrow >= s1 * p.slot) {
 #pragma unroll 1
-                for (int t = part; t < 4; t += L::kParts)
+                for (int t = isk; t < 4; t += 2)
 #pragma unroll 1
-                    for (int j = 0; j < D / 8; ++j)
-                        *reinterpret_cast<uint4*>(gbase + t * L::kTile + (j >> 3) * 16384 + swz(row, j & 7)) = make_uint4(0, 0, 0, 0);
+                    for (int j = ch0; j < ch0 + kCh; ++j)
+                        *reinterpret_cast<uint4*>(gbase + t * L::kTile + (j >> 3) * 16384 + swz(nrow, j & 7)) = make_uint4(0, 0, 0, 0);
             }
             // the row's sequence: (b, h), factor, first and last column it keeps
             const int seq = row / p.slot, tok = row - seq * p.slot, pair = pair0 + seq;
@@ -248,13 +255,7 @@ tc_short_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 cfac = stab_factor(p.m[pair - b * p.H], s_b);
             }
             const int lo = seq * p.slot, hi = live ? (p.causal ? row : lo + p.N - 1) : -1;
-            // norms: the first half of the warps the rows of q, the second those of k, kHalves threads (lanes l and
-            // l ^ 16) a row
             if (wait(B_FULL, par)) {
-                const int w0 = warp % (NW / 2), isk = warp / (NW / 2);
-                const int nrow = L::kHalves == 1 ? w0 * 32 + lane : w0 * 16 + (lane & 15);
-                constexpr int kCh = D / 8 / L::kHalves;
-                const int ch0 = L::kHalves == 1 ? 0 : (lane >> 4) * kCh;
                 uint8_t* tile = gbase + (isk ? L::kOffK : L::kOffQ);
                 float2 a0 = make_float2(0.f, 0.f), a1 = a0;
 #pragma unroll 1
@@ -358,7 +359,7 @@ tc_short_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 } else {
                     tc_fence_after();
                     // ---- dq (first half of the warps), dk (second half), kHalves threads a row; over the raw row
-                    const int isk = part / L::kHalves, half = part % L::kHalves;
+                    const int half = part % L::kHalves;
                     constexpr int kEc = D / L::kHalves;                       // columns of a thread
                     uint8_t* tile = gbase + (isk ? L::kOffK : L::kOffQ);
                     const uint32_t tacc = tmem + lane_base + (isk ? L::colB : L::colA);
