@@ -55,12 +55,16 @@ struct ShortParams {
     int wait_limit_kcycles;
 };
 
-template <int D, bool SLOTS>
+// What a tile holds: one sequence of dense tensors, several, or sequences in places of their own (SLOTS above).
+enum Tile { ONE, SEVERAL, PLACES };
+
+template <int D, Tile TILE>
 __global__ void __launch_bounds__(kThreads, SL<D>::kCtas)
 tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, ShortParams p) {
     using L = SL<D>;
     constexpr int NH = D / 64;
+    constexpr bool SLOTS = TILE == PLACES;
     // Tensor-memory columns, D = 128: scores, later the output accumulator 0..127 | masked bf16 scores 128..191.
     // D = 64: scores 0..127, then masked bf16 scores 0..63 | output accumulator 64..127.
     constexpr uint32_t colP = 0, colPt = D == 64 ? 0 : 128, colO = D == 64 ? 64 : 0;
@@ -78,7 +82,7 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const bool is_ctrl = warp == kWorkerWarps;
     const int row0 = (int)blockIdx.x * p.seqs_per_tile * p.N; // dense: first row of the tile in the list of B H N rows
     const int pair0 = (int)blockIdx.x * p.seqs_per_tile;
-    const int n_seq = SLOTS ? min(p.seqs_per_tile, p.BH - pair0) : p.seqs_per_tile;
+    const int n_seq = SLOTS ? min(p.seqs_per_tile, p.BH - pair0) : TILE == ONE ? 1 : p.seqs_per_tile;
 
     if (is_ctrl) {
         tmem_alloc(tmem_slot, L::kTmemCols);
@@ -113,9 +117,9 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // SLOTS: a pass takes the sequences s0 .. s1 - 1 of the tile: all of them, once.  Sequences that share a tile
     // meet in the second product as zeros times each other's v rows, which is no zero where a row is not finite:
     // then (some output is not finite) the first pass is not stored and every sequence gets a pass of its own.
-    // (Dense tensors: one pass, as the rows of all sequences are one copy.)
+    // (Dense tensors, where one copy brings the rows of all sequences: one pass, and the second product again below.)
     int n_pass = 1;
-    for (int pass = 0; pass < n_pass; ++pass) {
+    for (int pass = 0; pass < (SLOTS ? n_pass : 1); ++pass) {
     const uint32_t par = (uint32_t)(pass & 1);
     const int s0 = pass == 0 ? 0 : pass - 1, s1 = pass == 0 ? n_seq : pass;
     if (is_ctrl) {
@@ -170,7 +174,7 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 tc_commit(bars + B_OFULL);
                 ok = wait_or_abort(bars + B_EDONE, par, abort_flag);
             }
-            if (ok && !SLOTS) {
+            if (ok && !SLOTS && !(TILE == SEVERAL && *bad_flag)) {
 #pragma unroll
                 for (int hh = 0; hh < NH; ++hh)
                     if (hh * 64 < p.d_out) tma_store_4d(&tmO, base + L::kOffQ + hh * 16384, hh * 64, row0, 0, 0);
@@ -306,9 +310,15 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 uint32_t a[32];
                 tmem_ld32(tmem + lane_base + colO + c0, a);
                 tmem_wait_ld();
-                if (SLOTS) {
+                if (TILE != ONE) {
+                    const float2 zero = make_float2(0.f, 0.f);
+                    float2 f0 = zero, f1 = zero;
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) finite = fmaf(__uint_as_float(a[j]), 0.f, finite);
+                    for (int j = 0; j < 32; j += 4) {
+                        f0 = __ffma2_rn(make_float2(__uint_as_float(a[j]), __uint_as_float(a[j + 1])), zero, f0);
+                        f1 = __ffma2_rn(make_float2(__uint_as_float(a[j + 2]), __uint_as_float(a[j + 3])), zero, f1);
+                    }
+                    finite += (f0.x + f0.y) + (f1.x + f1.y);
                 }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -321,7 +331,7 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     *reinterpret_cast<uint4*>(gbase + L::kOffQ + (ch >> 3) * 16384u + swz(row, ch & 7)) = o;
                 }
             }
-            if (SLOTS && !(finite == 0.f)) *bad_flag = 1;
+            if (TILE != ONE && !(finite == 0.f)) *bad_flag = 1;
             fence_proxy_async();
             tc_fence_before();
             mbar_arrive(bars + B_EDONE);
@@ -335,6 +345,69 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     if (SLOTS && is_ctrl) tma_store_wait_all0();
     tc_fence_before();
     __syncthreads();
+    if (TILE == SEVERAL && *bad_flag && !*abort_flag) {
+        // The tile has not been stored: one sequence after the other, the masked scores, in tensor memory still, times
+        // v with the rows of the other sequences zeroed.  (FULL and OFULL have completed one phase.)
+        const int q4 = warp & 3, hf = warp >> 2, row = q4 * 32 + lane, pair = pair0 + row / p.N;
+        bool ok = true;
+        for (int sq = 0; sq < n_seq; ++sq) {
+            const uint32_t par = (uint32_t)(~sq & 1);
+            const int r0 = sq * p.N, r1 = r0 + p.N;
+            if (is_ctrl && lane == 0) {
+                mbar_expect_tx(bars + B_FULL, NH * (uint32_t)(n_seq * p.N) * 128u);
+                for (int hh = 0; hh < NH; ++hh) tma_load_4d(base + L::kOffV + hh * 16384, &tmV, bars + B_FULL, hh * 64, row0, 0, 0);
+            }
+            ok = wait_or_abort(bars + B_FULL, par, abort_flag);
+            if (!is_ctrl && (row < r0 || row >= r1))
+                for (int ch = hf * 4 * NH; ch < (hf + 1) * 4 * NH; ++ch)
+                    *reinterpret_cast<uint4*>(gbase + L::kOffV + (ch >> 3) * 16384u + swz(row, ch & 7)) = make_uint4(0, 0, 0, 0);
+            fence_proxy_async();
+            if (__syncthreads_or(!ok)) { ok = false; break; }
+            if (is_ctrl && lane == 0) {
+                tc_fence_after();
+                constexpr uint32_t idesc = instr_desc_bf16(128, D, false, true);
+                const uint32_t bl = smem_desc_lo(base + L::kOffV, 16384);
+                for (int kk = 0; kk < kRows / 16; ++kk)
+                    mma_ts_w(tmem + colO, tmem + colPt + kk * 8u, bl + kk * 128u, kDescHi, idesc, kk > 0);
+                tc_commit(bars + B_OFULL);
+            }
+            ok = wait_or_abort(bars + B_OFULL, par, abort_flag);
+            tc_fence_after();
+            if (!is_ctrl) {
+                float rx = 0.f;
+                if (row >= r0 && row < r1 && pair < p.BH) {
+                    const int b = pair / p.H;
+                    const float s_b = p.seq_len ? p.seq_len[b] : (p.seq_len_scalar > 0.f ? p.seq_len_scalar : (float)p.N);
+                    rx = stab_factor(p.m[pair - b * p.H], s_b) * reinterpret_cast<const float*>(gbase + L::kOffCtl + L::kOffRx)[row];
+                }
+#pragma unroll 1
+                for (int pc = 0; pc < D / 32; ++pc) {
+                    const int c0 = hf * (D / 2) + pc * 16;
+                    float a[16];
+                    __syncwarp();
+                    tmem_ld16(tmem + ((uint32_t)(q4 * 32) << 16) + colO + c0, reinterpret_cast<uint32_t*>(a));
+                    tmem_wait_ld();
+                    uint4 o[2];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) reinterpret_cast<uint32_t*>(o)[j] = pack_bf16(a[2 * j] * rx, a[2 * j + 1] * rx);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+                        if (row >= r0 && row < r1)
+                            *reinterpret_cast<uint4*>(gbase + L::kOffQ + (c0 >> 6) * 16384u + swz(row, ((c0 & 63) >> 3) + j)) = o[j];
+                }
+            }
+            fence_proxy_async();
+            tc_fence_before();
+            if (__syncthreads_or(!ok)) { ok = false; break; }
+        }
+        if (ok && is_ctrl && lane == 0) {
+            for (int hh = 0; hh < NH; ++hh)
+                if (hh * 64 < p.d_out) tma_store_4d(&tmO, base + L::kOffQ + hh * 16384, hh * 64, row0, 0, 0);
+            tma_store_commit();
+            tma_store_wait_all0();
+        }
+        __syncthreads();
+    }
     if (*abort_flag) {
         // A wait gave up: let the copies and products in flight land, then report where.
         for (int i = 0; i < 100; ++i) __nanosleep(1000);
@@ -347,9 +420,9 @@ tc_short_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     if (is_ctrl) tmem_dealloc(tmem, L::kTmemCols);
 }
 
-template <int D, bool SLOTS>
+template <int D, Tile TILE>
 cudaError_t launch_d(const CUtensorMap* tm, const ShortParams& p, int tiles, cudaStream_t st) {
-    auto kern = tc_short_fwd_kernel<D, SLOTS>;
+    auto kern = tc_short_fwd_kernel<D, TILE>;
     if (cudaError_t e = configure_smem_once(reinterpret_cast<const void*>(kern), SL<D>::kDynBytes); e != cudaSuccess)
         return e;
     const int prof = profile_begin_launch(5, st);
@@ -394,8 +467,9 @@ cudaError_t launch_tc_short_fwd(const void* q, const void* k, const void* v, voi
         p.head_first_mask |= (hf ? 1 : 0) << i;
     }
     const int tiles = (p.BH + p.seqs_per_tile - 1) / p.seqs_per_tile;
-    if (d == 64) return dense ? launch_d<64, false>(tm, p, tiles, st) : launch_d<64, true>(tm, p, tiles, st);
-    return dense ? launch_d<128, false>(tm, p, tiles, st) : launch_d<128, true>(tm, p, tiles, st);
+    if (!dense) return d == 64 ? launch_d<64, PLACES>(tm, p, tiles, st) : launch_d<128, PLACES>(tm, p, tiles, st);
+    if (p.seqs_per_tile > 1) return d == 64 ? launch_d<64, SEVERAL>(tm, p, tiles, st) : launch_d<128, SEVERAL>(tm, p, tiles, st);
+    return d == 64 ? launch_d<64, ONE>(tm, p, tiles, st) : launch_d<128, ONE>(tm, p, tiles, st);
 }
 
 }  // namespace cott

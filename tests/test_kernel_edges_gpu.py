@@ -673,15 +673,28 @@ def test_short_forward_memory_orders(N, dk, dv, causal):
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("bad", [float("nan"), float("inf")])
 @pytest.mark.parametrize("which", ["q", "k", "v"])
-def test_short_forward_keeps_sequences_apart(d, bad, which):
-    """A row that is not finite in one sequence of a tile of five: the others get the bits that they get without it."""
-    B, H, N = 60, 5, 20
+@pytest.mark.parametrize("layout", ["dense", "bnhd"])
+@pytest.mark.parametrize("N", [1, 20, 64])
+def test_short_forward_keeps_sequences_apart(N, layout, d, bad, which):
+    """Rows that are not finite in the last two sequences, which share a tile (with up to 42 more; in places of
+    whole eights of rows with up to ten): every other sequence gets the bits that it gets without them, and each of
+    the two those that it gets without the other."""
+    B, H = 60, 5
     c = synth.make_qkv(B, H, N, d, torch.bfloat16, 8800 + d)
     m = dev(c["m"])
-    ref = cott.fwd(*(_laid_out(c[x], "bnhd") for x in ("q", "k", "v")), m)
-    c[which][0, 2, 3] = bad
-    got = cott.fwd(*(_laid_out(c[x], "bnhd") for x in ("q", "k", "v")), m)
+    rows = [(B - 1, H - 2, 0), (B - 1, H - 1, N - 1)]
+
+    def call(which_rows):
+        x = {n: y.clone() for n, y in c.items()}
+        for r in which_rows:
+            x[which][r] = bad
+        return cott.fwd(*(_laid_out(x[n], layout) for n in ("q", "k", "v")), m)
+
+    ref, got = call([]), call(rows)
     keep = torch.ones(B, H, dtype=torch.bool)
-    keep[0, 2] = False
+    for r in rows:
+        keep[r[:2]] = False
+        x, y = got[r[:2]], call([r])[r[:2]]
+        assert torch.equal(x.isnan(), y.isnan()) and torch.equal(x.nan_to_num(), y.nan_to_num())
+        assert not torch.isfinite(x.float()).all()
     assert torch.equal(got[keep], ref[keep])
-    assert not torch.isfinite(got[0, 2].float()).all()
