@@ -9,15 +9,17 @@ import concurrent.futures
 import glob
 import hashlib
 import os
+import re
 import subprocess
+import sys
 import sysconfig
+import warnings
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
 CSRC = os.path.join(_PKG, "csrc")
 OBJ = os.path.join(_PKG, "build")
 LIB = os.path.join(_PKG, "libcott.so")
-BINDING = os.path.join(_PKG, "_cott_torch.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -77,15 +79,29 @@ def build(force: bool = False, verbose: bool = False, lib: str | None = None) ->
         if res.returncode != 0:
             raise RuntimeError("nvcc failed linking libcott.so")
     if lib == LIB:
-        build_binding(force, verbose)
+        try:
+            build_binding(force, verbose)
+        except (ImportError, OSError, RuntimeError) as e:
+            warnings.warn(f"the native half of the binding was not built, calls go through ctypes: {e}")
     return lib
+
+
+def binding_path() -> str:
+    """Where the native half of the Python binding lies that fits this interpreter and this torch: it is compiled
+    against the private layouts of both, so their versions are part of its name and no other one is ever loaded."""
+    import torch
+    versions = f"{sys.implementation.cache_tag}-torch{torch.__version__}-abi{int(torch._C._GLIBCXX_USE_CXX11_ABI)}"
+    return os.path.join(_PKG, f"_cott_torch.{re.sub('[^0-9A-Za-z.-]', '_', versions)}.so")
 
 
 def build_binding(force: bool = False, verbose: bool = False) -> str:
     """Compile ``csrc/cott_torch.cpp``, the native half of the Python binding, against torch and libcott.so."""
     src = os.path.join(CSRC, "cott_torch.cpp")
-    if not force and not _stale(BINDING, [src, os.path.join(_ROOT, "include", "cott.h")]):
-        return BINDING
+    path = binding_path()
+    if not force and not _stale(path, [src, os.path.join(_ROOT, "include", "cott.h"), os.path.abspath(__file__)]):
+        return path
+    if os.path.exists(path):
+        os.remove(path)               # (a compiler that fails leaves nothing old behind)
     import torch
     t = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
@@ -93,7 +109,7 @@ def build_binding(force: bool = False, verbose: bool = False) -> str:
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            *("-I" + p for p in (os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
                                 sysconfig.get_paths()["include"], os.path.join(cuda, "include"), os.path.join(_ROOT, "include"))),
-           src, "-o", BINDING, "-L" + os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python",
+           src, "-o", path, "-L" + os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python",
            "-L" + _PKG, "-l:libcott.so", "-Wl,-rpath,$ORIGIN"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if verbose or res.returncode != 0:
@@ -101,7 +117,7 @@ def build_binding(force: bool = False, verbose: bool = False) -> str:
         print(res.stderr)
     if res.returncode != 0:
         raise RuntimeError("the C++ compiler failed on cott_torch.cpp")
-    return BINDING
+    return path
 
 
 if __name__ == "__main__":

@@ -11,6 +11,8 @@ import ctypes
 import functools
 import importlib.util
 import os
+import types
+import warnings
 
 import torch
 
@@ -134,20 +136,26 @@ def _load():
 
 
 _native = None
-_NATIVE_PATH = os.path.join(_PKG, "_cott_torch.so")
+_NATIVE_CALLS = ("fwd", "fwd_stateful", "bwd", "bwd_stateful", "fwd_varlen", "bwd_varlen", "decode_step")
 
 
 def _load_native():
     """The native module with the plain forms of the calls below (``csrc/cott_torch.cpp``): each of its functions
-    returns None, having done nothing, for a call that is the Python code's, and an int for an error status."""
+    returns None, having done nothing, for a call that is the Python code's, and an int for an error status.
+    Where it has not been built for this interpreter and torch, every call is the Python code's."""
     global _native
     if _native is None:
         _load()
-        if not os.path.exists(_NATIVE_PATH):
-            raise RuntimeError(f"{_NATIVE_PATH} is missing: build it with `python -m paper_2409_18747_b200._build`")
-        spec = importlib.util.spec_from_file_location("_cott_torch", _NATIVE_PATH)
-        module = importlib.util.module_from_spec(spec)
-        spec.loader.exec_module(module)
+        from . import _build
+        path = _build.binding_path()
+        try:
+            spec = importlib.util.spec_from_file_location("_cott_torch", path)
+            module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(module)
+        except ImportError as e:
+            if os.path.exists(path):
+                warnings.warn(f"the native half of the binding does not load, calls go through ctypes: {e}")
+            module = types.SimpleNamespace(**{name: lambda *_: None for name in _NATIVE_CALLS})
         _native = module
     return _native
 

@@ -1,8 +1,11 @@
 """The C-ABI library loads, exports every symbol the header declares, and its host-only
 entry points behave.  No kernel is launched here (runs without a GPU)."""
+import contextlib
 import ctypes
 import os
 import re
+
+import pytest
 
 import paper_2409_18747_b200 as cott_pkg
 from paper_2409_18747_b200 import cott
@@ -256,3 +259,50 @@ def test_noalloc_is_not_refused_for_the_finer_groups_of_a_plan():
         if not os.path.exists("/dev/nvidia0"):
             assert lib.cott_fwd_noalloc(a, a, a, far, 1, BH, N, 128, 1, dt, ctypes.byref(sp), None) != -3
     assert lib.cott_fwd_noalloc(a, a, a, far, 64, 16, 8192, 128, 1, cott.BF16, ctypes.byref(sp), None) == -3
+
+
+def test_calls_go_through_ctypes_where_the_native_half_is_missing(monkeypatch, tmp_path):
+    """libcott.so alone is enough: without the native half, or with one that does not load, every call is the
+    Python code's."""
+    import torch
+    from paper_2409_18747_b200 import _build
+    q, m = torch.zeros((1, 1, 16, 64), dtype=torch.bfloat16), torch.zeros((1,))
+    broken = tmp_path / "broken.so"
+    broken.write_bytes(b"not a library")
+    for path in (tmp_path / "absent.so", broken):
+        monkeypatch.setattr(cott, "_native", None)
+        monkeypatch.setattr(_build, "binding_path", lambda: str(path))
+        with (pytest.warns(UserWarning, match="through ctypes") if path is broken else contextlib.nullcontext()):
+            assert all(getattr(cott._load_native(), name)(q) is None for name in cott._NATIVE_CALLS)
+        with pytest.raises(RuntimeError, match="CUDA tensors"):      # (the Python code's refusal)
+            cott.fwd(q, q, q, m)
+
+
+def test_library_is_built_where_the_native_half_cannot_be(monkeypatch, tmp_path):
+    """A compiler that is missing or fails on the native half: a warning, the library is there all the same, and
+    no native half of an earlier build stays behind."""
+    from paper_2409_18747_b200 import _build
+    old = tmp_path / "old.so"
+    monkeypatch.setattr(_build, "binding_path", lambda: str(old))
+    for cxx in ("/nonexistent/c++", "false"):
+        old.write_bytes(b"")
+        os.utime(old, (0, 0))                              # (older than its source)
+        monkeypatch.setenv("CXX", cxx)
+        with pytest.warns(UserWarning, match="native half"):
+            assert _build.build() == _build.LIB
+        assert not old.exists()
+
+
+def test_native_half_belongs_to_one_torch_and_interpreter(monkeypatch):
+    import sys
+    import torch
+    from paper_2409_18747_b200 import _build
+    here = _build.binding_path()
+    assert os.path.dirname(here) == os.path.dirname(_build.LIB)
+    with monkeypatch.context() as mp:
+        mp.setattr(torch, "__version__", "9.9.9")
+        assert _build.binding_path() != here
+    with monkeypatch.context() as mp:
+        mp.setattr(sys.implementation, "cache_tag", "cpython-999")
+        assert _build.binding_path() != here
+    assert _build.binding_path() == here
