@@ -95,7 +95,7 @@ def binding_path() -> str:
 
 
 def build_binding(force: bool = False, verbose: bool = False) -> str:
-    """Compile ``csrc/cott_torch.cpp``, the native half of the Python binding, against torch and libcott.so."""
+    """Compile ``csrc/cott_torch.cpp``, the native half of the Python binding, against torch."""
     src = os.path.join(CSRC, "cott_torch.cpp")
     path = binding_path()
     if not force and not _stale(path, [src, os.path.join(_ROOT, "include", "cott.h"), os.path.abspath(__file__)]):
@@ -109,8 +109,7 @@ def build_binding(force: bool = False, verbose: bool = False) -> str:
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            *("-I" + p for p in (os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
                                 sysconfig.get_paths()["include"], os.path.join(cuda, "include"), os.path.join(_ROOT, "include"))),
-           src, "-o", path, "-L" + os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python",
-           "-L" + _PKG, "-l:libcott.so", "-Wl,-rpath,$ORIGIN"]
+           src, "-o", path, "-L" + os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if verbose or res.returncode != 0:
         print(res.stdout)

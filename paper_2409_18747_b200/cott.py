@@ -145,13 +145,14 @@ def _load_native():
     Where it has not been built for this interpreter and torch, every call is the Python code's."""
     global _native
     if _native is None:
-        _load()
+        lib = _load()
         from . import _build
         path = _build.binding_path()
         try:
             spec = importlib.util.spec_from_file_location("_cott_torch", path)
             module = importlib.util.module_from_spec(spec)
             spec.loader.exec_module(module)
+            module.bind(*(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in module.entries))
         except ImportError as e:
             if os.path.exists(path):
                 warnings.warn(f"the native half of the binding does not load, calls go through ctypes: {e}")

@@ -15,9 +15,22 @@
 #include <c10/core/impl/TorchDispatchModeTLS.h>
 #include <c10/cuda/CUDAStream.h>
 #include <algorithm>
+#include <cstring>
 #include "cott.h"
 
 namespace {
+
+// The library that cott.py has loaded, whichever file that is: the module is linked against none, so that a program
+// has one copy of it, with one set of options.
+#define COTT_ENTRIES(X)                                                                                      \
+    X(cott_workspace_bytes_dkdv) X(cott_workspace_bytes_varlen) X(cott_fwd_strided) X(cott_fwd_stateful_strided)  \
+    X(cott_bwd_strided) X(cott_bwd_after_fwd) X(cott_bwd_stateful_strided) X(cott_fwd_varlen) X(cott_bwd_varlen)  \
+    X(cott_decode_step)
+struct Library {
+#define X(name) decltype(&::name) name;
+    COTT_ENTRIES(X)
+#undef X
+} lib;
 
 struct Other {};      // (thrown inside this file only: the call is left to the Python code)
 
@@ -147,7 +160,7 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         at::Tensor o = none(a[7]) ? at::Tensor() : plain(a[7]);
         if (o.defined()) layout(o);
         at::Tensor ws = none(a[8]) ? at::Tensor() : plain(a[8]);
-        const size_t need = ws.defined() ? 0 : cott_workspace_bytes_dkdv(COTT_OP_FWD, dt, B, H, N, d, d, causal);
+        const size_t need = ws.defined() ? 0 : lib.cott_workspace_bytes_dkdv(COTT_OP_FWD, dt, B, H, N, d, d, causal);
         if (need == (size_t)-1) throw Other();
         if (!o.defined()) o = at::empty_like(q);
         const Layout lo = layout(o);
@@ -155,7 +168,7 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (!ws.defined()) ws = room(need, q);
         void* st = stream();
         const cott_status rc = without_gil([&] {
-            return cott_fwd_strided(ptr(q), ptr(k), ptr(v), ptr(o), want_state ? fptr(state) : nullptr, B, H, N, d, causal, dt, lq.get(),
+            return lib.cott_fwd_strided(ptr(q), ptr(k), ptr(v), ptr(o), want_state ? fptr(state) : nullptr, B, H, N, d, causal, dt, lq.get(),
                                     lo.get(), &sp, ptr(ws), (size_t)ws.numel(), st);
         });
         if (rc != COTT_OK) return PyLong_FromLong(rc);
@@ -178,7 +191,7 @@ PyObject* fwd_stateful(PyObject*, PyObject* const* a, Py_ssize_t n) {
         at::Tensor o = none(a[7]) ? at::Tensor() : plain(a[7]);
         if (o.defined()) layout(o);
         at::Tensor ws = none(a[8]) ? at::Tensor() : plain(a[8]);
-        const size_t need = ws.defined() ? 0 : cott_workspace_bytes_dkdv(COTT_OP_FWD, dt, B, H, N, d, d, 1);
+        const size_t need = ws.defined() ? 0 : lib.cott_workspace_bytes_dkdv(COTT_OP_FWD, dt, B, H, N, d, d, 1);
         if (need == (size_t)-1) throw Other();
         if (!o.defined()) o = at::empty_like(q);
         const Layout lo = layout(o);
@@ -186,7 +199,7 @@ PyObject* fwd_stateful(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (!ws.defined()) ws = room(need, q);
         void* st = stream();
         const cott_status rc = without_gil([&] {
-            return cott_fwd_stateful_strided(ptr(q), ptr(k), ptr(v), ptr(o), state_in.defined() ? fptr(state_in) : nullptr,
+            return lib.cott_fwd_stateful_strided(ptr(q), ptr(k), ptr(v), ptr(o), state_in.defined() ? fptr(state_in) : nullptr,
                                              want_state ? fptr(state) : nullptr, B, H, N, d, dt, lq.get(), lo.get(), &sp, ptr(ws),
                                              (size_t)ws.numel(), st);
         });
@@ -213,7 +226,7 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
             layout(g[0], g[1], g[2]);
         }
         at::Tensor fws = none(a[9]) ? at::Tensor() : plain(a[9]);
-        const size_t need = ws.defined() ? 0 : cott_workspace_bytes_dkdv(COTT_OP_BWD, dt, B, H, N, d, d, causal);
+        const size_t need = ws.defined() ? 0 : lib.cott_workspace_bytes_dkdv(COTT_OP_BWD, dt, B, H, N, d, d, causal);
         if (need == (size_t)-1) throw Other();
         if (!given) for (int i = 0; i < 3; ++i) g[i] = at::empty_like(q);
         const Layout lg = layout(g[0], g[1], g[2]);
@@ -222,9 +235,9 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         void* st = stream();
         const cott_status rc = without_gil([&] {
             return fws.defined()
-                ? cott_bwd_after_fwd(ptr(q), ptr(k), ptr(v), ptr(d_o), ptr(g[0]), ptr(g[1]), ptr(g[2]), fptr(dm), B, H, N, d, causal, dt,
+                ? lib.cott_bwd_after_fwd(ptr(q), ptr(k), ptr(v), ptr(d_o), ptr(g[0]), ptr(g[1]), ptr(g[2]), fptr(dm), B, H, N, d, causal, dt,
                                      lq.get(), ld.get(), lg.get(), &sp, ptr(fws), ptr(ws), (size_t)ws.numel(), st)
-                : cott_bwd_strided(ptr(q), ptr(k), ptr(v), ptr(d_o), ptr(g[0]), ptr(g[1]), ptr(g[2]), fptr(dm), B, H, N, d, causal, dt,
+                : lib.cott_bwd_strided(ptr(q), ptr(k), ptr(v), ptr(d_o), ptr(g[0]), ptr(g[1]), ptr(g[2]), fptr(dm), B, H, N, d, causal, dt,
                                    lq.get(), ld.get(), lg.get(), &sp, ptr(ws), (size_t)ws.numel(), st);
         });
         if (rc != COTT_OK) return PyLong_FromLong(rc);
@@ -255,7 +268,7 @@ PyObject* bwd_stateful(PyObject*, PyObject* const* a, Py_ssize_t n) {
             three(a[10], g);
             layout(g[0], g[1], g[2]);
         }
-        const size_t need = ws.defined() ? 0 : cott_workspace_bytes_dkdv(COTT_OP_BWD, dt, B, H, N, d, d, 1);
+        const size_t need = ws.defined() ? 0 : lib.cott_workspace_bytes_dkdv(COTT_OP_BWD, dt, B, H, N, d, d, 1);
         if (need == (size_t)-1) throw Other();
         if (!given) { g[0] = at::empty_like(q); g[1] = at::empty_like(k); g[2] = at::empty_like(v); }
         const Layout lg = layout(g[0], g[1], g[2]);
@@ -264,7 +277,7 @@ PyObject* bwd_stateful(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (!ws.defined()) ws = room(need, q);
         void* st = stream();
         const cott_status rc = without_gil([&] {
-            return cott_bwd_stateful_strided(ptr(q), ptr(k), ptr(v), ptr(d_o), s[0].defined() ? fptr(s[0]) : nullptr,
+            return lib.cott_bwd_stateful_strided(ptr(q), ptr(k), ptr(v), ptr(d_o), s[0].defined() ? fptr(s[0]) : nullptr,
                                              s[1].defined() ? fptr(s[1]) : nullptr, ptr(g[0]), ptr(g[1]), ptr(g[2]),
                                              want ? fptr(ds) : nullptr, fptr(dm), B, H, N, d, d, dt, lq.get(), nullptr, ld.get(), lg.get(),
                                              nullptr, &sp, ptr(ws), (size_t)ws.numel(), st);
@@ -307,13 +320,13 @@ PyObject* fwd_varlen(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor &q = plain(a[0]), &k = plain(a[1]), &v = plain(a[2]), &cu = plain(a[4]);
         at::Tensor o = none(a[8]) ? at::Tensor() : plain(a[8]);
         at::Tensor ws = none(a[9]) ? at::Tensor() : plain(a[9]);
-        const size_t need = ws.defined() ? 0 : cott_workspace_bytes_varlen(COTT_OP_FWD, c.dt, c.B, c.H, c.T, c.longest, c.d, c.causal);
+        const size_t need = ws.defined() ? 0 : lib.cott_workspace_bytes_varlen(COTT_OP_FWD, c.dt, c.B, c.H, c.T, c.longest, c.d, c.causal);
         if (need == (size_t)-1) throw Other();
         if (!o.defined()) o = at::empty_like(q);
         if (!ws.defined()) ws = room(need, q);
         void* st = stream();
         const cott_status rc = without_gil([&] {
-            return cott_fwd_varlen(ptr(q), ptr(k), ptr(v), ptr(o), static_cast<const int*>(ptr(cu)), c.B, c.H, c.T, c.longest, c.d, c.causal,
+            return lib.cott_fwd_varlen(ptr(q), ptr(k), ptr(v), ptr(o), static_cast<const int*>(ptr(cu)), c.B, c.H, c.T, c.longest, c.d, c.causal,
                                    c.dt, &c.sp, ptr(ws), (size_t)ws.numel(), st);
         });
         if (rc != COTT_OK) return PyLong_FromLong(rc);
@@ -327,7 +340,7 @@ PyObject* bwd_varlen(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const PackedCall c = packed(a, 4, a[4], a[5], a[6], a[7], a[8]);
         const at::Tensor &q = plain(a[0]), &k = plain(a[1]), &v = plain(a[2]), &d_o = plain(a[3]), &cu = plain(a[5]);
         at::Tensor ws = none(a[9]) ? at::Tensor() : plain(a[9]);
-        const size_t need = ws.defined() ? 0 : cott_workspace_bytes_varlen(COTT_OP_BWD, c.dt, c.B, c.H, c.T, c.longest, c.d, c.causal);
+        const size_t need = ws.defined() ? 0 : lib.cott_workspace_bytes_varlen(COTT_OP_BWD, c.dt, c.B, c.H, c.T, c.longest, c.d, c.causal);
         if (need == (size_t)-1) throw Other();
         at::Tensor g[3];
         for (auto& x : g) x = at::empty_like(q);
@@ -335,7 +348,7 @@ PyObject* bwd_varlen(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (!ws.defined()) ws = room(need, q);
         void* st = stream();
         const cott_status rc = without_gil([&] {
-            return cott_bwd_varlen(ptr(q), ptr(k), ptr(v), ptr(d_o), ptr(g[0]), ptr(g[1]), ptr(g[2]), fptr(dm),
+            return lib.cott_bwd_varlen(ptr(q), ptr(k), ptr(v), ptr(d_o), ptr(g[0]), ptr(g[1]), ptr(g[2]), fptr(dm),
                                    static_cast<const int*>(ptr(cu)), c.B, c.H, c.T, c.longest, c.d, c.causal, c.dt, &c.sp, ptr(ws),
                                    (size_t)ws.numel(), st);
         });
@@ -356,18 +369,55 @@ PyObject* decode_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
         at::Tensor o = none(a[6]) ? at::empty_like(v) : plain(a[6]);
         PyObject* po = wrap(o);      // (before the state is updated: nothing may fail after that)
         void* st = stream();
-        const cott_status rc = without_gil([&] { return cott_decode_step(ptr(q), ptr(k), ptr(v), fptr(s), ptr(o), B, H, d, dt, &sp, st); });
+        const cott_status rc = without_gil([&] { return lib.cott_decode_step(ptr(q), ptr(k), ptr(v), fptr(s), ptr(o), B, H, d, dt, &sp, st); });
         if (rc == COTT_OK) return po;
         Py_XDECREF(po);
         return PyLong_FromLong(rc);
     });
 }
 
+// The address of a function of the library by its name, in the order of `entries`.
+const char* const entries[] = {
+#define X(name) #name,
+    COTT_ENTRIES(X)
+#undef X
+};
+constexpr Py_ssize_t kEntries = sizeof(entries) / sizeof(entries[0]);
+static_assert(sizeof(Library) == kEntries * sizeof(void*));
+PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (n != kEntries) { PyErr_SetString(PyExc_TypeError, "one address for each of `entries`"); return nullptr; }
+    void* addr[kEntries];
+    for (Py_ssize_t i = 0; i < n; ++i) {
+        addr[i] = PyLong_AsVoidPtr(a[i]);
+        if (!addr[i]) {
+            if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "a null address");
+            return nullptr;
+        }
+    }
+    memcpy(&lib, addr, sizeof(lib));
+    Py_RETURN_NONE;
+}
+
 #define FAST(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(name)), METH_FASTCALL, nullptr}
-PyMethodDef methods[] = {FAST(fwd), FAST(fwd_stateful), FAST(bwd), FAST(bwd_stateful), FAST(fwd_varlen), FAST(bwd_varlen), FAST(decode_step),
+PyMethodDef methods[] = {FAST(fwd), FAST(fwd_stateful), FAST(bwd), FAST(bwd_stateful), FAST(fwd_varlen), FAST(bwd_varlen), FAST(decode_step), FAST(bind),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_cott_torch", "Plain forms of the calls of cott.py.", -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__cott_torch(void) { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__cott_torch(void) {
+    PyObject* mod = PyModule_Create(&module);
+    if (!mod) return nullptr;
+    PyObject* names = PyTuple_New(kEntries);
+    for (Py_ssize_t i = 0; names && i < kEntries; ++i) {
+        PyObject* s = PyUnicode_FromString(entries[i]);
+        if (!s) { Py_CLEAR(names); break; }
+        PyTuple_SET_ITEM(names, i, s);
+    }
+    if (!names || PyModule_AddObject(mod, "entries", names) < 0) {
+        Py_XDECREF(names);
+        Py_DECREF(mod);
+        return nullptr;
+    }
+    return mod;
+}

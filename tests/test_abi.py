@@ -4,6 +4,9 @@ import contextlib
 import ctypes
 import os
 import re
+import shutil
+import subprocess
+import sys
 
 import pytest
 
@@ -294,7 +297,6 @@ def test_library_is_built_where_the_native_half_cannot_be(monkeypatch, tmp_path)
 
 
 def test_native_half_belongs_to_one_torch_and_interpreter(monkeypatch):
-    import sys
     import torch
     from paper_2409_18747_b200 import _build
     here = _build.binding_path()
@@ -306,3 +308,20 @@ def test_native_half_belongs_to_one_torch_and_interpreter(monkeypatch):
         mp.setattr(sys.implementation, "cache_tag", "cpython-999")
         assert _build.binding_path() != here
     assert _build.binding_path() == here
+
+
+def test_native_half_calls_the_library_that_was_loaded(tmp_path):
+    """A library that lies elsewhere (another build): the native half calls that one, and no second copy with
+    options of its own comes into the process."""
+    from paper_2409_18747_b200 import _build
+    if not os.path.exists(_build.binding_path()):
+        pytest.skip("the native half has not been built")
+    other = shutil.copy(cott_pkg.library_path(), tmp_path / "libcott_other.so")
+    code = f"""
+from paper_2409_18747_b200 import cott
+cott._LIB_PATH = {str(other)!r}
+assert len(cott._load_native().entries) >= 10
+libs = {{line.split()[-1] for line in open("/proc/self/maps") if "libcott" in line}}
+assert libs == {{{str(other)!r}}}, libs
+"""
+    subprocess.run([sys.executable, "-c", code], cwd=ROOT, check=True)
