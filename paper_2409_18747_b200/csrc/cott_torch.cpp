@@ -8,6 +8,7 @@
 // torch modes and transforms, unusual argument types, and every argument that the Python code refuses, so that
 // errors and rare forms have one implementation, there.  An error status of libcott is returned as an int.
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/utils/object_ptr.h>
 #include <torch/csrc/utils/python_arg_parser.h>
 #include <ATen/ATen.h>
 #include <ATen/PythonTorchFunctionTLS.h>
@@ -367,12 +368,10 @@ PyObject* decode_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const cott_dtype dt = dtype_of(q);
         const cott_scale_params sp = scale(a[4], a[5]);
         at::Tensor o = none(a[6]) ? at::empty_like(v) : plain(a[6]);
-        PyObject* po = wrap(o);      // (before the state is updated: nothing may fail after that)
+        THPObjectPtr po(wrap(o));    // (before the state is updated: nothing may fail after that)
         void* st = stream();
         const cott_status rc = without_gil([&] { return lib.cott_decode_step(ptr(q), ptr(k), ptr(v), fptr(s), ptr(o), B, H, d, dt, &sp, st); });
-        if (rc == COTT_OK) return po;
-        Py_XDECREF(po);
-        return PyLong_FromLong(rc);
+        return rc == COTT_OK ? po.release() : PyLong_FromLong(rc);
     });
 }
 

@@ -1,6 +1,7 @@
 """GPU parity at the sizes where a kernel or a branch of its dispatch can go wrong: edges of its
 tiles, remainders, the smallest and the largest of its range.  Oracle, metrics and gates are those
 of test_parity_gpu.py."""
+import sys
 import threading
 
 import pytest
@@ -611,8 +612,14 @@ def test_native_binding_holds_the_lock_after_a_refused_pointer():
     """torch refuses the data pointer of a workspace while the native half has the interpreter lock released: the
     lock is taken again and the Python code reports the refusal."""
     for name, args in _native_and_python_calls():
-        if name == "decode_step":
-            continue                                       # (no workspace)
+        if name == "decode_step":                          # (no workspace: the output, of which no reference stays behind)
+            out = torch.empty_like(args[2])
+            torch._C._set_throw_on_mutable_data_ptr(out)
+            before = sys.getrefcount(out)
+            with pytest.raises(RuntimeError):
+                cott.decode_step(*args[:-1], out=out)
+            assert sys.getrefcount(out) == before
+            continue
         at = {"bwd": 7, "bwd_varlen": 9, "bwd_stateful": 9, "fwd_varlen": 9}.get(name, 8)
         ws = torch.empty(1 << 24, dtype=torch.uint8, device="cuda")
         assert getattr(cott.cott._load_native(), name)(*args[:at], ws, *args[at + 1:]) is not None
