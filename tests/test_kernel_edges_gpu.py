@@ -1,6 +1,8 @@
 """GPU parity at the sizes where a kernel or a branch of its dispatch can go wrong: edges of its
 tiles, remainders, the smallest and the largest of its range.  Oracle, metrics and gates are those
 of test_parity_gpu.py."""
+import functools
+import inspect
 import sys
 import threading
 
@@ -398,15 +400,18 @@ def _laid_out(x, layout):
     return buf[:, :, 1].permute(0, 2, 1, 3)
 
 
-@pytest.mark.parametrize("N", [1, 2, 7, 8, 9, 24, 31, 64, 65, 100, 127, 128])
-@pytest.mark.parametrize("dk,dv", [(64, 64), (128, 128), (32, 32), (96, 40), (64, 128)])
-@pytest.mark.parametrize("causal", [True, False])
+def _short_cases(lengths):
+    """(N, dk, dv, causal) of calls that the kernels for at most 128 tokens take: bidirectional ones at d = 64 up to 64
+    tokens (with one sequence a tile two CTAs an SM of the one-launch bidirectional kernels are faster)."""
+    return [(N, dk, dv, causal) for causal in (True, False) for dk, dv in ((64, 64), (128, 128), (32, 32), (96, 40), (64, 128))
+            for N in lengths if causal or N <= 64 or max(dk, dv) > 64]
+
+
+@pytest.mark.parametrize("N,dk,dv,causal", _short_cases([1, 2, 7, 8, 9, 24, 31, 64, 65, 100, 127, 128]))
 def test_short_backward_tiles(N, dk, dv, causal):
     """The backward of at most 128 tokens: one to sixteen sequences a tile, places of whole eights of rows
     with and without rows to spare, a last tile that is not full, padded rows, every memory order."""
     B, H = 13, 23                                          # (enough for the rule to take this kernel)
-    if max(dk, dv) <= 64 and not causal and N > 64:
-        pytest.skip("two CTAs an SM of the one-launch bidirectional kernel are faster with one sequence a tile")
     layout = ("dense", "bnhd", "fused")[N % 3]
     c = synth.make_qkv(B, H, N, dk, torch.bfloat16, 8100 + N + dk, row_lognormal=True, with_do=True, d_v=dv)
     c["k"][0, 1, N // 2] = 0.0
@@ -432,6 +437,35 @@ def test_short_backward_tiles(N, dk, dv, causal):
     dk2 = again[1].clone(); dk2[z] = 0.0
     for x, y in zip((dq, dk_, dv_, dm), (again[0], dk2, again[2], again[3])):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("N", [1, 20, 65, 127, 128])
+@pytest.mark.parametrize("d,causal", [(64, True), (128, True), (128, False), (96, False)])
+def test_short_sequences_through_the_kernels_for_longer_ones(N, d, causal, option):
+    """short_bwd = 0 and short_fwd = 0, the way back to the kernels for longer sequences, whose walks then have one
+    chunk: the same call both ways against the definition."""
+    B, H = 13, 23
+    c = synth.make_qkv(B, H, N, d, torch.bfloat16, 8200 + N + d, with_do=True)
+    args = [_laid_out(c[x], "bnhd") for x in ("q", "k", "v", "d_o")]
+    m = dev(c["m"])
+    ref_o = oracle.fwd_quadratic(c["q"], c["k"], c["v"], c["m"], None, causal)
+    rq, rk, rv, rm = oracle.bwd_quadratic(c["q"], c["k"], c["v"], c["d_o"], c["m"], None, causal)
+    seen = []
+    for short in (0, 1):
+        option("short_bwd", short)
+        option("short_fwd", short)
+        o = cott.fwd(*args[:3], m, causal=causal)
+        dq, dk, dv, dm = cott.bwd(*args, m, causal=causal)
+        seen.append((o, dq, dk, dv))
+        if N == 1:
+            one_token_bounds((dq, dk, dv), (rq, rk, rv), c)
+            assert (dm == 0).all()
+            continue
+        for x, r in ((o, ref_o), (dq, rq), (dk, rk), (dv, rv)):
+            gate(x, r, torch.bfloat16)
+        gate_dm(dm, rm, 1e-2, dm_condition(rv, c["v"], c["m"], None), DM_COND_BF16)
+    # (other roundings: another kernel ran)
+    assert N == 1 or not all(torch.equal(x, y) for x, y in zip(*seen))
 
 
 @pytest.mark.parametrize("d", [64, 128])
@@ -485,7 +519,15 @@ def test_short_backward_rows_too_long_for_fp32(which, value, causal, N, dk, dv):
 @pytest.mark.parametrize("form", ["plain", "orders", "given", "per item", "subclass", "unequal"])
 def test_native_and_python_bindings_agree(form):
     """The native half of the binding and the Python code behind it, which takes what the native half leaves:
-    the same bits, the same strides, the tensors that were given handed back, the same refusals."""
+    the same bits, the same strides, the tensors that were given handed back, the same refusals.  The native half
+    is called by itself, so that it is seen to take what it should take and to leave the rest."""
+    native, native_takes = cott.cott._load_native(), form not in ("subclass", "unequal")
+
+    def by_native(name, *args, **kw):
+        call = inspect.signature(getattr(cott, name)).bind(*args, **kw)
+        call.apply_defaults()
+        return getattr(native, name)(*(x for key, x in call.arguments.items() if key != "stream"))
+
     B, H, N, d = 2, 3, 70, 64
     d_v = 96 if form == "unequal" else d
     order = (lambda x: _laid_out(x, "fused")) if form == "orders" else dev
@@ -517,7 +559,9 @@ def test_native_and_python_bindings_agree(form):
         rows = [x.permute(0, 2, 1, 3)[0].contiguous() for x in (q, k, v, d_o)]
         calls += [("fwd_varlen", (*rows[:3], m, cu, 50), dict(causal=False)), ("bwd_varlen", (*rows, m, cu, 50), {})]
     for name, args, kw in calls:
-        a = flat(getattr(cott, name)(*args, **kw))
+        a = by_native(name, *args, **kw)
+        assert (a is not None) == native_takes, name
+        a = flat(getattr(cott, name)(*args, **kw) if a is None else a)
         a = [x.clone(memory_format=torch.preserve_format) for x in a]
         b = flat(getattr(cott.cott, f"_{name}_any")(*args, **kw))
         assert len(a) == len(b)
@@ -528,11 +572,19 @@ def test_native_and_python_bindings_agree(form):
         assert all(x is y for x, y in zip(got, calls[3][2]["out"]))
     rows = [x[:, :, 0].contiguous() for x in (q, k, v)]
     s1, s2 = state.clone(), state.clone()
-    o1, o2 = cott.decode_step(*rows, s1, m, s), cott.cott._decode_step_any(*rows, s2, m, s)
+    o1, o2 = by_native("decode_step", *rows, s1, m, s), cott.cott._decode_step_any(*rows, s2, m, s)
+    assert (o1 is not None) == native_takes
+    o1 = cott.decode_step(*rows, s1, m, s) if o1 is None else o1
     assert torch.equal(o1, o2) and torch.equal(s1, s2)
-    for bad in (lambda f: f(q, k.transpose(2, 3), v, m), lambda f: f(q.half(), k, v, m), lambda f: f(q.cpu(), k, v, m),
-                lambda f: f(q, k, v, m.cpu()), lambda f: f(q[0], k[0], v[0], m), lambda f: f(q, k, v, m, -1.0),
-                lambda f: f(q, k, v, m, workspace=torch.empty(16, dtype=torch.uint8, device="cuda"))):
+    small = torch.empty(16, dtype=torch.uint8, device="cuda")
+    # (what the library refuses comes back from the native half as its status, what the Python code refuses as None)
+    for status, bad in ((None, lambda f: f(q, k.transpose(2, 3), v, m)), (None, lambda f: f(q.half(), k, v, m)),
+                        (None, lambda f: f(q.cpu(), k, v, m)), (None, lambda f: f(q, k, v, m.cpu())),
+                        (None, lambda f: f(q[0], k[0], v[0], m)), (torch.Tensor, lambda f: f(q, k, v, m, -1.0)),
+                        (-3, lambda f: f(q, k, v, m, workspace=small))):
+        answer = bad(functools.partial(by_native, "fwd"))
+        answer = torch.Tensor if isinstance(answer, torch.Tensor) else answer
+        assert answer == (status if native_takes else None)
         said = []
         for f in (cott.fwd, cott.cott._fwd_any):
             try:
@@ -629,6 +681,42 @@ def test_native_binding_holds_the_lock_after_a_refused_pointer():
         assert getattr(cott.cott._load_native(), name)(*args) is not None
 
 
+def test_native_binding_uses_the_current_stream():
+    """Two threads with a stream of their own as the current one: the calls run on it, behind what their inputs come
+    from there (the stream is kept busy first, and the inputs hold something else until then)."""
+    native = cott.cott._load_native()
+    calls = _native_and_python_calls()
+    want = {name: getattr(cott, name)(*(x.clone() if isinstance(x, torch.Tensor) else x for x in args)) for name, args in calls}
+    torch.cuda.synchronize()
+    said = []
+
+    def work():
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(5):
+                    for name, args in calls:
+                        late = [torch.zeros_like(x) if isinstance(x, torch.Tensor) and x.dtype != torch.int32 else x for x in args]
+                        torch.cuda.current_stream().synchronize()
+                        torch.cuda._sleep(200000)          # (0.1 ms)
+                        for x, y in zip(late, args):
+                            if x is not y:
+                                x.copy_(y)
+                        got = getattr(native, name)(*late)
+                        flat = lambda x: list(x) if isinstance(x, tuple) else [x]
+                        for x, y in zip(flat(got), flat(want[name])):
+                            assert torch.equal(x, y), name
+        except BaseException as e:
+            said.append(e)
+
+    threads = [threading.Thread(target=work) for _ in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    if said:
+        raise said[0]
+
+
 @pytest.mark.parametrize("name", ["bwd", "bwd_stateful"])
 def test_native_binding_while_another_thread_changes_the_list(name):
     """`out` given as a list whose items another thread replaces during the call, which runs without the
@@ -653,16 +741,12 @@ def test_native_binding_while_another_thread_changes_the_list(name):
         t.join()
 
 
-@pytest.mark.parametrize("N", [1, 2, 7, 8, 9, 31, 64, 65, 100, 128])
-@pytest.mark.parametrize("dk,dv", [(64, 64), (128, 128), (32, 32), (96, 40), (64, 128)])
-@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("N,dk,dv,causal", _short_cases([1, 2, 7, 8, 9, 31, 64, 65, 100, 128]))
 def test_short_forward_memory_orders(N, dk, dv, causal):
     """The forward of at most 128 tokens in memory orders that are not dense: places of whole eights of rows,
     a last tile that is not full; against the dense tensors' kernel, whose tiles hold the same rows (the
     scores and the sums over a row's own columns do not depend on where in a tile a sequence lies)."""
     B, H = 13, 23                                          # (enough for the rule to take this kernel)
-    if max(dk, dv) <= 64 and not causal and N > 64:
-        pytest.skip("the one-launch bidirectional kernel is faster with one sequence a tile")
     c = synth.make_qkv(B, H, N, dk, torch.bfloat16, 8700 + N + dk, row_lognormal=True, d_v=dv)
     c["k"][0, 1, N // 2] = 0.0
     m = dev(c["m"])

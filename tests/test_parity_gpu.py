@@ -1228,7 +1228,8 @@ def test_segment_backward_refuses_what_it_does_not_cover():
 
 
 # ------------------------------------------------------------------ a wait that runs out
-@pytest.mark.parametrize("op", ["fwd", "bwd", "bidir", "bidir_bwd", "bidir_bwd_walk", "short", "block"])
+@pytest.mark.parametrize("op", ["fwd", "bwd", "bidir", "bidir_bwd", "bidir_bwd_walk", "short", "block", "short_places",
+                                "short_bwd", "short_bwd64", "short_bwd64_two", "bwd128"])
 def test_bounded_wait_runs_out_and_reports(op, option, force_group):
     """Every device-side wait has a bound.  With the bound set to zero a wait gives up unless
     its hand-off is there within a few polls -- and the first tiles of a kernel cannot come
@@ -1237,17 +1238,22 @@ def test_bounded_wait_runs_out_and_reports(op, option, force_group):
     usable and the next call is correct.  (No GPU fault is involved: the kernels end normally.)
     One case per warp-specialised kernel: the generic walk, the fused backward (causal and
     bidirectional instance), the one-launch bidirectional backward, the bidirectional, the
-    short-sequence and the block forward."""
-    causal = op not in ("bidir", "bidir_bwd", "bidir_bwd_walk")
-    force_group(512 if causal else 4096)
+    short-sequence (dense, and in places of their own) and the block forward, the short-sequence
+    backward (its three instances) and the d = 128 backward."""
+    causal = op not in ("bidir", "bidir_bwd", "bidir_bwd_walk", "short_places", "short_bwd")
+    force_group(512 if causal and op != "bwd128" else 4096)
     if op == "bidir_bwd_walk":
         option("bidir_bwd", 0)
-    N = {"short": 64, "block": 16}.get(op, 1024)
-    c = synth.make_qkv(1, 2, N, 64, torch.bfloat16, 5400, with_do=True)
+    H, N, d = {"short": (2, 64, 64), "block": (2, 16, 64), "short_places": (2, 48, 128), "short_bwd": (2, 48, 128),
+               "short_bwd64": (150, 40, 64), "short_bwd64_two": (150, 128, 64), "bwd128": (2, 1024, 128)}.get(op, (2, 1024, 64))
+    kind = {"short": 6, "short_places": 6, "short_bwd": 9, "short_bwd64": 9, "short_bwd64_two": 9, "bwd128": 8}.get(op)
+    c = synth.make_qkv(1, H, N, d, torch.bfloat16, 5400, with_do=True)
     q, k, v, d_o, m = (dev(c[x]) for x in ("q", "k", "v", "d_o", "m"))
-    is_bwd = op in ("bwd", "bidir_bwd", "bidir_bwd_walk")
+    if op == "short_places":
+        q, k, v = (_as_bnhd(x) for x in (q, k, v))
+    is_bwd = "bwd" in op
     code = cott.cott.OP_BWD if is_bwd else cott.cott.OP_FWD
-    ws = torch.zeros(cott.workspace_bytes(code, cott.cott.BF16, 1, 2, N, 64, causal),
+    ws = torch.zeros(cott.workspace_bytes(code, cott.cott.BF16, 1, H, N, d, causal),
                      dtype=torch.uint8, device="cuda")
     state0 = torch.zeros((1, 2, 64, 64), dtype=torch.float32, device="cuda")
     if is_bwd:
@@ -1262,6 +1268,7 @@ def test_bounded_wait_runs_out_and_reports(op, option, force_group):
     words = ws[:12].view(torch.int32).cpu().numpy().view(np.uint32)
     assert words[0] == 1 and (words[1] >> 31) == 1               # where the first wait gave up
     assert ((words[1] >> 4) & 0x3FF) < 512                       # a barrier of the kernel's block
+    assert kind is None or words[2] >> 24 == kind                # the kernel that is meant
     option("wait_limit_kcycles", -1)
     out = call()
     assert cott.cott.last_async_status(ws) == 0
