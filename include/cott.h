@@ -120,7 +120,7 @@ extern volatile unsigned cott_option_changes;
  * launches and writes their durations in milliseconds to ms[] and their kind to kinds[]
  * (0 = partial-state pass, 1 = causal walk, 2 = read-out, 3 = fused backward walk (causal or
  * bidirectional), 4 = one-launch bidirectional forward, 5 = short-sequence forward, 6 = token-block
- * forward on a state, 7 = one-launch bidirectional backward; 17 = a causal walk that ran side by
+ * forward on a state, 7 = one-launch bidirectional backward, 8 = short-sequence backward; 17 = a causal walk that ran side by
  * side with a sibling walk of the same size on another stream of the library, in which case
  * its ms is half of the span the pair occupied, first start to last end); both are host
  * arrays of `cap` entries.  Returns the number of entries written, or -1 on a CUDA error.  Not thread-safe

@@ -658,9 +658,9 @@ static Bwd128Groups bwd128_groups(const Plan& p, int BH, int N, int causal, bool
     // chunk of 128 tokens a K walk takes 4.6 us and a Q walk 3.5; a walk cut in groups costs a state pass of
     // about 5 us and 0.9 us per chunk of its parts.  A single later group of the K walk leaves SMs idle in
     // its state pass: that pass is cut into up to four parts.  (Against half the plan's groups for both:
-    // B=3, H=16, N=2999 113 us / 127, B=1, H=40, N=4096 143 / 165, B=1, H=16, N=16384 224 / 254.  The chunks
-    // have since become 4.4 and 2.9 us, those calls 101, 121 and 214; with these figures in the sum below ten
-    // shapes from B H = 8 to 64 take the same time.)
+    // B=3, H=16, N=2999 113 us / 127, B=1, H=40, N=4096 143 / 165, B=1, H=16, N=16384 224 / 254.  Stamps of the
+    // present kernel on a full GPU: K chunks 4.7 to 5.1 us, Q chunks 3.2 to 3.7, and 14 us for a walk that reads four
+    // parts, which the sum below leaves out; with 4.4 and 2.9 in it ten shapes from B H = 8 to 64 take the same time.)
     const int chunks = (N + 127) / 128, slots = 148 / BH;
     double best = 1e30;
     // Of the numbers of groups with walks of one length only the least is looked at (others have the same walks
@@ -726,11 +726,6 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
         TcWalkArgs t;
         memset(&t, 0, sizeof(t));
         t.cu_seqlens = packed.cu_seqlens; t.total_tokens = packed.total_tokens;
-        // When two walks with one CTA per (b, h) fit on the GPU side by side but not two per
-        // (b, h) (74 / 2 < B*H <= 74), the dK^ and dV' streams run next to each other, each
-        // over the whole sequence as a single group (no partial-state pass, no scan), with the
-        // dQ^ stream's partial-state pass filling the SMs that are left; the dQ^ walk follows on
-        // the whole GPU.  Each side stream then carries one tensor-core kernel per call.
         // Short sequences: the quadratic form, several sequences per tile, one launch (cott_tc_short_bwd.cu), where
         // the kernels for longer ones, a CTA or two per (b, h), need more than a wave.  One call behind the
         // other, BH x N: causal d = 64 (one CTA a (b, h) and SM) 140 x 100 13.2 us against their 11.6, 228 x 79
@@ -823,6 +818,11 @@ static cott_status bwd_impl(const void* q, const void* k, const void* v, const v
             COTT_CUDA(launch_tc_bwd_fused(f, B, H, N, st));
             return COTT_OK;
         }
+        // When two walks with one CTA per (b, h) fit on the GPU side by side but not two per
+        // (b, h) (74 / 2 < B*H <= 74), the dK^ and dV' streams run next to each other, each
+        // over the whole sequence as a single group (no partial-state pass, no scan), with the
+        // dQ^ stream's partial-state pass filling the SMs that are left; the dQ^ walk follows on
+        // the whole GPU.  Each side stream then carries one tensor-core kernel per call.
         SideStreams* ss = nullptr;
         Plan pp = p;                       // plan of the two side-by-side streams
         // (d = 64 only: at d = 128 two such walks running at the same time once ended in launch

@@ -11,10 +11,15 @@
 // tiles in flight at this head size, so dQ, whose sum runs the other way, has CTAs of its own.  With
 // an all-ones mask (BIDIR) both sums are totals and only the products with them remain.
 //
-// What bounds it: the chain of one chunk (scores, mask, products, epilogue, state copy) on one SM, not
-// memory: two (b, h) on an idle GPU take as long a chunk as 64.  A K chunk takes 8400 cycles and a Q chunk
-// 5400; the products alone would keep the tensor core busy for 3600 and 2100, and shared memory (operands
-// of the products, tiles in and out, the workers' passes) for 6600 and 4900.
+// What bounds it: the chain of one chunk (scores, mask, products, epilogue, state copy) on one SM, stretched
+// where the other SMs load and store as well.  Stamps of every CTA, mean of a walk's chunks: K 4.3 us and Q 2.75
+// with two (b, h) on an idle GPU, K 5.1 and Q 3.7 with 64 (N=2048), K 4.8 and Q 3.3 at B=3, H=16, N=2999, K 5.0 and
+// Q 3.4 in 32 packed sequences.  The products alone would keep the tensor core busy for 1.8 and 1.1 us, and shared
+// memory (operands of the products, tiles in and out, the workers' passes) for 3.4 and 2.5.
+// Around its chunks a CTA spends 2 to 5 us until the first tile has landed and 2 us on dm and the exit, a walk that
+// sums four partial states 14 us more in reading them (a row a lane, uncoalesced), and the call 7 us on its launches.
+// So B=4, H=16, N=2048, one wave of 16 K chunks: 5 + 16 x 5.1 + 2 = 89 us of the kernel's 91; B=3, H=16, N=2999: 12 us
+// until the state pass is over and read, 24 Q chunks of 3.3, 2 = 93 of 97.
 // Measured, L2 cold: B=4, H=16, N=2048 99 us; B=3, H=16, N=2999 112 us; 32 packed sequences of 512 to
 // 2048 tokens, H=16, 378 us; B=10, H=12, N=5349, d=96 411 us.  With one slot for P in the Q walk and three
 // pairs of slots that took turns in the K walk, where every chunk waited for rows on their way out, and
@@ -73,16 +78,23 @@ struct Bwd128Params {
 };
 
 #ifdef COTT_TIMING
-// Debug build only: SM-clock stamps of CTAs 0 (K walk) and 1 (Q walk), first 16 chunks, eight slots for each of
-// six roles (0, 1: first thread of worker groups A, B; 2-5: score, product, state, copy threads).
-__device__ long long g_b128_stamps[2 * 6 * 16 * 8];
+// Debug build only.  SM-clock stamps of the first K walk (0) and the first Q walk (1) of (b, h) 0, found by what they do
+// and not by their place in the grid: up to 64 chunks, eight slots for each of six roles (0, 1: first thread of worker
+// groups A, B; 2-5: score, product, state, copy threads).  Nanosecond stamps of every CTA: start, wait for the kernel before
+// it over, first state written, first tile landed, last chunk done, exit.
+__device__ long long g_b128_stamps[2 * 6 * 64 * 8];
+__device__ long long g_b128_cta[8192 * 6];
+__device__ __forceinline__ long long global_ns() { long long t; asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t)); return t; }
 #define STAMP(role, c, slot)                                                                                 \
     do {                                                                                                     \
-        if (blockIdx.x < 2 && (c) < 16 && ((role) > 1 || threadIdx.x == ((role) ? kGroupA : 96)))                       \
-            g_b128_stamps[((blockIdx.x * 6 + (role)) * 16 + (c)) * 8 + (slot)] = clock64();                  \
+        if (bh == 0 && g == 0 && (c) < 64 && ((role) > 1 || threadIdx.x == ((role) ? kGroupA : 0)))          \
+            g_b128_stamps[(((kw ? 0 : 1) * 6 + (role)) * 64 + (c)) * 8 + (slot)] = clock64();                \
     } while (0)
+#define CTA_STAMP(thread, slot)                                                                              \
+    do { if (threadIdx.x == (thread) && blockIdx.x < 8192) g_b128_cta[blockIdx.x * 6 + (slot)] = global_ns(); } while (0)
 #else
 #define STAMP(role, c, slot) do { } while (0)
+#define CTA_STAMP(thread, slot) do { } while (0)
 #endif
 
 // tcgen05.mma chains (one thread).  K step kk of a K-major operand of 128 columns; of an MN-major
@@ -131,7 +143,8 @@ __device__ __forceinline__ void issue_update(uint32_t tS, uint32_t a, uint32_t b
 // Loops are kept rolled: five roles run different code on one SM, and with everything unrolled they
 // ran out of the instruction caches (ncu: 8.7 warps per issue stalled on "no instruction" against
 // 2.7 with the 16-column loops of the epilogues rolled: 141 us against 120 for B=4, H=16, N=2048;
-// rolling the product chains, the row norms and the two masks took the same case from 113 to 93).
+// rolling the product chains, the row norms and the two masks took the same case from 113 to 93; figures of
+// those steps, measured another way than the ones above).
 // Which walk a CTA runs is a compile-time property of its code (KW).
 template <bool KW, bool BIDIR, bool VARLEN>
 __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
@@ -160,6 +173,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
     float* dm_red = reinterpret_cast<float*>(gbase + L::kOffCtl + L::kOffDmRed);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    CTA_STAMP(0, 0);
     if (base & 1023u) {
         if (tid == 0 && atomicCAS(p.status, 0, 1) == 0) {
             p.status[1] = (int)0x80007FF0u;
@@ -240,6 +254,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    CTA_STAMP(0, 1);
 
     const float s_b = p.seq_len ? p.seq_len[bseq]
                                 : (p.seq_len_scalar > 0.f ? p.seq_len_scalar : (float)(VARLEN ? max(seq1 - seq0, 1) : p.N));
@@ -287,6 +302,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
     __syncthreads();
     tc_fence_after();
 
+    CTA_STAMP(0, 2);
     float dm_acc = 0.f;
     if (is_copy) {
         // ------------------------------------------------------------------ copy thread
@@ -389,6 +405,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
                 const bool acc = BIDIR || init_state || c > 0;
                 const uint32_t tO = tmem + (!kw && (c & 1) ? colSC2 : colO1);
                 if (!wait_or_abort(bar(B_FX, c), par(c), abort_flag)) break;
+                if (c == 0) CTA_STAMP((kWorkerWarps + 1) * 32, 3);
                 if (c >= 1 && !BIDIR && !wait_or_abort(bar(B_CP, c - 1), par(c - 1), abort_flag)) break;
                 STAMP(3, c, 0);
                 // the accumulator has been drained: one in the K walk, two in turn in the Q walk
@@ -646,6 +663,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
                 mbar_arrive(bar(B_E1, c));
                 STAMP(1, c, 5);
             }
+            CTA_STAMP(kGroupA, 4);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) dm_acc += __shfl_xor_sync(0xffffffffu, dm_acc, o);
             if (lane == 0) dm_red[w8] = dm_acc;
@@ -700,6 +718,7 @@ __device__ __forceinline__ void walk(const CUtensorMap& tmQ, const CUtensorMap& 
         }
     }
     if (is_score) tmem_dealloc(tmem, 512);
+    CTA_STAMP(0, 5);
 }
 
 template <bool BIDIR, bool VARLEN>
@@ -770,5 +789,8 @@ cudaError_t launch_tc_bwd128(const TcBwdFusedArgs& a, const Bwd128Groups& g, flo
 #ifdef COTT_TIMING
 extern "C" int cott_debug_b128_stamps(long long* out) {
     return (int)cudaMemcpyFromSymbol(out, cott::g_b128_stamps, sizeof(cott::g_b128_stamps));
+}
+extern "C" int cott_debug_b128_ctas(long long* out) {
+    return (int)cudaMemcpyFromSymbol(out, cott::g_b128_cta, sizeof(cott::g_b128_cta));
 }
 #endif

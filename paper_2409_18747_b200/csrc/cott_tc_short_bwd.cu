@@ -12,7 +12,7 @@
 // the element-wise product of the two score matrices, fp32.
 //
 // One CTA per tile: 16 warps of row workers (a quarter of a row's scores each, half of a row of dq or dk)
-// and one warp for copies and products; where the tiles of D = 64 are more than one wave, eight, with 97 KB and
+// and one warp for copies and products; where the tiles of D = 64 are more than one wave, eight, with 99.5 KB and
 // 256 tensor-memory columns, so that two CTAs share an SM.  D = 64 keeps P and G in one buffer in turn, D = 128
 // has one for each.  Bound by the chain of one tile (tiles land, norms, scores, masks, products, epilogues,
 // rows out), which is most of the 12 to 16 us of a call of one wave.  Against the kernels for longer
@@ -49,6 +49,7 @@ struct SBL {
     static constexpr int kOffLast = 480, kOffBad = 484;
     static constexpr int kDynBytes = kOffCtl + kOffX + (kHalves > 1 ? 2048 : 0) + 1024;
     static constexpr int kTmemCols = D == 64 ? 256 : 512;
+    static_assert(NW != 8 || (2 * (kDynBytes + 1024) <= 228 * 1024 && 2 * kTmemCols <= 512), "two CTAs an SM");
     // accumulators: scores P 0-127, G 128-255; D = 64: dV' over P (0-63), a 64-127, b 128-191; D = 128: dV' 256, a 384, b 0
     static constexpr uint32_t colP = 0, colG = 128, colV = D == 64 ? 0 : 256, colA = D == 64 ? 64 : 384, colB = D == 64 ? 128 : 0;
 };

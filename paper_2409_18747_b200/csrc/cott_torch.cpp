@@ -5,7 +5,7 @@
 //
 // Every function does exactly what the Python code behind it in cott.py does for the forms it knows, and
 // returns None -- before anything has been allocated or launched -- for all others: tensor subclasses, active
-// torch modes and transforms, unusual argument types, and every argument that the Python code refuses, so that
+// torch modes, levels of torch.func, unusual argument types, and every argument that the Python code refuses, so that
 // errors and rare forms have one implementation, there.  An error status of libcott is returned as an int.
 #include <torch/csrc/autograd/python_variable.h>
 #include <torch/csrc/utils/object_ptr.h>
